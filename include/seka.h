@@ -13,8 +13,7 @@
  *  - Pointers are DEVICE pointers unless the name starts with `h_`. The caller owns
  *    every buffer; the library keeps none and allocates no device memory.  Process state it
  *    does keep: the launch counter of seka_launch_count (atomic), the SM count of each
- *    device it has been called on, the driver entry point for tensor maps, the per-device
- *    address of the built-in scratch of seka_edit_keys_static, and eight events per device
+ *    device it has been called on, the driver entry point for tensor maps, and eight events per device
  *    that order the staging buffer of seka_attention_fwd_host between calls (all behind
  *    mutexes; calls may come from several host threads and for several devices).
  *  - Tensors are packed token-major: Q [T, Hq, d], K and V [T, Hkv, d], O [T, Hq, d],
@@ -80,7 +79,7 @@ size_t seka_workspace_bytes(const seka_shape* shape);
  * for highlighted tokens t of enabled heads h; every other row of K_out equals K_in
  * bit for bit.  K_out may alias K_in (in place: only edited rows are written).
  * fp32 tensors are edited in fp32 arithmetic; bf16 tensors accumulate in fp32 and round
- * once.  Uses `workspace` for the compacted list of highlighted tokens.
+ * once.  Uses `workspace` for the list of highlighted tiles.
  */
 seka_status seka_edit_keys(const seka_shape* shape, const void* K_in, void* K_out,
                            const uint8_t* mask, const float* U, const float* alpha,
@@ -168,27 +167,18 @@ seka_status seka_attention_fwd_host(const seka_shape* shape, const void* h_Q, co
  * Some hosts of this library may not call cudaMalloc at the point where the key cache has to be
  * edited: an inference server that hands its whole memory budget to a pre-sized KV-cache pool at
  * start-up, a plug-in that runs inside another framework's stream callback, or code that has
- * already frozen its allocator.  seka_edit_keys needs a scratch buffer (the compacted list of
- * highlighted tokens) that such a caller has nowhere to get.  This variant keeps that scratch in
- * a fixed array inside the library's device image instead; it takes the same tensors, minus
- * the workspace, and computes the same edit: in fp32 arithmetic with one rounding to the
- * tensor's type (for bf16 tensors seka_edit_keys uses a tensor-core kernel whose result can
- * differ from this one in the last bf16 place).
+ * already frozen its allocator.  seka_edit_keys needs a scratch buffer (the list of highlighted
+ * tokens) that such a caller has nowhere to get.  This variant takes the same tensors, minus the
+ * workspace, and computes the same edit in one launch that needs no scratch: in fp32 arithmetic
+ * with one rounding to the tensor's type (for bf16 tensors seka_edit_keys uses a tensor-core
+ * kernel whose result can differ from this one in the last bf16 place).
  *
  *  - Limit: total tokens <= SEKA_STATIC_MAX_TOKENS.  A larger shape is refused with
  *    SEKA_ERR_UNSUPPORTED before anything is launched; use seka_edit_keys with a workspace there.
- *  - Cost: every GPU that loads the library holds the array (4 * SEKA_STATIC_MAX_TOKENS + 256
- *    bytes) until the process exits, whether or not this entry point is ever called.  The
- *    kernel behind it (a warp per highlighted token, plain multiply-adds) is several times
- *    slower on large caches than the pipelined kernel of seka_edit_keys.
- *  - The call itself performs no cudaMalloc / cudaFree and uses no allocating library routine.
- *    The first call on each device looks up the array's device address (once, with that device
- *    current); make that first call outside any stream capture.
- *  - All calls on one device share the one array.  Its contents are whatever the previous call
- *    left; the call clears what it needs (the list counter) on `cuda_stream` first.  Two calls
- *    that may overlap on the GPU (different streams, or different host threads without ordering)
- *    race on the array: serialise them, or give the overlapping ones seka_edit_keys with
- *    separate workspaces.
+ *  - Cost: plain multiply-adds on every highlighted row, slower on large bf16 caches than the
+ *    tensor-core kernel of seka_edit_keys.
+ *  - The call itself performs no cudaMalloc / cudaFree and uses no allocating library routine, and
+ *    it keeps no state: calls may overlap, and may be captured into a graph from the first on.
  */
 #define SEKA_STATIC_MAX_TOKENS 262144
 seka_status seka_edit_keys_static(const seka_shape* shape, const void* K_in, void* K_out,

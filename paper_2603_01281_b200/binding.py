@@ -143,8 +143,7 @@ def seka_edit_keys(shape: SekaShape, K_in, K_out, mask, U, alpha, gain, head_ena
 
 
 def seka_edit_keys_static(shape: SekaShape, K_in, K_out, mask, U, alpha, gain, head_enable) -> None:
-    """seka_edit_keys for callers that cannot allocate: the scratch is a fixed array inside the library
-    (at most SEKA_STATIC_MAX_TOKENS tokens; calls that overlap on the GPU race on it)."""
+    """seka_edit_keys for callers that cannot allocate: one launch without scratch (at most SEKA_STATIC_MAX_TOKENS tokens)."""
     _check(load().seka_edit_keys_static(ctypes.byref(shape), _ptr(K_in), _ptr(K_out), _ptr(mask), _ptr(U),
                                         _ptr(alpha), _ptr(gain), _ptr(head_enable), _stream()),
            "seka_edit_keys_static")

@@ -1,19 +1,7 @@
 // Standalone key-editing kernel (the hook of Algorithm 1 / Algorithm 2 applied to a key tensor in HBM).
-#include <mutex>
-
 #include "seka_kernels.h"
 
 namespace seka {
-
-template <typename T> struct Elem;
-template <> struct Elem<float> {
-    static __device__ __forceinline__ float load(const float* p) { return *p; }
-    static __device__ __forceinline__ void store(float* p, float v) { *p = v; }
-};
-template <> struct Elem<__nv_bfloat16> {
-    static __device__ __forceinline__ float load(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-    static __device__ __forceinline__ void store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
-};
 
 __device__ __forceinline__ int find_sequence(const int* __restrict__ cu, int B, int L, int t) {
     if (cu == nullptr) return t / L;
@@ -25,70 +13,235 @@ __device__ __forceinline__ int find_sequence(const int* __restrict__ cu, int B, 
     return lo;
 }
 
-// One warp per (highlighted token, KV head) row, fp32 arithmetic:
-//   c = U_m^T k (lanes over the rank),  k' = k + g * sum_m alpha_m U_m c (lanes over head_dim).
-template <typename T, int D>
-__global__ void edit_rows_kernel(const T* K_in, T* K_out, const int* __restrict__ list,
-                                 const int* __restrict__ count, const float* __restrict__ U,
-                                 const float* __restrict__ alpha, const float* __restrict__ gain,
-                                 const uint8_t* __restrict__ head_enable, const int* __restrict__ cu, int B, int L,
-                                 int Hkv, int r, int M) {
-    constexpr int Q = D / 32;
-    const int lane = threadIdx.x & 31;
-    const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long items = (long long)(*count) * Hkv;
-    for (long long it = warp0; it < items; it += nwarps) {
-        const int h = (int)(it % Hkv);
-        if (head_enable != nullptr && head_enable[h] == 0) continue;
-        const int t = list[it / Hkv];
-        const int b = find_sequence(cu, B, L, t);
-        const float g = gain[b];
-        const size_t row = ((size_t)t * Hkv + h) * D;
-        float k[Q], dk[Q];
+// ---------------------------------------------------------------- fp32 arithmetic: a CTA per (64-token tile, KV head)
+//
+//   C = U_m^T k (highlighted rows x rank),  k' = k + g sum_m alpha_m U_m C,  both products as blocked fp32 multiply-adds.
+//
+// The CTA finds its highlighted rows itself (no list, no launch of its own for it), gathers them into shared memory, and
+// walks the rank 32 columns at a time: U's chunk [D x 32] is staged once for all rows of the tile, so an element of U is
+// read from global memory once per tile instead of once per row (one warp per row, everything through shuffles, was bound
+// by the latency of that chain).  With a second output tensor the rows that are not highlighted are copied in the same
+// pass, 16 bytes per lane; the loads go out before the highlight flags are known.  Bound by HBM where the copy dominates
+// (the fp32 layer of 6000 tokens x 16 heads x 64, rank 16, a tenth highlighted, into a second tensor: copy + list + a warp
+// per row 56 us per call, this 21 us), by the fp32 pipe where most rows are highlighted (4 D rank flops per row).
+constexpr int ER_ROWS = 64, ER_THREADS = 256, ER_CP = 36;     // tokens per tile; pitch (floats) of 32-column chunks: float4 reads of 8 rows meet 32 banks
+
+template <typename T> struct Row16;        // 16 bytes of a row <-> fp32 values
+template <> struct Row16<float> {
+    static constexpr int N = 4;
+    static __device__ __forceinline__ void unpack(const uint4& v, float* f) {
+        f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
+    }
+    static __device__ __forceinline__ void store4(float* dst, const float (&f)[4]) {
+        *reinterpret_cast<float4*>(dst) = make_float4(f[0], f[1], f[2], f[3]);
+    }
+};
+template <> struct Row16<__nv_bfloat16> {
+    static constexpr int N = 8;
+    static __device__ __forceinline__ void unpack(const uint4& v, float* f) {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int q = 0; q < Q; ++q) { k[q] = Elem<T>::load(K_in + row + q * 32 + lane); dk[q] = 0.f; }
+        for (int e = 0; e < 4; ++e) {
+            const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]));
+            f[2 * e] = x.x; f[2 * e + 1] = x.y;
+        }
+    }
+    static __device__ __forceinline__ void store4(__nv_bfloat16* dst, const float (&f)[4]) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]));
+    }
+};
+
+template <int D> constexpr size_t edit_rows_smem() { return sizeof(float) * (ER_ROWS * (D + 4) + D * ER_CP + ER_ROWS * ER_CP); }
+
+template <typename T, int D, bool COPY>
+__global__ void __launch_bounds__(ER_THREADS)
+edit_rows_kernel(const T* K_in, T* K_out, const uint8_t* __restrict__ mask, const float* __restrict__ U,
+                 const float* __restrict__ alpha, const float* __restrict__ gain,
+                 const uint8_t* __restrict__ head_enable, const int* __restrict__ cu, int n_tok, int B, int L,
+                 int Hkv, int r, int M, int heads_per_cta) {
+    using R = Row16<T>;
+    constexpr int KP = D + 4;                              // pitch of a key row in shared memory (16-byte aligned rows)
+    constexpr int UPR = D / R::N;                          // 16-byte units of a key row
+    constexpr int NV = ER_ROWS * UPR / ER_THREADS;         // units per thread
+    extern __shared__ __align__(16) float er_sm[];
+    float* Ks = er_sm;                                     // [64][KP]   highlighted rows, compacted
+    float* Us = Ks + ER_ROWS * KP;                         // [D][ER_CP] 32 columns of U_m
+    float* Cs = Us + D * ER_CP;                            // [64][ER_CP]
+    __shared__ int slot_of[ER_ROWS], row_of[ER_ROWS], seq_of[ER_ROWS], cnt_s[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int hgroups = (Hkv + heads_per_cta - 1) / heads_per_cta;
+    const int t0 = (int)(blockIdx.x / hgroups) * ER_ROWS, h0 = (int)(blockIdx.x % hgroups) * heads_per_cta;
+    const int h1 = h0 + heads_per_cta < Hkv ? h0 + heads_per_cta : Hkv;
+    const int n_rows = n_tok - t0 < ER_ROWS ? n_tok - t0 : ER_ROWS;
+
+    // a second tensor: the first head's rows are on their way while the flags are looked up
+    uint4 v[NV];
+    auto load_rows = [&](int h) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int u = q * ER_THREADS + tid, row = u / UPR, c = u % UPR;
+            if (row < n_rows) v[q] = *reinterpret_cast<const uint4*>(K_in + ((size_t)(t0 + row) * Hkv + h) * D + c * R::N);
+        }
+    };
+    if (COPY) load_rows(h0);
+    // highlighted rows of the tile, in order: slots 0 .. n_hot - 1
+    bool hl = false;
+    int b = 0;
+    if (tid < ER_ROWS) {
+        if (tid < n_rows && mask[t0 + tid] != 0) {
+            b = find_sequence(cu, B, L, t0 + tid);
+            hl = gain[b] != 0.f;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, hl);
+        if (lane == 0) cnt_s[warp] = __popc(bal);
+        slot_of[tid] = hl ? __popc(bal & ((1u << lane) - 1)) : -1;
+    }
+    __syncthreads();
+    const int n_hot = cnt_s[0] + cnt_s[1];
+    if (!COPY && n_hot == 0) return;
+    if (tid < ER_ROWS && hl) {
+        const int s = slot_of[tid] + (warp == 1 ? cnt_s[0] : 0);
+        slot_of[tid] = s; row_of[s] = tid; seq_of[s] = b;
+    }
+    __syncthreads();
+
+    for (int h = h0; h < h1; ++h) {
+        const bool on = n_hot > 0 && (head_enable == nullptr || head_enable[h] != 0);
+        if (COPY) {
+            if (h != h0) load_rows(h);
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const int u = q * ER_THREADS + tid, row = u / UPR, c = u % UPR;
+                if (row >= n_rows) continue;
+                const int s = on ? slot_of[row] : -1;
+                if (s < 0) *reinterpret_cast<uint4*>(K_out + ((size_t)(t0 + row) * Hkv + h) * D + c * R::N) = v[q];
+                else R::unpack(v[q], Ks + s * KP + c * R::N);
+            }
+        } else if (on) {
+            for (int u = tid; u < n_hot * UPR; u += ER_THREADS) {
+                const int s = u / UPR, c = u % UPR;
+                R::unpack(*reinterpret_cast<const uint4*>(K_in + ((size_t)(t0 + row_of[s]) * Hkv + h) * D + c * R::N), Ks + s * KP + c * R::N);
+            }
+        }
+        if (!on) continue;
+        // k' accumulates per thread: rows rg, rg + 16, ... (few highlighted rows still spread over all threads), 4 columns
+        // at 4 cg (and at 64 + 4 cg)
+        constexpr int NC = D / 64;
+        const int cg = tid & 15, rg = tid >> 4;
+        float acc[4][NC][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[i][c][e] = 0.f;
         for (int m = 0; m < M; ++m) {
-            const float a = g * (alpha != nullptr ? alpha[((size_t)b * Hkv + h) * M + m] : 1.f);
             const float* Um = U + ((size_t)m * Hkv + h) * D * r;
             for (int j0 = 0; j0 < r; j0 += 32) {
-                const int j = j0 + lane;
-                float c = 0.f;
+                const int rn = r - j0 < 32 ? r - j0 : 32;
+                // columns of the chunk that are worked on: 8, 16 or 32 (zero beyond the rank); a narrow chunk leaves lanes
+                // over, which then share the rows of U between them
+                const int rp = rn <= 8 ? 8 : (rn <= 16 ? 16 : 32), rs = rn <= 8 ? 3 : (rn <= 16 ? 4 : 5);
+                __syncthreads();                               // the previous chunk (or head) is through
+                for (int u = tid; u < D * rp; u += ER_THREADS) {
+                    const int i = u >> rs, j = u & (rp - 1);
+                    Us[i * ER_CP + j] = j < rn ? __ldg(Um + (size_t)i * r + j0 + j) : 0.f;
+                }
+                __syncthreads();
+                {   // C: warp w takes rows w, w + 8, ...; lane (s, j) column j, every (32 / rp)-th group of 4 dimensions
+                    const int j = lane & (rp - 1), ks = 32 >> rs, s4 = (lane >> rs) * 4;
+                    float c[8];
 #pragma unroll
-                for (int q = 0; q < Q; ++q)
-#pragma unroll 8
-                    for (int ii = 0; ii < 32; ++ii) {
-                        const float kv = __shfl_sync(0xffffffffu, k[q], ii);
-                        if (j < r) c = fmaf(__ldg(Um + (size_t)(q * 32 + ii) * r + j), kv, c);
+                    for (int i = 0; i < 8; ++i) c[i] = 0.f;
+                    for (int d0 = s4; d0 < D; d0 += 4 * ks) {
+                        float u4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) u4[e] = Us[(d0 + e) * ER_CP + j];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            if (warp + 8 * i >= n_hot) break;
+                            const float4 k4 = *reinterpret_cast<const float4*>(Ks + (warp + 8 * i) * KP + d0);
+                            c[i] = fmaf(k4.x, u4[0], fmaf(k4.y, u4[1], fmaf(k4.z, u4[2], fmaf(k4.w, u4[3], c[i]))));
+                        }
                     }
-                c *= a;
-                const int jn = min(32, r - j0);
-                for (int jj = 0; jj < jn; ++jj) {
-                    const float cj = __shfl_sync(0xffffffffu, c, jj);
 #pragma unroll
-                    for (int q = 0; q < Q; ++q) dk[q] = fmaf(__ldg(Um + (size_t)(q * 32 + lane) * r + j0 + jj), cj, dk[q]);
+                    for (int i = 0; i < 8; ++i) {
+                        const int s = warp + 8 * i;
+                        if (s >= n_hot) break;
+                        for (int o = rp; o < 32; o <<= 1) c[i] += __shfl_xor_sync(0xffffffffu, c[i], o);
+                        if (lane < rp) {
+                            const int sb = seq_of[s];
+                            const float a = gain[sb] * (alpha != nullptr ? alpha[((size_t)sb * Hkv + h) * M + m] : 1.f);
+                            Cs[s * ER_CP + j] = c[i] * a;
+                        }
+                    }
+                }
+                __syncthreads();
+                for (int jj = 0; jj < rn; jj += 4) {           // (columns up to the next multiple of 4 are zero)
+                    float4 u4[NC][4];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) u4[c][e] = *reinterpret_cast<const float4*>(Us + (c * 64 + cg * 4 + e) * ER_CP + jj);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (rg + 16 * i >= n_hot) break;
+                        const float4 c4 = *reinterpret_cast<const float4*>(Cs + (rg + 16 * i) * ER_CP + jj);
+#pragma unroll
+                        for (int c = 0; c < NC; ++c)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                acc[i][c][e] = fmaf(c4.x, u4[c][e].x, fmaf(c4.y, u4[c][e].y, fmaf(c4.z, u4[c][e].z, fmaf(c4.w, u4[c][e].w, acc[i][c][e]))));
+                    }
                 }
             }
         }
 #pragma unroll
-        for (int q = 0; q < Q; ++q) Elem<T>::store(K_out + row + q * 32 + lane, k[q] + dk[q]);
+        for (int i = 0; i < 4; ++i) {
+            const int s = rg + 16 * i;
+            if (s >= n_hot) break;
+            T* dst = K_out + ((size_t)(t0 + row_of[s]) * Hkv + h) * D;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const float4 k4 = *reinterpret_cast<const float4*>(Ks + s * KP + c * 64 + cg * 4);
+                const float o4[4] = {k4.x + acc[i][c][0], k4.y + acc[i][c][1], k4.z + acc[i][c][2], k4.w + acc[i][c][3]};
+                R::store4(dst + c * 64 + cg * 4, o4);
+            }
+        }
+        if (h + 1 < h1) __syncthreads();                       // the rows in shared memory are replaced
     }
 }
 
-template <typename T>
-static void launch_edit_rows(const seka_shape* s, const void* K_in, void* K_out, const int* list, const int* count,
-                             const float* U, const float* alpha, const float* gain, const uint8_t* he,
-                             cudaStream_t st) {
-    const int blocks = 148 * 8, threads = 256;
-    if (s->head_dim == 128)
-        edit_rows_kernel<T, 128><<<blocks, threads, 0, st>>>(
-            static_cast<const T*>(K_in), static_cast<T*>(K_out), list, count, U, alpha, gain, he, s->cu_seqlens,
-            s->batch, s->max_seqlen, s->n_kv_heads, s->rank, s->n_experts);
-    else
-        edit_rows_kernel<T, 64><<<blocks, threads, 0, st>>>(
-            static_cast<const T*>(K_in), static_cast<T*>(K_out), list, count, U, alpha, gain, he, s->cu_seqlens,
-            s->batch, s->max_seqlen, s->n_kv_heads, s->rank, s->n_experts);
+template <typename T, int D>
+static seka_status launch_edit_rows_t(const seka_shape* s, const void* K_in, void* K_out, const uint8_t* mask, const float* U,
+                                      const float* alpha, const float* gain, const uint8_t* he, cudaStream_t st) {
+    const int n_tok = shape_total_tokens(s);
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
+    const long long tiles = (n_tok + ER_ROWS - 1) / ER_ROWS;
+    // one head per CTA (a highlighted span then spreads over many SMs) until there are so many CTAs that the empty ones
+    // would cost more than the imbalance
+    long long hpc = tiles * s->n_kv_heads / (32LL * n_sm);
+    hpc = hpc < 1 ? 1 : (hpc > 4 ? 4 : hpc);
+    const long long grid = tiles * ((s->n_kv_heads + hpc - 1) / hpc);
+    if (grid > 0x7fffffffLL) return SEKA_ERR_UNSUPPORTED;
+    auto kern = K_in == K_out ? edit_rows_kernel<T, D, false> : edit_rows_kernel<T, D, true>;
+    constexpr size_t smem = edit_rows_smem<D>();
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
+    kern<<<(unsigned)grid, ER_THREADS, smem, st>>>(static_cast<const T*>(K_in), static_cast<T*>(K_out), mask, U, alpha, gain, he,
+                                                   s->cu_seqlens, n_tok, s->batch, s->max_seqlen, s->n_kv_heads, s->rank,
+                                                   s->n_experts, (int)hpc);
     ++g_launches;
+    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+}
+
+static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void* K_out, const uint8_t* mask, const float* U,
+                                    const float* alpha, const float* gain, const uint8_t* he, cudaStream_t st) {
+    if (s->dtype == SEKA_F32)
+        return s->head_dim == 128 ? launch_edit_rows_t<float, 128>(s, K_in, K_out, mask, U, alpha, gain, he, st)
+                                  : launch_edit_rows_t<float, 64>(s, K_in, K_out, mask, U, alpha, gain, he, st);
+    return s->head_dim == 128 ? launch_edit_rows_t<__nv_bfloat16, 128>(s, K_in, K_out, mask, U, alpha, gain, he, st)
+                              : launch_edit_rows_t<__nv_bfloat16, 64>(s, K_in, K_out, mask, U, alpha, gain, he, st);
 }
 
 // ---------------------------------------------------------------- bf16 tensors: one 128-token tile per step, on tcgen05
@@ -735,56 +888,21 @@ extern "C" seka_status seka_edit_keys(const seka_shape* shape, const void* K_in,
     if (!workspace || workspace_bytes < w.edit_total) return SEKA_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* ws = static_cast<char*>(workspace);
-    int* status = reinterpret_cast<int*>(ws);
-    int* list = reinterpret_cast<int*>(ws + w.list_off);
-    const size_t esz = shape->dtype == SEKA_F32 ? 4 : 2;
-    if (K_out != K_in) {
-        const size_t bytes = (size_t)T * shape->n_kv_heads * shape->head_dim * esz;
-        if (cudaMemcpyAsync(K_out, K_in, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return SEKA_ERR_CUDA;
-    }
     // bf16 tensors go through the tensor-core tile kernel (the projector products of all experts have to fit
     // into tensor memory); fp32 tensors, and banks too large for that, take the fp32 row kernel
     if (shape->dtype == SEKA_BF16 && (long long)shape->n_experts * shape->head_dim <= 512 && ((uintptr_t)workspace & 255) == 0) {
+        if (K_out != K_in) {
+            const size_t bytes = (size_t)T * shape->n_kv_heads * shape->head_dim * 2;
+            if (cudaMemcpyAsync(K_out, K_in, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return SEKA_ERR_CUDA;
+        }
         if (shape->head_dim == 128)
             return launch_edit_tiles<128>(shape, w, K_in, K_out, mask, U, alpha, gain, head_enable, ws, st);
         return launch_edit_tiles<64>(shape, w, K_in, K_out, mask, U, alpha, gain, head_enable, ws, st);
     }
-    launch_compact_mask(mask, T, list, status + 2, st);
-    if (shape->dtype == SEKA_F32)
-        launch_edit_rows<float>(shape, K_in, K_out, list, status + 2, U, alpha, gain, head_enable, st);
-    else
-        launch_edit_rows<__nv_bfloat16>(shape, K_in, K_out, list, status + 2, U, alpha, gain, head_enable, st);
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    return launch_edit_rows(shape, K_in, K_out, mask, U, alpha, gain, head_enable, st);
 }
 
-// ---------------------------------------------------------------- allocation-free variant
-namespace seka {
-
-// Scratch of seka_edit_keys_static, resident in the device image of every GPU that loads the
-// library: a 256-byte header whose first word is the list counter, then one int32 per token.
-// In host code this name is only a handle for cudaGetSymbolAddress, never a device pointer.
-static __device__ __align__(256) unsigned char g_static_scratch[256 + (size_t)SEKA_STATIC_MAX_TOKENS * 4];
-
-// Device address of the array on the current device, looked up once per device.
-static seka_status static_scratch_of_current_device(char** out) {
-    constexpr int kMaxDevices = 64;
-    static std::mutex mu;
-    static char* table[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SEKA_ERR_CUDA;
-    if (dev < 0 || dev >= kMaxDevices) return SEKA_ERR_UNSUPPORTED;
-    std::lock_guard<std::mutex> lock(mu);
-    if (table[dev] == nullptr) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || p == nullptr) return SEKA_ERR_CUDA;
-        table[dev] = static_cast<char*>(p);
-    }
-    *out = table[dev];
-    return SEKA_OK;
-}
-
-}  // namespace seka
-
+// ---------------------------------------------------------------- workspace-free variant: the fp32 row kernel needs no scratch
 extern "C" seka_status seka_edit_keys_static(const seka_shape* shape, const void* K_in, void* K_out,
                                              const uint8_t* mask, const float* U, const float* alpha,
                                              const float* gain, const uint8_t* head_enable, void* cuda_stream) {
@@ -792,25 +910,9 @@ extern "C" seka_status seka_edit_keys_static(const seka_shape* shape, const void
     seka_status stc = validate_shape(shape);
     if (stc != SEKA_OK) return stc;
     const int T = shape_total_tokens(shape);
-    if (T > SEKA_STATIC_MAX_TOKENS) return SEKA_ERR_UNSUPPORTED;   // beyond the built-in scratch
+    if (T > SEKA_STATIC_MAX_TOKENS) return SEKA_ERR_UNSUPPORTED;   // the documented limit of this entry point
     if (T == 0) return SEKA_OK;
     if (!K_in || !K_out || !mask || !U || !gain) return SEKA_ERR_INVALID_ARG;
     if (((uintptr_t)K_in | (uintptr_t)K_out) & 15) return SEKA_ERR_INVALID_ARG;
-    char* scratch = nullptr;
-    stc = static_scratch_of_current_device(&scratch);
-    if (stc != SEKA_OK) return stc;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    int* count = reinterpret_cast<int*>(scratch);
-    int* list = reinterpret_cast<int*>(scratch + 256);
-    const size_t esz = shape->dtype == SEKA_F32 ? 4 : 2;
-    if (K_out != K_in) {
-        const size_t bytes = (size_t)T * shape->n_kv_heads * shape->head_dim * esz;
-        if (cudaMemcpyAsync(K_out, K_in, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return SEKA_ERR_CUDA;
-    }
-    launch_compact_mask(mask, T, list, count, st);     // zeroes the counter on the stream first
-    if (shape->dtype == SEKA_F32)
-        launch_edit_rows<float>(shape, K_in, K_out, list, count, U, alpha, gain, head_enable, st);
-    else
-        launch_edit_rows<__nv_bfloat16>(shape, K_in, K_out, list, count, U, alpha, gain, head_enable, st);
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    return launch_edit_rows(shape, K_in, K_out, mask, U, alpha, gain, head_enable, static_cast<cudaStream_t>(cuda_stream));
 }

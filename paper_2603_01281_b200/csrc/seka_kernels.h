@@ -19,7 +19,6 @@ seka_status launch_prep_steering(const seka_shape* s, const SteerPlan& plan, con
 // `bh_info` (null: no steering) is the per-(sequence, KV head) byte the preparation launch wrote
 void launch_build_items(const Sched& sc, const int* cu, const uint8_t* bh_info, ItemRecord* items, int* count,
                         cudaStream_t st);
-void launch_compact_mask(const uint8_t* mask, int T, int* list, int* count, cudaStream_t st);
 void launch_convert_bf16(const float* Q, void* q16, size_t nq, const float* K, void* k16, const float* V, void* v16, size_t nk,
                          cudaStream_t st);
 

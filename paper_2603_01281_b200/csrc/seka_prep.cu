@@ -1,5 +1,5 @@
 // Small preparation kernels: dense edit operators and per-tile highlight flags for the fused kernel,
-// highlight-mask compaction, fp32 -> bf16 input conversion.
+// item table of packed batches, fp32 -> bf16 input conversion.
 #include "seka_kernels.h"
 #include "seka_route.cuh"
 
@@ -644,20 +644,6 @@ build_items_varlen_kernel(const Sched sc, const int* __restrict__ cu, const uint
     }
 }
 
-// Appends the indices of highlighted tokens to `list` (order within a warp preserved).
-__global__ void compact_mask_kernel(const uint8_t* __restrict__ mask, int T, int* __restrict__ list,
-                                    int* __restrict__ count) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool hl = t < T && mask[t] != 0;
-    const unsigned b = __ballot_sync(0xffffffffu, hl);
-    if (b == 0) return;
-    const int lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == 0) base = atomicAdd(count, __popc(b));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (hl) list[base + __popc(b & ((1u << lane) - 1))] = t;
-}
-
 // fp32 -> bf16 copies of Q, K and V in one launch (groups of four values; the three tensors one after another)
 struct ConvertArgs { const float4* in[3]; uint2* out[3]; size_t n4[3]; };
 __global__ void convert_f32_bf16_kernel(const ConvertArgs a) {
@@ -750,13 +736,6 @@ void launch_build_items(const Sched& sc, const int* cu, const uint8_t* bh_info, 
                         cudaStream_t st) {
     if (sc.rs <= 0) return;
     build_items_varlen_kernel<<<(unsigned)sc.rs, 1024, 0, st>>>(sc, cu, bh_info, items, count);
-    ++g_launches;
-}
-
-void launch_compact_mask(const uint8_t* mask, int T, int* list, int* count, cudaStream_t st) {
-    cudaMemsetAsync(count, 0, sizeof(int), st);
-    if (T == 0) return;
-    compact_mask_kernel<<<(T + 255) / 256, 256, 0, st>>>(mask, T, list, count);
     ++g_launches;
 }
 
