@@ -41,7 +41,6 @@ struct AttnParams {
     float* lse;
     const uint8_t* bh_info;       // [B, Hkv]: bit 0 the keys of this (sequence, KV head) are edited, bit 1 with the low parts
     const uint8_t* tile_hot;      // [B, n_qt]: key tile holds a highlighted token
-    const int* first_hot;         // [B]: first such tile of the sequence
     int* status;
     const ItemRecord* items;      // item table (packed batches), heaviest first
     const int* n_items;           // its length (device word)
@@ -69,10 +68,10 @@ struct Geo {
     static constexpr uint32_t TILE = (D / 64) * BLK_BYTES;         // a [128 x D] tile
     static constexpr int NXMAX = 3;                                // most stages of the key-side operand
     static constexpr uint32_t NBARS = 14 + 2 * NK + NXMAX;
-    // shared-memory copy of the per-(sequence, KV head) steering bytes and the per-sequence first highlighted tile
-    // (what fits beside the tiles; larger batches look them up in global memory)
-    static constexpr int INFO_HEADS = D == 128 ? 768 : 4096, INFO_SEQS = D == 128 ? 64 : 512;
-    static constexpr uint32_t INFO_BYTES = INFO_HEADS + INFO_SEQS * 4;
+    // shared-memory copy of the per-(sequence, KV head) steering bytes and of the tile flags, a bit each (what fits beside the
+    // tiles; larger batches look them up in global memory)
+    static constexpr int INFO_HEADS = D == 128 ? 768 : 2048, INFO_WORDS = D == 128 ? 128 : 512;
+    static constexpr uint32_t INFO_BYTES = INFO_HEADS + INFO_WORDS * 4;
 };
 
 struct SmemPlan {
@@ -154,7 +153,6 @@ struct Item {
     int hqA, hqB, qtA, qtB;     // query head and row-tile index of tile A / B
     int nA, nB, n_kv;           // key tiles of A / B (0: the tile lies beyond the sequence) and of the item
     bool steer;                 // the keys of this (sequence, KV head) are edited
-    bool hot_any;               // ... and one of the item's key tiles holds a highlighted token
     bool need_lo;               // ... and the low parts of the edited keys are multiplied too
 };
 
@@ -188,14 +186,37 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + sl.misc + 4);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // what does not depend on the launch before: barriers, tensor memory
+    if (tid == 0) {
+        mbar_init(q_full + 0, 1); mbar_init(q_full + 1, 1); mbar_init(k0_full, 1);
+        for (int i = 0; i < NK; ++i) { mbar_init(kv_full + i, 1); mbar_init(kv_free + i, 1); }
+        for (int i = 0; i < G::NXMAX; ++i) mbar_init(x_full + i, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(s_full + i, 1); mbar_init(p_full + i, 5); mbar_init(p_last + i, 4); mbar_init(o_full + i, 1);
+            mbar_init(o_drained + i, 4);
+        }
+        mbar_init(start_full, 1); mbar_init(drain, 1);
+        mbar_fence_init();
+        tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
+        if (p.plan.mode) tma_prefetch_desc(&tmX);
+    }
+    __syncwarp();
+    if (warp == 0) { tmem_alloc(tmem_holder, TMEM_COLS); tmem_relinquish(); }
+    pdl_wait();
     // an earlier launch (or CTA) gave up on this workspace: nothing is started (every role finds `ok` false)
     const bool dead = __syncthreads_or(*reinterpret_cast<volatile int*>(p.status) != 0);
     const int hook_skip = p.status[4];
     const uint64_t limit_ns = p.status[5] > 0 ? (uint64_t)p.status[5] * 1000ull : kWaitLimitNs;
-    // steering info is kept in shared memory when it fits (a look-up per work item then costs no trip to the caches)
-    const bool info_local = p.steer && p.sched.B * p.sched.Hkv <= G::INFO_HEADS && p.sched.B <= G::INFO_SEQS;
+    // steering info is kept in shared memory when it fits (a look-up then costs no trip to the caches): a byte per (sequence,
+    // KV head) and a bit per (sequence, key tile)
+    const bool info_local = p.steer && p.sched.B * p.sched.Hkv <= G::INFO_HEADS;
     uint8_t* info_bh = smem + sl.info;
-    int* info_first = reinterpret_cast<int*>(smem + sl.info + G::INFO_HEADS);
+    const int hot_words = (p.sched.n_qt + 31) / 32;
+    const bool hot_local = p.steer && p.sched.B * hot_words <= G::INFO_WORDS;
+    uint32_t* info_hot = reinterpret_cast<uint32_t*>(smem + sl.info + G::INFO_HEADS);
+    auto tile_is_hot = [&](int b, int j) -> bool {
+        return hot_local ? ((info_hot[b * hot_words + (j >> 5)] >> (j & 31)) & 1u) != 0 : __ldg(p.tile_hot + (size_t)b * p.sched.n_qt + j) != 0;
+    };
 
     // all lanes of a warp wait on the same barrier and then agree on the outcome
     auto warp_wait = [&](uint64_t* bar, uint32_t parity, int where) -> bool {
@@ -253,32 +274,20 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         it.nA = rec.n & 0xffff; it.nB = rec.n >> 16;
         it.n_kv = max(it.nA, it.nB);
         it.steer = steering && (rec.steer & 1) != 0 && p.plan.mode != 0;
-        it.hot_any = it.steer && (info_local ? info_first[it.b] : __ldg(p.first_hot + it.b)) < it.n_kv;
-        it.need_lo = it.hot_any && ((rec.steer & 2) != 0 || it.n_kv <= kLoTiles);
+        it.need_lo = it.steer && ((rec.steer & 2) != 0 || it.n_kv <= kLoTiles);
         return true;
     };
 
-    if (tid == 0) {
-        mbar_init(q_full + 0, 1); mbar_init(q_full + 1, 1); mbar_init(k0_full, 1);
-        for (int i = 0; i < NK; ++i) { mbar_init(kv_full + i, 1); mbar_init(kv_free + i, 1); }
-        for (int i = 0; i < G::NXMAX; ++i) mbar_init(x_full + i, 1);
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(s_full + i, 1); mbar_init(p_full + i, 5); mbar_init(p_last + i, 4); mbar_init(o_full + i, 1);
-            mbar_init(o_drained + i, 4);
-        }
-        mbar_init(start_full, 1); mbar_init(drain, 1);
-        *abort_flag = dead ? 1 : 0;
-        mbar_fence_init();
-        tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
-        if (p.plan.mode) tma_prefetch_desc(&tmX);
-    }
-    __syncwarp();
-    if (warp == 0) { tmem_alloc(tmem_holder, TMEM_COLS); tmem_relinquish(); }
+    if (tid == 0) *abort_flag = 0;
     // steering info into shared memory
-    if (info_local) {
+    if (info_local)
         for (int i = tid; i < p.sched.B * p.sched.Hkv; i += NTHREADS) info_bh[i] = p.bh_info[i];
-        for (int i = tid; i < p.sched.B; i += NTHREADS) info_first[i] = p.first_hot[i];
-    }
+    if (hot_local)
+        for (int w = warp; w < p.sched.B * hot_words; w += NTHREADS / 32) {
+            const int b = w / hot_words, j = (w - b * hot_words) * 32 + lane;
+            const uint32_t bits = __ballot_sync(0xffffffffu, j < p.sched.n_qt && p.tile_hot[(size_t)b * p.sched.n_qt + j] != 0);
+            if (lane == 0) info_hot[w] = bits;
+        }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -338,7 +347,6 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 ++n_hot;
             };
             while (ok && next_item(it, true)) {
-                const uint8_t* hot_g = p.tile_hot + (size_t)it.b * p.sched.n_qt;
                 // Q and the first K of an item may land once the last score product of the previous item is
                 // done (event n_kv - 1 of that item), its V/K pairs once its last step is done (event n_kv)
                 if (n_it > 0) {
@@ -357,7 +365,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                             tma_load_3d(smem + G::TILE + c * BLK_BYTES, &tmQ, q_full + 1, c * 64, it.hqB, it.seq0 + it.qtB * BM);
                     }
                     mbar_expect_tx(k0_full, G::TILE);
-                    const CUtensorMap* km0 = (staged && it.hot_any && hot_g[0] != 0) ? &tmX : &tmK;
+                    const CUtensorMap* km0 = (staged && it.steer && tile_is_hot(it.b, 0)) ? &tmX : &tmK;
 #pragma unroll
                     for (int c = 0; c < NBLK; ++c)
                         tma_load_3d(smem + sl.k + (pr % NK) * G::TILE + c * BLK_BYTES, km0, k0_full, c * 64, it.hkv, it.seq0);
@@ -365,7 +373,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 __syncwarp();
                 armed_q[0] = (n_it & 1) + 1; armed_k0 = (n_it & 1) + 1;
                 if (it.nB > 0) { armed_q[1] = (n_qb & 1) + 1; ++n_qb; }
-                if (it.need_lo && hot_g[0] != 0) {
+                if (it.need_lo && tile_is_hot(it.b, 0)) {
                     load_x(0, ev);
                     if (!ok) break;
                 }
@@ -382,7 +390,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         if (!ok) break;
                     }
                     const bool more = t + 1 < it.n_kv;
-                    const bool hot_n = more && it.hot_any && hot_g[t + 1] != 0;
+                    const bool hot_n = more && it.steer && tile_is_hot(it.b, t + 1);
                     const uint32_t g = pr + (uint32_t)t;
                     // (test hook: one pair of the first item of CTA 0 is left out altogether, so that its wait runs out)
                     const bool skip = hook_skip > 0 && n_it == 0 && blockIdx.x == 0 && t + 1 == hook_skip;
@@ -442,7 +450,6 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 __syncwarp();
             };
             while (ok && next_item(it, true)) {
-                const uint8_t* hot_g = p.tile_hot + (size_t)it.b * p.sched.n_qt;
                 const int nA = it.nA, nB = it.nB, n_kv = it.n_kv;
                 uint32_t x_stage = 0;      // stage that holds the low parts of the key tile being multiplied
                 // the low parts of the next edited key tile have landed (once per tile, before its first use)
@@ -498,8 +505,8 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     if (ok && nB > 0 && n_o[1] > 0) ok = warp_wait(o_drained + 1, (n_o[1] - 1) & 1, 47);
                 };
                 // do key tiles 0 and 1 take the low-part steps? (later ones are looked up one step ahead of their use)
-                const bool hot_cur = it.need_lo && hot_g[0] != 0;
-                bool hot_nxt = it.need_lo && n_kv > 1 && hot_g[1] != 0;
+                const bool hot_cur = it.need_lo && tile_is_hot(it.b, 0);
+                bool hot_nxt = it.need_lo && n_kv > 1 && tile_is_hot(it.b, 1);
                 // One thread issues for both tiles, in a fixed order (A then B in every step): the in-order tensor
                 // pipe then keeps the two tiles half a period apart (softmax of one tile under the MMAs of the other).
                 ok = warp_wait(start_full, n_it & 1, 20);
@@ -515,7 +522,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 for (int j = 0; j < n_kv && ok; ++j) {
                     const int j1 = j + 1;
                     const bool hot_j1 = hot_nxt && j1 < n_kv;
-                    hot_nxt = it.need_lo && j + 2 < n_kv && hot_g[j + 2] != 0;
+                    hot_nxt = it.need_lo && j + 2 < n_kv && tile_is_hot(it.b, j + 2);
                     bool x_seen = false;
                     // V of this step and K of the next have landed once p_full completes: the relay warp vouches
                     // for them there, so this warp has no waits of its own for operands (every wait here is a
@@ -701,6 +708,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     }
 
     // ---------------------------------------------------------------- teardown (also after an abort)
+    pdl_release();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -778,9 +786,10 @@ static seka_status launch_attn_t(const TileMaps& tm, const AttnParams& p, cudaSt
     // persistent CTAs, one per SM (the kernel needs the whole SM: all of tensor memory and most of shared memory)
     const unsigned grid = (unsigned)(p.sched.n_items_max < (long long)n_sm ? p.sched.n_items_max : (long long)n_sm);
     if (grid == 0) return SEKA_OK;
-    kern<<<grid, NTHREADS, dyn, st>>>(tm.q, tm.k, tm.v, tm.x, p);
-    g_launches.fetch_add(1);
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    // A launch of one item per CTA is placed under the tail of its preparation (one prompt of 777 tokens 32.6 -> 31.2 us, the
+    // toy layer 24.6 -> 21.2 us per call).  Longer ones are not: their CTAs then land on the SMs in the order in which these
+    // become free, and CTAs that share a KV head no longer sit next to each other (4 x 4096 tokens 589 -> 607 us).
+    return launch_kernel(p.sched.n_items_max <= (long long)grid, kern, grid, NTHREADS, dyn, st, tm.q, tm.k, tm.v, tm.x, p);
 }
 
 template <int D, typename OutT>
@@ -811,37 +820,48 @@ static seka_status attention_fwd_impl(const seka_shape* shape, const void* Q, co
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* ws = static_cast<char*>(workspace);
 
-    const void *q16 = Q, *k16 = K, *v16 = V;
-    if (shape->dtype == SEKA_F32) {
-        const size_t nq = (size_t)T * Hq * D, nk = (size_t)T * Hkv * D;
-        char* cq = ws + w.cvt_off;
-        char* ck = cq + align_up(nq * 2, 256);
-        char* cv = ck + align_up(nk * 2, 256);
-        launch_convert_bf16(static_cast<const float*>(Q), cq, nq, static_cast<const float*>(K), ck, static_cast<const float*>(V), cv, nk, st);
-        q16 = cq; k16 = ck; v16 = cv;
-    }
     AttnParams p;
     p.plan = make_steer_plan(shape, steer);
     p.sched = sched;
     void* X = ws + w.x_off;
     uint8_t* tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off);
-    int* first_hot = reinterpret_cast<int*>(ws + w.first_off);
     uint8_t* bh_info = reinterpret_cast<uint8_t*>(ws + w.info_off);
-    if (steer) {
-        // The tile kernels of the stand-alone edit write the side buffer (two small launches; in a routed call further
-        // blocks of the first one evaluate Eq. 6 with the routine of adaseka_route, so the coefficients, and with them
-        // everything after, are those of route-then-forward bit for bit).  Banks too wide for tensor memory
-        // (n_experts * head_dim > 512) take the one-launch preparation kernel.
-        if ((long long)shape->n_experts * D <= 512) {
-            const float* a = alpha;
-            if (sigma != nullptr) a = alpha_out != nullptr ? alpha_out : reinterpret_cast<float*>(ws + w.alpha_off);
-            stc = launch_stage_keys_pipe(shape, w, k16, X, mask, U, a, gain, head_enable, ws, st, Q, sigma, k_route);
-        } else {
-            stc = launch_prep_steering(shape, p.plan, k16, U, alpha, gain, head_enable, mask, X, tile_hot, first_hot, bh_info,
-                                       reinterpret_cast<int*>(ws), w.n_tiles, st, Q, sigma, k_route, alpha_out);
+    ItemRecord* items = reinterpret_cast<ItemRecord*>(ws + w.item_off);
+    int* n_items = reinterpret_cast<int*>(ws) + 3;
+    const bool table = shape->cu_seqlens != nullptr;
+
+    // The preparation: the edited keys of the tiles with highlighted tokens, the item table of a packed batch and the bf16
+    // copies of fp32 inputs, each in blocks of its own (nothing is launched if none of them is needed).
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
+    PrepJobs jobs = {};
+    jobs.sched = sched; jobs.cu = shape->cu_seqlens; jobs.items = items; jobs.item_count = n_items;
+    if (steer) jobs.steer = SteerIn{gain, alpha, head_enable, shape->n_experts, sigma != nullptr ? 1 : 0};
+    if (table) jobs.n_items_blocks = sched.rs;
+    const void *q16 = Q, *k16 = K, *v16 = V;
+    if (shape->dtype == SEKA_F32) {
+        const size_t nq = (size_t)T * Hq * D, nk = (size_t)T * Hkv * D;      // multiples of 4
+        char* cq = ws + w.cvt_off;
+        char* ck = cq + align_up(nq * 2, 256);
+        char* cv = ck + align_up(nk * 2, 256);
+        const void* in[3] = {Q, K, V};
+        char* out[3] = {cq, ck, cv};
+        for (int i = 0; i < 3; ++i) {
+            jobs.conv.in[i] = static_cast<const float4*>(in[i]); jobs.conv.out[i] = reinterpret_cast<uint2*>(out[i]);
+            jobs.conv.n4[i] = (i == 0 ? nq : nk) / 4;
         }
-        if (stc != SEKA_OK) return stc;
+        const long long want = (long long)((nq + 2 * nk) / (4 * 4 * PREP_THREADS)) + 1, most = 4LL * n_sm;
+        jobs.n_conv_blocks = (int)(want < most ? want : most);
+        q16 = cq; k16 = ck; v16 = cv;
     }
+    if (steer) {
+        RouteArgs route = {};
+        if (sigma != nullptr) route = RouteArgs{Q, shape->dtype == SEKA_F32 ? 1 : 0, sigma, k_route, Hq, alpha_out};
+        stc = launch_stage_keys(shape, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st);
+    } else {
+        stc = launch_prep_plain(jobs, st);
+    }
+    if (stc != SEKA_OK) return stc;
 
     TileMaps tm;
     if (!make_tile_map(&tm.q, q16, D, Hq, T, 128) || !make_tile_map(&tm.k, k16, D, Hkv, T, 128) ||
@@ -851,12 +871,9 @@ static seka_status attention_fwd_impl(const seka_shape* shape, const void* Q, co
     if (p.plan.mode != 0 && !make_tile_map(&tm.x, X, p.plan.xcols, Hkv, T, 128)) return SEKA_ERR_CUDA;
 
     p.O = O; p.lse = lse;
-    p.tile_hot = tile_hot; p.first_hot = first_hot; p.bh_info = bh_info; p.status = reinterpret_cast<int*>(ws);
+    p.tile_hot = tile_hot; p.bh_info = bh_info; p.status = reinterpret_cast<int*>(ws);
     p.steer = steer ? 1 : 0;
-    ItemRecord* items = reinterpret_cast<ItemRecord*>(ws + w.item_off);
-    const bool table = shape->cu_seqlens != nullptr;
-    if (table) launch_build_items(sched, shape->cu_seqlens, steer ? bh_info : nullptr, items, reinterpret_cast<int*>(ws) + 3, st);
-    p.items = items; p.n_items = reinterpret_cast<int*>(ws) + 3;
+    p.items = items; p.n_items = n_items;
     const float scale = shape->softmax_scale > 0.f ? shape->softmax_scale : 1.f / sqrtf((float)D);
     p.scale_log2 = scale * 1.4426950408889634f;
 

@@ -16,17 +16,15 @@ namespace seka {
 
 // ---------------------------------------------------------------- workspace layout
 // [0, 256)            status block: word 0 = seka_status, word 1 = where the wait gave up,
-//                     word 2 = number of highlighted tokens found by the compaction pass,
 //                     word 3 = number of work items in the item table of the fused kernel,
 //                     word 4 = test hook: the producer of CTA 0 leaves out the load of this V/K pair (1-based) of its
 //                              first item, so that a bounded wait runs out (0 = off),
 //                     word 5 = limit of every device-side wait of the fused kernel in microseconds (0 = 2 s)
-// [256, ...)          projector operands: the stand-alone edit keeps P[m][h] = U_m U_m^T here (two bf16 parts); the fused
-//                     kernel does not use it
-// then                one byte per (sequence, 128-key tile): the tile contains a highlighted token; then one int32
-//                     per sequence: its first such tile; then one byte per (sequence, KV head): steered / low parts used
+// [1024, ...)         (one expert) projectors P[h] = U_h U_h^T of the pipelined preparation, two bf16 parts
+// then                one byte per (sequence, 128-key tile): the tile contains a highlighted token; then one byte per
+//                     (sequence, KV head): steered / low parts used
 // then                item table of the fused kernel (32 bytes per unit, heaviest first)
-// then                compacted highlighted-token list (int32 per token)
+// then                (stand-alone edit) highlighted tokens, in segments: int32 per token; then a count per segment
 // then (fp32 inputs)  bf16 copies of Q, K, V
 // then                edited keys of the fused kernel, bf16 [T, Hkv, 2 d] (high | low parts; only rows of tiles that
 //                     hold a highlighted token are ever written or read)
@@ -40,7 +38,6 @@ constexpr size_t kStatusBytes = 256;
 // tensor-memory accumulator, by  S += Q (k'_lo)^T.  The low parts go through a small shared-memory ring of their own.
 struct SteerPlan {
     int mode;            // 0: no steering, 1: steering
-    int Rt;              // stacked rank M * r
     int xcols;           // bf16 columns of a side-buffer row: high parts [0, D), low parts [D, 2D)
     int nx;              // shared-memory stages of the low parts
 };
@@ -54,7 +51,7 @@ static inline int shape_total_tokens(const seka_shape* s) {
 // head_dim 128 leaves 32 KB of shared memory beside the Q, K and V tiles: one stage of low parts
 static inline SteerPlan make_steer_plan(const seka_shape* s, bool steer) {
     SteerPlan p;
-    p.mode = steer ? 1 : 0; p.Rt = s->rank * s->n_experts;
+    p.mode = steer ? 1 : 0;
     p.xcols = steer ? 2 * s->head_dim : 0;
     p.nx = steer ? (s->head_dim == 64 ? 3 : 1) : 0;
     return p;
@@ -135,16 +132,21 @@ SEKA_HD bool decode_item(const Sched& c, long long idx, const int* cu, ItemRecor
     return nA > 0;
 }
 
+// The stand-alone edit lists the highlighted tokens in segments of consecutive tokens, one block and one count each.
+constexpr int kMaxSegments = 1024;
+static inline int edit_segment_tokens(long long T) {
+    return (int)((T + (long long)kMaxSegments * 1024 - 1) / ((long long)kMaxSegments * 1024)) * 1024;
+}
+
 struct WorkspaceLayout {
-    size_t w_off, w_bytes;            // projector operands (see above)
-    size_t hot_off, hot_bytes;        // uint8 [B, ceil(max_seqlen / 128)], then int32 [B]
-    size_t first_off;                 // the int32 [B] inside the hot region
-    size_t info_off;                  // uint8 [B, Hkv] inside the hot region: bit 0 steered, bit 1 with the low parts
+    size_t w_off;                     // projectors P[h] as two bf16 parts (one expert)
+    size_t hot_off;                   // uint8 [B, ceil(max_seqlen / 128)]
+    size_t info_off;                  // uint8 [B, Hkv]: bit 0 steered, bit 1 with the low parts
     size_t item_off, item_bytes;      // ItemRecord [n_items_max]
     size_t list_off, list_bytes;      // int32 [total_tokens]
+    size_t count_off;                 // int32 [kMaxSegments]
     size_t cvt_off, cvt_bytes;        // bf16 copies of Q, K, V (fp32 inputs only)
     size_t x_off, x_bytes;            // edited keys of the fused kernel
-    size_t alpha_off;                 // fp32 [B, Hkv, M]: routing coefficients of a routed call that does not ask for them
     size_t edit_total;                // what the stand-alone edit needs (everything before the edited keys)
     size_t total;
     int n_tiles;                      // key tiles per sequence = ceil(max_seqlen / 128)
@@ -156,26 +158,23 @@ static inline WorkspaceLayout workspace_layout(const seka_shape* s) {
     const int D = s->head_dim;
     const SteerPlan plan = make_steer_plan(s, true);
     w.n_tiles = (s->max_seqlen + 127) / 128;
-    w.w_off = kStatusBytes;
-    w.w_bytes = align_up((size_t)2 * s->n_experts * s->n_kv_heads * D * D * 2, 1024);
-    w.hot_off = w.w_off + w.w_bytes;
-    w.first_off = w.hot_off + align_up((size_t)s->batch * w.n_tiles + 1, 256);
-    w.info_off = w.first_off + align_up((size_t)s->batch * 4 + 4, 256);
-    w.hot_bytes = (w.info_off - w.hot_off) + align_up((size_t)s->batch * s->n_kv_heads + 1, 256);
+    w.w_off = 1024;                   // (1024-byte aligned: read by TMA)
+    w.hot_off = w.w_off + (s->n_experts == 1 ? (size_t)2 * s->n_kv_heads * D * D * 2 : 0);
+    w.info_off = w.hot_off + align_up((size_t)s->batch * w.n_tiles + 1, 256);
     const Sched sc = make_sched(s);
-    w.item_off = w.hot_off + w.hot_bytes;
+    w.item_off = w.info_off + align_up((size_t)s->batch * s->n_kv_heads + 1, 256);
     w.item_bytes = align_up((size_t)sc.n_items_max * 32 + 32, 256);
     w.list_off = w.item_off + w.item_bytes;
     w.list_bytes = align_up(T * 4 + 4, 256);
-    w.cvt_off = w.list_off + w.list_bytes;
+    w.count_off = w.list_off + w.list_bytes;
+    w.cvt_off = w.count_off + kMaxSegments * 4;
     w.cvt_bytes = 0;
     if (s->dtype == SEKA_F32)
         w.cvt_bytes = align_up(T * s->n_q_heads * D * 2, 256) + 2 * align_up(T * s->n_kv_heads * D * 2, 256);
     w.edit_total = w.cvt_off + w.cvt_bytes;
     w.x_off = align_up(w.edit_total, 1024);
     w.x_bytes = align_up(T * s->n_kv_heads * plan.xcols * 2, 1024);
-    w.alpha_off = w.x_off + w.x_bytes;
-    w.total = w.alpha_off + align_up((size_t)s->batch * s->n_kv_heads * s->n_experts * 4 + 4, 256);
+    w.total = w.x_off + w.x_bytes;
     return w;
 }
 
@@ -207,6 +206,20 @@ __device__ __forceinline__ float alpha_max_of(const float* __restrict__ alpha, s
     for (int m = 0; m < M; ++m) a = fmaxf(a, fabsf(alpha[bh * M + m]));
     return a;
 }
+
+// ---------------------------------------------------------------- programmatic dependent launch
+// The kernels of one call, and of consecutive calls, may follow each other with the next one's blocks already placed: a
+// kernel lets its successor be launched early and touches global memory only after its predecessor has finished (both are
+// no-ops for a launch without the attribute).  Every thread of every block passes pdl_wait, so a kernel never finishes
+// before the one ahead of it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// ---------------------------------------------------------------- asynchronous 16-byte copies (zero-filled where `valid` is false)
+__device__ __forceinline__ void cp_async16(uint32_t smem_dst, const void* src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -433,6 +446,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// two fp32 values -> their high bf16 parts and their low bf16 parts, packed in pairs
+__device__ __forceinline__ void split_pair(float x, float y, uint32_t& hi, uint32_t& lo) {
+    hi = pack_bf16(x, y);
+    const float2 h = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&hi));
+    lo = pack_bf16(x - h.x, y - h.y);
 }
 
 #endif  // __CUDACC__

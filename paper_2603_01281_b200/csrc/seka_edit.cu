@@ -1,5 +1,6 @@
 // Standalone key-editing kernel (the hook of Algorithm 1 / Algorithm 2 applied to a key tensor in HBM).
 #include "seka_kernels.h"
+#include "seka_route.cuh"
 
 namespace seka {
 
@@ -244,15 +245,23 @@ static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void*
                               : launch_edit_rows_t<__nv_bfloat16, 64>(s, K_in, K_out, mask, U, alpha, gain, he, st);
 }
 
-// ---------------------------------------------------------------- bf16 tensors: one 128-token tile per step, on tcgen05
+// ---------------------------------------------------------------- bf16 tensors: 128 key rows per step, on tcgen05
 //
-// A CTA (8 warps) takes a contiguous run of the (KV head, highlighted tile) pairs, head-major, so that the projector
-// P[m][h] = U_m U_m^T (two bf16 parts, resident in shared memory) changes rarely: TMA stages the [128 x D] key tile,
-// the tensor core forms K P_m in tensor memory (two products per expert), every thread adds
-// g_b sum_m alpha_{b,h,m} (K P_m)[row] to half of its row in shared memory if the row is highlighted, and the warps
-// then write the highlighted rows out, 16 bytes per lane with the lanes of a row next to each other.
-// Unhighlighted rows are never written.  Two CTAs share an SM (96 KB of shared memory and M * D tensor-memory
-// columns each), so the loads, products and stores of different tiles overlap.
+// k' = k + sum_j c_j U[:, j] (U[:, j] . k) over the stacked columns j = (expert, direction), c_j = g_b alpha_{b,h,m(j)}: two
+// chained products per block of 64 columns,
+//     C = K U      (the key rows are exact in bf16, U as two bf16 parts),
+//     dK += (C diag(c)) U^T    (C scaled and split into two bf16 parts in tensor memory; three products of the parts),
+// so the edit is accurate to about 2^-17 of its size and no d x d projector is ever formed.  A step is 128 rows of one KV
+// head.  In the stand-alone edit they are the next 128 highlighted tokens, wherever they lie (a list made by the launch
+// before: only rows that change are read or written, and every CTA gets the same number of them); in the fused forward's
+// preparation (SIDE) they are the rows of one 128-key tile that holds a highlighted token, and k' of all of them goes to the
+// side buffer (rows of 2 D bf16: high parts [0, D), low parts [D, 2 D), the low parts only where the fused kernel reads them).
+//
+// The step is a chain (rows and U land, product, scale, product, add, write) that several CTAs per SM walk side by side; the
+// rows of a CTA's next step are fetched under the present one where shared memory has room for a second stage.
+// Measured: 144 x 4096 tokens x 8 heads x 128 in place, a tenth highlighted, 94 -> 72 us per call (whole 128-row tiles
+// through a projector, of which 58 % of the rows were written); one prompt of 777 tokens on 32/8 heads 42 -> 31 us per call
+// (four launches and two memsets before, two launches now).
 constexpr uint32_t EBLK = 128 * 128;        // one [128 x 64] bf16 block
 
 // all lanes of a warp wait on the same barrier and then agree on the outcome
@@ -260,218 +269,555 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     const bool ok = mbar_wait(bar, parity, abort_flag, status, where);
     return __all_sync(0xffffffffu, ok);
 }
-constexpr int EDIT_THREADS = 256;
+constexpr int ET_THREADS = 256, ET_WARPS = ET_THREADS / 32;
+constexpr int ET_UCOLS = 64;                // columns of U per block
 
-template <int D>
-struct EditSmem {
-    static constexpr uint32_t TILE = (D / 64) * EBLK;
-    static constexpr uint32_t PBLK = D * 128;
-    static constexpr uint32_t PMAT = (D / 64) * PBLK;       // one D x D bf16 matrix
-    static constexpr uint32_t K = 0;
-    static constexpr uint32_t P = K + TILE;                 // high part, then low part
-    static constexpr uint32_t FLAGS = P + 2 * PMAT;
-    static constexpr uint32_t BARS = FLAGS + 128;
-    static constexpr uint32_t MISC = BARS + 16;
-    static constexpr uint32_t DYN_BYTES = MISC + 16 + 1024;
+template <int D, bool SIDE>
+struct EtSmem {
+    static constexpr uint32_t TILE = (D / 64) * EBLK;       // 128 key rows
+    static constexpr uint32_t UMAT = D * 128;               // [D x 64] bf16
+    static constexpr int NS = D == 128 && SIDE ? 1 : 2;     // stages of key rows (two CTAs per SM leave room for one beside the low parts)
+    static constexpr uint32_t U = NS * TILE;                // high part, then low part
+    static constexpr uint32_t LO = U + 2 * UMAT;            // SIDE: low parts of the edited rows
+    static constexpr uint32_t ROUTE = LO + (SIDE ? TILE : 0);         // scratch and result of Eq. 6 (routed calls)
+    static constexpr uint32_t TMEM_COLS = D == 128 ? 256 : 128;       // 64 for C, D for dK
+    static constexpr int CTAS = D == 128 ? 2 : 3;           // per SM: tensor memory and shared memory (128), shared memory (64)
 };
 
-// SIDE: as in the pipelined kernel below, k' of every row of the tile that lies inside its sequence goes to the side
-// buffer of the fused forward (rows of 2 D bf16: high parts, then low parts where the fused kernel reads them).
-template <int D, bool SIDE>
-__global__ void __launch_bounds__(EDIT_THREADS)
-edit_tiles_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmP,
-                  __nv_bfloat16* __restrict__ K_out, const uint8_t* __restrict__ mask, const float* __restrict__ alpha,
-                  const float* __restrict__ gain, const uint8_t* __restrict__ head_enable,
-                  const int* __restrict__ cu_seqlens, const int* __restrict__ hot_list, const int* __restrict__ hot_count,
-                  int* status, int L, int Hkv, int M, int n_tiles, uint32_t tmem_cols) {
-    using SL = EditSmem<D>;
-    constexpr int NBLK = D / 64;
+// SIDE: a unit of work as the warp that looked at it left it
+struct __align__(16) UnitInfo { uint32_t bits[4]; int work, b, tok0, nvalid; float c; int with_lo, pad[2]; };
+
+struct TileArgs {
+    const void* K; __nv_bfloat16* out;
+    const uint8_t* mask; const float* U; const float* alpha; const float* gain; const uint8_t* head_enable; const int* cu;
+    const int* list; const int* counts; int n_seg, seg_tokens;                   // stand-alone edit: the highlighted tokens
+    uint8_t* tile_hot; uint8_t* bh_info;                                         // SIDE: written for the fused kernel
+    int* status;
+    int B, L, Hkv, r, M, n_tiles;
+    int n_route_blocks, n_tile_blocks;      // SIDE: routing blocks | item-table blocks | tile blocks | conversion blocks
+    RouteArgs route;
+    PrepJobs jobs;
+};
+
+template <int D, bool SIDE, typename KT>
+__global__ void __launch_bounds__(ET_THREADS, EtSmem<D, SIDE>::CTAS)
+edit_tiles_kernel(const __grid_constant__ TileArgs p) {
+    using SL = EtSmem<D, SIDE>;
+    constexpr int NS = SL::NS;
+    constexpr int UPR = D / 8;                          // 16-byte units (8 elements) of a key row
+    constexpr int RPP = ET_THREADS / UPR;               // rows a pass of the CTA loads
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sK = smem + SL::K;
-    uint8_t* flags = smem + SL::FLAGS;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + SL::BARS);
-    uint64_t* done = full + 1;
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + SL::MISC);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::MISC + 4);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row = tid & 127, half = tid >> 7;      // key row of the tile, and which half of its columns this thread updates
-    if (__syncthreads_or(*reinterpret_cast<volatile int*>(status) != 0)) return;
+    const int Hkv = p.Hkv, r = p.r, M = p.M;
+    const bool routed = SIDE && p.route.sigma != nullptr;
+    int blk = blockIdx.x;
+    if constexpr (SIDE) {
+        if (blk < p.n_route_blocks) {
+            // ------------------------------------------------ Eq. 6 of one (sequence, KV head), for the caller
+            pdl_wait();
+            pdl_release();
+            const double* a = route_group(p.route.Q, p.route.q_is_f32, p.U, p.route.sigma, p.cu, p.L, p.route.Hq, Hkv, D, r, M,
+                                          p.route.k_route, blk / Hkv, blk % Hkv, reinterpret_cast<double*>(smem));
+            for (int m = tid; m < M; m += ET_THREADS) p.route.alpha_out[(size_t)blk * M + m] = (float)a[m];
+            return;
+        }
+        blk -= p.n_route_blocks;
+        if (blk < p.jobs.n_items_blocks) {
+            pdl_wait();
+            pdl_release();
+            items_block(p.jobs.sched, p.jobs.cu, p.jobs.steer, p.jobs.items, p.jobs.item_count, blk);
+            return;
+        }
+        blk -= p.jobs.n_items_blocks;
+        if (blk >= p.n_tile_blocks) {
+            pdl_wait();
+            pdl_release();
+            convert_block(p.jobs.conv, blk - p.n_tile_blocks, p.jobs.n_conv_blocks);
+            return;
+        }
+    }
 
+    __shared__ __align__(8) uint64_t bars[2];           // C is ready, dK is ready
+    __shared__ uint32_t tmem_holder;
+    __shared__ int abort_s;
+    __shared__ int tok_s[2][SIDE ? 1 : 128], seq_s[2][SIDE ? 1 : 128];      // stand-alone: token (-1: none) and sequence of a row, per stage
+    __shared__ float c_s[2][SIDE ? 1 : 128];            // stand-alone: gain (one expert: times its coefficient) of a row, per stage
+    __shared__ UnitInfo look_s[ET_WARPS];               // SIDE: the units looked at last
+    __shared__ unsigned short exp_s[ET_UCOLS];          // expert of a column of the block
+    __shared__ int pre_s[SIDE ? 1 : kMaxSegments + 1];  // stand-alone: highlighted tokens before each segment
+    __shared__ int wsum_s[ET_WARPS];
+    volatile int* abort_flag = &abort_s;
     if (tid == 0) {
-        mbar_init(full, 1); mbar_init(done, 1);
-        *abort_flag = 0;
+        mbar_init(bars, 1); mbar_init(bars + 1, 1);
+        abort_s = 0;
         mbar_fence_init();
-        tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmP);
     }
     __syncwarp();
-    if (warp == 0) { tmem_alloc(tmem_holder, tmem_cols); tmem_relinquish(); }
+    if (warp == 0) { tmem_alloc(&tmem_holder, SL::TMEM_COLS); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_holder;
-    const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    constexpr uint32_t IDESC = umma_idesc_bf16(D, false);
-    constexpr uint32_t DESC_HI = umma_desc_hi_sw128(1024);
-    const uint32_t dK = umma_desc_lo(smem_u32(sK), 16), dP = umma_desc_lo(smem_u32(smem + SL::P), 16);
+    const uint32_t tC = tmem_holder, tD = tC + ET_UCOLS;
+    pdl_wait();
+    pdl_release();
+    bool ok = !__syncthreads_or(*reinterpret_cast<volatile int*>(p.status) != 0);
 
-    const int n_hot = *hot_count;
-    const long long n_work = (long long)n_hot * Hkv;
-    const long long per = (n_work + gridDim.x - 1) / gridDim.x;
-    const long long w0 = (long long)blockIdx.x * per, w1 = w0 + per < n_work ? w0 + per : n_work;
-    uint32_t n_full = 0, n_done = 0;
-    int resident = -1;          // (m, h) pair whose projector is in shared memory: m * Hkv + h
-    bool ok = true;
-    for (long long idx = w0; idx < w1 && ok; ++idx) {
-        const int h = (int)(idx / n_hot), tile = hot_list[idx % n_hot];
-        const int b = tile / n_tiles, t = tile % n_tiles;
-        const float g = gain[b];
-        if (g == 0.f || (head_enable != nullptr && head_enable[h] == 0)) continue;      // same for the whole CTA
-        const int seq0 = cu_seqlens ? cu_seqlens[b] : b * L;
-        const int Lb = (cu_seqlens ? cu_seqlens[b + 1] : (b + 1) * L) - seq0;
-        const int kpos = t * 128 + row;
-        const bool hl = kpos < Lb && mask[seq0 + kpos] != 0;
-        if (half == 0) flags[row] = hl ? 1 : 0;
-        const int nvalid = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
-        const bool with_lo = SIDE && (lo_needed(g, alpha_max_of(alpha, (size_t)b * Hkv + h, M)) || t < kLoTiles);
-        for (int m = 0; m < M && ok; ++m) {
-            const bool load_p = resident != m * Hkv + h;
-            if (m == 0 || load_p) {
-                if (tid == 0) {
-                    mbar_expect_tx(full, (m == 0 ? SL::TILE : 0u) + (load_p ? 2 * SL::PMAT : 0u));
-                    if (m == 0) {
+    uint8_t* sU = smem + SL::U;
+    constexpr uint32_t DESC_HI = umma_desc_hi_sw128(1024);
+    const uint32_t dK0 = umma_desc_lo(smem_u32(smem), 16), dU0 = umma_desc_lo(smem_u32(sU), EBLK);
+    const int row = tid & 127, half = tid >> 7;         // tensor-memory lane = key row, and which half of the columns
+    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+    const int R = r * M;
+    const bool u_vec = (r & 7) == 0 && (reinterpret_cast<uintptr_t>(p.U) & 15) == 0;
+
+    // ---------------------------------------------------- units of work
+    // The unit taken last: head, sequence, first token, rows (SIDE), whether its low parts are wanted, the flags of this
+    // thread's warp quarter, coefficient; stand-alone: chunk of the list.
+    int cur_h = 0, cur_b = 0, cur_tok0 = 0, cur_nvalid = 0, cur_lo = 0, cur_chunk = 0;
+    uint32_t cur_bits = 0;
+    float cur_c = 0.f;
+    int unit = blk, n_units = 0, n_hot = 0;
+    int look_pos = ET_WARPS;
+    if constexpr (SIDE) {
+        n_units = p.B * p.n_tiles * Hkv;
+    } else if (ok) {
+        // highlighted tokens before each segment, and in all
+        constexpr int PT = kMaxSegments / ET_THREADS;
+        int c[PT], sum = 0;
 #pragma unroll
-                        for (int c = 0; c < NBLK; ++c) tma_load_3d(sK + c * EBLK, &tmK, full, c * 64, h, seq0 + t * 128);
+        for (int q = 0; q < PT; ++q) { c[q] = tid * PT + q < p.n_seg ? p.counts[tid * PT + q] : 0; sum += c[q]; }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        if (lane == 31) wsum_s[warp] = incl;
+        __syncthreads();
+        int base = incl - sum;
+#pragma unroll
+        for (int w = 0; w < ET_WARPS; ++w) { if (w < warp) base += wsum_s[w]; n_hot += wsum_s[w]; }
+#pragma unroll
+        for (int q = 0; q < PT; ++q) { pre_s[tid * PT + q] = base; base += c[q]; }
+        __syncthreads();
+        n_units = ((n_hot + 127) / 128) * Hkv;
+    }
+    const int unit_step = SIDE ? p.n_tile_blocks : (int)gridDim.x;
+    auto next_index = [&](int u) { return u + unit_step < u ? 0x7fffffff : u + unit_step; };
+
+    // the next unit with work (false: none left); every thread gets the same answer
+    auto next_unit = [&]() -> bool {
+        if constexpr (!SIDE) {
+            while (unit < n_units) {
+                cur_chunk = unit / Hkv; cur_h = unit - cur_chunk * Hkv;
+                unit = next_index(unit);
+                if (p.head_enable == nullptr || p.head_enable[cur_h] != 0) return true;
+            }
+            return false;
+        } else {
+            while (true) {
+                if (look_pos == ET_WARPS) {             // a warp looks at each of the next eight units: one latency for all of them
+                    if (unit >= n_units) return false;
+                    __syncthreads();
+                    const long long u64 = unit + (long long)warp * unit_step;
+                    UnitInfo* info = look_s + warp;
+                    if (u64 < n_units) {
+                        const int u = (int)u64, bt = u / Hkv, h = u - bt * Hkv, b = bt / p.n_tiles, t = bt - b * p.n_tiles;
+                        const int seq0 = p.cu ? p.cu[b] : b * p.L;
+                        const int Lb = (p.cu ? p.cu[b + 1] : (b + 1) * p.L) - seq0;
+                        const float g = p.gain[b];
+                        const bool on = p.head_enable == nullptr || p.head_enable[h] != 0;
+                        const int sb = steer_byte(p.jobs.steer, b, h, Hkv);
+                        uint32_t any = 0;
+                        uint32_t bits[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int pos = t * 128 + q * 32 + lane;
+                            bits[q] = __ballot_sync(0xffffffffu, pos < Lb && p.mask[seq0 + pos] != 0);
+                            any |= bits[q];
+                        }
+                        if (lane == 0) {
+                            *reinterpret_cast<uint4*>(info->bits) = make_uint4(bits[0], bits[1], bits[2], bits[3]);
+                            info->work = (any != 0 && on && g != 0.f) ? 1 : 0;
+                            info->b = b; info->tok0 = seq0 + t * 128; info->nvalid = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
+                            info->c = g * (M == 1 && p.alpha != nullptr && !routed ? p.alpha[(size_t)b * Hkv + h] : 1.f);
+                            info->with_lo = (t < kLoTiles || (sb & 2) != 0) ? 1 : 0;
+                        }
+                        if (h == 0) {                   // what the fused kernel needs to know
+                            if (lane == 0) p.tile_hot[bt] = any != 0 ? 1 : 0;
+                            if (t == 0)
+                                for (int hh = lane; hh < Hkv; hh += 32) p.bh_info[(size_t)b * Hkv + hh] = (uint8_t)steer_byte(p.jobs.steer, b, hh, Hkv);
+                        }
+                    } else if (lane == 0) {
+                        info->work = 0;
                     }
-                    if (load_p) {
-#pragma unroll
-                        for (int part = 0; part < 2; ++part)
-#pragma unroll
-                            for (int c = 0; c < NBLK; ++c)
-                                tma_load_3d(smem + SL::P + part * SL::PMAT + c * SL::PBLK, &tmP, full, c * 64, 0,
-                                            ((part * M + m) * Hkv + h) * D);
+                    __syncthreads();
+                    look_pos = 0;
+                }
+                while (look_pos < ET_WARPS) {
+                    const int u = unit;
+                    unit = next_index(u);
+                    const UnitInfo& info = look_s[look_pos++];
+                    if (info.work) {
+                        cur_h = u % Hkv;
+                        cur_b = info.b; cur_tok0 = info.tok0; cur_nvalid = info.nvalid; cur_lo = info.with_lo; cur_c = info.c;
+                        cur_bits = info.bits[row >> 5];
+                        return true;
                     }
                 }
-                resident = m * Hkv + h;
-                ok = mbar_wait(full, n_full & 1, abort_flag, status, 60);
-                ++n_full;
-                ok = __syncthreads_and(ok);
-                if (!ok) break;
             }
+        }
+    };
+    // rows of the unit (stand-alone): the chunk's tokens, looked up in the segments (visible after the next barrier)
+    auto find_rows = [&](int st) {
+        if constexpr (!SIDE) {
+            if (tid >= 128) return;
+            const int q = cur_chunk * 128 + tid;
+            int tok = -1, b = 0;
+            float c = 0.f;
+            if (q < n_hot) {
+                int lo = 0, hi = p.n_seg - 1;           // largest segment with pre_s[seg] <= q (an empty one is never the largest)
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (pre_s[mid] <= q) lo = mid; else hi = mid - 1;
+                }
+                tok = p.list[(size_t)lo * p.seg_tokens + (q - pre_s[lo])];
+                b = find_sequence(p.cu, p.B, p.L, tok);
+                c = p.gain[b] * (M == 1 && p.alpha != nullptr ? p.alpha[(size_t)b * Hkv + cur_h] : 1.f);
+            }
+            tok_s[st][tid] = tok; seq_s[st][tid] = b; c_s[st][tid] = c;
+        }
+    };
+    // the unit's key rows on their way into stage st (128-byte swizzle; rows that do not exist are zero)
+    auto load_rows = [&](int st) {
+        const int c = tid % UPR;
+        const uint32_t base = smem_u32(smem) + st * SL::TILE + (c >> 3) * EBLK;
+#pragma unroll
+        for (int k = 0; k < 128 / RPP; ++k) {
+            const int rr = tid / UPR + k * RPP;
+            const int tok = SIDE ? cur_tok0 + rr : tok_s[st][SIDE ? 0 : rr];
+            const bool valid = SIDE ? rr < cur_nvalid : tok >= 0;
+            const size_t e = ((size_t)(valid ? tok : 0) * Hkv + cur_h) * D + c * 8;
+            const uint32_t dst = base + sw128_offset(rr, (c & 7) * 8);
+            if (sizeof(KT) == 2) {
+                cp_async16(dst, static_cast<const __nv_bfloat16*>(p.K) + e, valid);
+            } else {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b4 = a;
+                if (valid) {
+                    a = *reinterpret_cast<const float4*>(static_cast<const float*>(p.K) + e);
+                    b4 = *reinterpret_cast<const float4*>(static_cast<const float*>(p.K) + e + 4);
+                }
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pack_bf16(a.x, a.y)), "r"(pack_bf16(a.z, a.w)),
+                             "r"(pack_bf16(b4.x, b4.y)), "r"(pack_bf16(b4.z, b4.w)) : "memory");
+            }
+        }
+    };
+    // columns [j0, j0 + 64) of the stacked U of head h as two bf16 parts: [D x 64] blocks, 128-byte swizzle (K-major operand of
+    // the second product, MN-major of the first); zero up to the next multiple of 16 columns, undefined (and unused) beyond
+    auto stage_u = [&](int h, int j0) {
+        const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nu = (rc + 15) / 16 * 2;
+#pragma unroll 2
+        for (int u = tid; u < D * nu; u += ET_THREADS) {
+            const int i = u / nu, c8 = (u - i * nu) * 8;
+            float v[8];
+            if (u_vec && j0 + c8 + 8 <= R) {
+                const int m = (j0 + c8) / r, k = j0 + c8 - m * r;
+                const float4* src = reinterpret_cast<const float4*>(p.U + (((size_t)m * Hkv + h) * D + i) * r + k);
+                const float4 a = __ldg(src), b4 = __ldg(src + 1);
+                v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b4.x; v[5] = b4.y; v[6] = b4.z; v[7] = b4.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int j = j0 + c8 + e, m = j / r;
+                    v[e] = j < R ? __ldg(p.U + (((size_t)m * Hkv + h) * D + i) * r + (j - m * r)) : 0.f;
+                }
+            }
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) split_pair(v[2 * e], v[2 * e + 1], hi[e], lo[e]);
+            const uint32_t off = sw128_offset(i, c8);
+            *reinterpret_cast<uint4*>(sU + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(sU + SL::UMAT + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+        if (tid < ET_UCOLS) exp_s[tid] = (unsigned short)(j0 + tid < R ? (j0 + tid) / r : M - 1);
+    };
+
+    int st = 0, u_head = -1, routed_for = -1;           // stage, head whose only block of U is resident, (sequence, head) of the coefficients
+    uint32_t n_c = 0, n_d = 0;                          // products so far (phases)
+    float* alpha_r = reinterpret_cast<float*>(smem + SL::ROUTE);
+    bool have = ok && next_unit();
+    if (have) {
+        if (!SIDE) { find_rows(0); __syncthreads(); }
+        load_rows(0);
+    }
+    while (have) {
+        const int h = cur_h, b = cur_b, tok0 = cur_tok0, nvalid = cur_nvalid;
+        const bool with_lo = SIDE && cur_lo != 0;
+        if (u_head != h) { stage_u(h, 0); u_head = R <= ET_UCOLS ? h : -1; }
+        if (routed && routed_for != b * Hkv + h) {
+            // (the scratch starts behind the result: alpha_r holds M floats)
+            double* sm = reinterpret_cast<double*>(smem + SL::ROUTE + ((M * 4 + 15) & ~15));
+            const double* a = route_group(p.route.Q, p.route.q_is_f32, p.U, p.route.sigma, p.cu, p.L, p.route.Hq, Hkv, D, r, M,
+                                          p.route.k_route, b, h, sm);
+            for (int m = tid; m < M; m += ET_THREADS) alpha_r[m] = (float)a[m];
+            routed_for = b * Hkv + h;
+        }
+        cp_async_wait_all();
+        fence_proxy_async();
+        __syncthreads();                                // rows and U are in place
+        bool have_next = false;
+        const bool hl = SIDE ? ((cur_bits >> (row & 31)) & 1u) != 0 : tok_s[st][SIDE ? 0 : row] >= 0;
+        const float g = SIDE ? cur_c : c_s[st][SIDE ? 0 : row];
+        const int b_row = SIDE ? b : seq_s[st][SIDE ? 0 : row];
+        const bool warp_hl = __any_sync(0xffffffffu, hl);
+        for (int j0 = 0; j0 < R; j0 += ET_UCOLS) {
+            const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nks = (rc + 15) / 16;
+            if (j0 > 0) { stage_u(h, j0); fence_proxy_async(); __syncthreads(); }
             if (tid == 0) {
                 tc_fence_after();
-                // the high and the low part of the projector accumulate into the same columns
+                const uint32_t kd = dK0 + st * (SL::TILE >> 4);
+                constexpr uint32_t IDESC = umma_idesc_bf16(ET_UCOLS, true);
 #pragma unroll
                 for (int part = 0; part < 2; ++part)
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) {
-                        const uint32_t offk = ((uint32_t)(ks >> 2) * EBLK + (uint32_t)(ks & 3) * 32) >> 4;
-                        const uint32_t offp = ((uint32_t)part * SL::PMAT + (uint32_t)(ks >> 2) * SL::PBLK + (uint32_t)(ks & 3) * 32) >> 4;
-                        umma_ss(tmem_base + (uint32_t)m * D, dK + offk, DESC_HI, dP + offp, DESC_HI, IDESC, (ks > 0 || part) ? 1u : 0u);
-                    }
-                umma_commit(done);
+                    for (int ks = 0; ks < D / 16; ++ks)
+                        umma_ss(tC, kd + (((uint32_t)(ks >> 2) * EBLK + (uint32_t)(ks & 3) * 32) >> 4), DESC_HI,
+                                dU0 + (((uint32_t)part * SL::UMAT + (uint32_t)ks * 2048) >> 4), DESC_HI, IDESC, (ks > 0 || part) ? 1u : 0u);
+                umma_commit(bars);
             }
-            ok = mbar_wait(done, n_done & 1, abort_flag, status, 61);       // the projector may be replaced, K P_m may be read
-            ++n_done;
+            if (j0 == 0) {                              // under the product: what comes next
+                have_next = next_unit();
+                if (have_next) find_rows(st ^ 1);
+            }
+            ok = mbar_wait(bars, n_c & 1, abort_flag, p.status, 60);
+            ++n_c;
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok && warp_hl && half * 32 < rc) {
+                // 32 columns of C: times the row's coefficients, split, back over themselves (16 columns of high pairs, 16 of
+                // low); what the rows that are not highlighted get is never used
+                tc_fence_after();
+                const uint32_t tc = tC + lane_off + half * 32;
+                const float* a_row = routed ? alpha_r : (M > 1 && p.alpha != nullptr ? p.alpha + ((size_t)b_row * Hkv + h) * M : nullptr);
+                uint32_t v[32], hi[16], lo[16];
+                tmem_ld32(tc, v);
+                float c4[4] = {g, g, g, g};
+                if (a_row != nullptr && (r & 7) == 0) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) c4[q] *= a_row[exp_s[half * 32 + q * 8]];
+                }
+                tmem_wait_ld_on(v);
+                if (a_row != nullptr && (r & 7) != 0) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * a_row[exp_s[half * 32 + e]]);
+                }
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    split_pair(__uint_as_float(v[2 * e]) * c4[e >> 2], __uint_as_float(v[2 * e + 1]) * c4[e >> 2], hi[e], lo[e]);
+                tmem_st16(tc, hi);
+                tmem_st16(tc + 16, lo);
+                tmem_wait_st();
+            }
+            tc_fence_before();
             ok = __syncthreads_and(ok);
+            if (!ok) break;
+            if (tid == 0) {
+                tc_fence_after();
+                constexpr uint32_t IDESC = umma_idesc_bf16(D, false);
+                for (int ks = 0; ks < nks; ++ks) {
+                    const uint32_t a_hi = tC + (uint32_t)(ks >> 1) * 32 + (uint32_t)(ks & 1) * 8, a_lo = a_hi + 16;
+                    const uint32_t u_hi = dU0 + (((uint32_t)ks * 32) >> 4), u_lo = u_hi + (SL::UMAT >> 4);
+                    umma_ts(tD, a_hi, u_hi, DESC_HI, IDESC, (j0 > 0 || ks > 0) ? 1u : 0u);
+                    umma_ts(tD, a_lo, u_hi, DESC_HI, IDESC, 1u);
+                    umma_ts(tD, a_hi, u_lo, DESC_HI, IDESC, 1u);
+                }
+                umma_commit(bars + 1);
+            }
+            if (NS == 2 && j0 == 0 && have_next) load_rows(st ^ 1);
+            ok = mbar_wait(bars + 1, n_d & 1, abort_flag, p.status, 61);
+            ++n_d;
+            ok = __all_sync(0xffffffffu, ok);
+            if (R > ET_UCOLS) { ok = __syncthreads_and(ok); if (!ok) break; }      // (U is replaced next)
         }
-        if (!ok) break;
-        tc_fence_after();
-        // this thread's half row: k' = k + g sum_m alpha_m (K P_m)[row]
-        // (the tensor-memory loads are warp-wide instructions: every lane of a warp that has a highlighted row
-        // takes part in them, only the update of the row itself depends on the lane's own flag)
-        const bool warp_hl = __any_sync(0xffffffffu, hl);
-        if (warp_hl || with_lo) {
-            const bool side_lo = with_lo && row < nvalid;
-            __nv_bfloat16* xlo = K_out + ((size_t)(seq0 + t * 128 + (row < nvalid ? row : 0)) * Hkv + h) * (2 * D) + D;
+        if (!ok && R > ET_UCOLS) break;
+        uint8_t* sK = smem + st * SL::TILE;
+        uint8_t* sL = smem + SL::LO;
+        if (ok && (warp_hl || with_lo)) {
+            // k' = k + dK[row] for highlighted rows, half a row per thread, in place in the staged rows; low parts beside them
+            tc_fence_after();
 #pragma unroll 1
             for (int c = half * (D / 64); c < (half + 1) * (D / 64); ++c) {
-                float dk[32];
+                uint32_t v[32];
+                if (warp_hl) { tmem_ld32(tD + lane_off + c * 32, v); tmem_wait_ld_on(v); }     // warp-wide: every lane takes part
 #pragma unroll
-                for (int e = 0; e < 32; ++e) dk[e] = 0.f;
-                for (int m = 0; m < M && warp_hl; ++m) {
-                    const float cm = g * (alpha != nullptr ? alpha[((size_t)b * Hkv + h) * M + m] : 1.f);
-                    uint32_t v[32];
-                    tmem_ld32(t_lane + (uint32_t)m * D + c * 32, v);
-                    tmem_wait_ld_on(v);
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) dk[e] = fmaf(cm, __uint_as_float(v[e]), dk[e]);
-                }
-                uint4 lo4[4];
-                if (SIDE) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) lo4[q] = make_uint4(0u, 0u, 0u, 0u);
-                }
-                if (hl) {
-                    uint4* ptr[4];
-                    uint4 kv[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {      // 8 elements = one 16-byte unit of the swizzled row; reads before writes
-                        const int col = c * 32 + q * 8;
-                        ptr[q] = reinterpret_cast<uint4*>(sK + (col >> 6) * EBLK + sw128_offset(row, col & 63));
-                        kv[q] = *ptr[q];
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        uint32_t* w = reinterpret_cast<uint32_t*>(&kv[q]);
-                        uint32_t* l = reinterpret_cast<uint32_t*>(&lo4[q]);
+                for (int q = 0; q < 4; ++q) {          // 8 elements = one 16-byte unit of the swizzled row
+                    const uint32_t off = (uint32_t)((c * 32 + q * 8) >> 6) * EBLK + sw128_offset(row, (c * 32 + q * 8) & 63);
+                    uint4 l = make_uint4(0u, 0u, 0u, 0u);
+                    if (hl) {
+                        uint4 kv = *reinterpret_cast<uint4*>(sK + off);
+                        uint32_t* w = reinterpret_cast<uint32_t*>(&kv);
+                        uint32_t* lw = reinterpret_cast<uint32_t*>(&l);
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const float2 k2 = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[e]));
-                            const float x0 = k2.x + dk[q * 8 + 2 * e], x1 = k2.y + dk[q * 8 + 2 * e + 1];
-                            w[e] = pack_bf16(x0, x1);
-                            if (SIDE) {        // the low parts: what the rounding above dropped
-                                const float2 h2 = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[e]));
-                                l[e] = pack_bf16(x0 - h2.x, x1 - h2.y);
-                            }
+                            const float x0 = k2.x + __uint_as_float(v[q * 8 + 2 * e]), x1 = k2.y + __uint_as_float(v[q * 8 + 2 * e + 1]);
+                            if (SIDE) split_pair(x0, x1, w[e], lw[e]); else w[e] = pack_bf16(x0, x1);
                         }
+                        *reinterpret_cast<uint4*>(sK + off) = kv;
                     }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) *ptr[q] = kv[q];
-                }
-                if (SIDE && side_lo) {
-                    uint4* dst = reinterpret_cast<uint4*>(xlo + c * 32);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) dst[q] = lo4[q];
+                    if (with_lo) *reinterpret_cast<uint4*>(sL + off) = l;
                 }
                 __syncwarp();      // all lanes together again before the next warp-wide load
             }
         }
         tc_fence_before();
-        __syncthreads();
-        // write the highlighted rows out: D / 8 lanes per row, 16 bytes each; 16 rows per warp
-        constexpr int LPR = D / 8, RPI = 32 / LPR;
-#pragma unroll 1
-        for (int i = 0; i < 16 / RPI; ++i) {
-            const int r = warp * 16 + i * RPI + lane / LPR, col = (lane % LPR) * 8;
-            if (SIDE ? r < nvalid : flags[r] != 0) {
-                const uint4 v = *reinterpret_cast<const uint4*>(sK + (col >> 6) * EBLK + sw128_offset(r, col & 63));
-                *reinterpret_cast<uint4*>(K_out + ((size_t)(seq0 + t * 128 + r) * Hkv + h) * (SIDE ? 2 * D : D) + col) = v;
+        ok = __syncthreads_and(ok);
+        if (!ok) break;
+        // write the rows out: D / 8 lanes per row, 16 bytes each
+#pragma unroll 4
+        for (int k = 0; k < 128 / RPP; ++k) {
+            const int rr = tid / UPR + k * RPP, c = tid % UPR;
+            const int tok = SIDE ? tok0 + rr : tok_s[st][SIDE ? 0 : rr];
+            if (SIDE ? rr < nvalid : tok >= 0) {
+                const uint32_t off = (uint32_t)(c >> 3) * EBLK + sw128_offset(rr, (c & 7) * 8);
+                __nv_bfloat16* dst = p.out + ((size_t)tok * Hkv + h) * (SIDE ? 2 * D : D) + c * 8;
+                *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(sK + off);
+                if (with_lo) *reinterpret_cast<uint4*>(dst + D) = *reinterpret_cast<const uint4*>(sL + off);
             }
         }
-        __syncthreads();        // the tile and the flags are reused by the next step
+        have = have_next;
+        if (NS == 2) {
+            st ^= 1;                   // (this stage and the low parts are written again behind two barriers of the next step)
+        } else if (have) {
+            __syncthreads();
+            load_rows(0);
+        }
     }
+    cp_async_wait_all();
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
-        __syncwarp();
-        tmem_dealloc(tmem_base, tmem_cols);
-    }
+    if (warp == 0) tmem_dealloc(tC, SL::TMEM_COLS);
 }
 
-// ---------------------------------------------------------------- single projector (plain SEKA): the same work as a pipeline
+// List of the highlighted tokens (of sequences with a gain), a block per segment of consecutive tokens; with a second output
+// tensor further blocks copy the keys meanwhile (the rows that change are overwritten by the launch behind).
+__global__ void __launch_bounds__(256)
+edit_scan_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ gain, const int* __restrict__ cu, int T, int B, int L,
+                 int* __restrict__ list, int* __restrict__ counts, int seg_tokens, int n_seg, const uint4* __restrict__ src,
+                 uint4* __restrict__ dst, size_t n16) {
+    pdl_wait();
+    pdl_release();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if ((int)blockIdx.x >= n_seg) {
+        const size_t step = (size_t)(gridDim.x - n_seg) * 256;
+        for (size_t i0 = (size_t)(blockIdx.x - n_seg) * 256 + tid; i0 < n16; i0 += 4 * step) {
+            uint4 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i0 + q * step < n16) v[q] = src[i0 + q * step];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i0 + q * step < n16) dst[i0 + q * step] = v[q];
+        }
+        return;
+    }
+    __shared__ int wsum[8];
+    const int s0 = blockIdx.x * seg_tokens;
+    int* out = list + s0;
+    int total = 0;
+    for (int t0 = s0; t0 < s0 + seg_tokens && t0 < T; t0 += 1024) {        // 1024 tokens a round, four per thread
+        const int t = t0 + tid * 4;
+        unsigned bits = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) bits |= (t + q < T && mask[t + q] != 0) ? 1u << q : 0u;
+        if (bits != 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (((bits >> q) & 1u) && gain[find_sequence(cu, B, L, t + q)] == 0.f) bits &= ~(1u << q);
+        }
+        const int cnt = __popc(bits);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        int base = total + incl - cnt;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) { if (w < warp) base += wsum[w]; total += wsum[w]; }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if ((bits >> q) & 1u) out[base++] = t + q;
+        __syncthreads();
+    }
+    if (tid == 0) counts[blockIdx.x] = total;
+}
+
+template <int D, bool SIDE, typename KT>
+static seka_status launch_tiles_t(TileArgs& a, long long n_units, size_t smem, int extra_blocks, cudaStream_t st) {
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
+    auto kern = edit_tiles_kernel<D, SIDE, KT>;
+    if (smem > 220 * 1024) return SEKA_ERR_UNSUPPORTED;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
+    long long per_sm = (227 * 1024) / (smem + (SIDE ? 4 : 9) * 1024);
+    per_sm = per_sm > EtSmem<D, SIDE>::CTAS ? EtSmem<D, SIDE>::CTAS : (per_sm < 1 ? 1 : per_sm);
+    // one wave; a multiple of the KV heads, so that a CTA keeps its head (and its block of U)
+    long long g = per_sm * n_sm;
+    if (g > a.Hkv) g -= g % a.Hkv;
+    if (g > n_units) g = n_units;
+    a.n_tile_blocks = (int)g;
+    return launch_kernel(true, kern, (unsigned)(g + extra_blocks), ET_THREADS, smem, st, a);
+}
+
+template <int D, bool SIDE>
+static size_t tiles_smem(const seka_shape* s, bool routed, int k_route) {
+    return 1024 + EtSmem<D, SIDE>::ROUTE + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
+}
+
+static TileArgs tile_args(const seka_shape* s, const WorkspaceLayout& w, const void* K, void* out, const uint8_t* mask, const float* U,
+                          const float* alpha, const float* gain, const uint8_t* he, char* ws) {
+    TileArgs a = {};
+    a.K = K; a.out = static_cast<__nv_bfloat16*>(out);
+    a.mask = mask; a.U = U; a.alpha = alpha; a.gain = gain; a.head_enable = he; a.cu = s->cu_seqlens;
+    a.list = reinterpret_cast<int*>(ws + w.list_off); a.counts = reinterpret_cast<int*>(ws + w.count_off);
+    a.seg_tokens = edit_segment_tokens(shape_total_tokens(s));
+    a.n_seg = (shape_total_tokens(s) + a.seg_tokens - 1) / a.seg_tokens;
+    a.tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off); a.bh_info = reinterpret_cast<uint8_t*>(ws + w.info_off);
+    a.status = reinterpret_cast<int*>(ws);
+    a.B = s->batch; a.L = s->max_seqlen; a.Hkv = s->n_kv_heads; a.r = s->rank; a.M = s->n_experts; a.n_tiles = w.n_tiles;
+    return a;
+}
+
+static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout& w, const void* K_in, void* K_out, const uint8_t* mask,
+                                     const float* U, const float* alpha, const float* gain, const uint8_t* he, char* ws, cudaStream_t st) {
+    const int T = shape_total_tokens(s), Hkv = s->n_kv_heads, D = s->head_dim;
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
+    TileArgs a = tile_args(s, w, K_out, K_out, mask, U, alpha, gain, he, ws);
+    const bool copy = K_in != K_out;
+    const size_t n16 = copy ? (size_t)T * Hkv * D / 8 : 0;
+    size_t n_copy = (n16 + 4 * 256 - 1) / (4 * 256);
+    if (n_copy > (size_t)n_sm * 8) n_copy = (size_t)n_sm * 8;
+    seka_status stc = launch_kernel(true, edit_scan_kernel, (unsigned)(a.n_seg + n_copy), 256, 0, st, mask, gain, s->cu_seqlens, T, s->batch,
+                                    s->max_seqlen, const_cast<int*>(a.list), const_cast<int*>(a.counts), a.seg_tokens, a.n_seg,
+                                    static_cast<const uint4*>(K_in), static_cast<uint4*>(K_out), n16);
+    if (stc != SEKA_OK) return stc;
+    const long long units = (long long)((T + 127) / 128) * Hkv;
+    return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16>(a, units, tiles_smem<128, false>(s, false, 0), 0, st)
+                    : launch_tiles_t<64, false, __nv_bfloat16>(a, units, tiles_smem<64, false>(s, false, 0), 0, st);
+}
+
+// ---------------------------------------------------------------- many tiles, one projector: the preparation as a pipeline
 //
-// One persistent CTA per SM with three roles, so that several key tiles are in flight per SM and the tensor-core
-// product of one tile runs under the drain and write-out of the one before:
-//   warp 8   producer: walks this CTA's run of (KV head, highlighted tile) pairs, stages key tiles through a ring of
-//            NS shared-memory stages by TMA, writes the rows' highlight flags and the tile's coordinates beside them,
-//            and (re)loads the projector when the head changes (after the ring has drained);
+// Where the tiles of a plain-SEKA forward are many waves of CTAs, the chain above is bound by its instruction latencies
+// (about 5000 cycles per tile and SM at head_dim 64).  There one persistent CTA per SM with three roles does the same work from
+// the projector P[h] = U_h U_h^T (two bf16 parts, formed by the launch before), about 2700 cycles per tile and SM:
+//   warp 8   producer: walks this CTA's (sequence, tile) pairs of one KV head, stages the key tiles that hold a highlighted
+//            token through a ring of NS shared-memory stages by TMA, with the rows' highlight flags beside them;
 //   warp 9   MMA issuer: K P (two bf16 parts) into one of two sets of tensor-memory columns;
-//   warps 0-7  drain: half a key row per thread, k' = k + c (K P)[row] into the staged tile for highlighted rows,
-//            then the highlighted rows go out 16 bytes per lane; the stage and the columns are handed back.
+//   warps 0-7  drain: half a key row per thread, k' = k + c (K P)[row] into the staged tile for highlighted rows, low parts
+//            straight to global memory, then the rows go out 16 bytes per lane; stage and columns are handed back.
 constexpr int EP_THREADS = 320;
 
-struct EpMeta { int tok0, h, valid, p_gen; float c; int nvalid, with_lo, pad; };     // per stage: first token, head, end marker, projector generation, g * alpha, rows inside the sequence, low parts wanted (side mode)
+// per stage: highlighted rows, first token, rows inside the sequence, end marker, low parts wanted, g * alpha
+struct __align__(16) EpMeta { uint32_t bits[4]; int tok0, nvalid, valid, with_lo; float c; int pad[3]; };
 
 template <int D>
 struct EpSmem {
@@ -481,24 +827,19 @@ struct EpSmem {
     static constexpr int NS = D == 128 ? 4 : 8;             // key tiles in flight per SM
     static constexpr uint32_t K = 0;                        // NS stages
     static constexpr uint32_t P = K + NS * TILE;            // high part, then low part
-    static constexpr uint32_t FLAGS = P + 2 * PMAT;         // NS x 128 bytes
-    static constexpr uint32_t META = FLAGS + NS * 128;      // NS x 32 bytes
-    static constexpr uint32_t BARS = META + NS * 32;        // full[NS], free[NS], mma_done[2], cols_free[2], p_full, meet[2]
+    static constexpr uint32_t META = P + 2 * PMAT;          // NS x 48 bytes
+    static constexpr uint32_t BARS = META + NS * 48;        // full[NS], free[NS], mma_done[2], cols_free[2], p_full, meet[2]
     static constexpr uint32_t NBARS = 2 * NS + 7;
     static constexpr uint32_t MISC = BARS + NBARS * 8;
     static constexpr uint32_t DYN_BYTES = MISC + 16 + 1024;
 };
 
-// SIDE: instead of rewriting the highlighted rows of the key tensor, write k' of every row of the tile that lies inside
-// its sequence into the side buffer of the fused forward, rows of 2 D bf16: high parts [0, D), low parts [D, 2 D) (the low
-// parts only where the fused kernel reads them: see lo_needed; zero for rows that are not highlighted).
-template <int D, bool SIDE>
+template <int D>
 __global__ void __launch_bounds__(EP_THREADS, 1)
-edit_tiles_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmP,
-                       __nv_bfloat16* __restrict__ K_out, const uint8_t* __restrict__ mask, const float* __restrict__ alpha,
-                       const float* __restrict__ gain, const uint8_t* __restrict__ head_enable,
-                       const int* __restrict__ cu_seqlens, const int* __restrict__ hot_list, const int* __restrict__ hot_count,
-                       int* status, int L, int Hkv, int n_tiles) {
+stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmP, __nv_bfloat16* __restrict__ X,
+                       const uint8_t* __restrict__ mask, const float* __restrict__ alpha, const float* __restrict__ gain,
+                       const uint8_t* __restrict__ head_enable, const int* __restrict__ cu_seqlens,
+                       const uint8_t* __restrict__ tile_hot, int* status, int B, int L, int Hkv, int n_tiles) {
     using SL = EpSmem<D>;
     constexpr int EP_NS = SL::NS;
     constexpr int NBLK = D / 64;
@@ -515,8 +856,6 @@ edit_tiles_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + SL::MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::MISC + 4);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (__syncthreads_or(*reinterpret_cast<volatile int*>(status) != 0)) return;
-
     if (tid == 0) {
         for (int i = 0; i < EP_NS; ++i) { mbar_init(full + i, 2); mbar_init(freeb + i, 8); }
         for (int i = 0; i < 2; ++i) { mbar_init(mma_done + i, 1); mbar_init(cols_free + i, 8); mbar_init(meetb + i, 8); }
@@ -531,135 +870,104 @@ edit_tiles_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    pdl_wait();
+    pdl_release();
+    const bool dead = __syncthreads_or(*reinterpret_cast<volatile int*>(status) != 0);
 
-    if (warp == 8) {
+    if (dead) {
+        // an earlier launch gave up on this workspace
+    } else if (warp == 8) {
         // ------------------------------------------------------------ producer
-        const int n_hot = *hot_count;
-        const long long n_work = (long long)n_hot * Hkv;
-        const long long per = (n_work + gridDim.x - 1) / gridDim.x;
-        long long w0 = (long long)blockIdx.x * per;
-        if (w0 > n_work) w0 = n_work;                 // a CTA without work still pushes the end marker
-        const long long w1 = w0 + per < n_work ? w0 + per : n_work;
+        // Its units are (sequence, tile) pairs blk, blk + n, ... of one KV head (the grid is a multiple of Hkv).  One lane per
+        // unit fetches what a unit needs from global memory (flag, sequence bounds) for 32 units at a time; the highlight
+        // flags of a tile's rows are requested one tile ahead, so that the ring is not fed at the pace of memory round trips.
+        const int h = (int)blockIdx.x % Hkv, bt_step = (int)gridDim.x / Hkv, n_bt = B * n_tiles;
         uint32_t n_push = 0;      // stages filled so far
-        int p_gen = 0, cur_h = -1;
         bool ok = true;
-        // What a work unit needs from global memory (its entry of the list, the sequence bounds, gain, coefficient) is a
-        // chain of dependent loads; one lane per unit fetches it for 32 units at a time, and the highlight flags of a
-        // tile are requested one tile ahead, so that the ring is not fed at the pace of memory round trips.
-        uint8_t fl_next[4] = {0, 0, 0, 0};
-        bool have_next = false;
-        for (long long base = w0; base <= w1 && ok; base += 32) {
-            int h_l = 0, t_l = 0, seq0_l = 0, Lb_l = 0, lo_l = 0, skip_l = 1;
-            float c_l = 0.f;
-            {
-                const long long my = base + lane;
-                if (my < w1) {
-                    h_l = (int)(my / n_hot);
-                    const int tile = hot_list[my % n_hot];
-                    const int b = tile / n_tiles;
-                    t_l = tile % n_tiles;
-                    const float g = gain[b];
-                    const float a = alpha != nullptr ? alpha[(size_t)b * Hkv + h_l] : 1.f;
-                    skip_l = (g == 0.f || (head_enable != nullptr && head_enable[h_l] == 0)) ? 1 : 0;
-                    c_l = g * a;
-                    seq0_l = cu_seqlens ? cu_seqlens[b] : b * L;
-                    Lb_l = (cu_seqlens ? cu_seqlens[b + 1] : (b + 1) * L) - seq0_l;
-                    lo_l = (SIDE && (lo_needed(g, fabsf(a)) || t_l < kLoTiles)) ? 1 : 0;
-                }
+        const bool on = head_enable == nullptr || head_enable[h] != 0;
+        if (lane == 0 && on) {
+            mbar_expect_tx(p_full, 2 * SL::PMAT);
+#pragma unroll
+            for (int part = 0; part < 2; ++part)
+#pragma unroll
+                for (int cb = 0; cb < NBLK; ++cb)
+                    tma_load_3d(smem + SL::P + part * SL::PMAT + cb * SL::PBLK, &tmP, p_full, cb * 64, 0, (part * Hkv + h) * D);
+        }
+        __syncwarp();
+        auto push = [&](bool last, int tok0, int nvalid, int with_lo, float c, const uint32_t (&bits)[4]) {
+            const uint32_t s = n_push % EP_NS;
+            if (n_push >= EP_NS) {
+                ok = warp_wait(freeb + s, ((n_push / EP_NS) - 1) & 1, abort_flag, status, 63);
+                if (!ok) return;
             }
-            const int n_here = (int)((w1 - base + 1) < 32 ? (w1 - base + 1) : 32);      // units of this batch, end marker included
+            if (lane == 0) {
+                EpMeta* m = reinterpret_cast<EpMeta*>(smem + SL::META + s * 48);
+                m->tok0 = tok0; m->valid = last ? 0 : 1; m->c = c; m->nvalid = nvalid; m->with_lo = with_lo;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) m->bits[q] = bits[q];
+                if (!last) {
+                    mbar_expect_tx(full + s, SL::TILE);
+#pragma unroll
+                    for (int cb = 0; cb < NBLK; ++cb) tma_load_3d(smem + SL::K + s * SL::TILE + cb * EBLK, &tmK, full + s, cb * 64, h, tok0);
+                } else {
+                    mbar_arrive(full + s);
+                }
+                mbar_arrive(full + s);       // second arrival: flags and coordinates are in place
+            }
+            __syncwarp();
+            ++n_push;
+        };
+        for (long long base = (int)blockIdx.x / Hkv; base < n_bt && ok && on; base += 32LL * bt_step) {
+            const long long my = base + (long long)lane * bt_step;
+            int tok0_l = 0, nv_l = 0, lo_l = 0, hot_l = 0;
+            float c_l = 0.f;
+            if (my < n_bt) {
+                const int bt = (int)my, b = bt / n_tiles, t = bt - b * n_tiles;
+                const int seq0 = cu_seqlens ? cu_seqlens[b] : b * L;
+                const int Lb = (cu_seqlens ? cu_seqlens[b + 1] : (b + 1) * L) - seq0;
+                const float g = gain[b], a = alpha != nullptr ? alpha[(size_t)b * Hkv + h] : 1.f;
+                hot_l = (tile_hot[bt] != 0 && g != 0.f) ? 1 : 0;
+                c_l = g * a;
+                tok0_l = seq0 + t * 128; nv_l = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
+                lo_l = (lo_needed(g, fabsf(a)) || t < kLoTiles) ? 1 : 0;
+            }
+            unsigned todo = __ballot_sync(0xffffffffu, hot_l != 0);
+            uint32_t bits[4] = {0, 0, 0, 0};
             auto flags_of = [&](int k, uint8_t (&f)[4]) {      // highlight flags of unit k of the batch (4 rows per lane)
-                const int seq0 = __shfl_sync(0xffffffffu, seq0_l, k), t = __shfl_sync(0xffffffffu, t_l, k), Lb = __shfl_sync(0xffffffffu, Lb_l, k);
+                const int tok0 = __shfl_sync(0xffffffffu, tok0_l, k), nv = __shfl_sync(0xffffffffu, nv_l, k);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int kpos = t * 128 + q * 32 + lane;
-                    f[q] = (kpos < Lb && mask[seq0 + kpos] != 0) ? 1 : 0;
-                }
+                for (int q = 0; q < 4; ++q) f[q] = q * 32 + lane < nv ? mask[tok0 + q * 32 + lane] : 0;
             };
-            for (int k = 0; k < n_here && ok; ++k) {
-                const long long idx = base + k;
-                const bool last = idx >= w1;                    // one more stage after the work: the end marker
-                const int h = __shfl_sync(0xffffffffu, h_l, k), t = __shfl_sync(0xffffffffu, t_l, k);
-                const int seq0 = __shfl_sync(0xffffffffu, seq0_l, k), Lb = __shfl_sync(0xffffffffu, Lb_l, k);
-                const int with_lo = __shfl_sync(0xffffffffu, lo_l, k), skip = __shfl_sync(0xffffffffu, skip_l, k);
-                const float c = __shfl_sync(0xffffffffu, c_l, k);
-                uint8_t fl_cur[4] = {0, 0, 0, 0};
-                if (!last) {
-                    if (have_next) {
+            uint8_t fl[4];
+            if (todo) flags_of(__ffs(todo) - 1, fl);
+            while (todo && ok) {
+                const int k = __ffs(todo) - 1;
+                todo &= todo - 1;
+                uint8_t fl_next[4] = {0, 0, 0, 0};
+                if (todo) flags_of(__ffs(todo) - 1, fl_next);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) fl_cur[q] = fl_next[q];
-                    } else {
-                        flags_of(k, fl_cur);
-                    }
-                }
-                // the flags of the next unit of the batch are requested now and used in the next trip
-                have_next = k + 1 < n_here && base + k + 1 < w1;
-                if (have_next) flags_of(k + 1, fl_next);
-                if (!last) {
-                    if (skip) continue;
-                    if (h != cur_h) {
-                        // the projector changes: every tile of the old head must be through the tensor core (here: the
-                        // whole ring handed back), then the new one is loaded
-                        for (uint32_t q = n_push >= EP_NS ? n_push - EP_NS : 0; q < n_push && ok; ++q)
-                            ok = warp_wait(freeb + q % EP_NS, (q / EP_NS) & 1, abort_flag, status, 62);
-                        if (!ok) break;
-                        if (lane == 0) {
-                            mbar_expect_tx(p_full, 2 * SL::PMAT);
-#pragma unroll
-                            for (int part = 0; part < 2; ++part)
-#pragma unroll
-                                for (int cb = 0; cb < NBLK; ++cb)
-                                    tma_load_3d(smem + SL::P + part * SL::PMAT + cb * SL::PBLK, &tmP, p_full, cb * 64, 0, (part * Hkv + h) * D);
-                        }
-                        __syncwarp();
-                        cur_h = h; ++p_gen;
-                    }
-                }
-                const uint32_t s = n_push % EP_NS;
-                if (n_push >= EP_NS) {
-                    ok = warp_wait(freeb + s, ((n_push / EP_NS) - 1) & 1, abort_flag, status, 63);
-                    if (!ok) break;
-                }
-                uint8_t* fl = smem + SL::FLAGS + s * 128;
-                if (!last) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) fl[q * 32 + lane] = fl_cur[q];
-                }
-                if (lane == 0) {
-                    EpMeta* m = reinterpret_cast<EpMeta*>(smem + SL::META + s * 32);
-                    m->tok0 = seq0 + t * 128; m->h = h; m->valid = last ? 0 : 1; m->p_gen = p_gen; m->c = c;
-                    m->nvalid = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
-                    m->with_lo = last ? 0 : with_lo;
-                    if (!last) {
-                        mbar_expect_tx(full + s, SL::TILE);
-#pragma unroll
-                        for (int cb = 0; cb < NBLK; ++cb) tma_load_3d(smem + SL::K + s * SL::TILE + cb * EBLK, &tmK, full + s, cb * 64, h, seq0 + t * 128);
-                    } else {
-                        mbar_arrive(full + s);
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(full + s);       // second arrival: flags and coordinates are in place
-                ++n_push;
+                for (int q = 0; q < 4; ++q) { bits[q] = __ballot_sync(0xffffffffu, fl[q] != 0); fl[q] = fl_next[q]; }
+                push(false, __shfl_sync(0xffffffffu, tok0_l, k), __shfl_sync(0xffffffffu, nv_l, k), __shfl_sync(0xffffffffu, lo_l, k),
+                     __shfl_sync(0xffffffffu, c_l, k), bits);
             }
         }
+        if (ok) { const uint32_t none[4] = {0, 0, 0, 0}; push(true, 0, 0, 0, 0.f, none); }      // the end marker
+        if (on) warp_wait(p_full, 0, abort_flag, status, 62);      // (a CTA without work leaves only when the projector has landed)
     } else if (warp == 9) {
         // ------------------------------------------------------------ MMA issuer
         constexpr uint32_t IDESC = umma_idesc_bf16(D, false);
         constexpr uint32_t DESC_HI = umma_desc_hi_sw128(1024);
         const uint32_t dK = umma_desc_lo(smem_u32(smem + SL::K), 16), dP = umma_desc_lo(smem_u32(smem + SL::P), 16);
-        int seen_gen = 0;
         bool ok = true;
         for (uint32_t n = 0; ok; ++n) {
             const uint32_t s = n % EP_NS, cset = n & 1;
             ok = warp_wait(full + s, (n / EP_NS) & 1, abort_flag, status, 64);
             if (!ok) break;
-            const EpMeta m = *reinterpret_cast<const EpMeta*>(smem + SL::META + s * 32);
+            const EpMeta m = *reinterpret_cast<const EpMeta*>(smem + SL::META + s * 48);
             if (!m.valid) break;
-            if (m.p_gen != seen_gen) {
-                ok = warp_wait(p_full, (uint32_t)(m.p_gen - 1) & 1, abort_flag, status, 65);
+            if (n == 0) {
+                ok = warp_wait(p_full, 0, abort_flag, status, 65);
                 if (!ok) break;
-                seen_gen = m.p_gen;
             }
             if (n >= 2) {
                 ok = warp_wait(cols_free + cset, ((n >> 1) - 1) & 1, abort_flag, status, 66);
@@ -682,66 +990,44 @@ edit_tiles_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         }
     } else if (warp < 8) {
         // ------------------------------------------------------------ drain and write-out
-        const int row = tid & 127, half = tid >> 7;
+        const int row = tid & 127, half = tid >> 7, h = (int)blockIdx.x % Hkv;
         const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         bool ok = true;
         for (uint32_t n = 0; ok; ++n) {
             const uint32_t s = n % EP_NS, cset = n & 1;
             ok = warp_wait(full + s, (n / EP_NS) & 1, abort_flag, status, 67);
             if (!ok) break;
-            const EpMeta m = *reinterpret_cast<const EpMeta*>(smem + SL::META + s * 32);
+            const EpMeta m = *reinterpret_cast<const EpMeta*>(smem + SL::META + s * 48);
             if (!m.valid) break;
             uint8_t* sK = smem + SL::K + s * SL::TILE;
-            const uint8_t* fl = smem + SL::FLAGS + s * 128;
-            const bool hl = fl[row] != 0;
+            const uint32_t hl_bits = reinterpret_cast<const EpMeta*>(smem + SL::META + s * 48)->bits[warp & 3];
+            const bool hl = ((hl_bits >> lane) & 1u) != 0, warp_hl = hl_bits != 0, with_lo = m.with_lo != 0;
             ok = warp_wait(mma_done + cset, (n >> 1) & 1, abort_flag, status, 68);
             if (!ok) break;
             tc_fence_after();
-            // (the tensor-memory loads are warp-wide: every lane takes part, only the row update depends on the flag)
-            const bool side_lo = SIDE && m.with_lo != 0 && row < m.nvalid;
-            __nv_bfloat16* xlo = K_out + ((size_t)(m.tok0 + (row < m.nvalid ? row : 0)) * Hkv + m.h) * (2 * D) + D;
-            if (__any_sync(0xffffffffu, hl) || (SIDE && m.with_lo != 0)) {
-                const bool warp_hl = __any_sync(0xffffffffu, hl);
+            const bool side_lo = with_lo && row < m.nvalid;
+            __nv_bfloat16* xlo = X + ((size_t)(m.tok0 + (row < m.nvalid ? row : 0)) * Hkv + h) * (2 * D) + D;
+            if (warp_hl || with_lo) {
 #pragma unroll 1
                 for (int c = half * (D / 64); c < (half + 1) * (D / 64); ++c) {
                     uint32_t v[32];
-                    if (warp_hl) { tmem_ld32(t_lane + cset * D + c * 32, v); tmem_wait_ld_on(v); }
-                    uint4 lo4[4];
-                    if (SIDE) {
+                    if (warp_hl) { tmem_ld32(t_lane + cset * D + c * 32, v); tmem_wait_ld_on(v); }     // warp-wide: every lane takes part
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) lo4[q] = make_uint4(0u, 0u, 0u, 0u);
-                    }
-                    if (hl) {
-                        uint4* ptr[4];
-                        uint4 kv[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {      // 8 elements = one 16-byte unit of the swizzled row; reads before writes
-                            const int col = c * 32 + q * 8;
-                            ptr[q] = reinterpret_cast<uint4*>(sK + (col >> 6) * EBLK + sw128_offset(row, col & 63));
-                            kv[q] = *ptr[q];
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            uint32_t* w = reinterpret_cast<uint32_t*>(&kv[q]);
-                            uint32_t* l = reinterpret_cast<uint32_t*>(&lo4[q]);
+                    for (int q = 0; q < 4; ++q) {          // 8 elements = one 16-byte unit of the swizzled row
+                        const int col = c * 32 + q * 8;
+                        uint32_t lo[4] = {0u, 0u, 0u, 0u};
+                        if (hl) {
+                            uint4* ptr = reinterpret_cast<uint4*>(sK + (col >> 6) * EBLK + sw128_offset(row, col & 63));
+                            uint4 kv = *ptr;
+                            uint32_t* w = reinterpret_cast<uint32_t*>(&kv);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 const float2 k2 = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[e]));
-                                const float x0 = fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e]), k2.x), x1 = fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e + 1]), k2.y);
-                                w[e] = pack_bf16(x0, x1);
-                                if (SIDE) {        // the low parts: what the rounding above dropped
-                                    const float2 h2 = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[e]));
-                                    l[e] = pack_bf16(x0 - h2.x, x1 - h2.y);
-                                }
+                                split_pair(fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e]), k2.x), fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e + 1]), k2.y), w[e], lo[e]);
                             }
+                            *ptr = kv;
                         }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) *ptr[q] = kv[q];
-                    }
-                    if (side_lo) {
-                        uint4* dst = reinterpret_cast<uint4*>(xlo + c * 32);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) dst[q] = lo4[q];
+                        if (side_lo) *reinterpret_cast<uint4*>(xlo + col) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                     }
                     __syncwarp();      // all lanes together again before the next warp-wide load
                 }
@@ -756,9 +1042,9 @@ edit_tiles_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 #pragma unroll 1
             for (int i = 0; i < 16 / RPI; ++i) {
                 const int r = warp * 16 + i * RPI + lane / LPR, col = (lane % LPR) * 8;
-                if (SIDE ? r < m.nvalid : fl[r] != 0) {
+                if (r < m.nvalid) {
                     const uint4 v = *reinterpret_cast<const uint4*>(sK + (col >> 6) * EBLK + sw128_offset(r, col & 63));
-                    *reinterpret_cast<uint4*>(K_out + ((size_t)(m.tok0 + r) * Hkv + m.h) * (SIDE ? 2 * D : D) + col) = v;
+                    *reinterpret_cast<uint4*>(X + ((size_t)(m.tok0 + r) * Hkv + h) * (2 * D) + col) = v;
                 }
             }
             __syncwarp();
@@ -773,102 +1059,122 @@ edit_tiles_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     }
 }
 
-template <int D>
-static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout& w, const void* K_in, void* K_out,
-                                     const uint8_t* mask, const float* U, const float* alpha, const float* gain,
-                                     const uint8_t* he, char* ws, cudaStream_t st) {
-    using SL = EditSmem<D>;
-    // per-device facts: looked up per device; function attributes set on every call (they belong to the current device)
-    int n_sm = 0;
-    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
-    if (cudaFuncSetAttribute(edit_tiles_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SL::DYN_BYTES) != cudaSuccess)
-        return SEKA_ERR_CUDA;
-    int* status = reinterpret_cast<int*>(ws);
-    void* P = ws + w.w_off;
-    uint8_t* tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off);
-    int* hot_list = reinterpret_cast<int*>(ws + w.list_off);
-    if (launch_prep_edit(s, U, mask, P, tile_hot, w.n_tiles, hot_list, status + 2, st) != SEKA_OK) return SEKA_ERR_CUDA;
-    const int T = shape_total_tokens(s), Hkv = s->n_kv_heads, M = s->n_experts;
-    CUtensorMap tk, tp;
-    if (!make_tile_map(&tk, K_in, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * M * Hkv * D, D)) return SEKA_ERR_CUDA;
-    if (M == 1) {
-        using PL = EpSmem<D>;
-        if (cudaFuncSetAttribute(edit_tiles_pipe_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::DYN_BYTES) != cudaSuccess)
-            return SEKA_ERR_CUDA;
-        const long long work = (long long)s->batch * w.n_tiles * Hkv;
-        const unsigned gridp = (unsigned)(work < (long long)n_sm ? work : (long long)n_sm);
-        edit_tiles_pipe_kernel<D, false><<<gridp, EP_THREADS, PL::DYN_BYTES, st>>>(tk, tp, static_cast<__nv_bfloat16*>(K_out), mask, alpha, gain, he,
-                                                                          s->cu_seqlens, hot_list, status + 2, status, s->max_seqlen,
-                                                                          Hkv, w.n_tiles);
-        ++g_launches;
-        return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+// First launch of that path: blocks [0, n_p) form a 32 x 32 tile of P[h] each (bf16, high parts of all heads, then low parts);
+// then blocks with a warp per (sequence, key tile) for the tile flags and the steering bytes; then the item table.
+__global__ void __launch_bounds__(PREP_THREADS)
+prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ mask, __nv_bfloat16* __restrict__ P,
+                      uint8_t* __restrict__ tile_hot, uint8_t* __restrict__ bh_info, int B, int L, int Hkv, int D, int r, int n_tiles,
+                      int n_p, int n_flag, const __grid_constant__ PrepJobs jobs) {
+    const int tid = threadIdx.x;
+    pdl_wait();
+    pdl_release();
+    int blk = blockIdx.x;
+    if (blk < n_p) {
+        const int tiles = D / 32;
+        const int h = blk / (tiles * tiles), t = blk % (tiles * tiles);
+        const int i0 = (t / tiles) * 32, j0 = (t % tiles) * 32;
+        __shared__ float ui[32][33], uj[32][33];
+        const int tx = tid & 31, ty = tid >> 5;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* Uh = U + (size_t)h * D * r;
+        for (int k0 = 0; k0 < r; k0 += 32) {
+            __syncthreads();
+            for (int q = ty; q < 32; q += 8) {
+                const bool in = k0 + tx < r;
+                ui[q][tx] = in ? Uh[(size_t)(i0 + q) * r + k0 + tx] : 0.f;
+                uj[q][tx] = in ? Uh[(size_t)(j0 + q) * r + k0 + tx] : 0.f;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = ty + 8 * q;
+#pragma unroll 8
+                for (int k = 0; k < 32; ++k) acc[q] = fmaf(ui[i][k], uj[tx][k], acc[q]);
+            }
+        }
+        // two bf16 parts, P = hi + lo to about 2^-17: the edit keeps fp32-like accuracy on bf16 tensor cores
+        __nv_bfloat16* Phi = P + (size_t)h * D * D;
+        __nv_bfloat16* Plo = P + ((size_t)Hkv + h) * D * D;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const __nv_bfloat16 hi = __float2bfloat16_rn(acc[q]);
+            Phi[(size_t)(i0 + ty + 8 * q) * D + j0 + tx] = hi;
+            Plo[(size_t)(i0 + ty + 8 * q) * D + j0 + tx] = __float2bfloat16_rn(acc[q] - __bfloat162float(hi));
+        }
+        return;
     }
-    uint32_t cols = 32;
-    while (cols < (uint32_t)(M * D)) cols *= 2;
-    const int per_sm = (int)(512 / cols) < 2 ? (int)(512 / cols) : 2;          // tensor memory and shared memory per SM
-    const long long work_max = (long long)s->batch * w.n_tiles * Hkv;
-    const long long want = (long long)n_sm * per_sm;
-    const unsigned grid = (unsigned)(work_max < want ? work_max : want);
-    edit_tiles_kernel<D, false><<<grid, EDIT_THREADS, SL::DYN_BYTES, st>>>(tk, tp, static_cast<__nv_bfloat16*>(K_out), mask, alpha, gain, he,
-                                                         s->cu_seqlens, hot_list, status + 2, status, s->max_seqlen, Hkv, M,
-                                                         w.n_tiles, cols);
-    ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    blk -= n_p;
+    if (blk < n_flag) {
+        const int item = blk * (PREP_THREADS / 32) + (tid >> 5), lane = tid & 31;
+        if (item >= B * n_tiles) return;
+        const int b = item / n_tiles, t = item % n_tiles;
+        const int seq0 = jobs.cu ? jobs.cu[b] : b * L;
+        const int Lb = (jobs.cu ? jobs.cu[b + 1] : (b + 1) * L) - seq0;
+        bool any = false;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int pos = t * 128 + q * 32 + lane;
+            any = (pos < Lb && mask[seq0 + pos] != 0) || any;
+        }
+        any = __any_sync(0xffffffffu, any);
+        if (lane == 0) tile_hot[item] = any ? 1 : 0;
+        if (t == 0)
+            for (int h = lane; h < Hkv; h += 32) bh_info[(size_t)b * Hkv + h] = (uint8_t)steer_byte(jobs.steer, b, h, Hkv);
+        return;
+    }
+    items_block(jobs.sched, jobs.cu, jobs.steer, jobs.items, jobs.item_count, blk - n_flag);
 }
 
 template <int D>
-static seka_status stage_keys_pipe_t(const seka_shape* s, const WorkspaceLayout& w, const void* K16, void* X,
-                                     const uint8_t* mask, const float* U, const float* alpha, const float* gain,
-                                     const uint8_t* he, char* ws, cudaStream_t st, const void* Q_route, const float* sigma,
-                                     int k_route) {
+static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
+                                     const float* alpha, const float* gain, const uint8_t* he, char* ws, const PrepJobs& jobs,
+                                     cudaStream_t st) {
     using PL = EpSmem<D>;
+    const int T = shape_total_tokens(s), Hkv = s->n_kv_heads;
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
-    int* status = reinterpret_cast<int*>(ws);
     void* P = ws + w.w_off;
     uint8_t* tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off);
-    int* hot_list = reinterpret_cast<int*>(ws + w.list_off);
-    // routed call: `alpha` is where the preparation launch writes the coefficients (read by the tile kernel after it)
-    if (launch_prep_edit(s, U, mask, P, tile_hot, w.n_tiles, hot_list, status + 2, st, reinterpret_cast<int*>(ws + w.first_off),
-                         reinterpret_cast<uint8_t*>(ws + w.info_off), gain, alpha, he, Q_route, sigma, k_route,
-                         const_cast<float*>(alpha)) != SEKA_OK)
-        return SEKA_ERR_CUDA;
-    const int T = shape_total_tokens(s), Hkv = s->n_kv_heads, M = s->n_experts;
     CUtensorMap tk, tp;
-    if (!make_tile_map(&tk, K16, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * M * Hkv * D, D)) return SEKA_ERR_CUDA;
-    if (M > 1) {
-        // a bank of experts: one product pair per expert into its own tensor-memory columns, two CTAs per SM
-        using SL = EditSmem<D>;
-        if (cudaFuncSetAttribute(edit_tiles_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SL::DYN_BYTES) != cudaSuccess)
-            return SEKA_ERR_CUDA;
-        uint32_t cols = 32;
-        while (cols < (uint32_t)(M * D)) cols *= 2;
-        const int per_sm = (int)(512 / cols) < 2 ? (int)(512 / cols) : 2;
-        const long long work_max = (long long)s->batch * w.n_tiles * Hkv, want = (long long)n_sm * per_sm;
-        const unsigned grid_b = (unsigned)(work_max < want ? work_max : want);
-        edit_tiles_kernel<D, true><<<grid_b, EDIT_THREADS, SL::DYN_BYTES, st>>>(tk, tp, static_cast<__nv_bfloat16*>(X), mask, alpha, gain, he,
-                                                                              s->cu_seqlens, hot_list, status + 2, status, s->max_seqlen,
-                                                                              Hkv, M, w.n_tiles, cols);
-        ++g_launches;
-        return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
-    }
-    if (cudaFuncSetAttribute(edit_tiles_pipe_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::DYN_BYTES) != cudaSuccess)
-        return SEKA_ERR_CUDA;
-    const long long work = (long long)s->batch * w.n_tiles * Hkv;
-    const unsigned grid = (unsigned)(work < (long long)n_sm ? work : (long long)n_sm);
-    edit_tiles_pipe_kernel<D, true><<<grid, EP_THREADS, PL::DYN_BYTES, st>>>(tk, tp, static_cast<__nv_bfloat16*>(X), mask, alpha, gain, he,
-                                                                           s->cu_seqlens, hot_list, status + 2, status, s->max_seqlen,
-                                                                           Hkv, w.n_tiles);
-    ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    if (!make_tile_map(&tk, K, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * Hkv * D, D)) return SEKA_ERR_CUDA;
+    const int n_p = Hkv * (D / 32) * (D / 32), n_flag = (s->batch * w.n_tiles + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
+    seka_status stc = launch_kernel(true, prep_projector_kernel, (unsigned)(n_p + n_flag + jobs.n_items_blocks), PREP_THREADS, 0, st, U, mask,
+                                    static_cast<__nv_bfloat16*>(P), tile_hot, reinterpret_cast<uint8_t*>(ws + w.info_off), s->batch,
+                                    s->max_seqlen, Hkv, D, s->rank, w.n_tiles, n_p, n_flag, jobs);
+    if (stc != SEKA_OK) return stc;
+    auto kern = stage_keys_pipe_kernel<D>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::DYN_BYTES) != cudaSuccess) return SEKA_ERR_CUDA;
+    const unsigned grid = (unsigned)(n_sm / Hkv * Hkv);
+    return launch_kernel(true, kern, grid, EP_THREADS, PL::DYN_BYTES, st, tk, tp, reinterpret_cast<__nv_bfloat16*>(ws + w.x_off), mask, alpha,
+                         gain, he, s->cu_seqlens, tile_hot, reinterpret_cast<int*>(ws), s->batch, s->max_seqlen, Hkv, w.n_tiles);
 }
 
-seka_status launch_stage_keys_pipe(const seka_shape* s, const WorkspaceLayout& w, const void* K16, void* X,
-                                   const uint8_t* mask, const float* U, const float* alpha, const float* gain,
-                                   const uint8_t* head_enable, char* ws, cudaStream_t st, const void* Q_route,
-                                   const float* sigma, int k_route) {
-    return s->head_dim == 128 ? stage_keys_pipe_t<128>(s, w, K16, X, mask, U, alpha, gain, head_enable, ws, st, Q_route, sigma, k_route)
-                              : stage_keys_pipe_t<64>(s, w, K16, X, mask, U, alpha, gain, head_enable, ws, st, Q_route, sigma, k_route);
+seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
+                              const float* alpha, const float* gain, const uint8_t* head_enable, char* ws, const PrepJobs& jobs,
+                              const RouteArgs& route, cudaStream_t st) {
+    // The pipelined pair of launches from five waves of the chain on.  Measured per call, pipeline against chain: packed batch
+    // of 64 sequences, 16 heads of 64 (16384 units) 717 against 853 us; 4 x 4096 tokens x 8 heads of 128 (1024 units) 599
+    // against 597; one prompt of 777 tokens (56 units) 37 against 32.
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
+    const long long units = (long long)s->batch * w.n_tiles * s->n_kv_heads;
+    if (units > 0x7fffffffLL) return SEKA_ERR_UNSUPPORTED;
+    const int chain_ctas = s->head_dim == 128 ? EtSmem<128, true>::CTAS : EtSmem<64, true>::CTAS;
+    if (s->n_experts == 1 && route.sigma == nullptr && s->dtype == SEKA_BF16 && s->n_kv_heads <= n_sm && units > 5LL * chain_ctas * n_sm)
+        return s->head_dim == 128 ? launch_stage_pipe<128>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st)
+                                  : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st);
+    TileArgs a = tile_args(s, w, K, ws + w.x_off, mask, U, alpha, gain, head_enable, ws);
+    a.route = route; a.jobs = jobs;
+    const bool routed = route.sigma != nullptr;
+    a.n_route_blocks = routed && route.alpha_out != nullptr ? s->batch * s->n_kv_heads : 0;
+    const int extra = a.n_route_blocks + jobs.n_items_blocks + jobs.n_conv_blocks;
+    const bool f32 = s->dtype == SEKA_F32;
+    if (s->head_dim == 128) {
+        const size_t smem = tiles_smem<128, true>(s, routed, route.k_route);
+        return f32 ? launch_tiles_t<128, true, float>(a, units, smem, extra, st) : launch_tiles_t<128, true, __nv_bfloat16>(a, units, smem, extra, st);
+    }
+    const size_t smem = tiles_smem<64, true>(s, routed, route.k_route);
+    return f32 ? launch_tiles_t<64, true, float>(a, units, smem, extra, st) : launch_tiles_t<64, true, __nv_bfloat16>(a, units, smem, extra, st);
 }
 
 }  // namespace seka
@@ -888,17 +1194,8 @@ extern "C" seka_status seka_edit_keys(const seka_shape* shape, const void* K_in,
     if (!workspace || workspace_bytes < w.edit_total) return SEKA_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* ws = static_cast<char*>(workspace);
-    // bf16 tensors go through the tensor-core tile kernel (the projector products of all experts have to fit
-    // into tensor memory); fp32 tensors, and banks too large for that, take the fp32 row kernel
-    if (shape->dtype == SEKA_BF16 && (long long)shape->n_experts * shape->head_dim <= 512 && ((uintptr_t)workspace & 255) == 0) {
-        if (K_out != K_in) {
-            const size_t bytes = (size_t)T * shape->n_kv_heads * shape->head_dim * 2;
-            if (cudaMemcpyAsync(K_out, K_in, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return SEKA_ERR_CUDA;
-        }
-        if (shape->head_dim == 128)
-            return launch_edit_tiles<128>(shape, w, K_in, K_out, mask, U, alpha, gain, head_enable, ws, st);
-        return launch_edit_tiles<64>(shape, w, K_in, K_out, mask, U, alpha, gain, head_enable, ws, st);
-    }
+    // bf16 tensors go through the tensor-core tile kernel, fp32 tensors through the fp32 row kernel
+    if (shape->dtype == SEKA_BF16) return launch_edit_tiles(shape, w, K_in, K_out, mask, U, alpha, gain, head_enable, ws, st);
     return launch_edit_rows(shape, K_in, K_out, mask, U, alpha, gain, head_enable, st);
 }
 

@@ -5,44 +5,39 @@
 #include <stdint.h>
 
 #include "seka_common.cuh"
+#include "seka_prep.cuh"
 
 namespace seka {
 
-// Operand preparation of the fused kernel (tile flags, edited keys of the tiles with highlighted tokens; see seka_prep.cu).  With
-// `sigma` set, the routing coefficients of Eq. 6 are computed inside the launch from Q_route (the caller's Q in its own
-// dtype) instead of being read from `alpha`, and written to `alpha_out` if that is not null.
-seka_status launch_prep_steering(const seka_shape* s, const SteerPlan& plan, const void* K16, const float* U,
-                                 const float* alpha, const float* gain, const uint8_t* head_enable, const uint8_t* mask,
-                                 void* X, uint8_t* tile_hot, int* first_hot, uint8_t* bh_info, int* status, int n_tiles, cudaStream_t st,
-                                 const void* Q_route = nullptr, const float* sigma = nullptr, int k_route = 0,
-                                 float* alpha_out = nullptr);
-// `bh_info` (null: no steering) is the per-(sequence, KV head) byte the preparation launch wrote
-void launch_build_items(const Sched& sc, const int* cu, const uint8_t* bh_info, ItemRecord* items, int* count,
-                        cudaStream_t st);
-void launch_convert_bf16(const float* Q, void* q16, size_t nq, const float* K, void* k16, const float* V, void* v16, size_t nk,
-                         cudaStream_t st);
+// Jobs that ride along with the preparation launch (see seka_prep.cuh).
+struct PrepJobs {
+    int n_items_blocks, n_conv_blocks;      // blocks for the item table (packed batches) and for the conversion (fp32 inputs)
+    Sched sched;
+    const int* cu;
+    SteerIn steer;
+    ItemRecord* items;
+    int* item_count;
+    ConvertArgs conv;
+};
 
-// Preparation of the tile-wise edit: P[m][h] = U_m U_m^T (two bf16 parts), tile flags, list of the tiles that hold a
-// highlighted token; with `first_hot` / `bh_info` set also what the fused forward needs (see prep_edit_kernel); with
-// `sigma` set also the routing coefficients of Eq. 6 into `alpha_out` (further blocks of the same launch).
-seka_status launch_prep_edit(const seka_shape* s, const float* U, const uint8_t* mask, void* P, uint8_t* tile_hot, int n_tiles,
-                             int* hot_list, int* hot_count, cudaStream_t st, int* first_hot = nullptr, uint8_t* bh_info = nullptr,
-                             const float* gain = nullptr, const float* alpha = nullptr, const uint8_t* head_enable = nullptr,
-                             const void* Q_route = nullptr, const float* sigma = nullptr, int k_route = 0,
-                             float* alpha_out = nullptr);
+// The preparation of a forward without steering: `jobs` alone (nothing is launched if there are none).
+seka_status launch_prep_plain(const PrepJobs& jobs, cudaStream_t st);
+
+// Routing inside the preparation launch (Eq. 6); `sigma` null: the coefficients are given.
+struct RouteArgs {
+    const void* Q; int q_is_f32; const float* sigma; int k_route; int Hq; float* alpha_out;
+};
+
+// The preparation of a steered forward: edited keys of the tiles that hold a highlighted token into the side buffer
+// X [T, Hkv, 2 d] (high | low parts), tile flags, steering bytes, and `jobs`.  K is the caller's tensor in its own dtype.
+// With route.sigma set the coefficients are computed in the launch and written to route.alpha_out if that is not null.
+seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
+                              const float* alpha, const float* gain, const uint8_t* head_enable, char* ws, const PrepJobs& jobs,
+                              const RouteArgs& route, cudaStream_t st);
 
 // Eq. 6 for every (sequence, KV head): the launch behind adaseka_route
 seka_status launch_route(const seka_shape* s, const void* Q, const float* U, const float* sigma, int k_route,
                          float* alpha_out, cudaStream_t st);
-
-// The edited keys of the tiles that hold a highlighted token into the side buffer X [T, Hkv, 2 d] of the fused forward
-// (high | low parts), by the tile kernels of the stand-alone edit in their side mode (two launches with the
-// preparation): the pipelined kernel for one expert, the bank kernel for several (n_experts * d <= 512).
-// K16 is the bf16 key tensor; workspace regions as in workspace_layout.
-seka_status launch_stage_keys_pipe(const seka_shape* s, const WorkspaceLayout& w, const void* K16, void* X,
-                                   const uint8_t* mask, const float* U, const float* alpha, const float* gain,
-                                   const uint8_t* head_enable, char* ws, cudaStream_t st, const void* Q_route = nullptr,
-                                   const float* sigma = nullptr, int k_route = 0);
 
 // bf16 tensor [T, H, d] viewed as (d, H, T) for TMA: tiles of 64 x 1 x box_rows with the 128-byte swizzle.
 bool make_tile_map(CUtensorMap* m, const void* base, int d, int H, long long T, int box_rows = 128);
@@ -51,5 +46,21 @@ seka_status validate_shape(const seka_shape* s);
 
 // Number of SMs of the current device (looked up once per device, thread-safe).
 bool device_info(int* n_sm);
+
+// Launch whose status is that of the launch alone.  With `pdl` it may be placed while its predecessor in the stream drains
+// (the kernel begins with pdl_wait).
+template <typename... P, typename... A>
+static inline seka_status launch_kernel(bool pdl, void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                                        const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) return SEKA_ERR_CUDA;
+    ++g_launches;
+    return SEKA_OK;
+}
 
 }  // namespace seka

@@ -1,5 +1,5 @@
 // AdaSEKA routing coefficients (Eq. 6, Section 3.3) of one (sequence, KV head), as a device routine shared by the
-// stand-alone routing kernel and the operand preparation of the fused forward (so that both give the same bits).
+// stand-alone routing kernel and the preparation of the fused forward (so that both give the same bits).
 #pragma once
 
 #include "seka_common.cuh"
@@ -20,7 +20,7 @@ static inline int route_chunks(int M, int k_route) {
 __host__ __device__
 #endif
 static inline size_t route_smem_bytes(int D, int M, int k_route) {
-    return sizeof(double) * ((size_t)D + (size_t)M * k_route * route_chunks(M, k_route) + M + 1);
+    return sizeof(double) * ((size_t)D + (size_t)M * k_route * route_chunks(M, k_route) + M);
 }
 
 #ifdef __CUDACC__
@@ -35,14 +35,14 @@ __device__ __forceinline__ float route_load_q(const void* Q, int q_is_f32, size_
 // Every thread of the CTA calls this (it synchronises the CTA); `sm` holds route_smem_bytes() bytes.  The order of
 // every sum is fixed (it does not depend on the number of threads), so any kernel that calls this gets the same bits.
 // Returns the M coefficients (as doubles, in shared memory), valid for every thread on return.
-__device__ __forceinline__ const double* route_group(const void* Q, int q_is_f32, const float* __restrict__ U,
+__device__ __noinline__ static const double* route_group(const void* Q, int q_is_f32, const float* __restrict__ U,
                                                      const float* __restrict__ sigma, const int* __restrict__ cu_seqlens,
                                                      int L, int Hq, int Hkv, int D, int r, int M, int k_route,
                                                      int b, int h, double* sm) {
     const int C = route_chunks(M, k_route);
     double* qbar = sm;                          // [D]
     double* term = sm + D;                      // [M][C][k_route]: partial dot products
-    double* s = term + (size_t)M * C * k_route; // [M] (+ 1: the largest magnitude)
+    double* s = term + (size_t)M * C * k_route; // [M]
     const int G = Hq / Hkv, tid = threadIdx.x;
     const int last = (cu_seqlens ? cu_seqlens[b + 1] : (b + 1) * L) - 1;
     const int first = cu_seqlens ? cu_seqlens[b] : b * L;
@@ -68,27 +68,20 @@ __device__ __forceinline__ const double* route_group(const void* Q, int q_is_f32
         term[u] = dot * sg;
     }
     __syncthreads();
-    // pieces of a (expert, direction) pair in order, into the slot of piece 0; then the directions of an expert in order
-    for (int p = tid; p < M * k_route; p += blockDim.x) {
-        const int m = p / k_route, k = p - m * k_route;
+    // one warp per expert: each lane adds the pieces of its directions (lane, lane + 32, ...) in order, then the lanes are
+    // added pairwise (the same order whatever the number of warps)
+    const int lane = tid & 31;
+    for (int m = tid >> 5; m < M; m += blockDim.x >> 5) {
         double t = 0.0;
-        for (int c = 0; c < C; ++c) t += term[((size_t)m * C + c) * k_route + k];
-        term[(size_t)m * C * k_route + k] = t;
+        for (int k = lane; k < k_route; k += 32)
+            for (int c = 0; c < C; ++c) t += term[((size_t)m * C + c) * k_route + k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) s[m] = t;
     }
     __syncthreads();
-    for (int m = tid; m < M; m += blockDim.x) {
-        double tot = 0.0;
-        for (int k = 0; k < k_route; ++k) tot += term[(size_t)m * C * k_route + k];
-        s[m] = tot;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        double mx = 0.0;
-        for (int m = 0; m < M; ++m) mx = fmax(mx, fabs(s[m]));
-        s[M] = mx;
-    }
-    __syncthreads();
-    const double mx = s[M];
+    double mx = 0.0;
+    for (int m = 0; m < M; ++m) mx = fmax(mx, fabs(s[m]));
     __syncthreads();
     for (int m = tid; m < M; m += blockDim.x) s[m] = mx > 0.0 ? s[m] / mx : 0.0;
     __syncthreads();
