@@ -1,0 +1,49 @@
+"""Tile kernels of the key edit at the edges of their 128-row steps, 64-column blocks of stacked U and dispatch rule, against the
+fp64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2603_01281_b200 import binding, inputs
+
+import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("d,rank,experts,kv,lens,mask", [
+    (128, 32, 1, 2, [127], "all"), (128, 64, 1, 3, [128], "all"), (64, 16, 1, 2, [129], "all"), (64, 1, 1, 1, [1], "all"),
+    (128, 65, 1, 2, [300, 0, 41], "runs"), (128, 24, 3, 2, [513, 70], "runs"), (64, 7, 9, 2, [200, 200], "spans"),
+    (128, 128, 4, 2, [257], "spans"), (64, 64, 2, 5, [1024, 1025, 1], "runs"), (128, 16, 1, 2, [640], "none")])
+def test_edit_steps_and_blocks(d, rank, experts, kv, lens, mask, in_place):
+    w = inputs.make_custom(seed=90 + rank, dtype="bf16", lens=lens, n_q_heads=2 * kv, n_kv_heads=kv, head_dim=d, rank=rank,
+                           n_experts=experts, mask_kind=mask, highlight=0.3, gain=np.linspace(1.0, -0.5, len(lens)))
+    if len(lens) > 2:
+        w.gain[-1] = 0.0                                        # a sequence without a gain is not touched
+    alpha = np.random.default_rng(rank).uniform(-1, 1, size=(w.batch, kv, experts))
+    he = np.ones(kv, dtype=np.uint8)
+    he[-1] = kv == 1
+    ref = oracle.edit_keys(w.K, w.mask, w.cu_seqlens, w.U, alpha=alpha, gain=w.gain, head_enable=he)
+    got = H.run_edit(w, alpha=alpha, head_enable=he, in_place=in_place).double().cpu().numpy()
+    # one rounding of the result to bf16: half an ulp of the entry, at most 2^-8 of the row's largest
+    assert (np.abs(got - ref) / np.abs(ref).max(axis=-1, keepdims=True)).max() <= 2.0 ** -8
+    seq_gain = np.repeat(w.gain, np.diff(w.cu_seqlens))
+    same = ((w.mask == 0) | (seq_gain == 0))[:, None] | (he == 0)[None, :]
+    assert np.array_equal(got[same], w.K.astype(np.float64)[same])
+
+
+@pytest.mark.parametrize("d,seqs,kv", [(128, 92, 4), (128, 93, 4), (64, 139, 4), (64, 140, 4)])
+def test_preparation_on_both_sides_of_its_rule(d, seqs, kv):
+    """Four key tiles a sequence, so that 92 | 93 (139 | 140) sequences lie on the two sides of the line between the chain and the
+    pipelined preparation on a GPU of 148 SMs."""
+    lens = [400 + (37 * i) % 113 for i in range(seqs - 1)] + [512]
+    w = inputs.make_custom(seed=95, dtype="bf16", lens=lens, n_q_heads=kv, n_kv_heads=kv, head_dim=d, rank=16, mask_kind="runs",
+                           highlight=0.1, gain=[(0.5, 2.0, 0.0)[i % 3] for i in range(seqs)])
+    he = np.array([1, 0] + [1] * (kv - 2), dtype=np.uint8)
+    rows = H.sampled_rows(w, 8, seed=1)
+    O, LSE = H.run_fused(w, head_enable=he)
+    Oref, Lref, idx = H.oracle_rows(w, rows, head_enable=he)
+    H.check_attention(O[idx], Oref, "d%d %d sequences" % (d, seqs))
+    np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)       # the bound of the other forward tests
