@@ -7,7 +7,7 @@
 // contraction with the low parts, so that the logits are those of the fp32 k'.  The score matrix never reaches memory;
 // K and V are read only.
 //
-// One CTA (16 warps) owns two tiles of 128 queries that share a KV head ("A" and "B": two query heads of one group at
+// One CTA (12 warps) owns two tiles of 128 queries that share a KV head ("A" and "B": two query heads of one group at
 // the same rows, or two consecutive row tiles of one head when the group size is odd) and walks the key tiles
 // 0 .. diagonal.  Warp roles:
 //   warp 0        TMA producer: Q tiles, then K (or edited-key) and V tiles (128-byte swizzle) through two
@@ -21,18 +21,20 @@
 //                 softmax in base 2 with a lazily updated running maximum, P written back as bf16 over the consumed
 //                 score columns, O rescaled in tensor memory only when the maximum moved by more than 2^8; final
 //                 normalisation and store.
-// (Warps 3 and 12-15 only give their registers to the softmax warps.)
-// While one tile's softmax runs, the tensor core works on the other tile.  Every wait is bounded: a wait that runs
-// out raises the CTA's abort flag, every role leaves its loop, and the status word reports it.
+// (Warp 3 only gives its registers to the softmax warps.)
+// While one tile's softmax runs, the tensor core works on the other tile.  Items follow each other without a seam: the next
+// item's first key tile travels with this item's last value tile, its Q tiles follow the last score products, and the
+// first scores of a tile's next item are issued right behind its last P V, under the store of its output (before, every
+// item began with an empty tensor pipe and its operands on the way, about 8000 cycles).  Measured on 32 / 8 heads of 128:
+// 4 x 4096 tokens 0.495 -> 0.466 ms, one prompt of 4362 tokens 148 -> 139 us, 28 / 4 heads 1 x 32768 5.93 -> 5.69 ms
+// (unsteered, GPU rested between blocks).
+// Every wait is bounded: a wait that runs out raises the CTA's abort flag, every role leaves its loop, and the status word
+// reports it.
 #include <math.h>
 
 #include <mutex>
 
 #include "seka_kernels.h"
-
-#ifndef SEKA_POLY_PAIR_MASK
-#define SEKA_POLY_PAIR_MASK 0x0000u
-#endif
 
 namespace seka {
 
@@ -51,19 +53,24 @@ struct AttnParams {
 };
 
 constexpr int BM = 128, BN = 128;
-constexpr int NTHREADS = 512;
+constexpr int NTHREADS = 384;
 constexpr uint32_t BLK_BYTES = 128 * 128;   // one [128 x 64] bf16 block
 constexpr float LAZY_RESCALE_LOG2 = 8.0f;   // the running maximum is only raised when it moved by more than this
-// registers per thread after the roles split (the CTA owns the whole register file: 4 x 128 x (80+184+184+64) = 64 Ki)
-constexpr int REGS_CTRL = 80, REGS_SOFTMAX = 184, REGS_PROJ = 64;   // PROJ: the idle fourth warpgroup
-// which of the 16 element pairs of every 32-key chunk take the polynomial exp2 instead of the special-function unit
-constexpr uint32_t POLY_PAIR_MASK = SEKA_POLY_PAIR_MASK;
+// registers per thread after the roles split, out of the launch's 168 per thread (3 x 168 = 104 + 2 x 200)
+constexpr int REGS_CTRL = 104, REGS_SOFTMAX = 200;
+// Plain polls of a wait before it parks (see mbar_wait_limit).  One: a warp that polls takes issue slots from the softmax
+// warps of its scheduler (eight polls cost 1 % on 4 x 4096 tokens of 32 heads of 128, polling without end 4 %).
+constexpr int PLAIN_POLLS = 1;
+
 constexpr uint32_t SMEM_LIMIT = 227 * 1024;
 
 
 // Shared memory of one CTA.  Tiles first (each a multiple of 1024 bytes), then barriers and per-warp item slots.
 template <int D>
 struct Geo {
+    // P is handed to the tensor core in two pieces, so that most of P V runs under the last exponentials; 16-key blocks in the
+    // first piece (head_dim 64, whose P V is short: half)
+    static constexpr int KP1 = D == 128 ? 6 : 4;
     static constexpr int NK = D == 128 ? 2 : 3;                    // K and V ring depth
     static constexpr uint32_t TILE = (D / 64) * BLK_BYTES;         // a [128 x D] tile
     static constexpr int NXMAX = 3;                                // most stages of the key-side operand
@@ -85,7 +92,7 @@ __host__ __device__ inline SmemPlan smem_plan(const SteerPlan& sp) {
     s.k = 2 * G::TILE;
     s.v = s.k + G::NK * G::TILE;
     s.x = s.v + G::NK * G::TILE;
-    s.xb = sp.mode ? G::TILE : 0u;                                  // one stage of low parts: [128 x D]
+    s.xb = sp.mode ? G::TILE : 0u;                                 // one stage of low parts: [128 x D]
     s.bars = s.x + (uint32_t)sp.nx * s.xb;
     s.misc = s.bars + ((G::NBARS * 8 + 15) & ~15u);                 // 16-byte aligned: the item slots are filled by 16-byte async copies
     s.items = s.misc + 32;
@@ -110,41 +117,43 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-// 2^x for a pair of arguments on the FMA pipe: x = n + f with n = round(x), f in [-1/2, 1/2];
-// 2^f by a cubic fitted to relative error 7.5e-5 (far below the bf16 rounding of P), 2^n by adding n
-// to the exponent field.  Arguments below -126 (masked scores) give a value below 2^-125.
-__device__ __forceinline__ float2 exp2_poly2(float2 x) {
-    const float kMagic = 12582912.f;      // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
-    x.x = fmaxf(x.x, -126.f);
-    x.y = fmaxf(x.y, -126.f);
-    const float2 t = __fadd2_rn(x, make_float2(kMagic, kMagic));
-    const float2 n = __fadd2_rn(t, make_float2(-kMagic, -kMagic));
-    const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
-    float2 q = __ffma2_rn(f, make_float2(0.05517167f, 0.05517167f), make_float2(0.24261113f, 0.24261113f));
-    q = __ffma2_rn(q, f, make_float2(0.69326097f, 0.69326097f));
-    q = __ffma2_rn(q, f, make_float2(0.99992806f, 0.99992806f));
-    float2 r;
-    r.x = __int_as_float(__float_as_int(q.x) + (__float_as_int(t.x) << 23));
-    r.y = __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23));
-    return r;
+// 4 x 4 transpose among groups of four lanes: unit u (16 bytes) of lane q becomes unit q of lane u
+__device__ __forceinline__ void transpose4(uint4 (&a)[4], int lane) {
+    auto swap = [&](uint4& x, uint4& y, int bit) {       // the lane without `bit` gives y for its partner's x
+        const bool up = (lane & bit) != 0;
+        uint4 send = up ? x : y;
+        send.x = __shfl_xor_sync(0xffffffffu, send.x, bit); send.y = __shfl_xor_sync(0xffffffffu, send.y, bit);
+        send.z = __shfl_xor_sync(0xffffffffu, send.z, bit); send.w = __shfl_xor_sync(0xffffffffu, send.w, bit);
+        if (up) x = send; else y = send;
+    };
+    swap(a[0], a[2], 2); swap(a[1], a[3], 2);
+    swap(a[0], a[1], 1); swap(a[2], a[3], 1);
 }
-
-template <typename OutT> __device__ __forceinline__ void store_chunk32(OutT* dst, const uint32_t (&v)[32], float inv);
-template <> __device__ __forceinline__ void store_chunk32<__nv_bfloat16>(__nv_bfloat16* dst, const uint32_t (&v)[32], float inv) {
-    uint4* d4 = reinterpret_cast<uint4*>(dst);
+// 32 columns of the rows of a warp (lane = row), scaled, to global memory: four lanes write 64 contiguous bytes of a row
+// (a row per lane, 32 pieces of 16 bytes an instruction, took 2000 cycles of the load/store unit per tile).  `row0` points at
+// the columns in the row of lane 0, rows are `pitch` elements apart, `n_rows` of them exist.
+template <typename OutT> __device__ __forceinline__ void store_chunk32(OutT* row0, size_t pitch, int n_rows, const uint32_t (&v)[32], float inv, int lane) {
+    constexpr int EPU = 16 / (int)sizeof(OutT);          // elements of 16 bytes
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-        d4[c] = make_uint4(pack_bf16(__uint_as_float(v[8 * c]) * inv, __uint_as_float(v[8 * c + 1]) * inv),
-                           pack_bf16(__uint_as_float(v[8 * c + 2]) * inv, __uint_as_float(v[8 * c + 3]) * inv),
-                           pack_bf16(__uint_as_float(v[8 * c + 4]) * inv, __uint_as_float(v[8 * c + 5]) * inv),
-                           pack_bf16(__uint_as_float(v[8 * c + 6]) * inv, __uint_as_float(v[8 * c + 7]) * inv));
-}
-template <> __device__ __forceinline__ void store_chunk32<float>(float* dst, const uint32_t (&v)[32], float inv) {
-    float4* d4 = reinterpret_cast<float4*>(dst);
+    for (int half = 0; half < 32 / (4 * EPU); ++half) {
+        uint4 a[4];
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-        d4[c] = make_float4(__uint_as_float(v[4 * c]) * inv, __uint_as_float(v[4 * c + 1]) * inv,
-                            __uint_as_float(v[4 * c + 2]) * inv, __uint_as_float(v[4 * c + 3]) * inv);
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t* w = &v[half * 4 * EPU + u * EPU];
+            if constexpr (sizeof(OutT) == 2)
+                a[u] = make_uint4(pack_bf16(__uint_as_float(w[0]) * inv, __uint_as_float(w[1]) * inv), pack_bf16(__uint_as_float(w[2]) * inv, __uint_as_float(w[3]) * inv),
+                                  pack_bf16(__uint_as_float(w[4]) * inv, __uint_as_float(w[5]) * inv), pack_bf16(__uint_as_float(w[6]) * inv, __uint_as_float(w[7]) * inv));
+            else
+                a[u] = make_uint4(__float_as_uint(__uint_as_float(w[0]) * inv), __float_as_uint(__uint_as_float(w[1]) * inv),
+                                  __float_as_uint(__uint_as_float(w[2]) * inv), __float_as_uint(__uint_as_float(w[3]) * inv));
+        }
+        transpose4(a, lane);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = (lane & ~3) + k;
+            if (r < n_rows) *reinterpret_cast<uint4*>(row0 + (size_t)r * pitch + half * 4 * EPU + (lane & 3) * EPU) = a[k];
+        }
+    }
 }
 
 // One unit of work of a CTA: two 128-row query tiles that share a KV head of one sequence.
@@ -166,21 +175,20 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     constexpr int NBLK = D / 64;
     constexpr uint32_t TMEM_COLS = 512;
     constexpr uint32_t COL_S = 0, COL_O = 256;     // S_x at COL_S + 128 x, O_x at COL_O + D x
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    extern __shared__ __align__(1024) uint8_t smem[];
     const SmemPlan sl = smem_plan<D>(p.plan);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bars);
     uint64_t* q_full = bars;                 // [2]   Q tile landed
-    uint64_t* k0_full = q_full + 2;          // [1]   first key tile of the item landed
-    uint64_t* kv_full = k0_full + 1;         // [NK]  V(t) and K(t+1) landed (they are loaded as a pair)
-    uint64_t* kv_free = kv_full + NK;        // [NK]  one event per step: the tensor core is done with K(j+1) and V(j)
+    uint64_t* k0_full = q_full + 2;          // [1]   first key tile of the CTA's first item landed
+    uint64_t* kv_full = k0_full + 1;         // [NK]  V(g) and K(g+1) landed (they are loaded as a pair)
+    uint64_t* kv_free = kv_full + NK;        // [NK]  one event per step: the tensor core is done with K(g+1) and V(g)
     uint64_t* x_full = kv_free + NK;         // [3]   low parts of an edited tile landed
     uint64_t* s_full = x_full + G::NXMAX;    // [2]   scores of tile x are in tensor memory
     uint64_t* p_full = s_full + 2;           // [2]   4 softmax-warp arrivals (O_x rescaled, keys 0-95 of P_x written) + 1 from the relay
     uint64_t* p_last = p_full + 2;           // [2]   4 softmax-warp arrivals: keys 96-127 of P_x written
     uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished
     uint64_t* o_drained = o_full + 2;        // [2]   4 softmax-warp arrivals: O_x of the item has been read
-    uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles and first key tile of the item landed
+    uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles of the item landed
     uint64_t* drain = start_full + 1;        // [1]   every product issued has finished
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sl.misc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + sl.misc + 4);
@@ -220,7 +228,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
     // all lanes of a warp wait on the same barrier and then agree on the outcome
     auto warp_wait = [&](uint64_t* bar, uint32_t parity, int where) -> bool {
-        const bool ok = mbar_wait_limit(bar, parity, abort_flag, p.status, where, limit_ns);
+        const bool ok = mbar_wait_limit(bar, parity, abort_flag, p.status, where, limit_ns, PLAIN_POLLS);
         return __all_sync(0xffffffffu, ok);
     };
 
@@ -293,16 +301,38 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
 
-    // Running counts shared by all roles (each keeps its own copy; they advance identically):
-    //   n_it   items so far (phases of start_full, q_full[0], k0_full)
+    // Key tiles are numbered through, item after item: global tile g is tile g - pr of the item whose first tile is pr.  Pair g
+    // is V(g) and K(g+1), K(g+1) being the first key tile of the next item where V(g) is the last of this one; it uses
+    // stage g % NK of the V ring and (g + 1) % NK of the K ring.  Running counts shared by all roles (each keeps its own
+    // copy; they advance identically):
+    //   pr     first key tile of the present item
+    //   kv_free event g: the score products of key tile g and the P V of tile g - 1 are through (event 0: after the CTA's
+    //          first score products; event g + 1: after step g)
+    //   n_it   items so far (phases of start_full, q_full[0])
     //   n_o[x] items that had a tile x so far (phases of o_full, o_drained)
     //   n_qb   items with a tile B so far (phase of q_full[1])
     //   n_hot  edited key tiles whose low parts were loaded / used so far, over all items (stage and phase of x_full)
-    //   ev     kv_free events so far (n_kv + 1 per item: after the first score products, then after every step);
-    //          event j of an item covers the score products of its key tile j
-    //   pr     V/K pairs so far (n_kv per item); pair t of an item uses V stage (pr + t) % NK and K stage (pr + t + 1) % NK
     //   cx[x]  steps of tile x so far (phases of s_full, p_full, p_last)
     Item it;
+
+    // final normalisation and store of this warp's 32 rows of tile x of item `w` (`inv`: 1 / row sum of the lane's row)
+    auto store_tile = [&](int x, const Item& w, float inv) {
+        tc_fence_after();
+        const int q0 = (x ? w.qtB : w.qtA) * BM + (warp & 3) * 32;       // first query of the warp
+        const uint32_t tO = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + COL_O + D * x;
+        OutT* dst = static_cast<OutT*>(p.O) + ((size_t)(w.seq0 + q0) * p.sched.Hq + (x ? w.hqB : w.hqA)) * D;
+#pragma unroll 1
+        for (int c = 0; c < D / 32; ++c) {
+            uint32_t o[32];
+            tmem_ld32(tO + c * 32, o);
+            tmem_wait_ld_on(o);
+            store_chunk32<OutT>(dst + c * 32, (size_t)p.sched.Hq * D, w.Lb - q0, o, inv, lane);
+        }
+        tc_fence_before();
+        // O_x may be written again (the next item's first P V)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(o_drained + x);
+    };
 
     if (warp < 4) {
         reg_dec<REGS_CTRL>();
@@ -311,9 +341,9 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const bool leader = elect_one();
         if (warp == 0) {
             // ------------------------------------------------------------ TMA producer
-            const int nx = p.plan.nx;
+            const int n_x = p.plan.nx;
             const bool staged = p.plan.mode != 0;       // key tiles with highlighted tokens come from the side buffer
-            uint32_t ev = 0, pr = 0, n_it = 0, n_qb = 0, n_hot = 0;
+            uint32_t pr = 0, n_it = 0, n_qb = 0, n_hot = 0;
             uint32_t ev_seen = 0;            // events [0, ev_seen) are known to have completed
             uint32_t ev_hot[G::NXMAX] = {0, 0, 0};      // per stage of the key-side operand: event that releases it, + 1
             // parity + 1 of the last load armed on each barrier (0: none), for the teardown after an abort
@@ -326,74 +356,75 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 ok = warp_wait(kv_free + e % NK, (e / NK) & 1, where);
                 ev_seen = e + 1;
             };
-            // low parts of the edited key tile j of the item (event `e` covers its score products) into the next stage
-            auto load_x = [&](int j, uint32_t e) {
+            // low parts of the edited key tile j of item `w` (global tile g) into the next stage
+            auto load_x = [&](const Item& w, int j, uint32_t g) {
                 uint32_t st = 0, prev = 0;
 #pragma unroll
                 for (int i = 0; i < G::NXMAX; ++i)
-                    if ((int)(n_hot % (uint32_t)nx) == i) { st = i; prev = ev_hot[i]; ev_hot[i] = e + 1; }
+                    if ((int)(n_hot % (uint32_t)n_x) == i) { st = i; prev = ev_hot[i]; ev_hot[i] = g + 1; }
                 if (prev) see_event(prev - 1, 14);       // the tile that used this stage before is through the tensor core
                 if (!ok) return;
                 if (leader) {
                     mbar_expect_tx(x_full + st, sl.xb);
 #pragma unroll
                     for (int c = 0; c < NBLK; ++c)
-                        tma_load_3d(smem + sl.x + st * sl.xb + c * BLK_BYTES, &tmX, x_full + st, D + c * 64, it.hkv, it.seq0 + j * BN);
+                        tma_load_3d(smem + sl.x + st * sl.xb + c * BLK_BYTES, &tmX, x_full + st, D + c * 64, w.hkv, w.seq0 + j * BN);
                 }
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < G::NXMAX; ++i)
-                    if ((int)st == i) armed_x[i] = ((n_hot / (uint32_t)nx) & 1) + 1;
+                    if ((int)st == i) armed_x[i] = ((n_hot / (uint32_t)n_x) & 1) + 1;
                 ++n_hot;
             };
-            while (ok && next_item(it, true)) {
-                // Q and the first K of an item may land once the last score product of the previous item is
-                // done (event n_kv - 1 of that item), its V/K pairs once its last step is done (event n_kv)
-                if (n_it > 0) {
-                    see_event(ev - 2, 12);
-                    if (!ok) break;
-                }
+            auto load_q = [&](const Item& w) {
                 if (leader) {
                     mbar_expect_tx(q_full + 0, G::TILE);
 #pragma unroll
                     for (int c = 0; c < NBLK; ++c)
-                        tma_load_3d(smem + c * BLK_BYTES, &tmQ, q_full + 0, c * 64, it.hqA, it.seq0 + it.qtA * BM);
-                    if (it.nB > 0) {
+                        tma_load_3d(smem + c * BLK_BYTES, &tmQ, q_full + 0, c * 64, w.hqA, w.seq0 + w.qtA * BM);
+                    if (w.nB > 0) {
                         mbar_expect_tx(q_full + 1, G::TILE);
 #pragma unroll
                         for (int c = 0; c < NBLK; ++c)
-                            tma_load_3d(smem + G::TILE + c * BLK_BYTES, &tmQ, q_full + 1, c * 64, it.hqB, it.seq0 + it.qtB * BM);
+                            tma_load_3d(smem + G::TILE + c * BLK_BYTES, &tmQ, q_full + 1, c * 64, w.hqB, w.seq0 + w.qtB * BM);
                     }
-                    mbar_expect_tx(k0_full, G::TILE);
-                    const CUtensorMap* km0 = (staged && it.steer && tile_is_hot(it.b, 0)) ? &tmX : &tmK;
-#pragma unroll
-                    for (int c = 0; c < NBLK; ++c)
-                        tma_load_3d(smem + sl.k + (pr % NK) * G::TILE + c * BLK_BYTES, km0, k0_full, c * 64, it.hkv, it.seq0);
                 }
                 __syncwarp();
-                armed_q[0] = (n_it & 1) + 1; armed_k0 = (n_it & 1) + 1;
-                if (it.nB > 0) { armed_q[1] = (n_qb & 1) + 1; ++n_qb; }
-                if (it.need_lo && tile_is_hot(it.b, 0)) {
-                    load_x(0, ev);
-                    if (!ok) break;
+                armed_q[0] = (n_it & 1) + 1; ++n_it;
+                if (w.nB > 0) { armed_q[1] = (n_qb & 1) + 1; ++n_qb; }
+            };
+            bool have = ok && next_item(it, true);
+            if (have) {
+                load_q(it);
+                const bool hot = it.steer && tile_is_hot(it.b, 0);
+                if (leader) {
+                    mbar_expect_tx(k0_full, G::TILE);
+                    const CUtensorMap* km = (staged && hot) ? &tmX : &tmK;
+#pragma unroll
+                    for (int c = 0; c < NBLK; ++c) tma_load_3d(smem + sl.k + c * BLK_BYTES, km, k0_full, c * 64, it.hkv, it.seq0);
                 }
-                if (n_it > 0) {
-                    see_event(ev - 1, 13);
-                    if (!ok) break;
-                }
-                // V(t) and K(t+1) travel as a pair: both of their stages are released by the same event, the end
-                // of step t - NK of the MMA issuer (event t - NK + 1 of this item)
+                __syncwarp();
+                armed_k0 = 1;
+                if (hot && it.need_lo) load_x(it, 0, 0);
+            }
+            bool first = true;
+            while (ok && have) {
+                Item nx;
+                const bool more_items = next_item(nx, true);
+                // a pair's stages are released by the same event, the end of the step NK steps before
 #pragma unroll 1
                 for (int t = 0; t < it.n_kv; ++t) {
-                    if (t >= NK - 1) {
-                        see_event(ev + (uint32_t)(t - NK + 1), 10);
+                    const uint32_t g = pr + (uint32_t)t;
+                    if (g >= NK - 1) {
+                        see_event(g - (NK - 1), 10);
                         if (!ok) break;
                     }
-                    const bool more = t + 1 < it.n_kv;
-                    const bool hot_n = more && it.steer && tile_is_hot(it.b, t + 1);
-                    const uint32_t g = pr + (uint32_t)t;
+                    const bool inside = t + 1 < it.n_kv, more = inside || more_items;
+                    const Item& w = inside ? it : nx;
+                    const int j = inside ? t + 1 : 0;
+                    const bool hot_n = more && w.steer && tile_is_hot(w.b, j);
                     // (test hook: one pair of the first item of CTA 0 is left out altogether, so that its wait runs out)
-                    const bool skip = hook_skip > 0 && n_it == 0 && blockIdx.x == 0 && t + 1 == hook_skip;
+                    const bool skip = hook_skip > 0 && first && blockIdx.x == 0 && t + 1 == hook_skip;
                     if (leader && !skip) {
                         uint64_t* bar = kv_full + g % NK;
                         mbar_expect_tx(bar, more ? 2 * G::TILE : G::TILE);
@@ -404,8 +435,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                             const CUtensorMap* km = (staged && hot_n) ? &tmX : &tmK;
 #pragma unroll
                             for (int c = 0; c < NBLK; ++c)
-                                tma_load_3d(smem + sl.k + ((g + 1) % NK) * G::TILE + c * BLK_BYTES, km, bar, c * 64, it.hkv,
-                                            it.seq0 + (t + 1) * BN);
+                                tma_load_3d(smem + sl.k + ((g + 1) % NK) * G::TILE + c * BLK_BYTES, km, bar, c * 64, w.hkv, w.seq0 + j * BN);
                         }
                     }
                     __syncwarp();
@@ -414,12 +444,19 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         for (int i = 0; i < NK; ++i)
                             if ((int)(g % NK) == i) armed_kv[i] = ((g / NK) & 1) + 1;
                     }
-                    if (hot_n && it.need_lo) {
-                        load_x(t + 1, ev + (uint32_t)(t + 1));
+                    if (hot_n && w.need_lo) {
+                        load_x(w, j, g + 1);
                         if (!ok) break;
                     }
                 }
-                ev += it.n_kv + 1; pr += it.n_kv; ++n_it;
+                if (!ok) break;
+                pr += it.n_kv;
+                if (more_items) {
+                    see_event(pr - 1, 12);        // the last score products of the item are through: its Q tiles may be replaced
+                    if (!ok) break;
+                    load_q(nx);
+                }
+                it = nx; have = more_items; first = false;
             }
             if (*abort_flag) {
                 // loads that were armed may still be in flight: let them land before the shared memory is released
@@ -440,88 +477,108 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             const uint32_t dQ = umma_desc_lo(smem_u32(smem), 16), dK = umma_desc_lo(smem_u32(smem + sl.k), 16);
             const uint32_t dX = umma_desc_lo(smem_u32(smem + sl.x), 16);
             const uint32_t dV = umma_desc_lo(smem_u32(smem + sl.v), BLK_BYTES);
-            const uint32_t nx = p.plan.nx > 0 ? (uint32_t)p.plan.nx : 1u;
-            uint32_t ev = 0, pr = 0, n_it = 0, n_hot = 0;
+            const uint32_t n_x = p.plan.nx > 0 ? (uint32_t)p.plan.nx : 1u;
+            uint32_t n_it = 0, n_hot = 0;
             uint32_t cx[2] = {0, 0};      // steps of tile A / B so far
             uint32_t n_o[2] = {0, 0};     // items that had a tile A / B so far
             bool ok = !dead;
-            auto commit = [&](uint64_t* bar) {
-                if (leader) umma_commit(bar);
-                __syncwarp();
+            uint32_t x_stage = 0;         // stage that holds the low parts of the key tile being multiplied
+            // the low parts of the next edited key tile have landed (once per tile, before its first use)
+            auto see_x = [&]() {
+                x_stage = n_hot % n_x;
+                ok = warp_wait(x_full + x_stage, (n_hot / n_x) & 1, 32);
+                ++n_hot;
             };
-            while (ok && next_item(it, true)) {
-                const int nA = it.nA, nB = it.nB, n_kv = it.n_kv;
-                uint32_t x_stage = 0;      // stage that holds the low parts of the key tile being multiplied
-                // the low parts of the next edited key tile have landed (once per tile, before its first use)
-                auto see_x = [&]() {
-                    x_stage = n_hot % nx;
-                    ok = warp_wait(x_full + x_stage, (n_hot / nx) & 1, 32);
-                    ++n_hot;
-                };
-                // scores of tile x against key tile j; `hot`: the tile is an edited one whose low parts are multiplied too
-                auto issue_S = [&](int x, int j, bool hot) {
-                    const uint32_t kd = dK + ((pr + (uint32_t)j) % NK) * (G::TILE >> 4), qd = dQ + (uint32_t)x * (G::TILE >> 4);
-                    const uint32_t dst = tmem_base + COL_S + 128 * x;
-                    tc_fence_after();
-                    if (leader) {
+            // scores of tile x against the key tile in stage `st`; `hot`: the tile is an edited one whose low parts are multiplied too
+            auto issue_S = [&](int x, uint32_t st, bool hot) {
+                const uint32_t kd = dK + st * (G::TILE >> 4), qd = dQ + (uint32_t)x * (G::TILE >> 4);
+                const uint32_t dst = tmem_base + COL_S + 128 * x;
+                tc_fence_after();
+                if (leader) {
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        // 16 elements along the contraction = 32 bytes inside a 64-element block
+                        const uint32_t off = ((uint32_t)(ks >> 2) * BLK_BYTES + (uint32_t)(ks & 3) * 32) >> 4;
+                        umma_ss(dst, qd + off, DESC_HI, kd + off, DESC_HI, IDESC_S, ks > 0 ? 1u : 0u);
+                    }
+                    if (hot) {        // ... + Q (k'_lo)^T
+                        const uint32_t xd = dX + x_stage * (sl.xb >> 4);
 #pragma unroll
                         for (int ks = 0; ks < D / 16; ++ks) {
-                            // 16 elements along the contraction = 32 bytes inside a 64-element block
                             const uint32_t off = ((uint32_t)(ks >> 2) * BLK_BYTES + (uint32_t)(ks & 3) * 32) >> 4;
-                            umma_ss(dst, qd + off, DESC_HI, kd + off, DESC_HI, IDESC_S, ks > 0 ? 1u : 0u);
+                            umma_ss(dst, qd + off, DESC_HI, xd + off, DESC_HI, IDESC_S, 1u);
                         }
-                        if (hot) {        // ... + Q (k'_lo)^T
-                            const uint32_t xd = dX + x_stage * (sl.xb >> 4);
-#pragma unroll
-                            for (int ks = 0; ks < D / 16; ++ks) {
-                                const uint32_t off = ((uint32_t)(ks >> 2) * BLK_BYTES + (uint32_t)(ks & 3) * 32) >> 4;
-                                umma_ss(dst, qd + off, DESC_HI, xd + off, DESC_HI, IDESC_S, 1u);
-                            }
-                        }
-                        umma_commit(s_full + x);
                     }
-                    __syncwarp();
-                };
-                // P V of tile x and key tile j, key blocks [ks0, ks1) of 16 keys (2048 bytes of the V tile, 8 columns of P)
-                auto issue_PV = [&](int x, int j, int ks0, int ks1, bool last) {
-                    const uint32_t vd = dV + ((pr + (uint32_t)j) % NK) * (G::TILE >> 4);
-                    const uint32_t dst = tmem_base + COL_O + D * x, src = tmem_base + COL_S + 128 * x;
-                    tc_fence_after();
-                    if (leader) {
+                    umma_commit(s_full + x);
+                }
+                __syncwarp();
+            };
+            // P V of tile x with the value tile in stage `st`, key blocks [ks0, ks1) of 16 keys (2048 bytes of V, 8 columns of P)
+            auto issue_PV = [&](int x, uint32_t st, bool fresh, int ks0, int ks1, bool last) {
+                const uint32_t vd = dV + st * (G::TILE >> 4);
+                const uint32_t dst = tmem_base + COL_O + D * x, src = tmem_base + COL_S + 128 * x;
+                tc_fence_after();
+                if (leader) {
 #pragma unroll
-                        for (int ks = 0; ks < BN / 16; ++ks)
-                            if (ks >= ks0 && ks < ks1)
-                                umma_ts(dst, src + (uint32_t)ks * 8, vd + (uint32_t)ks * (2048 >> 4), DESC_HI, IDESC_PV,
-                                        (j > 0 || ks > 0) ? 1u : 0u);
-                        if (last) umma_commit(o_full + x);
-                    }
-                    __syncwarp();
+                    for (int ks = 0; ks < BN / 16; ++ks)
+                        if (ks >= ks0 && ks < ks1)
+                            umma_ts(dst, src + (uint32_t)ks * 8, vd + (uint32_t)ks * (2048 >> 4), DESC_HI, IDESC_PV,
+                                    (!fresh || ks > 0) ? 1u : 0u);
+                    if (last) umma_commit(o_full + x);
+                }
+                __syncwarp();
+            };
+            // P of tile x and step j has been handed over: P V with the value tile in stage `st`.  Before an item's first P V
+            // writes O_x, the O_x of the last item that had a tile x has been read (its phases count those items only, and each
+            // is seen, in order, by the next item that has the tile: a parity wait cannot tell a phase from the one two later).
+            auto step_PV = [&](int x, uint32_t st, int j, int n) {
+                if (j == 0 && n_o[x] > 0) {
+                    ok = warp_wait(o_drained + x, (n_o[x] - 1) & 1, 46 + x);
+                    if (!ok) return;
+                }
+                issue_PV(x, st, j == 0, 0, G::KP1, false);
+                ok = warp_wait(p_last + x, (cx[x] + j) & 1, 28 + x);
+                if (!ok) return;
+                issue_PV(x, st, j == 0, G::KP1, BN / 16, j == n - 1);
+            };
+            auto commit_event = [&](uint32_t st) {
+                if (leader) umma_commit(kv_free + st);
+                __syncwarp();
+            };
+            uint32_t st = 0;              // stage of the present value tile (of key tile g; the next key tile is in the stage after it)
+            bool have = ok && next_item(it, true);
+            if (have) {
+                ok = warp_wait(start_full, 0, 20);
+                const bool hot = it.need_lo && tile_is_hot(it.b, 0);
+                if (ok && hot) see_x();
+                if (ok) {
+                    issue_S(0, 0, hot);
+                    if (it.nB > 0) issue_S(1, 0, hot);
+                    commit_event(0);
+                }
+            }
+            // One thread issues for both tiles, in a fixed order (A then B in every step): the in-order tensor
+            // pipe then keeps the two tiles half a period apart (softmax of one tile under the MMAs of the other).
+            while (ok && have) {
+                Item nx;
+                const bool more = next_item(nx, true);
+                const int nA = it.nA, nB = it.nB, n_kv = it.n_kv;
+                ++n_it;
+                bool started = false;          // the next item's operands have been seen
+                bool hot0 = false;             // its first key tile takes the low parts
+                auto start_next = [&]() {
+                    if (started) return;
+                    started = true;
+                    ok = warp_wait(start_full, n_it & 1, 21);
+                    hot0 = nx.need_lo && tile_is_hot(nx.b, 0);
+                    if (ok && hot0) see_x();
                 };
-                // The O_x of the last item that had a tile x has been read.  Its phases count those items only, and each is
-                // seen, in order, by the next item that has the tile: a warp that could arrive for items in which it has
-                // nothing to do would run ahead, and a parity wait cannot tell a phase from the one two later.
-                auto see_drained = [&]() {
-                    if (n_o[0] > 0) ok = warp_wait(o_drained + 0, (n_o[0] - 1) & 1, 46);
-                    if (ok && nB > 0 && n_o[1] > 0) ok = warp_wait(o_drained + 1, (n_o[1] - 1) & 1, 47);
-                };
-                // do key tiles 0 and 1 take the low-part steps? (later ones are looked up one step ahead of their use)
-                const bool hot_cur = it.need_lo && tile_is_hot(it.b, 0);
                 bool hot_nxt = it.need_lo && n_kv > 1 && tile_is_hot(it.b, 1);
-                // One thread issues for both tiles, in a fixed order (A then B in every step): the in-order tensor
-                // pipe then keeps the two tiles half a period apart (softmax of one tile under the MMAs of the other).
-                ok = warp_wait(start_full, n_it & 1, 20);
-                if (!ok) break;
-                if (hot_cur) { see_x(); if (!ok) break; }
-                issue_S(0, 0, hot_cur);
-                if (nB > 0) issue_S(1, 0, hot_cur);
-                commit(kv_free + ev % NK);
-                ++ev;
-                see_drained();          // before the item's first P V writes O_x again
-                if (!ok) break;
 #pragma unroll 1
-                for (int j = 0; j < n_kv && ok; ++j) {
+                for (int j = 0; j < n_kv; ++j) {
                     const int j1 = j + 1;
-                    const bool hot_j1 = hot_nxt && j1 < n_kv;
+                    const uint32_t st1 = st + 1 == (uint32_t)NK ? 0u : st + 1;
+                    const bool hot_j1 = hot_nxt && j1 < n_kv, turn = j1 == n_kv && more;      // turn: on to the next item's scores
                     hot_nxt = it.need_lo && j + 2 < n_kv && tile_is_hot(it.b, j + 2);
                     bool x_seen = false;
                     // V of this step and K of the next have landed once p_full completes: the relay warp vouches
@@ -529,48 +586,64 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     // bubble in the tensor pipe: its queue is only a couple of MMAs deep)
                     if (j < nA) {
                         ok = warp_wait(p_full + 0, (cx[0] + j) & 1, 24);
+                        if (ok) step_PV(0, st, j, nA);
                         if (!ok) break;
-                        issue_PV(0, j, 0, 6, false);
-                        ok = warp_wait(p_last + 0, (cx[0] + j) & 1, 28);
-                        if (!ok) break;
-                        issue_PV(0, j, 6, 8, j == nA - 1);
                         if (j1 < nA) {
                             if (hot_j1) { see_x(); x_seen = true; if (!ok) break; }
-                            issue_S(0, j1, hot_j1);
+                            issue_S(0, st1, hot_j1);
+                        } else if (turn) {
+                            start_next();
+                            if (!ok) break;
+                            issue_S(0, st1, hot0);
                         }
                     }
                     if (j < nB) {
                         ok = warp_wait(p_full + 1, (cx[1] + j) & 1, 26);
                         if (!ok) break;
-                        issue_PV(1, j, 0, 6, false);
-                        ok = warp_wait(p_last + 1, (cx[1] + j) & 1, 29);
+                        if (turn && j >= nA) {        // tile A has been through for a step: it goes on first
+                            start_next();
+                            if (!ok) break;
+                            issue_S(0, st1, hot0);
+                        }
+                        step_PV(1, st, j, nB);
                         if (!ok) break;
-                        issue_PV(1, j, 6, 8, j == nB - 1);
                     }
                     if (j1 < nB) {
                         if (hot_j1 && !x_seen) { see_x(); if (!ok) break; }      // tile A does not use this key tile
-                        issue_S(1, j1, hot_j1);
+                        issue_S(1, st1, hot_j1);
+                    } else if (turn && nx.nB > 0) {
+                        start_next();
+                        if (!ok) break;
+                        issue_S(1, st1, hot0);
                     }
-                    commit(kv_free + ev % NK);      // K(j+1) and V(j) may be overwritten
-                    ++ev;
+                    commit_event(st1);     // K(g+1) and V(g) may be overwritten
+                    st = st1;
                 }
-                pr += n_kv; cx[0] += nA; cx[1] += nB; ++n_it;
+                if (!ok) break;
+                cx[0] += nA; cx[1] += nB;
                 ++n_o[0];
                 if (nB > 0) ++n_o[1];
+                it = nx; have = more;
             }
         } else if (warp == 2) {
             // ------------------------------------------------------------ operand relay: "the operands have landed", once per
-            // item for Q and the first K, and per step "V(j) and K(j+1) landed" as a fifth arrival on the
+            // item for Q (and the CTA's first K), and per step "V(g) and K(g+1) landed" as a fifth arrival on the
             // P hand-off barrier, so that the MMA issuer waits on one barrier per hand-off
             uint32_t pr = 0, n_it = 0, n_qb = 0, cx[2] = {0, 0};
             bool ok = !dead;
-            while (ok && next_item(it)) {
+            auto q_landed = [&](const Item& w) {
                 ok = warp_wait(q_full + 0, n_it & 1, 21);
-                if (ok && it.nB > 0) { ok = warp_wait(q_full + 1, n_qb & 1, 22); ++n_qb; }
-                if (ok) ok = warp_wait(k0_full, n_it & 1, 23);
-                if (!ok) break;
-                if (lane == 0) mbar_arrive(start_full);
+                ++n_it;
+                if (ok && w.nB > 0) { ok = warp_wait(q_full + 1, n_qb & 1, 22); ++n_qb; }
+                if (ok && n_it == 1) ok = warp_wait(k0_full, 0, 23);
+                if (ok && lane == 0) mbar_arrive(start_full);
                 __syncwarp();
+            };
+            bool have = ok && next_item(it);
+            if (have) q_landed(it);
+            while (ok && have) {
+                Item nx;
+                const bool more = next_item(nx);
 #pragma unroll 1
                 for (int j = 0; j < it.n_kv; ++j) {
                     const uint32_t g = pr + j;
@@ -581,17 +654,18 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         if (j < it.nB) mbar_arrive(p_full + 1);
                     }
                     __syncwarp();
+                    // the next item's Q tiles: loaded when this item's last score products are through, so they land while its
+                    // last softmax runs
+                    if (j + 1 == it.n_kv && more) { q_landed(nx); if (!ok) break; }
                     // stay within the phase: the next arrival may only come after this phase has completed
                     if (j < it.nA) ok = warp_wait(p_full + 0, (cx[0] + j) & 1, 33);
                     if (ok && j < it.nB) ok = warp_wait(p_full + 1, (cx[1] + j) & 1, 34);
                     if (!ok) break;
                 }
-                pr += it.n_kv; cx[0] += it.nA; cx[1] += it.nB; ++n_it;
+                pr += it.n_kv; cx[0] += it.nA; cx[1] += it.nB;
+                it = nx; have = more;
             }
         }
-    } else if (warp >= 12) {
-        // (these warps only hand their registers to the softmax warps)
-        reg_dec<REGS_PROJ>();
     } else {
         // ------------------------------------------------------------ softmax of tile x, one query row per thread
         reg_inc<REGS_SOFTMAX>();
@@ -654,18 +728,12 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     for (int e2 = 0; e2 < 16; ++e2) {
                         const int e = 32 * c + 2 * e2;
                         const float2 arg = __ffma2_rn(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), sc2, nm2);
-                        float2 pe;
-                        if ((POLY_PAIR_MASK >> e2) & 1u) {
-                            pe = exp2_poly2(arg);
-                        } else {
-                            pe.x = fast_exp2(arg.x);
-                            pe.y = fast_exp2(arg.y);
-                        }
+                        const float2 pe = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
                         sum[e2 & 1] = __fadd2_rn(sum[e2 & 1], pe);
                         pk16[e2] = pack_bf16(pe.x, pe.y);
                     }
                     tmem_st16(tS + c * 16, pk16);     // P (bf16 pairs) over score columns that are already in registers
-                    if (c == 2) {                     // keys 0-95 are in place: the tensor core may start on them
+                    if (2 * c + 2 == G::KP1) {      // the first piece is in place: the tensor core may start on it
                         tmem_wait_st();
                         tc_fence_before();
                         __syncwarp();
@@ -682,27 +750,14 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             if (!ok) break;
             cX += nX;
             if (nX > 0) {
-                ok = warp_wait(o_full + x, n_o & 1, 44 + x);
-                ++n_o;
-                if (!ok) break;
-                // final normalisation and store
-                tc_fence_after();
-                const int qpos = qtX * BM + row;
-                const bool valid = qpos < it.Lb;
-                const size_t orow = (size_t)(it.seq0 + (valid ? qpos : 0)) * p.sched.Hq + hqX;
                 const float inv = 1.f / l_run;
-                uint32_t o[32];
-#pragma unroll 1
-                for (int c = 0; c < D / 32; ++c) {
-                    tmem_ld32(tO + c * 32, o);
-                    tmem_wait_ld();
-                    if (valid) store_chunk32<OutT>(static_cast<OutT*>(p.O) + orow * D + c * 32, o, inv);
-                }
-                if (valid && p.lse != nullptr) p.lse[orow] = (m_run + log2f(l_run)) * 0.6931471805599453f;
-                tc_fence_before();
-                // O_x may be written again (the next item's first P V)
-                __syncwarp();
-                if (lane == 0) mbar_arrive(o_drained + x);
+                const int qpos = qtX * BM + row;
+                if (p.lse != nullptr && qpos < it.Lb)
+                    p.lse[(size_t)(it.seq0 + qpos) * p.sched.Hq + hqX] = (m_run + log2f(l_run)) * 0.6931471805599453f;
+                ok = warp_wait(o_full + x, n_o & 1, 44 + x);
+                if (!ok) break;
+                store_tile(x, it, inv);
+                ++n_o;
             }
         }
     }
@@ -775,12 +830,12 @@ struct TileMaps { CUtensorMap q, k, v, x; };
 template <int D, typename OutT, bool TABLE>
 static seka_status launch_attn_t(const TileMaps& tm, const AttnParams& p, cudaStream_t st) {
     const SmemPlan sl = smem_plan<D>(p.plan);
-    const uint32_t dyn = sl.total + 1024;      // slack for the 1024-byte alignment
+    const uint32_t dyn = sl.total;
     if (dyn > SMEM_LIMIT) return SEKA_ERR_UNSUPPORTED;
     auto kern = seka_attn_fwd_kernel<D, OutT, TABLE>;
     // the attribute belongs to the function on the current device: set on every call (a cheap driver call), so that a
     // process that drives several devices, or calls from several threads, needs no bookkeeping here
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess) return SEKA_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return SEKA_ERR_CUDA;
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     // persistent CTAs, one per SM (the kernel needs the whole SM: all of tensor memory and most of shared memory)
@@ -864,11 +919,11 @@ static seka_status attention_fwd_impl(const seka_shape* shape, const void* Q, co
     if (stc != SEKA_OK) return stc;
 
     TileMaps tm;
-    if (!make_tile_map(&tm.q, q16, D, Hq, T, 128) || !make_tile_map(&tm.k, k16, D, Hkv, T, 128) ||
-        !make_tile_map(&tm.v, v16, D, Hkv, T, 128))
+    if (!make_tile_map(&tm.q, q16, D, Hq, T, BM) || !make_tile_map(&tm.k, k16, D, Hkv, T, BN) ||
+        !make_tile_map(&tm.v, v16, D, Hkv, T, BN))
         return SEKA_ERR_CUDA;
     tm.x = tm.k;      // never dereferenced without steering
-    if (p.plan.mode != 0 && !make_tile_map(&tm.x, X, p.plan.xcols, Hkv, T, 128)) return SEKA_ERR_CUDA;
+    if (p.plan.mode != 0 && !make_tile_map(&tm.x, X, p.plan.xcols, Hkv, T, BN)) return SEKA_ERR_CUDA;
 
     p.O = O; p.lse = lse;
     p.tile_hot = tile_hot; p.bh_info = bh_info; p.status = reinterpret_cast<int*>(ws);

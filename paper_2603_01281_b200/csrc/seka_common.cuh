@@ -267,9 +267,9 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s; a whole launch takes 
 constexpr int kPlainPolls = 8;
 
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                int* status, int where, uint64_t limit_ns) {
+                                                int* status, int where, uint64_t limit_ns, int plain_polls = kPlainPolls) {
 #pragma unroll 1
-    for (int i = 0; i < kPlainPolls; ++i)
+    for (int i = 0; i < plain_polls; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     uint64_t t0 = 0;
     while (true) {
