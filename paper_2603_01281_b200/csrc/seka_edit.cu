@@ -259,6 +259,8 @@ static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void*
 //
 // The step is a chain (rows and U land, product, scale, product, add, write) that several CTAs per SM walk side by side; the
 // rows of a CTA's next step are fetched under the present one where shared memory has room for a second stage.
+// Registers and code are kept small (16 columns at a time, short unrolls): a launch is often one or two steps per CTA, bound
+// by fetching its instructions, and spilled registers tripled the time of a step at head_dim 64.
 // Measured: 144 x 4096 tokens x 8 heads x 128 in place, a tenth highlighted, 94 -> 72 us per call (whole 128-row tiles
 // through a projector, of which 58 % of the rows were written); one prompt of 777 tokens on 32/8 heads 42 -> 31 us per call
 // (four launches and two memsets before, two launches now).
@@ -277,15 +279,14 @@ struct EtSmem {
     static constexpr uint32_t TILE = (D / 64) * EBLK;       // 128 key rows
     static constexpr uint32_t UMAT = D * 128;               // [D x 64] bf16
     static constexpr int NS = D == 128 && SIDE ? 1 : 2;     // stages of key rows (two CTAs per SM leave room for one beside the low parts)
-    static constexpr uint32_t U = NS * TILE;                // high part, then low part
-    static constexpr uint32_t LO = U + 2 * UMAT;            // SIDE: low parts of the edited rows
-    static constexpr uint32_t ROUTE = LO + (SIDE ? TILE : 0);         // scratch and result of Eq. 6 (routed calls)
+    static constexpr uint32_t U = NS * TILE;                // blocks of U (high part, then low part each); SIDE: then the low
+                                                            // parts of the edited rows; then scratch and result of Eq. 6
     static constexpr uint32_t TMEM_COLS = D == 128 ? 256 : 128;       // 64 for C, D for dK
     static constexpr int CTAS = D == 128 ? 2 : 3;           // per SM: tensor memory and shared memory (128), shared memory (64)
 };
 
 // SIDE: a unit of work as the warp that looked at it left it
-struct __align__(16) UnitInfo { uint32_t bits[4]; int work, b, tok0, nvalid; float c; int with_lo, pad[2]; };
+struct __align__(16) UnitInfo { uint32_t bits[4]; int work, b, tok0, nvalid; float c; int with_lo, h, pad; };
 
 struct TileArgs {
     const void* K; __nv_bfloat16* out;
@@ -294,7 +295,8 @@ struct TileArgs {
     uint8_t* tile_hot; uint8_t* bh_info;                                         // SIDE: written for the fused kernel
     int* status;
     int B, L, Hkv, r, M, n_tiles;
-    int n_route_blocks, n_tile_blocks;      // SIDE: routing blocks | item-table blocks | tile blocks | conversion blocks
+    int u_blocks;                           // blocks of U that stay in shared memory (all of them, or one that is replaced)
+    int n_tile_blocks;                      // SIDE: item-table blocks | tile blocks | conversion blocks
     RouteArgs route;
     PrepJobs jobs;
 };
@@ -313,16 +315,6 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     const bool routed = SIDE && p.route.sigma != nullptr;
     int blk = blockIdx.x;
     if constexpr (SIDE) {
-        if (blk < p.n_route_blocks) {
-            // ------------------------------------------------ Eq. 6 of one (sequence, KV head), for the caller
-            pdl_wait();
-            pdl_release();
-            const double* a = route_group(p.route.Q, p.route.q_is_f32, p.U, p.route.sigma, p.cu, p.L, p.route.Hq, Hkv, D, r, M,
-                                          p.route.k_route, blk / Hkv, blk % Hkv, reinterpret_cast<double*>(smem));
-            for (int m = tid; m < M; m += ET_THREADS) p.route.alpha_out[(size_t)blk * M + m] = (float)a[m];
-            return;
-        }
-        blk -= p.n_route_blocks;
         if (blk < p.jobs.n_items_blocks) {
             pdl_wait();
             pdl_release();
@@ -344,7 +336,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     __shared__ int tok_s[2][SIDE ? 1 : 128], seq_s[2][SIDE ? 1 : 128];      // stand-alone: token (-1: none) and sequence of a row, per stage
     __shared__ float c_s[2][SIDE ? 1 : 128];            // stand-alone: gain (one expert: times its coefficient) of a row, per stage
     __shared__ UnitInfo look_s[ET_WARPS];               // SIDE: the units looked at last
-    __shared__ unsigned short exp_s[ET_UCOLS];          // expert of a column of the block
+    __shared__ unsigned short exp_s[2 * ET_UCOLS];      // expert of a column of the blocks in shared memory
     __shared__ int pre_s[SIDE ? 1 : kMaxSegments + 1];  // stand-alone: highlighted tokens before each segment
     __shared__ int wsum_s[ET_WARPS];
     volatile int* abort_flag = &abort_s;
@@ -379,8 +371,13 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     float cur_c = 0.f;
     int unit = blk, n_units = 0, n_hot = 0;
     int look_pos = ET_WARPS;
+    // SIDE: a CTA keeps its (sequence, KV head) as long as there are enough CTAs (its block of U and its routed coefficients
+    // then serve all its units): `per` CTAs share the tiles of a pair, or a CTA takes several pairs one after another.
+    const int BH = p.B * Hkv, per = SIDE ? (p.n_tile_blocks >= BH ? p.n_tile_blocks / BH : 1) : 1;
     if constexpr (SIDE) {
-        n_units = p.B * p.n_tiles * Hkv;
+        if (p.n_tile_blocks >= BH) n_units = blk < per * BH ? (p.n_tiles - blk / BH + per - 1) / per : 0;
+        else n_units = (BH - blk + p.n_tile_blocks - 1) / p.n_tile_blocks * p.n_tiles;
+        unit = 0;                                       // units are counted per CTA
     } else if (ok) {
         // highlighted tokens before each segment, and in all
         constexpr int PT = kMaxSegments / ET_THREADS;
@@ -400,15 +397,18 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         __syncthreads();
         n_units = ((n_hot + 127) / 128) * Hkv;
     }
-    const int unit_step = SIDE ? p.n_tile_blocks : (int)gridDim.x;
-    auto next_index = [&](int u) { return u + unit_step < u ? 0x7fffffff : u + unit_step; };
+    auto unit_pair = [&](int u, int& t) -> int {        // (SIDE) pair b * Hkv + h and tile of unit u of this CTA
+        if (p.n_tile_blocks >= BH) { t = blk / BH + u * per; return blk % BH; }
+        t = u % p.n_tiles;
+        return blk + u / p.n_tiles * p.n_tile_blocks;
+    };
 
     // the next unit with work (false: none left); every thread gets the same answer
     auto next_unit = [&]() -> bool {
         if constexpr (!SIDE) {
             while (unit < n_units) {
                 cur_chunk = unit / Hkv; cur_h = unit - cur_chunk * Hkv;
-                unit = next_index(unit);
+                unit = unit + (int)gridDim.x < unit ? 0x7fffffff : unit + (int)gridDim.x;
                 if (p.head_enable == nullptr || p.head_enable[cur_h] != 0) return true;
             }
             return false;
@@ -417,10 +417,10 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                 if (look_pos == ET_WARPS) {             // a warp looks at each of the next eight units: one latency for all of them
                     if (unit >= n_units) return false;
                     __syncthreads();
-                    const long long u64 = unit + (long long)warp * unit_step;
                     UnitInfo* info = look_s + warp;
-                    if (u64 < n_units) {
-                        const int u = (int)u64, bt = u / Hkv, h = u - bt * Hkv, b = bt / p.n_tiles, t = bt - b * p.n_tiles;
+                    if (unit + warp < n_units) {
+                        int t;
+                        const int bh = unit_pair(unit + warp, t), b = bh / Hkv, h = bh - b * Hkv;
                         const int seq0 = p.cu ? p.cu[b] : b * p.L;
                         const int Lb = (p.cu ? p.cu[b + 1] : (b + 1) * p.L) - seq0;
                         const float g = p.gain[b];
@@ -437,12 +437,12 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                         if (lane == 0) {
                             *reinterpret_cast<uint4*>(info->bits) = make_uint4(bits[0], bits[1], bits[2], bits[3]);
                             info->work = (any != 0 && on && g != 0.f) ? 1 : 0;
-                            info->b = b; info->tok0 = seq0 + t * 128; info->nvalid = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
+                            info->b = b; info->h = h; info->tok0 = seq0 + t * 128; info->nvalid = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
                             info->c = g * (M == 1 && p.alpha != nullptr && !routed ? p.alpha[(size_t)b * Hkv + h] : 1.f);
                             info->with_lo = (t < kLoTiles || (sb & 2) != 0) ? 1 : 0;
                         }
                         if (h == 0) {                   // what the fused kernel needs to know
-                            if (lane == 0) p.tile_hot[bt] = any != 0 ? 1 : 0;
+                            if (lane == 0) p.tile_hot[(size_t)b * p.n_tiles + t] = any != 0 ? 1 : 0;
                             if (t == 0)
                                 for (int hh = lane; hh < Hkv; hh += 32) p.bh_info[(size_t)b * Hkv + hh] = (uint8_t)steer_byte(p.jobs.steer, b, hh, Hkv);
                         }
@@ -453,11 +453,10 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                     look_pos = 0;
                 }
                 while (look_pos < ET_WARPS) {
-                    const int u = unit;
-                    unit = next_index(u);
+                    ++unit;
                     const UnitInfo& info = look_s[look_pos++];
                     if (info.work) {
-                        cur_h = u % Hkv;
+                        cur_h = info.h;
                         cur_b = info.b; cur_tok0 = info.tok0; cur_nvalid = info.nvalid; cur_lo = info.with_lo; cur_c = info.c;
                         cur_bits = info.bits[row >> 5];
                         return true;
@@ -490,7 +489,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     auto load_rows = [&](int st) {
         const int c = tid % UPR;
         const uint32_t base = smem_u32(smem) + st * SL::TILE + (c >> 3) * EBLK;
-#pragma unroll
+#pragma unroll 2
         for (int k = 0; k < 128 / RPP; ++k) {
             const int rr = tid / UPR + k * RPP;
             const int tok = SIDE ? cur_tok0 + rr : tok_s[st][SIDE ? 0 : rr];
@@ -512,37 +511,63 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     };
     // columns [j0, j0 + 64) of the stacked U of head h as two bf16 parts: [D x 64] blocks, 128-byte swizzle (K-major operand of
     // the second product, MN-major of the first); zero up to the next multiple of 16 columns, undefined (and unused) beyond
-    auto stage_u = [&](int h, int j0) {
+    auto stage_u = [&](int h, int j0, int slot) {
+        uint8_t* sB = sU + slot * (2 * SL::UMAT);
         const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nu = (rc + 15) / 16 * 2;
-#pragma unroll 2
-        for (int u = tid; u < D * nu; u += ET_THREADS) {
-            const int i = u / nu, c8 = (u - i * nu) * 8;
-            float v[8];
-            if (u_vec && j0 + c8 + 8 <= R) {
-                const int m = (j0 + c8) / r, k = j0 + c8 - m * r;
-                const float4* src = reinterpret_cast<const float4*>(p.U + (((size_t)m * Hkv + h) * D + i) * r + k);
-                const float4 a = __ldg(src), b4 = __ldg(src + 1);
-                v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b4.x; v[5] = b4.y; v[6] = b4.z; v[7] = b4.w;
-            } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int j = j0 + c8 + e, m = j / r;
-                    v[e] = j < R ? __ldg(p.U + (((size_t)m * Hkv + h) * D + i) * r + (j - m * r)) : 0.f;
+        if (u_vec) {
+#pragma unroll 1
+            for (int u = tid; u < D * nu; u += ET_THREADS) {
+                const int i = u / nu, c8 = (u - i * nu) * 8;
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b4 = a;
+                if (j0 + c8 < R) {                          // (rank a multiple of 8: eight columns of one expert)
+                    const int m = (j0 + c8) / r, k = j0 + c8 - m * r;
+                    const float4* src = reinterpret_cast<const float4*>(p.U + (((size_t)m * Hkv + h) * D + i) * r + k);
+                    a = __ldg(src); b4 = __ldg(src + 1);
                 }
+                uint32_t hi[4], lo[4];
+                split_pair(a.x, a.y, hi[0], lo[0]); split_pair(a.z, a.w, hi[1], lo[1]);
+                split_pair(b4.x, b4.y, hi[2], lo[2]); split_pair(b4.z, b4.w, hi[3], lo[3]);
+                const uint32_t off = sw128_offset(i, c8);
+                *reinterpret_cast<uint4*>(sB + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4*>(sB + SL::UMAT + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
-            uint32_t hi[4], lo[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) split_pair(v[2 * e], v[2 * e + 1], hi[e], lo[e]);
-            const uint32_t off = sw128_offset(i, c8);
-            *reinterpret_cast<uint4*>(sU + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(sU + SL::UMAT + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        } else {
+#pragma unroll 1
+            for (int u = tid; u < D * nu * 4; u += ET_THREADS) {        // two columns at a time
+                const int i = u / (nu * 4), c2 = (u - i * (nu * 4)) * 2, j = j0 + c2, m0 = j / r, m1 = (j + 1) / r;
+                const float x = j < R ? __ldg(p.U + (((size_t)m0 * Hkv + h) * D + i) * r + (j - m0 * r)) : 0.f;
+                const float y = j + 1 < R ? __ldg(p.U + (((size_t)m1 * Hkv + h) * D + i) * r + (j + 1 - m1 * r)) : 0.f;
+                uint32_t hi, lo;
+                split_pair(x, y, hi, lo);
+                const uint32_t off = sw128_offset(i, c2);
+                *reinterpret_cast<uint32_t*>(sB + off) = hi;
+                *reinterpret_cast<uint32_t*>(sB + SL::UMAT + off) = lo;
+            }
         }
-        if (tid < ET_UCOLS) exp_s[tid] = (unsigned short)(j0 + tid < R ? (j0 + tid) / r : M - 1);
+        if (tid < ET_UCOLS) exp_s[slot * ET_UCOLS + tid] = (unsigned short)(j0 + tid < R ? (j0 + tid) / r : M - 1);
     };
 
     int st = 0, u_head = -1, routed_for = -1;           // stage, head whose only block of U is resident, (sequence, head) of the coefficients
     uint32_t n_c = 0, n_d = 0;                          // products so far (phases)
-    float* alpha_r = reinterpret_cast<float*>(smem + SL::ROUTE);
+    const bool resident = R <= ET_UCOLS * p.u_blocks;
+    uint8_t* sL = smem + SL::U + p.u_blocks * (2 * SL::UMAT);
+    float* alpha_r = reinterpret_cast<float*>(sL + (SIDE ? SL::TILE : 0));
+    // Eq. 6 of a pair b * Hkv + h into alpha_r (the scratch starts behind the result)
+    auto route_pair = [&](int bh) {
+        double* sm = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(alpha_r) + ((M * 4 + 15) & ~15));
+        const double* a = route_group(p.route.Q, p.route.q_is_f32, p.U, p.route.sigma, p.cu, p.L, p.route.Hq, Hkv, D, r, M,
+                                      p.route.k_route, bh / Hkv, bh % Hkv, sm);
+        for (int m = tid; m < M; m += ET_THREADS) alpha_r[m] = (float)a[m];
+        routed_for = bh;
+    };
+    if (routed && ok && p.route.alpha_out != nullptr && blk < BH) {
+        // the first CTA of a pair leaves its coefficients for the caller
+        for (int bh = blk; bh < BH; bh += p.n_tile_blocks) {
+            route_pair(bh);
+            __syncthreads();
+            for (int m = tid; m < M; m += ET_THREADS) p.route.alpha_out[(size_t)bh * M + m] = alpha_r[m];
+        }
+    }
     bool have = ok && next_unit();
     if (have) {
         if (!SIDE) { find_rows(0); __syncthreads(); }
@@ -551,15 +576,13 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     while (have) {
         const int h = cur_h, b = cur_b, tok0 = cur_tok0, nvalid = cur_nvalid;
         const bool with_lo = SIDE && cur_lo != 0;
-        if (u_head != h) { stage_u(h, 0); u_head = R <= ET_UCOLS ? h : -1; }
-        if (routed && routed_for != b * Hkv + h) {
-            // (the scratch starts behind the result: alpha_r holds M floats)
-            double* sm = reinterpret_cast<double*>(smem + SL::ROUTE + ((M * 4 + 15) & ~15));
-            const double* a = route_group(p.route.Q, p.route.q_is_f32, p.U, p.route.sigma, p.cu, p.L, p.route.Hq, Hkv, D, r, M,
-                                          p.route.k_route, b, h, sm);
-            for (int m = tid; m < M; m += ET_THREADS) alpha_r[m] = (float)a[m];
-            routed_for = b * Hkv + h;
+        if (u_head != h) {
+            stage_u(h, 0, 0);
+            if (resident && R > ET_UCOLS) stage_u(h, ET_UCOLS, 1);
+            u_head = resident ? h : -1;
         }
+        const bool read_back = routed && BH > p.n_tile_blocks && p.route.alpha_out != nullptr;      // written by this CTA above
+        if (routed && !read_back && routed_for != b * Hkv + h) route_pair(b * Hkv + h);
         cp_async_wait_all();
         fence_proxy_async();
         __syncthreads();                                // rows and U are in place
@@ -570,17 +593,22 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         const bool warp_hl = __any_sync(0xffffffffu, hl);
         for (int j0 = 0; j0 < R; j0 += ET_UCOLS) {
             const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nks = (rc + 15) / 16;
-            if (j0 > 0) { stage_u(h, j0); fence_proxy_async(); __syncthreads(); }
+            if (j0 > 0 && !resident) { stage_u(h, j0, 0); fence_proxy_async(); __syncthreads(); }
+            const int slot = resident ? j0 / ET_UCOLS : 0;
+            const uint32_t dU = dU0 + slot * ((2 * SL::UMAT) >> 4);
+            const unsigned short* ex = exp_s + slot * ET_UCOLS + half * 32;
             if (tid == 0) {
                 tc_fence_after();
                 const uint32_t kd = dK0 + st * (SL::TILE >> 4);
                 constexpr uint32_t IDESC = umma_idesc_bf16(ET_UCOLS, true);
+#pragma unroll 1
+                for (int pb = 0; pb < 2 * (D / 64); ++pb) {         // part of U, 64 dimensions
+                    const uint32_t kb = kd + (uint32_t)(pb % (D / 64)) * (EBLK >> 4);
+                    const uint32_t ub = dU + (((uint32_t)(pb / (D / 64)) * SL::UMAT + (uint32_t)(pb % (D / 64)) * 8192) >> 4);
 #pragma unroll
-                for (int part = 0; part < 2; ++part)
-#pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks)
-                        umma_ss(tC, kd + (((uint32_t)(ks >> 2) * EBLK + (uint32_t)(ks & 3) * 32) >> 4), DESC_HI,
-                                dU0 + (((uint32_t)part * SL::UMAT + (uint32_t)ks * 2048) >> 4), DESC_HI, IDESC, (ks > 0 || part) ? 1u : 0u);
+                    for (int ks = 0; ks < 4; ++ks)
+                        umma_ss(tC, kb + (uint32_t)(ks * 32 >> 4), DESC_HI, ub + (uint32_t)(ks * 2048 >> 4), DESC_HI, IDESC, (ks > 0 || pb > 0) ? 1u : 0u);
+                }
                 umma_commit(bars);
             }
             if (j0 == 0) {                              // under the product: what comes next
@@ -591,28 +619,29 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             ++n_c;
             ok = __all_sync(0xffffffffu, ok);
             if (ok && warp_hl && half * 32 < rc) {
-                // 32 columns of C: times the row's coefficients, split, back over themselves (16 columns of high pairs, 16 of
-                // low); what the rows that are not highlighted get is never used
+                // C times the row's coefficients, split, back over itself; what the rows that are not highlighted get is never used
                 tc_fence_after();
                 const uint32_t tc = tC + lane_off + half * 32;
-                const float* a_row = routed ? alpha_r : (M > 1 && p.alpha != nullptr ? p.alpha + ((size_t)b_row * Hkv + h) * M : nullptr);
-                uint32_t v[32], hi[16], lo[16];
-                tmem_ld32(tc, v);
-                float c4[4] = {g, g, g, g};
-                if (a_row != nullptr && (r & 7) == 0) {
+                const float* a_row = read_back ? p.route.alpha_out + (size_t)(b * Hkv + h) * M : routed ? alpha_r : (M > 1 && p.alpha != nullptr ? p.alpha + ((size_t)b_row * Hkv + h) * M : nullptr);
+                // (16 columns at a time: few registers and little code, most launches make one or two steps and are bound by
+                // fetching their instructions)
+#pragma unroll 1
+                for (int q = 0; q < 2 && half * 32 + q * 16 < rc; ++q) {
+                    uint32_t v[16], hl8[8];
+                    tmem_ld16(tc + q * 16, v);
+                    float ca = g, cb = g;
+                    if (a_row != nullptr && (r & 7) == 0) { ca *= a_row[ex[q * 16]]; cb *= a_row[ex[q * 16 + 8]]; }
+                    tmem_wait_ld_on16(v);
+                    if (a_row != nullptr && (r & 7) != 0) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) c4[q] *= a_row[exp_s[half * 32 + q * 8]];
+                        for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * a_row[ex[q * 16 + e]]);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) split_pair(__uint_as_float(v[2 * e]) * (e < 4 ? ca : cb), __uint_as_float(v[2 * e + 1]) * (e < 4 ? ca : cb), v[e], hl8[e]);
+                    // a 16-column operand block: high pairs in its first eight columns, low pairs in the others
+                    tmem_st8(tc + q * 16, v);
+                    tmem_st8(tc + q * 16 + 8, hl8);
                 }
-                tmem_wait_ld_on(v);
-                if (a_row != nullptr && (r & 7) != 0) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * a_row[exp_s[half * 32 + e]]);
-                }
-#pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    split_pair(__uint_as_float(v[2 * e]) * c4[e >> 2], __uint_as_float(v[2 * e + 1]) * c4[e >> 2], hi[e], lo[e]);
-                tmem_st16(tc, hi);
-                tmem_st16(tc + 16, lo);
                 tmem_wait_st();
             }
             tc_fence_before();
@@ -621,9 +650,10 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             if (tid == 0) {
                 tc_fence_after();
                 constexpr uint32_t IDESC = umma_idesc_bf16(D, false);
+#pragma unroll 1
                 for (int ks = 0; ks < nks; ++ks) {
-                    const uint32_t a_hi = tC + (uint32_t)(ks >> 1) * 32 + (uint32_t)(ks & 1) * 8, a_lo = a_hi + 16;
-                    const uint32_t u_hi = dU0 + (((uint32_t)ks * 32) >> 4), u_lo = u_hi + (SL::UMAT >> 4);
+                    const uint32_t a_hi = tC + (uint32_t)ks * 16, a_lo = a_hi + 8;
+                    const uint32_t u_hi = dU + (((uint32_t)ks * 32) >> 4), u_lo = u_hi + (SL::UMAT >> 4);
                     umma_ts(tD, a_hi, u_hi, DESC_HI, IDESC, (j0 > 0 || ks > 0) ? 1u : 0u);
                     umma_ts(tD, a_lo, u_hi, DESC_HI, IDESC, 1u);
                     umma_ts(tD, a_hi, u_lo, DESC_HI, IDESC, 1u);
@@ -634,21 +664,20 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             ok = mbar_wait(bars + 1, n_d & 1, abort_flag, p.status, 61);
             ++n_d;
             ok = __all_sync(0xffffffffu, ok);
-            if (R > ET_UCOLS) { ok = __syncthreads_and(ok); if (!ok) break; }      // (U is replaced next)
+            if (!resident) { ok = __syncthreads_and(ok); if (!ok) break; }      // (U is replaced next)
         }
-        if (!ok && R > ET_UCOLS) break;
+        if (!ok && !resident) break;
         uint8_t* sK = smem + st * SL::TILE;
-        uint8_t* sL = smem + SL::LO;
         if (ok && (warp_hl || with_lo)) {
             // k' = k + dK[row] for highlighted rows, half a row per thread, in place in the staged rows; low parts beside them
             tc_fence_after();
 #pragma unroll 1
-            for (int c = half * (D / 64); c < (half + 1) * (D / 64); ++c) {
-                uint32_t v[32];
-                if (warp_hl) { tmem_ld32(tD + lane_off + c * 32, v); tmem_wait_ld_on(v); }     // warp-wide: every lane takes part
+            for (int c = half * (D / 32); c < (half + 1) * (D / 32); ++c) {      // 16 columns
+                uint32_t v[16];
+                if (warp_hl) { tmem_ld16(tD + lane_off + c * 16, v); tmem_wait_ld_on16(v); }     // warp-wide: every lane takes part
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {          // 8 elements = one 16-byte unit of the swizzled row
-                    const uint32_t off = (uint32_t)((c * 32 + q * 8) >> 6) * EBLK + sw128_offset(row, (c * 32 + q * 8) & 63);
+                for (int q = 0; q < 2; ++q) {          // 8 elements = one 16-byte unit of the swizzled row
+                    const uint32_t off = (uint32_t)((c * 16) >> 6) * EBLK + sw128_offset(row, ((c * 16) & 63) + q * 8);
                     uint4 l = make_uint4(0u, 0u, 0u, 0u);
                     if (hl) {
                         uint4 kv = *reinterpret_cast<uint4*>(sK + off);
@@ -671,7 +700,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         ok = __syncthreads_and(ok);
         if (!ok) break;
         // write the rows out: D / 8 lanes per row, 16 bytes each
-#pragma unroll 4
+#pragma unroll 2
         for (int k = 0; k < 128 / RPP; ++k) {
             const int rr = tid / UPR + k * RPP, c = tid % UPR;
             const int tok = SIDE ? tok0 + rr : tok_s[st][SIDE ? 0 : rr];
@@ -758,17 +787,26 @@ static seka_status launch_tiles_t(TileArgs& a, long long n_units, size_t smem, i
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
     long long per_sm = (227 * 1024) / (smem + (SIDE ? 4 : 9) * 1024);
     per_sm = per_sm > EtSmem<D, SIDE>::CTAS ? EtSmem<D, SIDE>::CTAS : (per_sm < 1 ? 1 : per_sm);
-    // one wave; a multiple of the KV heads, so that a CTA keeps its head (and its block of U)
+    // one wave; a multiple of the (sequence, KV head) pairs or at least of the KV heads, so that a CTA keeps its block of U
     long long g = per_sm * n_sm;
-    if (g > a.Hkv) g -= g % a.Hkv;
     if (g > n_units) g = n_units;
+    if (SIDE && g >= (long long)a.B * a.Hkv) g -= g % ((long long)a.B * a.Hkv);
+    else if (g > a.Hkv) g -= g % a.Hkv;
     a.n_tile_blocks = (int)g;
     return launch_kernel(true, kern, (unsigned)(g + extra_blocks), ET_THREADS, smem, st, a);
 }
 
+// Stacked ranks of 65 to 128 keep both blocks of U in shared memory at head_dim 64, where that leaves room for two CTAs (38
+// sequences of 487 tokens, 8 heads, 4 experts of rank 32, routed: see below); at head_dim 128 the blocks are replaced per step.
+static int u_blocks_of(const seka_shape* s) {
+    const int R = s->rank * s->n_experts;
+    return s->head_dim == 64 && R > ET_UCOLS && R <= 2 * ET_UCOLS ? 2 : 1;
+}
+
 template <int D, bool SIDE>
 static size_t tiles_smem(const seka_shape* s, bool routed, int k_route) {
-    return 1024 + EtSmem<D, SIDE>::ROUTE + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
+    using SL = EtSmem<D, SIDE>;
+    return 1024 + SL::U + u_blocks_of(s) * 2 * SL::UMAT + (SIDE ? SL::TILE : 0) + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
 }
 
 static TileArgs tile_args(const seka_shape* s, const WorkspaceLayout& w, const void* K, void* out, const uint8_t* mask, const float* U,
@@ -780,7 +818,7 @@ static TileArgs tile_args(const seka_shape* s, const WorkspaceLayout& w, const v
     a.seg_tokens = edit_segment_tokens(shape_total_tokens(s));
     a.n_seg = (shape_total_tokens(s) + a.seg_tokens - 1) / a.seg_tokens;
     a.tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off); a.bh_info = reinterpret_cast<uint8_t*>(ws + w.info_off);
-    a.status = reinterpret_cast<int*>(ws);
+    a.status = reinterpret_cast<int*>(ws); a.u_blocks = u_blocks_of(s);
     a.B = s->batch; a.L = s->max_seqlen; a.Hkv = s->n_kv_heads; a.r = s->rank; a.M = s->n_experts; a.n_tiles = w.n_tiles;
     return a;
 }
@@ -1152,22 +1190,22 @@ static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout&
 seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
                               const float* alpha, const float* gain, const uint8_t* head_enable, char* ws, const PrepJobs& jobs,
                               const RouteArgs& route, cudaStream_t st) {
-    // The pipelined pair of launches from five waves of the chain on.  Measured per call, pipeline against chain: packed batch
-    // of 64 sequences, 16 heads of 64 (16384 units) 717 against 853 us; 4 x 4096 tokens x 8 heads of 128 (1024 units) 599
-    // against 597; one prompt of 777 tokens (56 units) 37 against 32.
+    // The pipelined pair of launches from four waves of the chain on.  Measured preparations, pipeline against chain: packed
+    // batch of 64 sequences, 16 heads of 64, short runs (16384 units) 105 against 132 us; 64 x 1024 tokens, 4 heads of 64 /
+    // 128, all highlighted (2048 units) 32 against 36 / 50 against 56; 38 x 487, 8 heads of 64, 44 % (1216 units) 25 against
+    // 21; 4 x 4096 tokens, 8 heads of 128, a tenth (1024 units) 18 against 16; 4362 tokens, 8 heads (280) 19 against 13.
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     const long long units = (long long)s->batch * w.n_tiles * s->n_kv_heads;
     if (units > 0x7fffffffLL) return SEKA_ERR_UNSUPPORTED;
     const int chain_ctas = s->head_dim == 128 ? EtSmem<128, true>::CTAS : EtSmem<64, true>::CTAS;
-    if (s->n_experts == 1 && route.sigma == nullptr && s->dtype == SEKA_BF16 && s->n_kv_heads <= n_sm && units > 5LL * chain_ctas * n_sm)
+    if (s->n_experts == 1 && route.sigma == nullptr && s->dtype == SEKA_BF16 && s->n_kv_heads <= n_sm && units > 4LL * chain_ctas * n_sm)
         return s->head_dim == 128 ? launch_stage_pipe<128>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st)
                                   : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st);
     TileArgs a = tile_args(s, w, K, ws + w.x_off, mask, U, alpha, gain, head_enable, ws);
     a.route = route; a.jobs = jobs;
     const bool routed = route.sigma != nullptr;
-    a.n_route_blocks = routed && route.alpha_out != nullptr ? s->batch * s->n_kv_heads : 0;
-    const int extra = a.n_route_blocks + jobs.n_items_blocks + jobs.n_conv_blocks;
+    const int extra = jobs.n_items_blocks + jobs.n_conv_blocks;
     const bool f32 = s->dtype == SEKA_F32;
     if (s->head_dim == 128) {
         const size_t smem = tiles_smem<128, true>(s, routed, route.k_route);

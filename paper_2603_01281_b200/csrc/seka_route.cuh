@@ -57,15 +57,35 @@ __device__ __noinline__ static const double* route_group(const void* Q, int q_is
     }
     __syncthreads();
     const int rows = D / C;                     // D is 64 or 128, C divides it
-    for (int u = tid; u < M * C * k_route; u += blockDim.x) {
-        const int k = u % k_route, mc = u / k_route, c = mc % C, m = mc / C;
-        const float* Um = U + (((size_t)m * Hkv + h) * D + (size_t)c * rows) * r + k;   // neighbouring threads: neighbouring columns
-        const double sg = (double)sigma[((size_t)m * Hkv + h) * r + k];
-        const double* qc = qbar + c * rows;
-        double dot = 0.0;
-#pragma unroll 16
-        for (int i = 0; i < rows; ++i) dot += qc[i] * (double)Um[(size_t)i * r];
-        term[u] = dot * sg;
+    if ((r & 3) == 0 && (k_route & 3) == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0) {
+        // four directions per thread: a quarter of the rounds, each one memory latency
+        const int k4 = k_route >> 2;
+        for (int u = tid; u < M * C * k4; u += blockDim.x) {
+            const int k = (u % k4) * 4, mc = u / k4, c = mc % C, m = mc / C;
+            const float* Um = U + (((size_t)m * Hkv + h) * D + (size_t)c * rows) * r + k;
+            const float* sg = sigma + ((size_t)m * Hkv + h) * r + k;
+            const double* qc = qbar + c * rows;
+            double dot[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+            for (int i = 0; i < rows; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(Um + (size_t)i * r);
+                const double q = qc[i];
+                dot[0] += q * (double)x.x; dot[1] += q * (double)x.y; dot[2] += q * (double)x.z; dot[3] += q * (double)x.w;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) term[(size_t)mc * k_route + k + e] = dot[e] * (double)sg[e];
+        }
+    } else {
+        for (int u = tid; u < M * C * k_route; u += blockDim.x) {
+            const int k = u % k_route, mc = u / k_route, c = mc % C, m = mc / C;
+            const float* Um = U + (((size_t)m * Hkv + h) * D + (size_t)c * rows) * r + k;   // neighbouring threads: neighbouring columns
+            const double sg = (double)sigma[((size_t)m * Hkv + h) * r + k];
+            const double* qc = qbar + c * rows;
+            double dot = 0.0;
+#pragma unroll 8
+            for (int i = 0; i < rows; ++i) dot += qc[i] * (double)Um[(size_t)i * r];
+            term[u] = dot * sg;
+        }
     }
     __syncthreads();
     // one warp per expert: each lane adds the pieces of its directions (lane, lane + 32, ...) in order, then the lanes are
