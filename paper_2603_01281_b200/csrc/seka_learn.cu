@@ -11,11 +11,11 @@
 //                         item i while item i + 1 accumulates in the other half of tensor memory.
 //   learn_reduce_kernel   sums the per-chunk partials in chunk order, scales by 1 / n.
 //   learn_dist_kernel     D = mean over the answer tokens of ||h+ - h-||_2, per slot (fixed summation order).
-//   learn_svd_kernel      one CTA per matrix: one-sided Jacobi (Hestenes) in fp64 on the columns of Omega held in
-//                         shared memory; every pair of columns meets once per sweep (ordering by recursive halving,
-//                         four lanes per pair, one column of each pair resident in registers); on convergence the
-//                         column norms are the singular values and the normalised columns the left singular
-//                         vectors; sorted descending; the rank of Eq. 3 from the sorted values.
+//   learn_svd_kernel      one CTA per matrix, fp64: QR of Omega^T, then one-sided Jacobi (Hestenes) on the columns of R^T;
+//                         half of the columns in registers, half in shared memory; every pair of columns meets once per
+//                         sweep (ordering by recursive halving); on convergence the column norms are the singular
+//                         values and the normalised columns the left singular vectors; sorted descending; the rank of
+//                         Eq. 3 from the sorted values.
 #include <math.h>
 
 #include "seka_kernels.h"
@@ -290,225 +290,424 @@ __global__ void learn_dist_reduce_kernel(const float* __restrict__ part_sum, con
     }
 }
 
-// ------------------------------------------------------------------------------------ SVD (one-sided Jacobi, fp64)
-constexpr int SV_LP = 4;                        // lanes that share a column pair: eight pairs per warp
-constexpr int SV_PAD = 4;                       // doubles of padding per column (32 bytes: the eight 32-byte pieces a warp
-                                                // touches in neighbouring columns fall on different banks)
-constexpr int SV_THREADS = 64 * SV_LP;          // 64 pairs per round at head_dim 128
+// ------------------------------------------------------------------------------------ SVD (QR + one-sided Jacobi, fp64)
+constexpr int SV_LP = 8;                        // lanes of a group
+constexpr int SV_PAD = 2;                       // doubles of padding per column (columns stay on 16-byte boundaries)
 constexpr int SV_MAX_SWEEPS = 60;
+constexpr size_t svd_smem_bytes(int d) { return sizeof(double) * (size_t)(d / 2) * (d + SV_PAD); }
 
-// One CTA per (sign, slot).  G (column-major, fp64, shared memory) starts as Omega; plane rotations from the right
-// make its columns mutually orthogonal: Omega V = U S.  Outputs: U [d x d] row-major with the singular vectors as
-// columns, S descending, and the smallest k with sum_{i<=k} S_i >= gamma * sum_i S_i (Eq. 3).
-__global__ void __launch_bounds__(SV_THREADS, 1)
-learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ omega_neg, int slots, int d, float gamma,
+// approximations to about 2^-22; arguments of the fp32 normal range
+__device__ __forceinline__ float svd_rcp(float v) { float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
+__device__ __forceinline__ float svd_rsqrt(float v) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
+
+// A plane rotation of the columns x, y by the angle theta as three shears, in place:
+//   x += al y,  y += be x,  x += al y   with  al = -tan(theta / 2), be = sin(theta):   x' = c x - s y,  y' = s x + c y.
+// Three multiply-adds per row, no scale factors to keep.  tan(theta / 2) needs no more than single precision: an error eps
+// leaves eps times the old inner product behind, which the next sweep removes; the rotation itself is orthogonal to fp64
+// because be and c follow from the rounded tan(theta / 2) in fp64.
+struct SvdRotation {
+    double td, be;                              // tan(theta / 2), sin(theta)
+    float tab;                                  // tan(theta) * (x . y): the squared norms become aa - tab, bb + tab
+};
+
+// `aa`, `bb`: squared norms, `dot` = x . y.  No branches: a pair that is orthogonal already gets the angle zero.  `cos2`,
+// `lean2`: see the end of a sweep below.
+__device__ __forceinline__ bool svd_rotation(float aa, float bb, double dot, SvdRotation& r, float& cos2, float& lean2) {
+    const float ra = svd_rcp(aa), rb = svd_rcp(bb);
+    const float ab = (float)dot, cc = (ab * ra) * (ab * rb);
+    // |cos| > 1e-13 (well above the rounding noise of the inner product), as a product of ratios so that columns of very
+    // different size neither overflow nor underflow the test
+    const bool turn = fminf(aa, bb) > 1e-37f && cc > 1e-26f;
+    // (cos, sin) of the doubled angle ~ (|bb - aa|, 2 ab), brought to the order of one by a power of two
+    const float df = bb - aa, t2ab = 2.f * ab;
+    const float sc = __int_as_float(0x7f000000 - (__float_as_int(fmaxf(fabsf(df), fabsf(t2ab))) & 0x7f800000));
+    const float dn = fabsf(df) * sc, tn = (df >= 0.f ? t2ab : -t2ab) * sc;
+    const float ih = svd_rsqrt(fmaf(dn, dn, tn * tn));
+    const float u = fmaf(0.5f * dn, ih, 0.5f), iu = svd_rsqrt(u), cs = u * iu;       // cos^2(theta), 1 / cos(theta), cos(theta)
+    const float s2 = tn * ih;                                                       // sin(2 theta)
+    const float tau = turn ? 0.5f * s2 * svd_rcp(cs + u) : 0.f;
+    const float t = 0.5f * s2 * (iu * iu);
+    // sin(theta) = 2 tau / (1 + tau^2) in fp64: cos^2(theta / 2) = (1 + cos(theta)) / 2 is the reciprocal to single
+    // precision, one step of third order makes it exact
+    const double td = (double)tau, r0 = (double)(turn ? fmaf(0.5f, cs, 0.5f) : 1.f), p = (td + td) * r0;
+    const double e = fma(-fma(td, td, 1.0), r0, 1.0);
+    r.td = td;
+    r.be = fma(p, fma(e, e, e), p);
+    r.tab = turn ? t * ab : 0.f;
+    if (turn) {
+        cos2 = fmaxf(cos2, cc);
+        lean2 = fmaxf(lean2, t * t * fmaxf(aa * rb, bb * ra));
+    }
+    return turn;
+}
+
+// One CTA per (sign, slot).  Outputs: U [D x D] row-major with the left singular vectors of Omega as columns, S descending,
+// and the smallest k with sum_{i<=k} S_i >= gamma * sum_i S_i (Eq. 3).
+//
+// 1. Householder QR of Omega^T with its columns (the rows of Omega) taken by falling norm:  Omega^T P = Q R, so Omega has the
+//    left singular vectors and the singular values of L = P R^T, whose rows stand in the order of Omega's.  Omega^T is
+//    held by columns; step k finishes entry k of every column, so what the last step leaves is L, row by row.
+//    L is far closer to orthogonal columns than Omega is (Drmac and Veselic's preconditioning of the Jacobi method): 5-6
+//    sweeps instead of 10-12 on learned cross-covariances, for the price of about one sweep.
+// 2. One-sided Jacobi (Hestenes): plane rotations from the right make the columns of L mutually orthogonal, L J = U S.
+//
+// Half of the columns live in registers, half in shared memory: two CTAs fit on an SM and their rounds overlap.  A group of
+// SV_LP lanes holds two columns (x0, x1); lane lg holds the rows 2 SV_LP e + 2 lg + {0, 1}.
+//
+// Ordering of a sweep (every pair of columns meets once): level m = D / 2, D / 4, ..., 2 cuts the D / 2 column positions of
+// either kind into blocks of m.  In round r of the level, the group whose columns are the 2i-th and (2i + 1)-th of its block
+// meets the ((2i + r) mod m)-th column of the block in shared memory: one read and one write of that column for two rotations.
+// Both inner products are formed at once: the second, with the column that the first rotation leaves, follows from x0 . x1,
+// which is formed once a level and carried along (what the single-precision angle leaves of x0' . y' is neglected there: a
+// relative 2^-22 of a product that shrinks quadratically).  Between levels the groups of the second half of a block swap their
+// columns with the ones in shared memory half a block before: pairs within either half meet next.  The last level rotates
+// x0 against x1, swaps both with shared memory, and rotates again.
+//
+// End: a sweep without a rotation, or one after which no pair can have a cosine above 1e-13: with c the largest
+// cosine of the sweep and l the largest |t| max(|A| / |B|, |B| / |A|) (how far a rotation leans a column, relative to its length),
+// a pair made orthogonal meets at most 2 (D - 1) more rotations, each of which changes its cosine by at most l c.
+//
+// What bounds it: the shared-memory reads and writes of the visiting columns and the latency of a round (inner products,
+// angle, update: a chain of dependent operations).  128 registers a thread are what two CTAs leave: half of the visiting
+// column is read a second time rather than held through the angles (with all of it held the spills cost 10 %).
+// Measured, 576 matrices of 128 x 128: 5.99 -> 2.79 ms (before: no QR, one column per group resident, the whole matrix in
+// shared memory and so one CTA per SM, scaled rotations).
+template <int D>
+__global__ void __launch_bounds__(2 * D, D == 128 ? 2 : 4)
+learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ omega_neg, int slots, float gamma,
                  float* __restrict__ U_pos, float* __restrict__ U_neg, float* __restrict__ S_pos, float* __restrict__ S_neg,
                  int* __restrict__ k_pos, int* __restrict__ k_neg, int* __restrict__ sweeps_out) {
-    extern __shared__ double sv_sm[];
-    const int ldg = d + SV_PAD;             // column stride: the pad staggers neighbouring columns over the banks
-    double* G = sv_sm;                      // [d][ldg], column j at G + j * ldg
-    double* sig = G + (size_t)d * ldg;      // [d]
-    int* order = reinterpret_cast<int*>(sig + d);   // [d]: position of column j in the sorted output
-    __shared__ int rotated;
-    __shared__ double pr[64], scl[128], iscl[128], scale;
-    __shared__ float nrm2[128];
+    constexpr int NT = 2 * D, NP = D / 2, LDG = D + SV_PAD;       // threads, columns of either kind, column stride
+    constexpr int NE = D / (2 * SV_LP), HE = NE / 2;              // row pairs per lane; those of the first D / 2 rows
+    extern __shared__ __align__(16) double sv_sm[];
+    double* G = sv_sm;                      // [NP][LDG]: the columns in shared memory
+    __shared__ __align__(16) double vbuf[2][D];
+    __shared__ double sig[D], beta[2];
+    __shared__ float nrm2[NP], red[NT / 32];
+    __shared__ int order[D];
+    __shared__ unsigned worst[2];           // bits of the largest cos2, lean2 of a sweep
     const int sign = blockIdx.x / slots, slot = blockIdx.x % slots;
-    const float* om = (sign == 0 ? omega_pos : omega_neg) + (size_t)slot * d * d;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n_warps = SV_THREADS / 32;
-    for (int idx = tid; idx < d * d; idx += SV_THREADS) {
-        const int i = idx / d, j = idx - i * d;     // Omega[i][j], coalesced read
-        G[(size_t)j * ldg + i] = (double)om[idx];
+    const float* om = (sign == 0 ? omega_pos : omega_neg) + (size_t)slot * D * D;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = tid / SV_LP, lg = tid % SV_LP;      // group, lane within the group
+    const unsigned group_mask = 0xffu << (lane & ~(SV_LP - 1));
+    auto group_sum = [&](double v) {
+#pragma unroll
+        for (int o = SV_LP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(group_mask, v, o);
+        return v;
+    };
+    double2* gp0 = reinterpret_cast<double2*>(G + (size_t)(2 * g) * LDG) + lg;          // the two positions that the group
+    double2* gp1 = reinterpret_cast<double2*>(G + (size_t)(2 * g + 1) * LDG) + lg;      // folds, swaps and reduces
+
+    // ---- Omega^T by columns, its largest entry scaled to 2^40 (the squares of the norms have to fit fp32: 2^-125 to 2^94)
+    double2 x0[NE], x1[NE], y[NE];
+    float mx = 0.f;
+    {
+        auto row = [&](int j, int e) {
+            const float2 v = *reinterpret_cast<const float2*>(om + (size_t)j * D + 2 * SV_LP * e + 2 * lg);
+            mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
+            return make_double2((double)v.x, (double)v.y);
+        };
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            x0[e] = row(2 * g, e);
+            x1[e] = row(2 * g + 1, e);
+            gp0[SV_LP * e] = row(NP + 2 * g, e);
+            gp1[SV_LP * e] = row(NP + 2 * g + 1, e);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[warp] = mx;
+    __syncthreads();
+    mx = 0.f;
+    for (int w = 0; w < NT / 32; ++w) mx = fmaxf(mx, red[w]);
+    const double scale = (double)mx * 0x1p-40, inv_scale = mx > 0.f ? 1.0 / scale : 0.0;
+    {
+        double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;
+        auto scaled = [&](double2& v, double& n) {
+            v.x *= inv_scale; v.y *= inv_scale;
+            n = fma(v.x, v.x, fma(v.y, v.y, n));
+        };
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            scaled(x0[e], n0);
+            scaled(x1[e], n1);
+            double2 v = gp0[SV_LP * e];
+            scaled(v, n2); gp0[SV_LP * e] = v;
+            v = gp1[SV_LP * e];
+            scaled(v, n3); gp1[SV_LP * e] = v;
+        }
+        n0 = group_sum(n0); n1 = group_sum(n1); n2 = group_sum(n2); n3 = group_sum(n3);
+        if (lg == 0) { sig[2 * g] = n0; sig[2 * g + 1] = n1; sig[NP + 2 * g] = n2; sig[NP + 2 * g + 1] = n3; }
     }
     __syncthreads();
-    // scale the matrix to unit largest entry (squares of column norms stay far from under- and overflow)
-    {
-        double mx = 0.0;
-        for (int idx = tid; idx < d * d; idx += SV_THREADS) mx = fmax(mx, fabs(G[(size_t)(idx / d) * ldg + idx % d]));
+    if (tid < D) {
+        int rk = 0;
+#pragma unroll 4
+        for (int i = 0; i < D; ++i) rk += (sig[i] > sig[tid] || (sig[i] == sig[tid] && i < tid)) ? 1 : 0;
+        order[rk] = tid;
+    }
+    __syncthreads();
+
+    // ---- QR: one barrier per step; the owner of the next pivot column publishes its reflector I - beta v v^T
+    auto publish = [&](int k) {
+        const int j = order[k], jj = j & (NP - 1);
+        if ((jj >> 1) != g) return;
+        const double2* c = (jj & 1) == 0 ? gp0 : gp1;
+        double n0 = 0.0, n1 = 0.0, pv = 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 0) pr[warp] = mx;
-        __syncthreads();
-        if (tid == 0) {
-            double m2 = 0.0;
-            for (int w = 0; w < n_warps; ++w) m2 = fmax(m2, pr[w]);
-            scale = m2;
+        for (int e = 0; e < NE; ++e) {
+            const int i = 2 * SV_LP * e + 2 * lg;
+            y[e] = c[SV_LP * e];
+            if (j < NP) y[e] = (jj & 1) == 0 ? x0[e] : x1[e];
+            if (i < k) y[e].x = 0.0;
+            if (i + 1 < k) y[e].y = 0.0;
+            if (i == k) pv = y[e].x;
+            if (i + 1 == k) pv = y[e].y;
+            n0 = fma(y[e].x, y[e].x, n0);
+            n1 = fma(y[e].y, y[e].y, n1);
         }
-        __syncthreads();
-        const double inv = scale > 0.0 ? 1.0 / scale : 0.0;
-        for (int idx = tid; idx < d * d; idx += SV_THREADS) G[(size_t)(idx / d) * ldg + idx % d] *= inv;
+        n0 = group_sum(n0 + n1);
+        // the norm to 2^-42 (it only decides how close to zero the column is brought), beta = 2 / (v . v) to fp64
+        const double r = (double)svd_rsqrt((float)n0), n = n0 * (r * fma(-0.5 * n0, r * r, 1.5));
+        const bool some = n0 > 1e-36;           // (columns below 2^-100 of the largest entry: no reflection)
+        const double vk = some ? pv + (pv < 0.0 ? -n : n) : 0.0, vv = fma(vk, vk, fma(-pv, pv, n0));
+        const double q = (double)svd_rcp((float)vv), e1 = fma(-vv, q, 1.0);
+        if (((k >> 1) & (SV_LP - 1)) == lg) beta[k & 1] = some ? 2.0 * fma(q, fma(e1, e1, e1), q) : 0.0;     // the lane of row k
+        double2* vb = reinterpret_cast<double2*>(vbuf[k & 1]) + lg;
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const int i = 2 * SV_LP * e + 2 * lg;
+            vb[SV_LP * e] = make_double2(i == k ? vk : y[e].x, i + 1 == k ? vk : y[e].y);
+        }
+    };
+    publish(0);
+    __syncthreads();
+#pragma unroll 1
+    for (int k = 0; k < D; ++k) {
+        const double2* vb = reinterpret_cast<const double2*>(vbuf[k & 1]) + lg;
+        double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
+        auto dots = [&](int e) {
+            const double2 v = vb[SV_LP * e], c3 = gp1[SV_LP * e];
+            y[e] = gp0[SV_LP * e];
+            d0 = fma(v.x, x0[e].x, fma(v.y, x0[e].y, d0));
+            d1 = fma(v.x, x1[e].x, fma(v.y, x1[e].y, d1));
+            d2 = fma(v.x, y[e].x, fma(v.y, y[e].y, d2));
+            d3 = fma(v.x, c3.x, fma(v.y, c3.y, d3));
+        };
+        auto update = [&](int e) {
+            const double2 v = vb[SV_LP * e];
+            double2 c = gp1[SV_LP * e];
+            x0[e].x = fma(d0, v.x, x0[e].x); x0[e].y = fma(d0, v.y, x0[e].y);
+            x1[e].x = fma(d1, v.x, x1[e].x); x1[e].y = fma(d1, v.y, x1[e].y);
+            gp0[SV_LP * e] = make_double2(fma(d2, v.x, y[e].x), fma(d2, v.y, y[e].y));
+            c.x = fma(d3, v.x, c.x); c.y = fma(d3, v.y, c.y);
+            gp1[SV_LP * e] = c;
+        };
+        // the reflector is zero above row k: the first half of the rows is finished after half of the steps
+        if (k < D / 2) {
+#pragma unroll
+            for (int e = 0; e < HE; ++e) dots(e);
+        }
+#pragma unroll
+        for (int e = HE; e < NE; ++e) dots(e);
+        const double nb = -beta[k & 1];
+        d0 = nb * group_sum(d0); d1 = nb * group_sum(d1); d2 = nb * group_sum(d2); d3 = nb * group_sum(d3);
+        if (k < D / 2) {
+#pragma unroll
+            for (int e = 0; e < HE; ++e) update(e);
+        }
+#pragma unroll
+        for (int e = HE; e < NE; ++e) update(e);
+        if (k + 1 < D) publish(k + 1);
         __syncthreads();
     }
-    constexpr int RPL = 128 / SV_LP;                // rows per lane at d = 128 (d = 64 uses the first half)
-    const int per_lane = d / SV_LP;
-    const int n_pairs = d / 2;
-    // Scaled (fast) rotations: column j of the matrix is scl[j] * g_j with g_j the stored column.  A rotation
-    //   A' = c (A - t B),  B' = c (B + t A)   becomes   g_a' = g_a - (t s_b / s_a) g_b,  g_b' = g_b + (t s_a / s_b) g_a
-    // (two multiply-adds per row instead of four operations) with s_a' = c s_a, s_b' = c s_b; the reciprocals are
-    // tracked too (1 / c = (1 + t^2) c), so no division is needed for the ratios.  The scales are folded back into
-    // the columns at the start of every sweep (c >= 1 / sqrt 2 per rotation, 127 rotations per sweep at most).
-    //
-    // Ordering of a sweep (every pair of columns meets once, d - 1 rounds of d / 2 disjoint pairs): level l cuts
-    // the columns into blocks of 2 m, m = d / 2, d / 4, ..., 1; in round r of the level the i-th column of the first
-    // half of a block meets the ((i + r) mod m)-th column of its second half.  A group of SV_LP lanes owns one
-    // first-half column for the whole level and keeps it in registers; only the second-half columns go through
-    // shared memory (read, rotated, written back in place), and there is one barrier per round, since every group
-    // works out its own rotation.
-    //
-    // What bounds the kernel is the fp64 pipe (one warp instruction every 8-11 cycles per scheduler on this part),
-    // so the aim is few fp64 warp instructions per round: several pairs share a warp (the scalar work of a rotation
-    // is then issued once for all of them), the tangent and the squared norms are fp32, only what decides the
-    // orthogonality of the result stays fp64.
-    for (int j = tid; j < d; j += SV_THREADS) { scl[j] = 1.0; iscl[j] = 1.0; }
-    const int grp = lane / SV_LP, lg = lane % SV_LP;
-    const int hw = (32 / SV_LP) * warp + grp;       // pair slot of a round
-    const bool active = hw < n_pairs;
+
+    // ---- column j, entry k  ->  column k, entry j, through the shared half
+    {
+        auto at = [&](int c, int i) -> double& { return G[(size_t)c * LDG + i]; };
+        auto i0 = [&](int e) { return 2 * SV_LP * e + 2 * lg; };
+#pragma unroll
+        for (int e = 0; e < HE; ++e) {
+            y[e] = make_double2(at(i0(e), 2 * g), at(i0(e) + 1, 2 * g));
+            y[HE + e] = make_double2(at(i0(e), 2 * g + 1), at(i0(e) + 1, 2 * g + 1));
+        }
+        for (int idx = tid; idx < NP * NP; idx += NT) {         // the quarter that stays in shared memory
+            const int c = idx / NP, i = idx % NP;
+            if (i < c) { const double u = at(c, NP + i); at(c, NP + i) = at(i, NP + c); at(i, NP + c) = u; }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < HE; ++e) { gp0[SV_LP * e] = x0[e]; gp1[SV_LP * e] = x1[e]; }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < HE; ++e) {
+            x0[e] = make_double2(at(i0(e), 2 * g), at(i0(e) + 1, 2 * g));
+            x1[e] = make_double2(at(i0(e), 2 * g + 1), at(i0(e) + 1, 2 * g + 1));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < HE; ++e) {
+            at(i0(e), 2 * g) = x0[HE + e].x; at(i0(e) + 1, 2 * g) = x0[HE + e].y;
+            at(i0(e), 2 * g + 1) = x1[HE + e].x; at(i0(e) + 1, 2 * g + 1) = x1[HE + e].y;
+            x0[HE + e] = y[e];
+            x1[HE + e] = y[HE + e];
+        }
+        __syncthreads();
+    }
+
+    // ---- Jacobi
+    double nx0, nx1, ny0, ny1;              // squared norms of the group's columns and of the two at its positions
+    auto norms = [&]() {
+        auto add = [](const double2& v, double& n) { n = fma(v.x, v.x, fma(v.y, v.y, n)); };
+        nx0 = nx1 = ny0 = ny1 = 0.0;
+#pragma unroll
+        for (int e = 0; e < NE; ++e) { add(x0[e], nx0); add(x1[e], nx1); add(gp0[SV_LP * e], ny0); add(gp1[SV_LP * e], ny1); }
+        nx0 = group_sum(nx0); nx1 = group_sum(nx1); ny0 = group_sum(ny0); ny1 = group_sum(ny1);
+    };
+    float aa0, aa1;
+    // x0, x1 <-> the columns at positions q and q + 1
+    auto swap_columns = [&](int q) {
+        double2* c0 = reinterpret_cast<double2*>(G + (size_t)q * LDG) + lg;
+        double2* c1 = reinterpret_cast<double2*>(G + (size_t)(q + 1) * LDG) + lg;
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            double2 v = c0[SV_LP * e]; c0[SV_LP * e] = x0[e]; x0[e] = v;
+            v = c1[SV_LP * e]; c1[SV_LP * e] = x1[e]; x1[e] = v;
+        }
+        const float n0 = nrm2[q], n1 = nrm2[q + 1];
+        __syncwarp(group_mask);
+        if (lg == 0) { nrm2[q] = aa0; nrm2[q + 1] = aa1; }
+        aa0 = n0; aa1 = n1;
+    };
+    auto resident_dot = [&]() {
+        double a = 0.0, b = 0.0;
+#pragma unroll
+        for (int e = 0; e < NE; ++e) { a = fma(x0[e].x, x1[e].x, a); b = fma(x0[e].y, x1[e].y, b); }
+        return group_sum(a + b);
+    };
+    // a block's columns change hands: the warps of the block (8 columns per warp) wait for one another.  Every block of every
+    // level has a barrier of its own (1, 2 | 3 .. 6): one block may be a level ahead of another
+    auto block_sync = [&](int m) {
+        __syncwarp();
+        if (m == NP) __syncthreads();
+        else if (m > 8) asm volatile("bar.sync %0, %1;" ::"r"(NP / m - 1 + 2 * g / m), "r"(m * 4) : "memory");
+    };
     int sweep = 0;
     for (; sweep < SV_MAX_SWEEPS; ++sweep) {
-        if (tid == 0) rotated = 0;
+        norms();                            // exact at the start of every sweep; inside it they follow the rotations in fp32,
+        aa0 = (float)nx0; aa1 = (float)nx1; // as they only feed the tangent
+        if (lg == 0) { nrm2[2 * g] = (float)ny0; nrm2[2 * g + 1] = (float)ny1; }
+        if (tid == 0) { worst[0] = 0u; worst[1] = 0u; }
         __syncthreads();
-        // fold the scales, and the squared column norms, exact at the start of every sweep; inside the sweep they
-        // follow the rotations (A' . A' = A . A - t A . B,  B' . B' = B . B + t A . B) in fp32: they only feed the
-        // tangent.  A pair then costs one inner product.
-        for (int j = warp; j < d; j += n_warps) {
-            const double sj = scl[j];
-            double ss = 0.0;
-            for (int i = lane; i < d; i += 32) {
-                const double v = G[(size_t)j * ldg + i] * sj;
-                G[(size_t)j * ldg + i] = v;
-                ss = fma(v, v, ss);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-            __syncwarp();
-            if (lane == 0) { nrm2[j] = (float)ss; scl[j] = 1.0; iscl[j] = 1.0; }
-        }
-        __syncthreads();
-        for (int m = n_pairs; m >= 1; m >>= 1) {
-            // the resident column of this group for the level, with its scale, reciprocal scale and squared norm
-            const int blk = hw / m, idx = hw - blk * m;
-            const int ca = blk * 2 * m + idx;
-            double x[RPL];
-            double sa = 1.0, isa = 1.0;
-            float aa = 0.f, saf = 1.f;
-            if (active) {
-                const double* ga = G + (size_t)ca * ldg;
-#pragma unroll
-                for (int e = 0; e < RPL; ++e)
-                    if (e < per_lane) x[e] = ga[lg + SV_LP * e];
-                sa = scl[ca]; isa = iscl[ca]; aa = nrm2[ca]; saf = (float)sa;
-            }
+        float cos2 = 0.f, lean2 = 0.f;
+#pragma unroll 1
+        for (int m = NP; m >= 2; m >>= 1) {
+            const int idx = (2 * g) & (m - 1), p0 = 2 * g - idx;        // position in the block, first position of the block
+            double g01 = resident_dot();
+#pragma unroll 1
             for (int r = 0; r < m; ++r) {
-                if (active) {
-                    int ib = idx + r;
-                    if (ib >= m) ib -= m;
-                    const int cb = blk * 2 * m + m + ib;
-                    double* gb = G + (size_t)cb * ldg;
-                    double y[RPL];
-                    double dsum[4] = {0.0, 0.0, 0.0, 0.0};      // four chains: dependent fp64 operations are slow
+                const int q = p0 + ((idx + r) & (m - 1));
+                double2* gb = reinterpret_cast<double2*>(G + (size_t)q * LDG) + lg;
+                double a0 = 0.0, b0 = 0.0, a1 = 0.0, b1 = 0.0;
 #pragma unroll
-                    for (int e = 0; e < RPL; ++e) {
-                        if (e < per_lane) {
-                            y[e] = gb[lg + SV_LP * e];
-                            dsum[e & 3] = fma(x[e], y[e], dsum[e & 3]);
-                        }
-                    }
-                    double dot = (dsum[0] + dsum[1]) + (dsum[2] + dsum[3]);
+                for (int e = 0; e < NE; ++e) {
+                    y[e] = gb[SV_LP * e];
+                    a0 = fma(x0[e].x, y[e].x, a0); a1 = fma(x1[e].x, y[e].x, a1);
+                    b0 = fma(x0[e].y, y[e].y, b0); b1 = fma(x1[e].y, y[e].y, b1);
+                }
+                const float bb = nrm2[q];
+                const double d0 = group_sum(a0 + b0), d1 = group_sum(a1 + b1);
+                // every lane of the group holds the same sums and works out the same rotations
+                SvdRotation u, v;
+                asm volatile("" ::: "memory");         // (the second half of the column is read again below)
+                bool any = svd_rotation(aa0, bb, d0, u, cos2, lean2);
+                any |= svd_rotation(aa1, bb + u.tab, fma(u.be, fma(-u.td, d1, g01), d1), v, cos2, lean2);
+                if (__any_sync(0xffffffffu, any)) {
+                    g01 = fma(-u.be, fma(u.td, g01, d1), g01);
+                    aa0 = fmaxf(aa0 - u.tab, 0.f); aa1 = fmaxf(aa1 - v.tab, 0.f);
+                    if (lg == 0) nrm2[q] = bb + u.tab + v.tab;
 #pragma unroll
-                    for (int o = SV_LP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);   // within the group
-                    // every lane of the group holds the same sums and works out the same rotation
-                    const double sb = scl[cb], isb = iscl[cb];
-                    const float bb = nrm2[cb];
-                    // The tangent of the rotation angle needs no more than single precision: an error eps in t leaves
-                    // eps times the old inner product behind, which the next sweep removes; the rotation itself stays
-                    // exact because the same t goes into both columns and into the scales.
-                    const float ab = saf * (float)sb * (float)dot;
-                    float tf = 0.f;
-                    // |cos| > 1e-13 (well above the rounding noise of the inner product), as a product of ratios so
-                    // that columns of very different size neither overflow nor underflow the test
-                    if (aa > 0.f && bb > 0.f && (ab / aa) * (ab / bb) > 1e-26f) {
-                        const float df = bb - aa, t2ab = 2.f * ab;
-                        const float mf = fmaxf(fabsf(df), fabsf(t2ab));
-                        const float dn = df / mf, tn = t2ab / mf;
-                        tf = (dn >= 0.f ? tn : -tn) / (fabsf(dn) + sqrtf(fmaf(dn, dn, tn * tn)));
-                    }
-                    if (tf != 0.f) {                    // the same decision on all lanes of the group
-                        // the cosine: one Newton step in fp64 from an fp32 seed
-                        const double t = (double)tf;
-                        const double t2 = fma(t, t, 1.0);
-                        const double c0 = (double)rsqrtf(fmaf(tf, tf, 1.f));
-                        const double cs = c0 * fma(-0.5 * t2, c0 * c0, 1.5), ics = t2 * cs;
-                        const double ta = t * sb * isa, tb = t * sa * isb;
-#pragma unroll
-                        for (int e = 0; e < RPL; ++e) {
-                            if (e < per_lane) {
-                                const double xo = x[e];
-                                x[e] = fma(-ta, y[e], xo);
-                                gb[lg + SV_LP * e] = fma(tb, xo, y[e]);
-                            }
-                        }
-                        if (lg == 0) {
-                            scl[cb] = cs * sb; iscl[cb] = isb * ics; nrm2[cb] = bb + tf * ab;
-                            rotated = 1;
-                        }
-                        sa *= cs; isa *= ics; saf = (float)sa; aa = fmaxf(aa - tf * ab, 0.f);
+                    for (int e = 0; e < NE; ++e) {
+                        double2 c = e < HE ? y[e] : gb[SV_LP * e];
+                        x0[e].x = fma(-u.td, c.x, x0[e].x); x0[e].y = fma(-u.td, c.y, x0[e].y);
+                        c.x = fma(u.be, x0[e].x, c.x); c.y = fma(u.be, x0[e].y, c.y);
+                        x0[e].x = fma(-u.td, c.x, x0[e].x); x0[e].y = fma(-u.td, c.y, x0[e].y);
+                        x1[e].x = fma(-v.td, c.x, x1[e].x); x1[e].y = fma(-v.td, c.y, x1[e].y);
+                        c.x = fma(v.be, x1[e].x, c.x); c.y = fma(v.be, x1[e].y, c.y);
+                        x1[e].x = fma(-v.td, c.x, x1[e].x); x1[e].y = fma(-v.td, c.y, x1[e].y);
+                        gb[SV_LP * e] = c;
                     }
                 }
-                __syncthreads();                        // the second-half columns change hands
+                block_sync(m);
             }
-            // the level ends: the resident columns go back
-            if (active) {
-                double* ga = G + (size_t)ca * ldg;
-#pragma unroll
-                for (int e = 0; e < RPL; ++e)
-                    if (e < per_lane) ga[lg + SV_LP * e] = x[e];
-                if (lg == 0) { scl[ca] = sa; iscl[ca] = isa; nrm2[ca] = aa; }
+            if (m > 2) {
+                if (idx >= m / 2) swap_columns(2 * g - m / 2);
+                block_sync(m);
             }
-            __syncthreads();
         }
-        if (rotated == 0) break;                    // a whole sweep without a rotation: the columns are orthogonal
-        __syncthreads();
-    }
-    // fold the scales of the last sweep
-    for (int j = warp; j < d; j += n_warps) {
-        const double sj = scl[j];
-        for (int i = lane; i < d; i += 32) G[(size_t)j * ldg + i] *= sj;
-    }
-    __syncthreads();
-    // singular values = column norms
-    for (int j = warp; j < d; j += n_warps) {
-        double ss = 0.0;
-        for (int i = lane; i < d; i += 32) ss = fma(G[(size_t)j * ldg + i], G[(size_t)j * ldg + i], ss);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            SvdRotation u;
+            if (svd_rotation(aa0, aa1, resident_dot(), u, cos2, lean2)) {
+                aa0 = fmaxf(aa0 - u.tab, 0.f); aa1 += u.tab;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) sig[j] = sqrt(ss);           // of the scaled matrix; the scale goes back on at the output
+                for (int e = 0; e < NE; ++e) {
+                    x0[e].x = fma(-u.td, x1[e].x, x0[e].x); x0[e].y = fma(-u.td, x1[e].y, x0[e].y);
+                    x1[e].x = fma(u.be, x0[e].x, x1[e].x); x1[e].y = fma(u.be, x0[e].y, x1[e].y);
+                    x0[e].x = fma(-u.td, x1[e].x, x0[e].x); x0[e].y = fma(-u.td, x1[e].y, x0[e].y);
+                }
+            }
+            if (h == 0) swap_columns(2 * g);
+        }
+        if (lg == 0) { atomicMax(&worst[0], __float_as_uint(cos2)); atomicMax(&worst[1], __float_as_uint(lean2)); }
+        __syncthreads();
+        constexpr float stop = 1e-13f / (2 * (D - 1));
+        const bool done = __uint_as_float(worst[0]) * __uint_as_float(worst[1]) < stop * stop;
+        __syncthreads();
+        if (done) break;
     }
+    norms();                                        // singular values = column norms
+    if (lg == 0) { sig[2 * g] = sqrt(nx0); sig[2 * g + 1] = sqrt(nx1); sig[NP + 2 * g] = sqrt(ny0); sig[NP + 2 * g + 1] = sqrt(ny1); }
     __syncthreads();
     // descending order (ties: the earlier column first)
-    for (int j = tid; j < d; j += SV_THREADS) {
-        int r = 0;
-        for (int i = 0; i < d; ++i) r += (sig[i] > sig[j] || (sig[i] == sig[j] && i < j)) ? 1 : 0;
-        order[j] = r;
+    if (tid < D) {
+        int rk = 0;
+#pragma unroll 4
+        for (int i = 0; i < D; ++i) rk += (sig[i] > sig[tid] || (sig[i] == sig[tid] && i < tid)) ? 1 : 0;
+        order[tid] = rk;
     }
     __syncthreads();
-    float* Uo = (sign == 0 ? U_pos : U_neg) + (size_t)slot * d * d;
-    float* So = (sign == 0 ? S_pos : S_neg) + (size_t)slot * d;
-    for (int idx = tid; idx < d * d; idx += SV_THREADS) {
-        const int i = idx / d, j = idx - i * d;     // component i of column j
-        const double s = sig[j];
-        Uo[(size_t)i * d + order[j]] = s > 0.0 ? (float)(G[(size_t)j * ldg + i] / s) : 0.f;
-    }
-    for (int j = tid; j < d; j += SV_THREADS) So[order[j]] = (float)(sig[j] * scale);
+    float* Uo = (sign == 0 ? U_pos : U_neg) + (size_t)slot * D * D;
+    float* So = (sign == 0 ? S_pos : S_neg) + (size_t)slot * D;
+    auto write_half = [&](int c0) {
+        for (int idx = tid; idx < D * NP; idx += NT) {
+            const int i = idx / NP, j = idx % NP;   // component i of column j
+            const double sv = sig[c0 + j];
+            Uo[(size_t)i * D + order[c0 + j]] = sv > 0.0 ? (float)(G[(size_t)j * LDG + i] / sv) : 0.f;
+        }
+    };
+    write_half(NP);
+    if (tid < D) So[order[tid]] = (float)(sig[tid] * scale);        // the scale of the matrix goes back on
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < NE; ++e) { gp0[SV_LP * e] = x0[e]; gp1[SV_LP * e] = x1[e]; }
+    __syncthreads();
+    write_half(0);
+    __syncthreads();
+    if (tid < D) G[order[tid]] = sig[tid];          // the matrix has been written out: its first entries take the sorted values
     __syncthreads();
     if (tid == 0) {
         // Eq. 3 on the sorted values, in fp64
-        double* sorted = G;                         // the matrix has been written out: reuse its first d entries
-        for (int j = 0; j < d; ++j) sorted[order[j]] = sig[j];
         double total = 0.0;
-        for (int j = 0; j < d; ++j) total += sorted[j];
+#pragma unroll 4
+        for (int j = 0; j < D; ++j) total += G[j];
         double run = 0.0;
-        int k = d;
-        for (int j = 0; j < d; ++j) {
-            run += sorted[j];
+        int k = D;
+#pragma unroll 1
+        for (int j = 0; j < D; ++j) {
+            run += G[j];
             if (run >= (double)gamma * total) { k = j + 1; break; }
         }
         (sign == 0 ? k_pos : k_neg)[slot] = k;
@@ -588,8 +787,7 @@ extern "C" seka_status seka_learn_projections(const seka_learn_shape* shape, con
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     if (cudaFuncSetAttribute(learn_cov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LC_DYN_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(learn_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * (128 * (128 + SV_PAD) + 128) + sizeof(int) * 128)) != cudaSuccess)
+        cudaFuncSetAttribute(learn_svd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)svd_smem_bytes(128)) != cudaSuccess)
         return SEKA_ERR_CUDA;
 
     // cross-covariances: columns in groups of 128 (one head of 128, or two neighbouring heads of 64)
@@ -619,9 +817,9 @@ extern "C" seka_status seka_learn_projections(const seka_learn_shape* shape, con
     ++g_launches;
 
     // SVD of every Omega, rank rule
-    const size_t sv_smem = sizeof(double) * ((size_t)d * (d + SV_PAD) + d) + sizeof(int) * d;
-    learn_svd_kernel<<<2 * slots, SV_THREADS, sv_smem, st>>>(omega_pos, omega_neg, slots, d, shape->gamma, U_pos, U_neg,
-                                                           S_pos, S_neg, k_pos, k_neg, reinterpret_cast<int*>(ws + pl.sweeps_off));
+    auto svd = d == 128 ? learn_svd_kernel<128> : learn_svd_kernel<64>;
+    svd<<<2 * slots, 2 * d, svd_smem_bytes(d), st>>>(omega_pos, omega_neg, slots, shape->gamma, U_pos, U_neg, S_pos, S_neg, k_pos, k_neg,
+                                                     reinterpret_cast<int*>(ws + pl.sweeps_off));
     ++g_launches;
     return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
 }
