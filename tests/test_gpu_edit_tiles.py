@@ -34,9 +34,9 @@ def test_edit_steps_and_blocks(d, rank, experts, kv, lens, mask, in_place):
     assert np.array_equal(got[same], w.K.astype(np.float64)[same])
 
 
-@pytest.mark.parametrize("d,seqs,kv", [(128, 92, 4), (128, 93, 4), (64, 139, 4), (64, 140, 4)])
+@pytest.mark.parametrize("d,seqs,kv", [(128, 74, 4), (128, 75, 4), (64, 111, 4), (64, 112, 4)])
 def test_preparation_on_both_sides_of_its_rule(d, seqs, kv):
-    """Four key tiles a sequence, so that 92 | 93 (139 | 140) sequences lie on the two sides of the line between the chain and the
+    """Four key tiles a sequence, so that 74 | 75 (111 | 112) sequences lie on the two sides of the line between the chain and the
     pipelined preparation on a GPU of 148 SMs."""
     lens = [400 + (37 * i) % 113 for i in range(seqs - 1)] + [512]
     w = inputs.make_custom(seed=95, dtype="bf16", lens=lens, n_q_heads=kv, n_kv_heads=kv, head_dim=d, rank=16, mask_kind="runs",
