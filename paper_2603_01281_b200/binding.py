@@ -202,7 +202,8 @@ def seka_learn_projections(h, h_pos, h_neg, answer_tokens, gamma: float) -> dict
     nbytes = int(load().seka_learn_workspace_bytes(ctypes.byref(shp)))
     if nbytes == 0:
         raise SekaError(SEKA_ERR_UNSUPPORTED, "seka_learn_workspace_bytes")
-    ws = torch.zeros(nbytes, dtype=torch.uint8, device=h.device)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=h.device)
+    ws[:256].zero_()                        # the status block; the launches write the rest before they read it
     f32 = dict(dtype=torch.float32, device=h.device)
     out = {"omega_pos": torch.empty((slots, d, d), **f32), "omega_neg": torch.empty((slots, d, d), **f32),
            "U_pos": torch.empty((slots, d, d), **f32), "U_neg": torch.empty((slots, d, d), **f32),

@@ -8,9 +8,9 @@
 //                         streams 128-token tiles of h, h+, h- with TMA through two stages; one thread issues
 //                         tcgen05 products with BOTH operands MN-major (the token axis is the contraction) into two
 //                         128 x 128 accumulators in tensor memory; four warps drain the finished accumulators of
-//                         item i while item i + 1 accumulates in the other half of tensor memory.
-//   learn_reduce_kernel   sums the per-chunk partials in chunk order, scales by 1 / n.
-//   learn_dist_kernel     D = mean over the answer tokens of ||h+ - h-||_2, per slot (fixed summation order).
+//                         item i while item i + 1 accumulates in the other half of tensor memory; four more warps
+//                         sum ||h+ - h-||_2 over the answer tokens from the same staged tiles.
+//   learn_reduce_kernel   sums the per-chunk partials in chunk order, scales by 1 / n; D = mean of the distances.
 //   learn_svd_kernel      one CTA per matrix, fp64: QR of Omega^T, then one-sided Jacobi (Hestenes) on the columns of R^T;
 //                         half of the columns in registers, half in shared memory; every pair of columns meets once per
 //                         sweep (ordering by recursive halving); on convergence the column norms are the singular
@@ -24,7 +24,7 @@ namespace seka {
 namespace {
 
 // ------------------------------------------------------------------------------------ cross-covariances
-constexpr int LC_THREADS = 192;                 // warp 0 producer, warp 1 MMA issuer, warps 2..5 drain
+constexpr int LC_THREADS = 320;                 // warp 0 producer, warp 1 MMA issuer, warps 2..5 drain, warps 6..9 distances
 constexpr int LC_TOK = 128;                     // tokens per stage
 constexpr int LC_NS = 2;
 constexpr uint32_t LC_BLK = 128 * 128;          // [128 tokens x 64 columns] block, 128-byte swizzle
@@ -37,6 +37,9 @@ constexpr uint32_t LC_TMEM_COLS = 512;          // two sets of (Omega+, Omega-) 
 
 struct LearnCovParams {
     float* part;            // [n_chunks][slots][2][d][d]
+    double* dist;           // [n_chunks][4][slots]: sums of the distances, one per distance warp
+    int* count;             // [n_chunks][4]: answer tokens
+    const uint8_t* answer;  // [n_tokens] or null: all
     int n_tokens, n_groups, d, slots, chunk_tokens, n_chunks;
     int* status;
 };
@@ -56,7 +59,7 @@ learn_cov_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant_
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + LC_BARS);
     uint64_t* full = bars;              // [2] the three tiles of a stage have landed
-    uint64_t* empty = bars + 2;         // [2] the products that read the stage have finished
+    uint64_t* empty = bars + 2;         // [2] the products that read the stage have finished, the four distance warps have read it
     uint64_t* acc_full = bars + 4;      // [2] every product of an item has finished: its accumulators can be read
     uint64_t* acc_free = bars + 6;      // [2] four drain-warp arrivals: the accumulators have been read
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + LC_MISC);
@@ -65,7 +68,7 @@ learn_cov_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant_
     if (__syncthreads_or(*reinterpret_cast<volatile int*>(p.status) != 0)) return;
 
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); mbar_init(acc_full + i, 1); mbar_init(acc_free + i, 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 5); mbar_init(acc_full + i, 1); mbar_init(acc_free + i, 4); }
         *abort_flag = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmH); tma_prefetch_desc(&tmP); tma_prefetch_desc(&tmN);
@@ -144,7 +147,7 @@ learn_cov_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant_
                 ++n_pop;
             }
         }
-    } else {
+    } else if (warp < 6) {
         // ------------------------------------------------------------ drain: accumulators -> per-chunk partials
         const int q = warp & 3;                                        // the quarter of tensor-memory lanes this warp may read
         const int row = q * 32 + lane;
@@ -183,6 +186,71 @@ learn_cov_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant_
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_free + set);
         }
+    } else {
+        // ------------------------------------------------------------ distances: a lane per token of the stage
+        // The tiles are on chip already, so the distances cost no traffic: a pass of their own over h+ and h- took 413 us
+        // beside 1031 us of products (288 slots of 128, 32k tokens, 30 % answer tokens); in here they add 56.
+        const int w4 = warp - 6, row = w4 * 32 + lane, per = 128 / p.d;         // row of the stage, slots per group
+        uint32_t n_pop = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+            const int g = item % p.n_groups, c = item / p.n_groups;
+            const int t0 = c * p.chunk_tokens, t1 = min(p.n_tokens, t0 + p.chunk_tokens);
+            const int n_tiles = (t1 - t0 + LC_TOK - 1) / LC_TOK;
+            double sum0 = 0.0, sum1 = 0.0;
+            int count = 0;
+            for (int t = 0; t < n_tiles; ++t) {
+                const uint32_t s = n_pop % LC_NS;
+                const int tok = t0 + t * LC_TOK + row;
+                const bool on = tok < t1 && (p.answer == nullptr || p.answer[tok] != 0);
+                ok = lc_wait(full + s, (n_pop / LC_NS) & 1, abort_flag, p.status, 74);
+                if (!ok) break;
+                if (on) {
+                    const uint8_t* hp = smem + s * LC_STAGE + LC_TILE + row * 128;
+                    float ss[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+                    for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+                        for (int ch = 0; ch < 8; ++ch) {
+                            const uint8_t* at = hp + blk * LC_BLK + ((ch ^ (row & 7)) << 4);        // 128-byte swizzle
+                            const uint4 a4 = *reinterpret_cast<const uint4*>(at), b4 = *reinterpret_cast<const uint4*>(at + LC_TILE);
+                            const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
+                                const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
+                                const float dx = a.x - b.x, dy = a.y - b.y;
+                                ss[blk][0] = fmaf(dx, dx, ss[blk][0]);
+                                ss[blk][1] = fmaf(dy, dy, ss[blk][1]);
+                            }
+                        }
+                    const float q0 = ss[0][0] + ss[0][1], q1 = ss[1][0] + ss[1][1];
+                    if (per == 1) {
+                        sum0 += (double)sqrtf(q0 + q1);
+                    } else {
+                        sum0 += (double)sqrtf(q0);
+                        sum1 += (double)sqrtf(q1);
+                    }
+                    ++count;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty + s);
+                ++n_pop;
+            }
+            if (!ok) break;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sum0 += __shfl_xor_sync(0xffffffffu, sum0, o);
+                sum1 += __shfl_xor_sync(0xffffffffu, sum1, o);
+                count += __shfl_xor_sync(0xffffffffu, count, o);
+            }
+            if (lane == 0) {
+                double* dst = p.dist + (size_t)(c * 4 + w4) * p.slots + g * per;
+                dst[0] = sum0;
+                if (per == 2) dst[1] = sum1;
+                if (g == 0) p.count[c * 4 + w4] = count;
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -192,102 +260,37 @@ learn_cov_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant_
     }
 }
 
-// omega[sign][slot][i][j] = sum over chunks (in order) of the partials, divided by the number of tokens
-__global__ void learn_reduce_kernel(const float* __restrict__ part, float* __restrict__ omega_pos,
-                                    float* __restrict__ omega_neg, int slots, int d, int n_chunks, float inv_n) {
-    const size_t per = (size_t)d * d, total = (size_t)slots * 2 * per;
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+// omega[sign][slot][i][j] = sum over chunks (in order) of the partials, divided by the number of tokens; four entries a thread.
+// The blocks after those: D[slot] = mean of the distances, a warp per slot (lane i adds the sums i, i + 32, ... in order).
+// Bound by the partials' bytes: 3 chunks of 288 slots of 128 (151 MB) 110 -> 29 us (one entry a thread before).
+constexpr int LR_THREADS = 256;
+__global__ void __launch_bounds__(LR_THREADS)
+learn_reduce_kernel(const LearnCovParams p, float* __restrict__ omega_pos, float* __restrict__ omega_neg, float* __restrict__ D,
+                    unsigned n_omega_blocks, float inv_n) {
+    if (blockIdx.x >= n_omega_blocks) {
+        const int slot = (int)(blockIdx.x - n_omega_blocks) * (LR_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+        if (slot >= p.slots) return;
+        double t = 0.0;
+        int n = 0;
+        for (int c = lane; c < 4 * p.n_chunks; c += 32) { t += p.dist[(size_t)c * p.slots + slot]; n += p.count[c]; }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { t += __shfl_xor_sync(0xffffffffu, t, o); n += __shfl_xor_sync(0xffffffffu, n, o); }
+        if (lane == 0) D[slot] = n > 0 ? (float)(t / (double)n) : 0.f;
+        return;
+    }
+    const size_t per = (size_t)p.d * p.d / 4, total = (size_t)p.slots * 2 * per;
+    const size_t idx = (size_t)blockIdx.x * LR_THREADS + threadIdx.x;
     if (idx >= total) return;
-    float acc = 0.f;
-    for (int c = 0; c < n_chunks; ++c) acc += part[(size_t)c * total + idx];
+    const float4* src = reinterpret_cast<const float4*>(p.part) + idx;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int c = 0; c < p.n_chunks; ++c) {
+        const float4 v = __ldcs(src + (size_t)c * total);
+        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
     const size_t slot = idx / (2 * per), rest = idx % (2 * per);
     float* out = rest < per ? omega_pos : omega_neg;
-    out[slot * per + rest % per] = acc * inv_n;
-}
-
-// ------------------------------------------------------------------------------------ head-selection distance
-// Block b takes a range of tokens; every slot has one owner (a fixed group of lanes of one warp), which keeps the
-// slot's running sum in shared memory: one writer per slot, fixed order.
-constexpr int LD_THREADS = 256;
-__global__ void learn_dist_kernel(const __nv_bfloat16* __restrict__ hp, const __nv_bfloat16* __restrict__ hn,
-                                  const uint8_t* __restrict__ answer, int n, int slots, int d, int tokens_per_block,
-                                  float* __restrict__ part_sum, int* __restrict__ part_count) {
-    extern __shared__ float acc[];                  // [slots]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int s = threadIdx.x; s < slots; s += LD_THREADS) acc[s] = 0.f;
-    __syncthreads();
-    const int t0 = blockIdx.x * tokens_per_block, t1 = min(n, t0 + tokens_per_block);
-    int count = 0;
-    for (int t = t0; t < t1; ++t) {
-        if (answer != nullptr && answer[t] == 0) continue;
-        ++count;
-        // A row (one token of one slot) is d / 8 lanes of 16 bytes, so one warp load covers 2 (d = 128) or 4 (d = 64)
-        // neighbouring slots: 512 contiguous bytes.  Four such loads per tensor are in flight before the sums.
-        const int lpr = d / 8, rpw = 32 / lpr;              // lanes per row, rows per warp load
-        const int sub = lane / lpr;
-        const int n_q = (slots + rpw - 1) / rpw;
-        for (int q0 = warp; q0 < n_q; q0 += 4 * (LD_THREADS / 32)) {
-            float ss[4];
-            uint4 a4[4], b4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int sl = (q0 + u * (LD_THREADS / 32)) * rpw + sub;
-                a4[u] = make_uint4(0u, 0u, 0u, 0u); b4[u] = a4[u];
-                if (q0 + u * (LD_THREADS / 32) < n_q && sl < slots) {
-                    const size_t off = ((size_t)t * slots + sl) * d + (size_t)(lane % lpr) * 8;
-                    a4[u] = *reinterpret_cast<const uint4*>(hp + off);
-                    b4[u] = *reinterpret_cast<const uint4*>(hn + off);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t* aw = reinterpret_cast<const uint32_t*>(&a4[u]);
-                const uint32_t* bw = reinterpret_cast<const uint32_t*>(&b4[u]);
-                float acc2 = 0.f;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-                    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
-                    const float dx = a.x - b.x, dy = a.y - b.y;
-                    acc2 = fmaf(dx, dx, fmaf(dy, dy, acc2));
-                }
-                ss[u] = acc2;
-            }
-            for (int o = lpr / 2; o > 0; o >>= 1) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) ss[u] += __shfl_xor_sync(0xffffffffu, ss[u], o);
-            }
-            if (lane % lpr == 0) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int sl = (q0 + u * (LD_THREADS / 32)) * rpw + sub;
-                    if (q0 + u * (LD_THREADS / 32) < n_q && sl < slots) acc[sl] += sqrtf(ss[u]);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    for (int s = threadIdx.x; s < slots; s += LD_THREADS) part_sum[(size_t)blockIdx.x * slots + s] = acc[s];
-    if (threadIdx.x == 0) part_count[blockIdx.x] = count;
-}
-
-// One CTA per slot: thread i adds the partials of blocks i, i + 256, ... in order, then thread 0 adds the 256 sums in order.
-__global__ void learn_dist_reduce_kernel(const float* __restrict__ part_sum, const int* __restrict__ part_count,
-                                         int n_blocks, int slots, float* __restrict__ D) {
-    __shared__ double tot[256];
-    __shared__ long long cnt[256];
-    const int s = blockIdx.x, i = threadIdx.x;
-    double t = 0.0;
-    long long c = 0;
-    for (int b = i; b < n_blocks; b += 256) { t += (double)part_sum[(size_t)b * slots + s]; c += part_count[b]; }
-    tot[i] = t; cnt[i] = c;
-    __syncthreads();
-    if (i == 0) {
-        double tt = 0.0;
-        long long cc = 0;
-        for (int k = 0; k < 256; ++k) { tt += tot[k]; cc += cnt[k]; }
-        D[s] = cc > 0 ? (float)(tt / (double)cc) : 0.f;
-    }
+    reinterpret_cast<float4*>(out)[slot * per + rest % per] = make_float4(acc.x * inv_n, acc.y * inv_n, acc.z * inv_n, acc.w * inv_n);
 }
 
 // ------------------------------------------------------------------------------------ SVD (QR + one-sided Jacobi, fp64)
@@ -370,7 +373,7 @@ __device__ __forceinline__ bool svd_rotation(float aa, float bb, double dot, Svd
 // What bounds it: the shared-memory reads and writes of the visiting columns and the latency of a round (inner products,
 // angle, update: a chain of dependent operations).  128 registers a thread are what two CTAs leave: half of the visiting
 // column is read a second time rather than held through the angles (with all of it held the spills cost 10 %).
-// Measured, 576 matrices of 128 x 128: 5.99 -> 2.79 ms (before: no QR, one column per group resident, the whole matrix in
+// Measured, 576 matrices of 128 x 128: 5.99 -> 2.64 ms (before: no QR, one column per group resident, the whole matrix in
 // shared memory and so one CTA per SM, scaled rotations).
 template <int D>
 __global__ void __launch_bounds__(2 * D, D == 128 ? 2 : 4)
@@ -716,7 +719,7 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
 }
 
 struct LearnPlan {
-    int n_groups, chunk_tokens, n_chunks, dist_tokens, dist_blocks;
+    int n_groups, chunk_tokens, n_chunks;
     size_t part_off, part_bytes, dsum_off, dsum_bytes, dcnt_off, dcnt_bytes, sweeps_off, sweeps_bytes, total;
 };
 
@@ -743,15 +746,12 @@ LearnPlan learn_plan(const seka_learn_shape* s) {
     chunk = (chunk + LC_TOK - 1) / LC_TOK * LC_TOK;
     pl.chunk_tokens = (int)chunk;
     pl.n_chunks = (int)((s->n_tokens + chunk - 1) / chunk);
-    pl.dist_tokens = 8;
-    pl.dist_blocks = (s->n_tokens + pl.dist_tokens - 1) / pl.dist_tokens;
-    if (pl.dist_blocks > 8192) { pl.dist_tokens = (s->n_tokens + 8191) / 8192; pl.dist_blocks = (s->n_tokens + pl.dist_tokens - 1) / pl.dist_tokens; }
     pl.part_off = kStatusBytes;
     pl.part_bytes = align_up((size_t)pl.n_chunks * s->n_slots * 2 * d * d * sizeof(float), 256);
     pl.dsum_off = pl.part_off + pl.part_bytes;
-    pl.dsum_bytes = align_up((size_t)pl.dist_blocks * s->n_slots * sizeof(float), 256);
+    pl.dsum_bytes = align_up((size_t)pl.n_chunks * 4 * s->n_slots * sizeof(double), 256);
     pl.dcnt_off = pl.dsum_off + pl.dsum_bytes;
-    pl.dcnt_bytes = align_up((size_t)pl.dist_blocks * sizeof(int), 256);
+    pl.dcnt_bytes = align_up((size_t)pl.n_chunks * 4 * sizeof(int), 256);
     pl.sweeps_off = pl.dcnt_off + pl.dcnt_bytes;
     pl.sweeps_bytes = align_up((size_t)2 * s->n_slots * sizeof(int), 256);
     pl.total = pl.sweeps_off + pl.sweeps_bytes;
@@ -797,23 +797,17 @@ extern "C" seka_status seka_learn_projections(const seka_learn_shape* shape, con
         return SEKA_ERR_CUDA;
     LearnCovParams p;
     p.part = reinterpret_cast<float*>(ws + pl.part_off);
+    p.dist = reinterpret_cast<double*>(ws + pl.dsum_off);
+    p.count = reinterpret_cast<int*>(ws + pl.dcnt_off);
+    p.answer = answer_tokens;
     p.n_tokens = n; p.n_groups = pl.n_groups; p.d = d; p.slots = slots;
     p.chunk_tokens = pl.chunk_tokens; p.n_chunks = pl.n_chunks; p.status = reinterpret_cast<int*>(ws);
     const int n_items = pl.n_groups * pl.n_chunks;
     learn_cov_kernel<<<n_items < n_sm ? n_items : n_sm, LC_THREADS, LC_DYN_BYTES, st>>>(tmH, tmP, tmN, p);
     ++g_launches;
-    const size_t total = (size_t)slots * 2 * d * d;
-    learn_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(p.part, omega_pos, omega_neg, slots, d, pl.n_chunks, 1.f / (float)n);
-    ++g_launches;
-
-    // head-selection distance
-    float* dsum = reinterpret_cast<float*>(ws + pl.dsum_off);
-    int* dcnt = reinterpret_cast<int*>(ws + pl.dcnt_off);
-    learn_dist_kernel<<<pl.dist_blocks, LD_THREADS, slots * sizeof(float), st>>>(
-        static_cast<const __nv_bfloat16*>(h_pos), static_cast<const __nv_bfloat16*>(h_neg), answer_tokens, n, slots, d,
-        pl.dist_tokens, dsum, dcnt);
-    ++g_launches;
-    learn_dist_reduce_kernel<<<slots, 256, 0, st>>>(dsum, dcnt, pl.dist_blocks, slots, D);
+    const unsigned omega_blocks = (unsigned)(((size_t)slots * 2 * d * d / 4 + LR_THREADS - 1) / LR_THREADS);
+    const unsigned dist_blocks = (unsigned)((slots + LR_THREADS / 32 - 1) / (LR_THREADS / 32));
+    learn_reduce_kernel<<<omega_blocks + dist_blocks, LR_THREADS, 0, st>>>(p, omega_pos, omega_neg, D, omega_blocks, 1.f / (float)n);
     ++g_launches;
 
     // SVD of every Omega, rank rule
