@@ -313,9 +313,9 @@ struct SvdRotation {
     float tab;                                  // tan(theta) * (x . y): the squared norms become aa - tab, bb + tab
 };
 
-// `aa`, `bb`: squared norms, `dot` = x . y.  No branches: a pair that is orthogonal already gets the angle zero.  `cos2`,
-// `lean2`: see the end of a sweep below.
-__device__ __forceinline__ bool svd_rotation(float aa, float bb, double dot, SvdRotation& r, float& cos2, float& lean2) {
+// `aa`, `bb`: squared norms, `dot` = x . y.  No branches: a pair that is orthogonal already gets the angle zero.  `lean2`:
+// see the end of a sweep below.
+__device__ __forceinline__ bool svd_rotation(float aa, float bb, double dot, SvdRotation& r, float& lean2) {
     const float ra = svd_rcp(aa), rb = svd_rcp(bb);
     const float ab = (float)dot, cc = (ab * ra) * (ab * rb);
     // |cos| > 1e-13 (well above the rounding noise of the inner product), as a product of ratios so that columns of very
@@ -337,10 +337,7 @@ __device__ __forceinline__ bool svd_rotation(float aa, float bb, double dot, Svd
     r.td = td;
     r.be = fma(p, fma(e, e, e), p);
     r.tab = turn ? t * ab : 0.f;
-    if (turn) {
-        cos2 = fmaxf(cos2, cc);
-        lean2 = fmaxf(lean2, t * t * fmaxf(aa * rb, bb * ra));
-    }
+    if (turn) lean2 = fmaxf(lean2, t * t * fmaxf(aa * rb, bb * ra));
     return turn;
 }
 
@@ -359,21 +356,24 @@ __device__ __forceinline__ bool svd_rotation(float aa, float bb, double dot, Svd
 //
 // Ordering of a sweep (every pair of columns meets once): level m = D / 2, D / 4, ..., 2 cuts the D / 2 column positions of
 // either kind into blocks of m.  In round r of the level, the group whose columns are the 2i-th and (2i + 1)-th of its block
-// meets the ((2i + r) mod m)-th column of the block in shared memory: one read and one write of that column for two rotations.
+// meets the columns 2 ((i + r) mod (m / 2)) and the one after it of the block in shared memory: one read and one write of a
+// column for two rotations, a barrier for four.
 // Both inner products are formed at once: the second, with the column that the first rotation leaves, follows from x0 . x1,
 // which is formed once a level and carried along (what the single-precision angle leaves of x0' . y' is neglected there: a
 // relative 2^-22 of a product that shrinks quadratically).  Between levels the groups of the second half of a block swap their
 // columns with the ones in shared memory half a block before: pairs within either half meet next.  The last level rotates
 // x0 against x1, swaps both with shared memory, and rotates again.
 //
-// End: a sweep without a rotation, or one after which no pair can have a cosine above 1e-13: with c the largest
-// cosine of the sweep and l the largest |t| max(|A| / |B|, |B| / |A|) (how far a rotation leans a column, relative to its length),
-// a pair made orthogonal meets at most 2 (D - 1) more rotations, each of which changes its cosine by at most l c.
+// End: a sweep without a rotation, or one after which no pair can have a cosine above 1e-13: with l the largest
+// |t| max(|A| / |B|, |B| / |A|) of the sweep (how far a rotation leans a column, relative to its length; never less than the
+// cosine that it removes), a pair made orthogonal meets at most 2 (D - 1) more rotations, each of which changes its cosine by at
+// most l^2.
 //
 // What bounds it: the shared-memory reads and writes of the visiting columns and the latency of a round (inner products,
-// angle, update: a chain of dependent operations).  128 registers a thread are what two CTAs leave: half of the visiting
-// column is read a second time rather than held through the angles (with all of it held the spills cost 10 %).
-// Measured, 576 matrices of 128 x 128: 5.99 -> 2.64 ms (before: no QR, one column per group resident, the whole matrix in
+// angle, update: a chain of dependent operations).  128 registers a thread are what two CTAs leave: at D = 128 the
+// visiting column is read a second time rather than held through the angles (all / half of it held: 17 % / 1 % slower; at
+// D = 64 there is room, and a second read costs 3 %).
+// Measured, 576 matrices of 128 x 128: 5.99 -> 2.55 ms (before: no QR, one column per group resident, the whole matrix in
 // shared memory and so one CTA per SM, scaled rotations).
 template <int D>
 __global__ void __launch_bounds__(2 * D, D == 128 ? 2 : 4)
@@ -388,7 +388,7 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
     __shared__ double sig[D], beta[2];
     __shared__ float nrm2[NP], red[NT / 32];
     __shared__ int order[D];
-    __shared__ unsigned worst[2];           // bits of the largest cos2, lean2 of a sweep
+    __shared__ unsigned worst;              // bits of the largest lean2 of a sweep
     const int sign = blockIdx.x / slots, slot = blockIdx.x % slots;
     const float* om = (sign == 0 ? omega_pos : omega_neg) + (size_t)slot * D * D;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -602,16 +602,16 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
         norms();                            // exact at the start of every sweep; inside it they follow the rotations in fp32,
         aa0 = (float)nx0; aa1 = (float)nx1; // as they only feed the tangent
         if (lg == 0) { nrm2[2 * g] = (float)ny0; nrm2[2 * g + 1] = (float)ny1; }
-        if (tid == 0) { worst[0] = 0u; worst[1] = 0u; }
+        if (tid == 0) worst = 0u;
         __syncthreads();
-        float cos2 = 0.f, lean2 = 0.f;
+        float lean2 = 0.f;
 #pragma unroll 1
         for (int m = NP; m >= 2; m >>= 1) {
             const int idx = (2 * g) & (m - 1), p0 = 2 * g - idx;        // position in the block, first position of the block
             double g01 = resident_dot();
 #pragma unroll 1
             for (int r = 0; r < m; ++r) {
-                const int q = p0 + ((idx + r) & (m - 1));
+                const int q = p0 + ((idx + r) & (m - 2)) + (r & 1);
                 double2* gb = reinterpret_cast<double2*>(G + (size_t)q * LDG) + lg;
                 double a0 = 0.0, b0 = 0.0, a1 = 0.0, b1 = 0.0;
 #pragma unroll
@@ -624,16 +624,16 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
                 const double d0 = group_sum(a0 + b0), d1 = group_sum(a1 + b1);
                 // every lane of the group holds the same sums and works out the same rotations
                 SvdRotation u, v;
-                asm volatile("" ::: "memory");         // (the second half of the column is read again below)
-                bool any = svd_rotation(aa0, bb, d0, u, cos2, lean2);
-                any |= svd_rotation(aa1, bb + u.tab, fma(u.be, fma(-u.td, d1, g01), d1), v, cos2, lean2);
+                if (D == 128) asm volatile("" ::: "memory");       // (read again below, not held through the angles)
+                bool any = svd_rotation(aa0, bb, d0, u, lean2);
+                any |= svd_rotation(aa1, bb + u.tab, fma(u.be, fma(-u.td, d1, g01), d1), v, lean2);
                 if (__any_sync(0xffffffffu, any)) {
                     g01 = fma(-u.be, fma(u.td, g01, d1), g01);
                     aa0 = fmaxf(aa0 - u.tab, 0.f); aa1 = fmaxf(aa1 - v.tab, 0.f);
                     if (lg == 0) nrm2[q] = bb + u.tab + v.tab;
 #pragma unroll
                     for (int e = 0; e < NE; ++e) {
-                        double2 c = e < HE ? y[e] : gb[SV_LP * e];
+                        double2 c = D == 128 ? gb[SV_LP * e] : y[e];
                         x0[e].x = fma(-u.td, c.x, x0[e].x); x0[e].y = fma(-u.td, c.y, x0[e].y);
                         c.x = fma(u.be, x0[e].x, c.x); c.y = fma(u.be, x0[e].y, c.y);
                         x0[e].x = fma(-u.td, c.x, x0[e].x); x0[e].y = fma(-u.td, c.y, x0[e].y);
@@ -643,7 +643,7 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
                         gb[SV_LP * e] = c;
                     }
                 }
-                block_sync(m);
+                if (r & 1) block_sync(m);
             }
             if (m > 2) {
                 if (idx >= m / 2) swap_columns(2 * g - m / 2);
@@ -653,7 +653,7 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
             SvdRotation u;
-            if (svd_rotation(aa0, aa1, resident_dot(), u, cos2, lean2)) {
+            if (svd_rotation(aa0, aa1, resident_dot(), u, lean2)) {
                 aa0 = fmaxf(aa0 - u.tab, 0.f); aa1 += u.tab;
 #pragma unroll
                 for (int e = 0; e < NE; ++e) {
@@ -664,10 +664,9 @@ learn_svd_kernel(const float* __restrict__ omega_pos, const float* __restrict__ 
             }
             if (h == 0) swap_columns(2 * g);
         }
-        if (lg == 0) { atomicMax(&worst[0], __float_as_uint(cos2)); atomicMax(&worst[1], __float_as_uint(lean2)); }
+        if (lg == 0) atomicMax(&worst, __float_as_uint(lean2));
         __syncthreads();
-        constexpr float stop = 1e-13f / (2 * (D - 1));
-        const bool done = __uint_as_float(worst[0]) * __uint_as_float(worst[1]) < stop * stop;
+        const bool done = __uint_as_float(worst) < 1e-13f / (2 * (D - 1));
         __syncthreads();
         if (done) break;
     }
