@@ -7,8 +7,10 @@
 //                         consumer warps take 16 tokens of each stage, form the scores of the whole query
 //                         group (query heads of the KV head padded to the 16 rows of mma.sync m16n8k16),
 //                         keep a private online softmax and accumulate P V in registers; the warps' states
-//                         are merged in shared memory and written as one partial (m, l, unnormalised o).
-//   decode_combine_kernel merges the partials of a (sequence, query head) and normalises.
+//                         are merged in shared memory.  Where the chunks of a (sequence, KV head) are one
+//                         cluster, its CTAs merge their states through distributed shared memory and write
+//                         the output; otherwise each writes a partial (m, l, unnormalised o).
+//   decode_combine_kernel merges the partials of a (sequence, query head) and normalises, a warp each.
 #include <math.h>
 
 #include "seka_kernels.h"
@@ -21,6 +23,7 @@ constexpr int DEC_CONSUMERS = 4;                       // warps; each owns 16 to
 constexpr int DEC_THREADS = (DEC_CONSUMERS + 1) * 32;  // + one producer warp
 constexpr int DEC_MAX_GROUP = 16;                      // query heads per KV head (rows of one MMA)
 constexpr int DEC_SM_COUNT = 148;                      // used for sizing the split only
+constexpr int DEC_MAX_CLUSTER = 8;                     // chunks of a (sequence, KV head) that merge in a cluster
 
 template <int D>
 struct DecSmem {
@@ -34,7 +37,7 @@ struct DecSmem {
     static constexpr int BYTES = MISC_OFF + 16;
     static constexpr int DYN_BYTES = BYTES + 1024;                 // room to align the base to 1024 bytes
     static constexpr int MERGE_STRIDE = D + 2;                     // floats per row: o[D], m, l
-    static_assert(DEC_CONSUMERS * 16 * MERGE_STRIDE * 4 <= NSTAGE * STAGE_BYTES, "merge area aliases the stages");
+    static_assert((DEC_CONSUMERS + 1) * 16 * MERGE_STRIDE * 4 <= NSTAGE * STAGE_BYTES, "merge area aliases the stages");
 };
 
 struct DecodeParams {
@@ -44,6 +47,7 @@ struct DecodeParams {
     const int* cu_seqlens;
     int B, L, Hq, Hkv, G;
     int chunk, n_splits;        // cached tokens per CTA (a multiple of 64), chunks per sequence at max_seqlen
+    int direct;                 // the n_splits CTAs of a (sequence, KV head) are a cluster that writes the output
     float scale_log2;
     float* part_o;              // [B, Hkv, n_splits, G, D] unnormalised outputs
     float* part_ml;             // [B, Hkv, n_splits, G, 2] running maximum (log2 domain) and sum
@@ -65,6 +69,17 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ float ld_cluster_f32(uint32_t local_addr, uint32_t rank) {
+    uint32_t a;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local_addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // HALF: the query group has at most 8 heads, so rows 8..15 of every MMA are padding and their softmax is skipped.
 template <int D, bool HALF>
 __global__ void __launch_bounds__(DEC_THREADS, DecSmem<D>::CTAS_PER_SM)
@@ -79,19 +94,22 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
 
     const int split = blockIdx.x, hkv = blockIdx.y, b = blockIdx.z;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int seq0, Lb;
-    if (p.cu_seqlens != nullptr) { seq0 = p.cu_seqlens[b]; Lb = p.cu_seqlens[b + 1] - seq0; }
-    else { seq0 = b * p.L; Lb = p.L; }
-    const int k_begin = split * p.chunk;
-    if (k_begin >= Lb) return;                              // the whole CTA leaves before any barrier exists
-    const int k_end = min(Lb, k_begin + p.chunk);
-    const int n_stage = (k_end - k_begin + DEC_STAGE_KEYS - 1) / DEC_STAGE_KEYS;
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < SL::NSTAGE; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], DEC_CONSUMERS); }
         *abort_flag = 0;
         mbar_fence_init();
+        tma_prefetch_desc(&tk);
+        tma_prefetch_desc(&tv);
     }
+    pdl_wait();
+    pdl_release();
+    int seq0, Lb;
+    if (p.cu_seqlens != nullptr) { seq0 = p.cu_seqlens[b]; Lb = p.cu_seqlens[b + 1] - seq0; }
+    else { seq0 = b * p.L; Lb = p.L; }
+    const int k_begin = split * p.chunk;
+    if (k_begin >= Lb && !p.direct) return;                 // the whole CTA leaves
+    const int k_end = min(Lb, k_begin + p.chunk);
+    const int n_stage = k_begin < k_end ? (k_end - k_begin + DEC_STAGE_KEYS - 1) / DEC_STAGE_KEYS : 0;
     __syncthreads();
 
     const int G = p.G;
@@ -104,8 +122,6 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
     if (warp == DEC_CONSUMERS) {
         // ------------------------------------------------ producer: one lane streams the K and V tiles
         if (lane == 0) {
-            tma_prefetch_desc(&tk);
-            tma_prefetch_desc(&tv);
             int issued = 0;
             bool ok = true;
             for (int i = 0; i < n_stage; ++i) {
@@ -239,7 +255,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
 
     // ---------------------------------------------------- merge the four warps' states, write the partial
     __syncthreads();                                        // every stage has been consumed (or the CTA has aborted)
-    if (*abort_flag) return;
+    if (*abort_flag && !p.direct) return;                   // (the status tells; a CTA of a cluster stays for its peers)
     float* mg = reinterpret_cast<float*>(smem);             // [warp][16 rows][D + 2]
     if (warp < DEC_CONSUMERS) {
         l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
@@ -263,6 +279,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
     }
     __syncthreads();
     const size_t item = ((size_t)b * p.Hkv + hkv) * p.n_splits + split;
+    float* res = mg + DEC_CONSUMERS * 16 * SL::MERGE_STRIDE;        // [G][D + 2]: this CTA's state where a cluster merges
     for (int idx = threadIdx.x; idx < G * D; idx += DEC_THREADS) {
         const int g = idx / D, c = idx - g * D;
         float mw[DEC_CONSUMERS], M = -INFINITY;
@@ -275,42 +292,115 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
             acc = fmaf(mg[((size_t)w * 16 + g) * SL::MERGE_STRIDE + c], f, acc);
             lsum = fmaf(mg[((size_t)w * 16 + g) * SL::MERGE_STRIDE + D + 1], f, lsum);
         }
-        p.part_o[(item * G + g) * D + c] = acc;
-        if (c == 0) { p.part_ml[(item * G + g) * 2] = M; p.part_ml[(item * G + g) * 2 + 1] = lsum; }
+        if (p.direct) {
+            res[g * SL::MERGE_STRIDE + c] = acc;
+            if (c == 0) { res[g * SL::MERGE_STRIDE + D] = M; res[g * SL::MERGE_STRIDE + D + 1] = lsum; }
+        } else {
+            p.part_o[(item * G + g) * D + c] = acc;
+            if (c == 0) *reinterpret_cast<float2*>(p.part_ml + (item * G + g) * 2) = make_float2(M, lsum);
+        }
     }
+    if (!p.direct) return;
+
+    // ---------------------------------------------------- the cluster merges: every CTA a part of the group's output
+    cluster_sync();
+    const int ns = (Lb + p.chunk - 1) / p.chunk;            // CTAs that held cached tokens (ranks 0 .. ns - 1)
+    const uint32_t res_addr = smem_u32(res);
+    for (int idx = split * DEC_THREADS + threadIdx.x; idx < G * D; idx += p.n_splits * DEC_THREADS) {
+        const int g = idx / D, c = idx - g * D;
+        const uint32_t row = res_addr + (uint32_t)(g * SL::MERGE_STRIDE) * 4u;
+        float m[DEC_MAX_CLUSTER], l[DEC_MAX_CLUSTER], o1[DEC_MAX_CLUSTER], M = -INFINITY;
+#pragma unroll
+        for (int r = 0; r < DEC_MAX_CLUSTER; ++r) {
+            m[r] = -INFINITY; l[r] = 0.f; o1[r] = 0.f;
+            if (r < ns) {
+                m[r] = ld_cluster_f32(row + D * 4, r); l[r] = ld_cluster_f32(row + D * 4 + 4, r); o1[r] = ld_cluster_f32(row + c * 4, r);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < DEC_MAX_CLUSTER; ++r) M = fmaxf(M, m[r]);
+        float acc = 0.f, lsum = 0.f;
+#pragma unroll
+        for (int r = 0; r < DEC_MAX_CLUSTER; ++r) {
+            const float f = m[r] == -INFINITY ? 0.f : fast_exp2(m[r] - M);
+            lsum = fmaf(l[r], f, lsum);
+            acc = fmaf(o1[r], f, acc);
+        }
+        const bool any = lsum > 0.f;
+        const size_t hq = (size_t)b * p.Hq + (size_t)hkv * G + g;
+        p.O[hq * D + c] = __float2bfloat16(any ? acc / lsum : 0.f);
+        if (p.lse != nullptr && c == 0) p.lse[hq] = any ? (M + log2f(lsum)) * 0.6931471805599453f : -INFINITY;
+    }
+    cluster_sync();                                         // nobody leaves while its state is read
 }
 
-// One CTA per (sequence, query head), one thread per output element.
-__global__ void decode_combine_kernel(const DecodeParams p, int D) {
-    const int b = blockIdx.x / p.Hq, hq = blockIdx.x - b * p.Hq;
+// A warp per (sequence, query head): lanes load the chunks' (m, l) side by side, then every lane sums D / 32 columns, eight
+// chunks' loads in flight.  Bound by two dependent loads; placed while the split kernel drains.  The pair of launches for 64
+// sequences of 4096 tokens (32 query heads on 8 of 128): 159.6 -> 156.4 us a step, for one of 32768 36.8 -> 31.3.
+constexpr int DEC_COMBINE_WARPS = 4;
+template <int D>
+__global__ void __launch_bounds__(DEC_COMBINE_WARPS * 32)
+decode_combine_kernel(const DecodeParams p) {
+    constexpr int V = D / 32;
+    const int row = (int)blockIdx.x * DEC_COMBINE_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_release();
+    if (row >= p.B * p.Hq) return;
+    const int b = row / p.Hq, hq = row - b * p.Hq;
     const int hkv = hq / p.G, g = hq - hkv * p.G;
-    const int c = threadIdx.x;
     const int Lb = p.cu_seqlens != nullptr ? p.cu_seqlens[b + 1] - p.cu_seqlens[b] : p.L;
     const int ns = (Lb + p.chunk - 1) / p.chunk;            // chunks that held cached tokens
     const size_t item0 = ((size_t)b * p.Hkv + hkv) * p.n_splits;
-    float M = -INFINITY;
-    for (int s = 0; s < ns; ++s) M = fmaxf(M, p.part_ml[((item0 + s) * p.G + g) * 2]);
-    float acc = 0.f, l = 0.f;
-    for (int s = 0; s < ns; ++s) {
-        const float ms = p.part_ml[((item0 + s) * p.G + g) * 2];
-        const float f = ms == -INFINITY ? 0.f : fast_exp2(ms - M);
-        l = fmaf(p.part_ml[((item0 + s) * p.G + g) * 2 + 1], f, l);
-        acc = fmaf(p.part_o[((item0 + s) * p.G + g) * D + c], f, acc);
+    float M = -INFINITY, l = 0.f, acc[V] = {};
+    for (int s0 = 0; s0 < ns; s0 += 32) {
+        const int n = min(32, ns - s0);
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (lane < n) ml = *reinterpret_cast<const float2*>(p.part_ml + ((item0 + s0 + lane) * p.G + g) * 2);
+        float mx = fmaxf(M, ml.x);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float keep = M == -INFINITY ? 0.f : fast_exp2(M - mx), f = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - mx);
+        l = fmaf(l, keep, ml.y * f);                        // per lane until the end
+        M = mx;
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[e] *= keep;
+        const float* src = p.part_o + ((item0 + s0) * p.G + g) * D + lane * V;
+#pragma unroll 8
+        for (int i = 0; i < n; ++i) {
+            const float fi = __shfl_sync(0xffffffffu, f, i);
+            float v[V];
+            if (V == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(src + (size_t)i * p.G * D);
+            else *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(src + (size_t)i * p.G * D);
+#pragma unroll
+            for (int e = 0; e < V; ++e) acc[e] = fmaf(v[e], fi, acc[e]);
+        }
     }
-    const bool any = ns > 0 && l > 0.f;
-    p.O[((size_t)b * p.Hq + hq) * D + c] = __float2bfloat16(any ? acc / l : 0.f);
-    if (p.lse != nullptr && c == 0)
-        p.lse[(size_t)b * p.Hq + hq] = any ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    uint32_t* out = reinterpret_cast<uint32_t*>(p.O + (size_t)row * D + lane * V);
+#pragma unroll
+    for (int e = 0; e < V / 2; ++e) out[e] = pack_bf16(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+    if (p.lse != nullptr && lane == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
 }
 
 struct DecodePlan {
-    int chunk, n_splits;
+    int chunk, n_splits, direct;
     size_t ml_off, ml_bytes, o_off, o_bytes, total;
 };
 
 // Chunks of cached tokens.  A CTA has a fixed cost (query fragments, the merge of its warps, its partial), so chunks
 // are long: about three waves of CTAs over the SMs, at least 1024 tokens each.  Where that would leave SMs without
 // work (few sequences), the chunks shrink until one wave is full, down to 256 tokens.
+//
+// Where a power of two of chunks (up to a portable cluster of 8) per (sequence, KV head) fits one wave, those CTAs are a
+// cluster and the step is one launch.  Two launches cost 2 to 10 us more: 32 query heads on 8 of 128, one sequence of 512 /
+// 4096 tokens 6.5 -> 4.2 / 11.2 -> 6.9 us, 3 ragged sequences up to 6000 12.3 -> 8.5, 16 of 2048 28.6 -> 24.2, 4 of 32768
+// 97 -> 81 (90.8 in two launches of the present kernels).  The exceptions:
+//   - fewer CTAs than SMs with long chunks: one sequence of 16384 takes 16.3 us in 64 chunks of 2048, 15.7 in two launches;
+//   - batches whose longest sequence is far above the mean (lengths are known on the device only): one CTA
+//     would stream its long chunk alone, so chunks are limited to 2048 tokens there.
+// Workspace: that of the two launches in every case, a function of batch, heads and max_seqlen alone.
 DecodePlan decode_plan(const seka_shape* s) {
     DecodePlan d;
     const int G = s->n_q_heads / s->n_kv_heads;
@@ -333,6 +423,15 @@ DecodePlan decode_plan(const seka_shape* s) {
     d.o_off = d.ml_off + d.ml_bytes;
     d.o_bytes = align_up(items * s->head_dim * sizeof(float) + 16, 256);
     d.total = d.o_off + d.o_bytes;
+
+    d.direct = d.n_splits == 1;
+    int cl = 1;
+    while (cl < DEC_MAX_CLUSTER && pairs * 2 * cl <= slots && s->max_seqlen > 128 * cl) cl *= 2;
+    const int part = ((s->max_seqlen + cl - 1) / cl + DEC_STAGE_KEYS - 1) / DEC_STAGE_KEYS * DEC_STAGE_KEYS;
+    const bool even = (long long)s->max_seqlen * s->batch <= 3LL * shape_total_tokens(s);
+    if (pairs > 0 && pairs <= slots && part > 0 && (part <= 1024 || (pairs * cl >= DEC_SM_COUNT && (even || part <= 2048)))) {
+        d.chunk = part; d.n_splits = cl; d.direct = 1;
+    }
     return d;
 }
 
@@ -353,9 +452,7 @@ seka_status launch_split(const CUtensorMap& tk, const CUtensorMap& tv, const Dec
     if (cudaFuncSetAttribute(decode_split_kernel<D, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)SL::DYN_BYTES) != cudaSuccess) return SEKA_ERR_CUDA;
     dim3 grid((unsigned)p.n_splits, (unsigned)p.Hkv, (unsigned)p.B);
-    decode_split_kernel<D, HALF><<<grid, DEC_THREADS, SL::DYN_BYTES, st>>>(tk, tv, p);
-    ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    return launch_cluster(true, p.direct ? (unsigned)p.n_splits : 1u, decode_split_kernel<D, HALF>, grid, DEC_THREADS, SL::DYN_BYTES, st, tk, tv, p);
 }
 
 }  // namespace
@@ -387,7 +484,7 @@ extern "C" seka_status seka_decode_attention(const seka_shape* shape, const void
     p.Q = static_cast<const __nv_bfloat16*>(Q); p.O = static_cast<__nv_bfloat16*>(O); p.lse = lse;
     p.cu_seqlens = shape->cu_seqlens;
     p.B = shape->batch; p.L = shape->max_seqlen; p.Hq = shape->n_q_heads; p.Hkv = Hkv; p.G = shape->n_q_heads / Hkv;
-    p.chunk = plan.chunk; p.n_splits = plan.n_splits;
+    p.chunk = plan.chunk; p.n_splits = plan.n_splits; p.direct = plan.direct && T > 0 && shape->max_seqlen > 0;
     const float scale = shape->softmax_scale > 0.f ? shape->softmax_scale : 1.f / sqrtf((float)D);
     p.scale_log2 = scale * 1.4426950408889634f;
     p.part_ml = reinterpret_cast<float*>(ws + plan.ml_off);
@@ -401,9 +498,9 @@ extern "C" seka_status seka_decode_attention(const seka_shape* shape, const void
         const bool half = p.G <= 8;
         seka_status s2 = D == 128 ? (half ? launch_split<128, true>(tk, tv, p, st) : launch_split<128, false>(tk, tv, p, st))
                                   : (half ? launch_split<64, true>(tk, tv, p, st) : launch_split<64, false>(tk, tv, p, st));
-        if (s2 != SEKA_OK) return s2;
+        if (s2 != SEKA_OK || p.direct) return s2;
     }
-    decode_combine_kernel<<<(unsigned)(p.B * p.Hq), D, 0, st>>>(p, D);
-    ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    const unsigned grid = (unsigned)((p.B * p.Hq + DEC_COMBINE_WARPS - 1) / DEC_COMBINE_WARPS);
+    return D == 128 ? launch_kernel(true, decode_combine_kernel<128>, grid, DEC_COMBINE_WARPS * 32, 0, st, p)
+                    : launch_kernel(true, decode_combine_kernel<64>, grid, DEC_COMBINE_WARPS * 32, 0, st, p);
 }

@@ -48,19 +48,31 @@ seka_status validate_shape(const seka_shape* s);
 bool device_info(int* n_sm);
 
 // Launch whose status is that of the launch alone.  With `pdl` it may be placed while its predecessor in the stream drains
-// (the kernel begins with pdl_wait).
+// (the kernel begins with pdl_wait).  `cluster`: CTAs of a cluster along x.
 template <typename... P, typename... A>
-static inline seka_status launch_kernel(bool pdl, void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
-                                        const A&... args) {
+static inline seka_status launch_cluster(bool pdl, unsigned cluster, void (*kern)(P...), dim3 grid, unsigned threads, size_t smem,
+                                         cudaStream_t st, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if (pdl) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = at; cfg.numAttrs = n;
     if (cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) return SEKA_ERR_CUDA;
     ++g_launches;
     return SEKA_OK;
+}
+template <typename... P, typename... A>
+static inline seka_status launch_kernel(bool pdl, void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                                        const A&... args) {
+    return launch_cluster(pdl, 1u, kern, grid, threads, smem, st, args...);
 }
 
 }  // namespace seka

@@ -1,0 +1,41 @@
+"""The decode step on both sides of its dispatch: chunks of a (sequence, KV head) merged inside a cluster of 1, 2, 4 or 8 CTAs,
+and by the second launch."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2603_01281_b200 import binding, inputs
+
+import helpers as H
+import test_gpu_decode as T
+
+pytestmark = pytest.mark.gpu
+
+
+def _launches(f):
+    n = binding.load().seka_launch_count()
+    out = f()
+    return out, binding.load().seka_launch_count() - n
+
+
+@pytest.mark.parametrize("d,Hq,Hkv,lens,launches", [
+    (128, 1, 1, [128], 1), (128, 1, 1, [129], 1), (128, 4, 1, [1025, 0, 1, 128, 64], 1),        # clusters of 1, 2, 8 (ranks without tokens)
+    (128, 16, 1, [8192, 300], 1), (128, 9, 1, [8193, 7000], 2),                                 # the longest chunk of few CTAs
+    (64, 2, 2, [8192], 1), (64, 2, 2, [8193], 2),
+    (128, 8, 8, [700 - 17 * i for i in range(18)], 1), (128, 8, 8, [700 - 17 * i for i in range(19)], 1),       # 144 | 152 pairs: 2 | 1
+    (128, 8, 8, [1100 - 27 * i for i in range(37)], 1), (128, 8, 8, [1100 - 27 * i for i in range(38)], 2),         # 296 | 304 pairs: one wave
+    (64, 12, 12, [1100 - 27 * i for i in range(37)], 1), (64, 12, 12, [1100 - 27 * i for i in range(38)], 2),       # 444 | 456 pairs
+    (128, 8, 8, [2560] + [30] * 36, 2), (128, 8, 8, [2560] * 14 + [30] * 23, 1),                # 296 pairs of up to 2560: uneven | even
+])
+def test_decode_on_both_sides_of_its_dispatch(d, Hq, Hkv, lens, launches):
+    w = inputs.make_custom(seed=41, dtype="bf16", lens=lens, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, rank=8)
+    dev = H.device_tensors(w)
+    q = T._last_queries(w)
+    (O, LSE), n = _launches(lambda: T._run_decode(w, dev, dev["K"], q))
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert n == launches, (n, launches)
+    Oref, Lref = oracle.decode_attention(q, w.K, w.V, w.cu_seqlens)
+    for b in np.flatnonzero(np.asarray(lens) == 0):
+        assert np.all(O[b] == 0) and np.all(np.isneginf(LSE[b]))
+    T._check(O, LSE, Oref, Lref)
