@@ -90,15 +90,19 @@ def status_string(status: int) -> str:
     return load().seka_status_string(int(status)).decode()
 
 
-def _ptr(t: Optional[torch.Tensor]):
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
     assert t.is_contiguous(), "tensors passed to the library must be contiguous"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    """The current stream of the current device, as torch.cuda.current_stream().cuda_stream gives it, without building the
+    stream object (3.2 us of a call; the raw lookup takes 0.1)."""
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(status: int, where: str) -> None:
