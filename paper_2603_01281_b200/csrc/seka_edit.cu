@@ -261,7 +261,7 @@ static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void*
 // rows of a CTA's next step are fetched under the present one where shared memory has room for a second stage.
 // Registers and code are kept small (16 columns at a time, short unrolls): a launch is often one or two steps per CTA, bound
 // by fetching its instructions, and spilled registers tripled the time of a step at head_dim 64.
-// Measured: 144 x 4096 tokens x 8 heads x 128 in place, a tenth highlighted, 94 -> 72 us per call (whole 128-row tiles
+// Measured: 144 x 4096 tokens x 8 heads x 128 in place, a tenth highlighted, 94 -> 69 us per call (whole 128-row tiles
 // through a projector, of which 58 % of the rows were written); one prompt of 777 tokens on 32/8 heads 42 -> 31 us per call
 // (four launches and two memsets before, two launches now).
 constexpr uint32_t EBLK = 128 * 128;        // one [128 x 64] bf16 block
@@ -274,15 +274,16 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 constexpr int ET_THREADS = 256, ET_WARPS = ET_THREADS / 32;
 constexpr int ET_UCOLS = 64;                // columns of U per block
 
-template <int D, bool SIDE>
+template <int D, bool SIDE, bool PACK = false>
 struct EtSmem {
     static constexpr uint32_t TILE = (D / 64) * EBLK;       // 128 key rows
     static constexpr uint32_t UMAT = D * 128;               // [D x 64] bf16
     static constexpr int NS = D == 128 && SIDE ? 1 : 2;     // stages of key rows (two CTAs per SM leave room for one beside the low parts)
     static constexpr uint32_t U = NS * TILE;                // blocks of U (high part, then low part each); SIDE: then the low
                                                             // parts of the edited rows; then scratch and result of Eq. 6
+    static constexpr uint32_t UBLK = PACK ? UMAT : 2 * UMAT;          // a block of U with its low part
     static constexpr uint32_t TMEM_COLS = D == 128 ? 256 : 128;       // 64 for C, D for dK
-    static constexpr int CTAS = D == 128 ? 2 : 3;           // per SM: tensor memory and shared memory (128), shared memory (64)
+    static constexpr int CTAS = D == 128 ? 2 : PACK ? 4 : 3;          // per SM: tensor memory (shared memory for 64 unpacked)
 };
 
 // SIDE: a unit of work as the warp that looked at it left it
@@ -301,10 +302,13 @@ struct TileArgs {
     PrepJobs jobs;
 };
 
-template <int D, bool SIDE, typename KT>
-__global__ void __launch_bounds__(ET_THREADS, EtSmem<D, SIDE>::CTAS)
+// PACK (stacked rank of at most 32): both parts of U stand in one block, the low part from column 32 on, so that one product
+// forms K times either part and both halves of the threads scale C.  Before / with it: 36 layers as above 74 -> 69 us, 64 x 4096
+// tokens x 8 heads x 64, half highlighted, 96 -> 78 us (a fourth CTA per SM fits there).
+template <int D, bool SIDE, typename KT, bool PACK>
+__global__ void __launch_bounds__(ET_THREADS, EtSmem<D, SIDE, PACK>::CTAS)
 edit_tiles_kernel(const __grid_constant__ TileArgs p) {
-    using SL = EtSmem<D, SIDE>;
+    using SL = EtSmem<D, SIDE, PACK>;
     constexpr int NS = SL::NS;
     constexpr int UPR = D / 8;                          // 16-byte units (8 elements) of a key row
     constexpr int RPP = ET_THREADS / UPR;               // rows a pass of the CTA loads
@@ -512,7 +516,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     // columns [j0, j0 + 64) of the stacked U of head h as two bf16 parts: [D x 64] blocks, 128-byte swizzle (K-major operand of
     // the second product, MN-major of the first); zero up to the next multiple of 16 columns, undefined (and unused) beyond
     auto stage_u = [&](int h, int j0, int slot) {
-        uint8_t* sB = sU + slot * (2 * SL::UMAT);
+        uint8_t* sB = sU + slot * SL::UBLK;
         const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nu = (rc + 15) / 16 * 2;
         if (u_vec) {
 #pragma unroll 1
@@ -527,9 +531,8 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                 uint32_t hi[4], lo[4];
                 split_pair(a.x, a.y, hi[0], lo[0]); split_pair(a.z, a.w, hi[1], lo[1]);
                 split_pair(b4.x, b4.y, hi[2], lo[2]); split_pair(b4.z, b4.w, hi[3], lo[3]);
-                const uint32_t off = sw128_offset(i, c8);
-                *reinterpret_cast<uint4*>(sB + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                *reinterpret_cast<uint4*>(sB + SL::UMAT + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                *reinterpret_cast<uint4*>(sB + sw128_offset(i, c8)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4*>(PACK ? sB + sw128_offset(i, c8 + 32) : sB + SL::UMAT + sw128_offset(i, c8)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
         } else {
 #pragma unroll 1
@@ -539,9 +542,8 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                 const float y = j + 1 < R ? __ldg(p.U + (((size_t)m1 * Hkv + h) * D + i) * r + (j + 1 - m1 * r)) : 0.f;
                 uint32_t hi, lo;
                 split_pair(x, y, hi, lo);
-                const uint32_t off = sw128_offset(i, c2);
-                *reinterpret_cast<uint32_t*>(sB + off) = hi;
-                *reinterpret_cast<uint32_t*>(sB + SL::UMAT + off) = lo;
+                *reinterpret_cast<uint32_t*>(sB + sw128_offset(i, c2)) = hi;
+                *reinterpret_cast<uint32_t*>(PACK ? sB + sw128_offset(i, c2 + 32) : sB + SL::UMAT + sw128_offset(i, c2)) = lo;
             }
         }
         if (tid < ET_UCOLS) exp_s[slot * ET_UCOLS + tid] = (unsigned short)(j0 + tid < R ? (j0 + tid) / r : M - 1);
@@ -550,7 +552,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     int st = 0, u_head = -1, routed_for = -1;           // stage, head whose only block of U is resident, (sequence, head) of the coefficients
     uint32_t n_c = 0, n_d = 0;                          // products so far (phases)
     const bool resident = R <= ET_UCOLS * p.u_blocks;
-    uint8_t* sL = smem + SL::U + p.u_blocks * (2 * SL::UMAT);
+    uint8_t* sL = smem + SL::U + p.u_blocks * SL::UBLK;
     float* alpha_r = reinterpret_cast<float*>(sL + (SIDE ? SL::TILE : 0));
     // Eq. 6 of a pair b * Hkv + h into alpha_r (the scratch starts behind the result)
     auto route_pair = [&](int bh) {
@@ -595,14 +597,15 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nks = (rc + 15) / 16;
             if (j0 > 0 && !resident) { stage_u(h, j0, 0); fence_proxy_async(); __syncthreads(); }
             const int slot = resident ? j0 / ET_UCOLS : 0;
-            const uint32_t dU = dU0 + slot * ((2 * SL::UMAT) >> 4);
-            const unsigned short* ex = exp_s + slot * ET_UCOLS + half * 32;
+            const uint32_t dU = dU0 + slot * (SL::UBLK >> 4);
+            const int jh = half * (PACK ? 16 : 32);     // first column of this half of the threads
+            const unsigned short* ex = exp_s + slot * ET_UCOLS + jh;
             if (tid == 0) {
                 tc_fence_after();
                 const uint32_t kd = dK0 + st * (SL::TILE >> 4);
                 constexpr uint32_t IDESC = umma_idesc_bf16(ET_UCOLS, true);
 #pragma unroll 1
-                for (int pb = 0; pb < 2 * (D / 64); ++pb) {         // part of U, 64 dimensions
+                for (int pb = 0; pb < (PACK ? 1 : 2) * (D / 64); ++pb) {        // part of U (packed: both side by side), 64 dimensions
                     const uint32_t kb = kd + (uint32_t)(pb % (D / 64)) * (EBLK >> 4);
                     const uint32_t ub = dU + (((uint32_t)(pb / (D / 64)) * SL::UMAT + (uint32_t)(pb % (D / 64)) * 8192) >> 4);
 #pragma unroll
@@ -618,20 +621,27 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             ok = mbar_wait(bars, n_c & 1, abort_flag, p.status, 60);
             ++n_c;
             ok = __all_sync(0xffffffffu, ok);
-            if (ok && warp_hl && half * 32 < rc) {
+            if (ok && warp_hl && jh < rc) {
                 // C times the row's coefficients, split, back over itself; what the rows that are not highlighted get is never used
                 tc_fence_after();
-                const uint32_t tc = tC + lane_off + half * 32;
+                const uint32_t tc = tC + lane_off + jh;
                 const float* a_row = read_back ? p.route.alpha_out + (size_t)(b * Hkv + h) * M : routed ? alpha_r : (M > 1 && p.alpha != nullptr ? p.alpha + ((size_t)b_row * Hkv + h) * M : nullptr);
                 // (16 columns at a time: few registers and little code, most launches make one or two steps and are bound by
                 // fetching their instructions)
 #pragma unroll 1
-                for (int q = 0; q < 2 && half * 32 + q * 16 < rc; ++q) {
+                for (int q = 0; q < (PACK ? 1 : 2) && jh + q * 16 < rc; ++q) {
                     uint32_t v[16], hl8[8];
                     tmem_ld16(tc + q * 16, v);
                     float ca = g, cb = g;
                     if (a_row != nullptr && (r & 7) == 0) { ca *= a_row[ex[q * 16]]; cb *= a_row[ex[q * 16 + 8]]; }
                     tmem_wait_ld_on16(v);
+                    if constexpr (PACK) {           // K times the low part
+                        uint32_t v2[16];
+                        tmem_ld16(tc + 32, v2);
+                        tmem_wait_ld_on16(v2);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(v2[e]));
+                    }
                     if (a_row != nullptr && (r & 7) != 0) {
 #pragma unroll
                         for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * a_row[ex[q * 16 + e]]);
@@ -653,7 +663,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
 #pragma unroll 1
                 for (int ks = 0; ks < nks; ++ks) {
                     const uint32_t a_hi = tC + (uint32_t)ks * 16, a_lo = a_hi + 8;
-                    const uint32_t u_hi = dU + (((uint32_t)ks * 32) >> 4), u_lo = u_hi + (SL::UMAT >> 4);
+                    const uint32_t u_hi = dU + (((uint32_t)ks * 32) >> 4), u_lo = u_hi + ((PACK ? 64 : SL::UMAT) >> 4);
                     umma_ts(tD, a_hi, u_hi, DESC_HI, IDESC, (j0 > 0 || ks > 0) ? 1u : 0u);
                     umma_ts(tD, a_lo, u_hi, DESC_HI, IDESC, 1u);
                     umma_ts(tD, a_hi, u_lo, DESC_HI, IDESC, 1u);
@@ -778,15 +788,16 @@ edit_scan_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ gai
     if (tid == 0) counts[blockIdx.x] = total;
 }
 
-template <int D, bool SIDE, typename KT>
+template <int D, bool SIDE, typename KT, bool PACK = false>
 static seka_status launch_tiles_t(TileArgs& a, long long n_units, size_t smem, int extra_blocks, cudaStream_t st) {
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
-    auto kern = edit_tiles_kernel<D, SIDE, KT>;
+    auto kern = edit_tiles_kernel<D, SIDE, KT, PACK>;
+    constexpr int CTAS = EtSmem<D, SIDE, PACK>::CTAS;
     if (smem > 220 * 1024) return SEKA_ERR_UNSUPPORTED;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
     long long per_sm = (227 * 1024) / (smem + (SIDE ? 4 : 9) * 1024);
-    per_sm = per_sm > EtSmem<D, SIDE>::CTAS ? EtSmem<D, SIDE>::CTAS : (per_sm < 1 ? 1 : per_sm);
+    per_sm = per_sm > CTAS ? CTAS : (per_sm < 1 ? 1 : per_sm);
     // one wave; a multiple of the (sequence, KV head) pairs or at least of the KV heads, so that a CTA keeps its block of U
     long long g = per_sm * n_sm;
     if (g > n_units) g = n_units;
@@ -803,10 +814,10 @@ static int u_blocks_of(const seka_shape* s) {
     return s->head_dim == 64 && R > ET_UCOLS && R <= 2 * ET_UCOLS ? 2 : 1;
 }
 
-template <int D, bool SIDE>
+template <int D, bool SIDE, bool PACK = false>
 static size_t tiles_smem(const seka_shape* s, bool routed, int k_route) {
-    using SL = EtSmem<D, SIDE>;
-    return 1024 + SL::U + u_blocks_of(s) * 2 * SL::UMAT + (SIDE ? SL::TILE : 0) + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
+    using SL = EtSmem<D, SIDE, PACK>;
+    return 1024 + SL::U + u_blocks_of(s) * SL::UBLK + (SIDE ? SL::TILE : 0) + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
 }
 
 static TileArgs tile_args(const seka_shape* s, const WorkspaceLayout& w, const void* K, void* out, const uint8_t* mask, const float* U,
@@ -838,6 +849,10 @@ static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout&
                                     static_cast<const uint4*>(K_in), static_cast<uint4*>(K_out), n16);
     if (stc != SEKA_OK) return stc;
     const long long units = (long long)((T + 127) / 128) * Hkv;
+    // (the fused forward's preparation stays unpacked: its launches are a step or two per CTA, and gain nothing)
+    if (s->rank * s->n_experts <= ET_UCOLS / 2)
+        return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16, true>(a, units, tiles_smem<128, false, true>(s, false, 0), 0, st)
+                        : launch_tiles_t<64, false, __nv_bfloat16, true>(a, units, tiles_smem<64, false, true>(s, false, 0), 0, st);
     return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16>(a, units, tiles_smem<128, false>(s, false, 0), 0, st)
                     : launch_tiles_t<64, false, __nv_bfloat16>(a, units, tiles_smem<64, false>(s, false, 0), 0, st);
 }

@@ -16,7 +16,10 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("d,rank,experts,kv,lens,mask", [
     (128, 32, 1, 2, [127], "all"), (128, 64, 1, 3, [128], "all"), (64, 16, 1, 2, [129], "all"), (64, 1, 1, 1, [1], "all"),
     (128, 65, 1, 2, [300, 0, 41], "runs"), (128, 24, 3, 2, [513, 70], "runs"), (64, 7, 9, 2, [200, 200], "spans"),
-    (128, 128, 4, 2, [257], "spans"), (64, 64, 2, 5, [1024, 1025, 1], "runs"), (128, 16, 1, 2, [640], "none")])
+    (128, 128, 4, 2, [257], "spans"), (64, 64, 2, 5, [1024, 1025, 1], "runs"), (128, 16, 1, 2, [640], "none"),
+    # both sides of a stacked rank of 32, where U changes its layout
+    (128, 33, 1, 2, [300], "all"), (64, 32, 1, 2, [300, 77], "runs"), (64, 33, 1, 2, [300], "runs"), (128, 8, 4, 3, [257, 130], "spans"),
+    (64, 11, 3, 2, [140], "all"), (128, 17, 1, 2, [190, 66], "all"), (64, 3, 10, 1, [513], "runs")])
 def test_edit_steps_and_blocks(d, rank, experts, kv, lens, mask, in_place):
     w = inputs.make_custom(seed=90 + rank, dtype="bf16", lens=lens, n_q_heads=2 * kv, n_kv_heads=kv, head_dim=d, rank=rank,
                            n_experts=experts, mask_kind=mask, highlight=0.3, gain=np.linspace(1.0, -0.5, len(lens)))
