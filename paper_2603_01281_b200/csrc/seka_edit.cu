@@ -24,7 +24,7 @@ __device__ __forceinline__ int find_sequence(const int* __restrict__ cu, int B, 
 // by the latency of that chain).  With a second output tensor the rows that are not highlighted are copied in the same
 // pass, 16 bytes per lane; the loads go out before the highlight flags are known.  Bound by HBM where the copy dominates
 // (the fp32 layer of 6000 tokens x 16 heads x 64, rank 16, a tenth highlighted, into a second tensor: copy + list + a warp
-// per row 56 us per call, this 21 us), by the fp32 pipe where most rows are highlighted (4 D rank flops per row).
+// per row 56 us per call, this 19 us; 21 without its placement under the tail of the launch before), by the fp32 pipe where most rows are highlighted (4 D rank flops per row).
 constexpr int ER_ROWS = 64, ER_THREADS = 256, ER_CP = 36;     // tokens per tile; pitch (floats) of 32-column chunks: float4 reads of 8 rows meet 32 banks
 
 template <typename T> struct Row16;        // 16 bytes of a row <-> fp32 values
@@ -75,6 +75,8 @@ edit_rows_kernel(const T* K_in, T* K_out, const uint8_t* __restrict__ mask, cons
     const int h1 = h0 + heads_per_cta < Hkv ? h0 + heads_per_cta : Hkv;
     const int n_rows = n_tok - t0 < ER_ROWS ? n_tok - t0 : ER_ROWS;
 
+    pdl_wait();
+    pdl_release();
     // a second tensor: the first head's rows are on their way while the flags are looked up
     uint4 v[NV];
     auto load_rows = [&](int h) {
@@ -229,11 +231,8 @@ static seka_status launch_edit_rows_t(const seka_shape* s, const void* K_in, voi
     auto kern = K_in == K_out ? edit_rows_kernel<T, D, false> : edit_rows_kernel<T, D, true>;
     constexpr size_t smem = edit_rows_smem<D>();
     if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
-    kern<<<(unsigned)grid, ER_THREADS, smem, st>>>(static_cast<const T*>(K_in), static_cast<T*>(K_out), mask, U, alpha, gain, he,
-                                                   s->cu_seqlens, n_tok, s->batch, s->max_seqlen, s->n_kv_heads, s->rank,
-                                                   s->n_experts, (int)hpc);
-    ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? SEKA_OK : SEKA_ERR_CUDA;
+    return launch_kernel(true, kern, (unsigned)grid, ER_THREADS, smem, st, static_cast<const T*>(K_in), static_cast<T*>(K_out), mask, U, alpha,
+                         gain, he, s->cu_seqlens, n_tok, s->batch, s->max_seqlen, s->n_kv_heads, s->rank, s->n_experts, (int)hpc);
 }
 
 static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void* K_out, const uint8_t* mask, const float* U,
