@@ -270,7 +270,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     const bool ok = mbar_wait(bar, parity, abort_flag, status, where);
     return __all_sync(0xffffffffu, ok);
 }
-constexpr int ET_THREADS = 256, ET_WARPS = ET_THREADS / 32;
+constexpr int ET_THREADS = 256, ET_SMALL = 512;
 constexpr int ET_UCOLS = 64;                // columns of U per block
 
 template <int D, bool SIDE, bool PACK = false>
@@ -304,13 +304,22 @@ struct TileArgs {
 // PACK (stacked rank of at most 32): both parts of U stand in one block, the low part from column 32 on, so that one product
 // forms K times either part and both halves of the threads scale C.  Before / with it: 36 layers as above 74 -> 69 us, 64 x 4096
 // tokens x 8 heads x 64, half highlighted, 96 -> 78 us (a fourth CTA per SM fits there).
-template <int D, bool SIDE, typename KT, bool PACK>
-__global__ void __launch_bounds__(ET_THREADS, EtSmem<D, SIDE, PACK>::CTAS)
+//
+// NTH = ET_SMALL: the preparation of a small launch, one step per CTA and one CTA per SM.  Its time is the chain's latency, so
+// four threads share a row, and the rows, U and what tells whether the step has work are all asked for at once (one trip to
+// memory instead of four; rows and U are wasted where the tile turns out not to be highlighted).  Before / with it, per call of
+// the fused forward: one prompt of 777 tokens on 32/8 heads of 128 30.4 -> 28.3 us, 2 tiles x 4 heads of 64 in fp32 19.4 -> 16.1,
+// 700 tokens with four routed experts 38 -> 34 (the step itself 19100 -> 12100 cycles in the first).
+template <int D, bool SIDE, typename KT, bool PACK, int NTH>
+__global__ void __launch_bounds__(NTH, NTH == ET_THREADS ? EtSmem<D, SIDE, PACK>::CTAS : 1)
 edit_tiles_kernel(const __grid_constant__ TileArgs p) {
+    constexpr bool SMALL = NTH == ET_SMALL;
+    static_assert(!SMALL || (SIDE && !PACK), "the small form is one of the preparation");
+    constexpr int NW = NTH / 32, PARTS = NTH / 128;     // warps; threads per row
     using SL = EtSmem<D, SIDE, PACK>;
     constexpr int NS = SL::NS;
     constexpr int UPR = D / 8;                          // 16-byte units (8 elements) of a key row
-    constexpr int RPP = ET_THREADS / UPR;               // rows a pass of the CTA loads
+    constexpr int RPP = NTH / UPR;                      // rows a pass of the CTA loads
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -321,6 +330,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         if (blk < p.jobs.n_items_blocks) {
             pdl_wait();
             pdl_release();
+            if (tid >= PREP_THREADS) return;
             items_block(p.jobs.sched, p.jobs.cu, p.jobs.steer, p.jobs.items, p.jobs.item_count, blk);
             return;
         }
@@ -338,10 +348,10 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     __shared__ int abort_s;
     __shared__ int tok_s[2][SIDE ? 1 : 128], seq_s[2][SIDE ? 1 : 128];      // stand-alone: token (-1: none) and sequence of a row, per stage
     __shared__ float c_s[2][SIDE ? 1 : 128];            // stand-alone: gain (one expert: times its coefficient) of a row, per stage
-    __shared__ UnitInfo look_s[ET_WARPS];               // SIDE: the units looked at last
+    __shared__ UnitInfo look_s[NW];               // SIDE: the units looked at last
     __shared__ unsigned short exp_s[2 * ET_UCOLS];      // expert of a column of the blocks in shared memory
     __shared__ int pre_s[SIDE ? 1 : kMaxSegments + 1];  // stand-alone: highlighted tokens before each segment
-    __shared__ int wsum_s[ET_WARPS];
+    __shared__ int wsum_s[NW];
     volatile int* abort_flag = &abort_s;
     if (tid == 0) {
         mbar_init(bars, 1); mbar_init(bars + 1, 1);
@@ -356,12 +366,13 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     const uint32_t tC = tmem_holder, tD = tC + ET_UCOLS;
     pdl_wait();
     pdl_release();
-    bool ok = !__syncthreads_or(*reinterpret_cast<volatile int*>(p.status) != 0);
+    const int dead = *reinterpret_cast<volatile int*>(p.status);
+    bool ok = SMALL || !__syncthreads_or(dead != 0);
 
     uint8_t* sU = smem + SL::U;
     constexpr uint32_t DESC_HI = umma_desc_hi_sw128(1024);
     const uint32_t dK0 = umma_desc_lo(smem_u32(smem), 16), dU0 = umma_desc_lo(smem_u32(sU), EBLK);
-    const int row = tid & 127, half = tid >> 7;         // tensor-memory lane = key row, and which half of the columns
+    const int row = tid & 127, part = tid >> 7;         // tensor-memory lane = key row, and which part of the columns
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const int R = r * M;
     const bool u_vec = (r & 7) == 0 && (reinterpret_cast<uintptr_t>(p.U) & 15) == 0;
@@ -373,17 +384,18 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     uint32_t cur_bits = 0;
     float cur_c = 0.f;
     int unit = blk, n_units = 0, n_hot = 0;
-    int look_pos = ET_WARPS;
+    int look_pos = NW;
     // SIDE: a CTA keeps its (sequence, KV head) as long as there are enough CTAs (its block of U and its routed coefficients
     // then serve all its units): `per` CTAs share the tiles of a pair, or a CTA takes several pairs one after another.
     const int BH = p.B * Hkv, per = SIDE ? (p.n_tile_blocks >= BH ? p.n_tile_blocks / BH : 1) : 1;
     if constexpr (SIDE) {
-        if (p.n_tile_blocks >= BH) n_units = blk < per * BH ? (p.n_tiles - blk / BH + per - 1) / per : 0;
+        if (SMALL) n_units = 0;                         // (the only one is taken below)
+        else if (p.n_tile_blocks >= BH) n_units = blk < per * BH ? (p.n_tiles - blk / BH + per - 1) / per : 0;
         else n_units = (BH - blk + p.n_tile_blocks - 1) / p.n_tile_blocks * p.n_tiles;
         unit = 0;                                       // units are counted per CTA
     } else if (ok) {
         // highlighted tokens before each segment, and in all
-        constexpr int PT = kMaxSegments / ET_THREADS;
+        constexpr int PT = kMaxSegments / NTH;
         int c[PT], sum = 0;
 #pragma unroll
         for (int q = 0; q < PT; ++q) { c[q] = tid * PT + q < p.n_seg ? p.counts[tid * PT + q] : 0; sum += c[q]; }
@@ -394,7 +406,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         __syncthreads();
         int base = incl - sum;
 #pragma unroll
-        for (int w = 0; w < ET_WARPS; ++w) { if (w < warp) base += wsum_s[w]; n_hot += wsum_s[w]; }
+        for (int w = 0; w < NW; ++w) { if (w < warp) base += wsum_s[w]; n_hot += wsum_s[w]; }
 #pragma unroll
         for (int q = 0; q < PT; ++q) { pre_s[tid * PT + q] = base; base += c[q]; }
         __syncthreads();
@@ -417,7 +429,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             return false;
         } else {
             while (true) {
-                if (look_pos == ET_WARPS) {             // a warp looks at each of the next eight units: one latency for all of them
+                if (look_pos == NW) {             // a warp looks at each of the next units, one a warp: one latency for all of them
                     if (unit >= n_units) return false;
                     __syncthreads();
                     UnitInfo* info = look_s + warp;
@@ -455,7 +467,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                     __syncthreads();
                     look_pos = 0;
                 }
-                while (look_pos < ET_WARPS) {
+                while (look_pos < NW) {
                     ++unit;
                     const UnitInfo& info = look_s[look_pos++];
                     if (info.work) {
@@ -519,11 +531,11 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         const int rc = R - j0 < ET_UCOLS ? R - j0 : ET_UCOLS, nu = (rc + 15) / 16 * 2;
         if (u_vec) {
 #pragma unroll 1
-            for (int u = tid; u < D * nu; u += ET_THREADS) {
+            for (int u = tid; u < D * nu; u += NTH) {
                 const int i = u / nu, c8 = (u - i * nu) * 8;
                 float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b4 = a;
                 if (j0 + c8 < R) {                          // (rank a multiple of 8: eight columns of one expert)
-                    const int m = (j0 + c8) / r, k = j0 + c8 - m * r;
+                    const int m = M == 1 ? 0 : (j0 + c8) / r, k = j0 + c8 - m * r;
                     const float4* src = reinterpret_cast<const float4*>(p.U + (((size_t)m * Hkv + h) * D + i) * r + k);
                     a = __ldg(src); b4 = __ldg(src + 1);
                 }
@@ -535,7 +547,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             }
         } else {
 #pragma unroll 1
-            for (int u = tid; u < D * nu * 4; u += ET_THREADS) {        // two columns at a time
+            for (int u = tid; u < D * nu * 4; u += NTH) {        // two columns at a time
                 const int i = u / (nu * 4), c2 = (u - i * (nu * 4)) * 2, j = j0 + c2, m0 = j / r, m1 = (j + 1) / r;
                 const float x = j < R ? __ldg(p.U + (((size_t)m0 * Hkv + h) * D + i) * r + (j - m0 * r)) : 0.f;
                 const float y = j + 1 < R ? __ldg(p.U + (((size_t)m1 * Hkv + h) * D + i) * r + (j + 1 - m1 * r)) : 0.f;
@@ -558,21 +570,55 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         double* sm = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(alpha_r) + ((M * 4 + 15) & ~15));
         const double* a = route_group(p.route.Q, p.route.q_is_f32, p.U, p.route.sigma, p.cu, p.L, p.route.Hq, Hkv, D, r, M,
                                       p.route.k_route, bh / Hkv, bh % Hkv, sm);
-        for (int m = tid; m < M; m += ET_THREADS) alpha_r[m] = (float)a[m];
+        for (int m = tid; m < M; m += NTH) alpha_r[m] = (float)a[m];
         routed_for = bh;
     };
+    bool have = false;
+    if constexpr (SMALL) {
+        const int t = blk / BH, bh = blk % BH;
+        cur_b = bh / Hkv; cur_h = bh - cur_b * Hkv;
+        const int seq0 = p.cu ? p.cu[cur_b] : cur_b * p.L;
+        const int Lb = (p.cu ? p.cu[cur_b + 1] : (cur_b + 1) * p.L) - seq0;
+        cur_tok0 = seq0 + t * 128; cur_nvalid = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
+        load_rows(0);
+        const int m = row < cur_nvalid ? p.mask[cur_tok0 + row] : 0;
+        const float g = p.gain[cur_b];
+        const int on = p.head_enable == nullptr ? 1 : p.head_enable[cur_h];
+        const bool one = M == 1 && p.alpha != nullptr && !routed;
+        const float a1 = one ? p.alpha[bh] : 1.f;
+        if (resident) {
+            stage_u(cur_h, 0, 0);
+            if (R > ET_UCOLS) stage_u(cur_h, ET_UCOLS, 1);
+            u_head = cur_h;
+        }
+        const float amax = one ? fabsf(a1) : routed ? 1.f : alpha_max_of(p.alpha, (size_t)bh, M);       // (as in steer_byte)
+        cur_c = g * a1;
+        cur_lo = t < kLoTiles || lo_needed(g, amax);
+        cur_bits = __ballot_sync(0xffffffffu, m != 0);
+        if (lane == 0) wsum_s[warp] = cur_bits != 0;
+        ok = !__syncthreads_or(dead != 0);
+        const int any = wsum_s[0] | wsum_s[1] | wsum_s[2] | wsum_s[3];
+        if (cur_h == 0) {                               // what the fused kernel needs to know
+            if (tid == 0) p.tile_hot[(size_t)cur_b * p.n_tiles + t] = any != 0 ? 1 : 0;
+            if (t == 0)
+                for (int hh = tid; hh < Hkv; hh += NTH) p.bh_info[(size_t)cur_b * Hkv + hh] = (uint8_t)steer_byte(p.jobs.steer, cur_b, hh, Hkv);
+        }
+        have = ok && any && on && g != 0.f;
+    }
     if (routed && ok && p.route.alpha_out != nullptr && blk < BH) {
         // the first CTA of a pair leaves its coefficients for the caller
         for (int bh = blk; bh < BH; bh += p.n_tile_blocks) {
             route_pair(bh);
             __syncthreads();
-            for (int m = tid; m < M; m += ET_THREADS) p.route.alpha_out[(size_t)bh * M + m] = alpha_r[m];
+            for (int m = tid; m < M; m += NTH) p.route.alpha_out[(size_t)bh * M + m] = alpha_r[m];
         }
     }
-    bool have = ok && next_unit();
-    if (have) {
-        if (!SIDE) { find_rows(0); __syncthreads(); }
-        load_rows(0);
+    if constexpr (!SMALL) {
+        have = ok && next_unit();
+        if (have) {
+            if (!SIDE) { find_rows(0); __syncthreads(); }
+            load_rows(0);
+        }
     }
     while (have) {
         const int h = cur_h, b = cur_b, tok0 = cur_tok0, nvalid = cur_nvalid;
@@ -597,7 +643,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
             if (j0 > 0 && !resident) { stage_u(h, j0, 0); fence_proxy_async(); __syncthreads(); }
             const int slot = resident ? j0 / ET_UCOLS : 0;
             const uint32_t dU = dU0 + slot * (SL::UBLK >> 4);
-            const int jh = half * (PACK ? 16 : 32);     // first column of this half of the threads
+            const int jh = part * (PACK ? 16 : 64 / PARTS);         // first column of this part of the threads
             const unsigned short* ex = exp_s + slot * ET_UCOLS + jh;
             if (tid == 0) {
                 tc_fence_after();
@@ -628,7 +674,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
                 // (16 columns at a time: few registers and little code, most launches make one or two steps and are bound by
                 // fetching their instructions)
 #pragma unroll 1
-                for (int q = 0; q < (PACK ? 1 : 2) && jh + q * 16 < rc; ++q) {
+                for (int q = 0; q < (PACK ? 1 : 4 / PARTS) && jh + q * 16 < rc; ++q) {
                     uint32_t v[16], hl8[8];
                     tmem_ld16(tc + q * 16, v);
                     float ca = g, cb = g;
@@ -678,10 +724,10 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         if (!ok && !resident) break;
         uint8_t* sK = smem + st * SL::TILE;
         if (ok && (warp_hl || with_lo)) {
-            // k' = k + dK[row] for highlighted rows, half a row per thread, in place in the staged rows; low parts beside them
+            // k' = k + dK[row] for highlighted rows, 1 / PARTS of a row per thread, in place in the staged rows; low parts beside them
             tc_fence_after();
 #pragma unroll 1
-            for (int c = half * (D / 32); c < (half + 1) * (D / 32); ++c) {      // 16 columns
+            for (int c = part * (D / 16 / PARTS); c < (part + 1) * (D / 16 / PARTS); ++c) {      // 16 columns
                 uint32_t v[16];
                 if (warp_hl) { tmem_ld16(tD + lane_off + c * 16, v); tmem_wait_ld_on16(v); }     // warp-wide: every lane takes part
 #pragma unroll
@@ -709,7 +755,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         ok = __syncthreads_and(ok);
         if (!ok) break;
         // write the rows out: D / 8 lanes per row, 16 bytes each
-#pragma unroll 2
+#pragma unroll SMALL ? 4 : 2
         for (int k = 0; k < 128 / RPP; ++k) {
             const int rr = tid / UPR + k * RPP, c = tid % UPR;
             const int tok = SIDE ? tok0 + rr : tok_s[st][SIDE ? 0 : rr];
@@ -787,11 +833,11 @@ edit_scan_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ gai
     if (tid == 0) counts[blockIdx.x] = total;
 }
 
-template <int D, bool SIDE, typename KT, bool PACK = false>
+template <int D, bool SIDE, typename KT, bool PACK = false, int NTH = ET_THREADS>
 static seka_status launch_tiles_t(TileArgs& a, long long n_units, size_t smem, int extra_blocks, cudaStream_t st) {
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
-    auto kern = edit_tiles_kernel<D, SIDE, KT, PACK>;
+    auto kern = edit_tiles_kernel<D, SIDE, KT, PACK, NTH>;
     constexpr int CTAS = EtSmem<D, SIDE, PACK>::CTAS;
     if (smem > 220 * 1024) return SEKA_ERR_UNSUPPORTED;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
@@ -803,7 +849,7 @@ static seka_status launch_tiles_t(TileArgs& a, long long n_units, size_t smem, i
     if (SIDE && g >= (long long)a.B * a.Hkv) g -= g % ((long long)a.B * a.Hkv);
     else if (g > a.Hkv) g -= g % a.Hkv;
     a.n_tile_blocks = (int)g;
-    return launch_kernel(true, kern, (unsigned)(g + extra_blocks), ET_THREADS, smem, st, a);
+    return launch_kernel(true, kern, (unsigned)(g + extra_blocks), NTH, smem, st, a);
 }
 
 // Stacked ranks of 65 to 128 keep both blocks of U in shared memory at head_dim 64, where that leaves room for two CTAs (38
@@ -1221,6 +1267,14 @@ seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, con
     const bool routed = route.sigma != nullptr;
     const int extra = jobs.n_items_blocks + jobs.n_conv_blocks;
     const bool f32 = s->dtype == SEKA_F32;
+    if (units + extra <= n_sm) {                // one step per CTA, one CTA per SM: the small form (more CTAs than SMs would queue)
+        const size_t smem = s->head_dim == 128 ? tiles_smem<128, true>(s, routed, route.k_route) : tiles_smem<64, true>(s, routed, route.k_route);
+        if (s->head_dim == 128)
+            return f32 ? launch_tiles_t<128, true, float, false, ET_SMALL>(a, units, smem, extra, st)
+                       : launch_tiles_t<128, true, __nv_bfloat16, false, ET_SMALL>(a, units, smem, extra, st);
+        return f32 ? launch_tiles_t<64, true, float, false, ET_SMALL>(a, units, smem, extra, st)
+                   : launch_tiles_t<64, true, __nv_bfloat16, false, ET_SMALL>(a, units, smem, extra, st);
+    }
     if (s->head_dim == 128) {
         const size_t smem = tiles_smem<128, true>(s, routed, route.k_route);
         return f32 ? launch_tiles_t<128, true, float>(a, units, smem, extra, st) : launch_tiles_t<128, true, __nv_bfloat16>(a, units, smem, extra, st);

@@ -28,10 +28,10 @@ __device__ __forceinline__ int steer_byte(const SteerIn& s, int b, int h, int Hk
 
 // One of `n_blocks` blocks that share the conversion; four 16-byte loads of a thread are in flight together.
 __device__ __noinline__ static void convert_block(const ConvertArgs& a, int block, int n_blocks) {
-    const size_t step = (size_t)n_blocks * PREP_THREADS;
+    const size_t step = (size_t)n_blocks * blockDim.x;
 #pragma unroll
     for (int t = 0; t < 3; ++t) {
-        for (size_t i0 = (size_t)block * PREP_THREADS + threadIdx.x; i0 < a.n4[t]; i0 += 4 * step) {
+        for (size_t i0 = (size_t)block * blockDim.x + threadIdx.x; i0 < a.n4[t]; i0 += 4 * step) {
             float4 v[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q)

@@ -50,3 +50,23 @@ def test_preparation_on_both_sides_of_its_rule(d, seqs, kv):
     Oref, Lref, idx = H.oracle_rows(w, rows, head_enable=he)
     H.check_attention(O[idx], Oref, "d%d %d sequences" % (d, seqs))
     np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)       # the bound of the other forward tests
+
+
+@pytest.mark.parametrize("d,seqs,kv,L,rank,experts,dtype,varlen", [
+    (128, 37, 4, 100, 32, 1, "bf16", False), (128, 38, 4, 100, 32, 1, "bf16", False),      # 148 | 152 steps: small form | not
+    (64, 37, 4, 100, 16, 1, "bf16", False), (64, 38, 4, 100, 16, 1, "bf16", True),
+    (128, 2, 2, 300, 65, 1, "bf16", True), (128, 3, 2, 129, 24, 3, "bf16", False),         # U in blocks that are replaced
+    (64, 3, 3, 257, 33, 3, "bf16", True), (64, 2, 2, 128, 7, 1, "bf16", False),
+    (64, 3, 4, 130, 8, 1, "f32", False), (128, 2, 3, 200, 16, 2, "f32", True)])
+def test_small_preparation(d, seqs, kv, L, rank, experts, dtype, varlen):
+    lens = [L if not varlen or i == 0 else (0 if i == 1 and seqs > 2 else max(1, L - 31 * i % L)) for i in range(seqs)]
+    w = inputs.make_custom(seed=97, dtype=dtype, lens=lens, n_q_heads=2 * kv, n_kv_heads=kv, head_dim=d, rank=rank, n_experts=experts,
+                           mask_kind="runs", highlight=0.2, gain=[(0.5, 2.0, 0.0)[i % 3] for i in range(seqs)])
+    w.Q, w.K, w.V = (inputs.round_to_bf16(x) for x in (w.Q, w.K, w.V))      # (fp32 inputs are rounded on the way in)
+    alpha = np.random.default_rng(rank).uniform(-1, 1, size=(w.batch, kv, experts)).astype(np.float32)
+    he = np.array([1] * (kv - 1) + [0], dtype=np.uint8)
+    rows = H.sampled_rows(w, 8, seed=1)
+    O, LSE = H.run_fused(w, alpha=alpha, head_enable=he, force_varlen=varlen)
+    Oref, Lref, idx = H.oracle_rows(w, rows, alpha=alpha, head_enable=he)
+    H.check_attention(O[idx], Oref, "d%d %d sequences" % (d, seqs))
+    np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)       # the bound of the other forward tests
