@@ -910,8 +910,12 @@ static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout&
 //   warp 8   producer: walks this CTA's (sequence, tile) pairs of one KV head, stages the key tiles that hold a highlighted
 //            token through a ring of NS shared-memory stages by TMA, with the rows' highlight flags beside them;
 //   warp 9   MMA issuer: K P (two bf16 parts) into one of two sets of tensor-memory columns;
-//   warps 0-7  drain: half a key row per thread, k' = k + c (K P)[row] into the staged tile for highlighted rows, low parts
-//            straight to global memory, then the rows go out 16 bytes per lane; stage and columns are handed back.
+//   warps 0-7  drain: half a key row per thread, k' = k + c (K P)[row] into the staged tile for highlighted rows, the low parts
+//            beside it, then the rows go out 16 bytes per lane; stage and columns are handed back.
+// Bound by the writes (twice what it reads).  At head_dim 64 the low parts go through shared memory as well (a row per lane
+// they were 16-byte pieces, two to a sector) and two CTAs fit an SM: 16384 tiles of 16 heads 98 -> 77 us (the second CTA alone
+// 92, three of them 94).  At head_dim 128 shared memory is full of P and key tiles: low parts go straight to global memory
+// (through shared memory with two key stages instead of four: 101 against 93 us on 64 x 1024 tokens of 8 heads).
 constexpr int EP_THREADS = 320;
 
 // per stage: highlighted rows, first token, rows inside the sequence, end marker, low parts wanted, g * alpha
@@ -922,10 +926,13 @@ struct EpSmem {
     static constexpr uint32_t TILE = (D / 64) * EBLK;
     static constexpr uint32_t PBLK = D * 128;
     static constexpr uint32_t PMAT = (D / 64) * PBLK;
-    static constexpr int NS = D == 128 ? 4 : 8;             // key tiles in flight per SM
+    static constexpr int NS = D == 128 ? 4 : 3;             // stages of key tiles
+    static constexpr int CTAS = D == 128 ? 1 : 2;           // per SM (the projector of 128 leaves room for one)
     static constexpr uint32_t K = 0;                        // NS stages
     static constexpr uint32_t P = K + NS * TILE;            // high part, then low part
-    static constexpr uint32_t META = P + 2 * PMAT;          // NS x 48 bytes
+    static constexpr bool LOW = D == 64;                    // the low parts go out through shared memory (two tiles), as whole rows
+    static constexpr uint32_t L = P + 2 * PMAT;
+    static constexpr uint32_t META = L + (LOW ? 2 * TILE : 0);        // NS x 48 bytes
     static constexpr uint32_t BARS = META + NS * 48;        // full[NS], free[NS], mma_done[2], cols_free[2], p_full, meet[2]
     static constexpr uint32_t NBARS = 2 * NS + 7;
     static constexpr uint32_t MISC = BARS + NBARS * 8;
@@ -933,7 +940,7 @@ struct EpSmem {
 };
 
 template <int D>
-__global__ void __launch_bounds__(EP_THREADS, 1)
+__global__ void __launch_bounds__(EP_THREADS, EpSmem<D>::CTAS)
 stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmP, __nv_bfloat16* __restrict__ X,
                        const uint8_t* __restrict__ mask, const float* __restrict__ alpha, const float* __restrict__ gain,
                        const uint8_t* __restrict__ head_enable, const int* __restrict__ cu_seqlens,
@@ -1125,7 +1132,11 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
                             }
                             *ptr = kv;
                         }
-                        if (side_lo) *reinterpret_cast<uint4*>(xlo + col) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                        if (SL::LOW) {          // (the tile before last is out: its writers have met since)
+                            if (with_lo) *reinterpret_cast<uint4*>(smem + SL::L + cset * SL::TILE + (col >> 6) * EBLK + sw128_offset(row, col & 63)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                        } else if (side_lo) {
+                            *reinterpret_cast<uint4*>(xlo + col) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                        }
                     }
                     __syncwarp();      // all lanes together again before the next warp-wide load
                 }
@@ -1142,7 +1153,9 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
                 const int r = warp * 16 + i * RPI + lane / LPR, col = (lane % LPR) * 8;
                 if (r < m.nvalid) {
                     const uint4 v = *reinterpret_cast<const uint4*>(sK + (col >> 6) * EBLK + sw128_offset(r, col & 63));
-                    *reinterpret_cast<uint4*>(X + ((size_t)(m.tok0 + r) * Hkv + h) * (2 * D) + col) = v;
+                    __nv_bfloat16* dst = X + ((size_t)(m.tok0 + r) * Hkv + h) * (2 * D) + col;
+                    *reinterpret_cast<uint4*>(dst) = v;
+                    if (SL::LOW && with_lo) *reinterpret_cast<uint4*>(dst + D) = *reinterpret_cast<const uint4*>(smem + SL::L + cset * SL::TILE + (col >> 6) * EBLK + sw128_offset(r, col & 63));
                 }
             }
             __syncwarp();
@@ -1242,7 +1255,7 @@ static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout&
     if (stc != SEKA_OK) return stc;
     auto kern = stage_keys_pipe_kernel<D>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::DYN_BYTES) != cudaSuccess) return SEKA_ERR_CUDA;
-    const unsigned grid = (unsigned)(n_sm / Hkv * Hkv);
+    const unsigned grid = (unsigned)(PL::CTAS * n_sm / Hkv * Hkv);
     return launch_kernel(true, kern, grid, EP_THREADS, PL::DYN_BYTES, st, tk, tp, reinterpret_cast<__nv_bfloat16*>(ws + w.x_off), mask, alpha,
                          gain, he, s->cu_seqlens, tile_hot, reinterpret_cast<int*>(ws), s->batch, s->max_seqlen, Hkv, w.n_tiles);
 }
@@ -1251,9 +1264,9 @@ seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, con
                               const float* alpha, const float* gain, const uint8_t* head_enable, char* ws, const PrepJobs& jobs,
                               const RouteArgs& route, cudaStream_t st) {
     // The pipelined pair of launches from four waves of the chain on.  Measured preparations, pipeline against chain: packed
-    // batch of 64 sequences, 16 heads of 64, short runs (16384 units) 105 against 132 us; 64 x 1024 tokens, 4 heads of 64 /
-    // 128, all highlighted (2048 units) 32 against 36 / 50 against 56; 38 x 487, 8 heads of 64, 44 % (1216 units) 25 against
-    // 21; 4 x 4096 tokens, 8 heads of 128, a tenth (1024 units) 18 against 16; 4362 tokens, 8 heads (280) 19 against 13.
+    // batch of 64 sequences, 16 heads of 64, short runs (16384 units) 84 against 132 us; 64 x 1024 tokens, 4 heads of 64 /
+    // 128, all highlighted (2048 units) 26 against 36 / 50 against 56; 46 x 500, 8 heads of 64, 44 % (1472 units) 29 against
+    // 30, 12 x 500 (384 units) 15 against 13; 4 x 4096 tokens, 8 heads of 128, a tenth (1024 units) 18 against 16; 4362 tokens, 8 heads (280) 19 against 13.
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     const long long units = (long long)s->batch * w.n_tiles * s->n_kv_heads;
