@@ -255,7 +255,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
 
     // ---------------------------------------------------- merge the four warps' states, write the partial
     __syncthreads();                                        // every stage has been consumed (or the CTA has aborted)
-    if (*abort_flag && !p.direct) return;                   // (the status tells; a CTA of a cluster stays for its peers)
+    if (*abort_flag && (!p.direct || p.n_splits == 1)) return;      // (the status tells; a CTA of a cluster stays for its peers)
     float* mg = reinterpret_cast<float*>(smem);             // [warp][16 rows][D + 2]
     if (warp < DEC_CONSUMERS) {
         l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
@@ -292,7 +292,11 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
             acc = fmaf(mg[((size_t)w * 16 + g) * SL::MERGE_STRIDE + c], f, acc);
             lsum = fmaf(mg[((size_t)w * 16 + g) * SL::MERGE_STRIDE + D + 1], f, lsum);
         }
-        if (p.direct) {
+        if (p.direct && p.n_splits == 1) {                  // nobody to merge with
+            const size_t hq = (size_t)b * p.Hq + (size_t)hkv * G + g;
+            p.O[hq * D + c] = __float2bfloat16(lsum > 0.f ? acc / lsum : 0.f);
+            if (p.lse != nullptr && c == 0) p.lse[hq] = lsum > 0.f ? (M + log2f(lsum)) * 0.6931471805599453f : -INFINITY;
+        } else if (p.direct) {
             res[g * SL::MERGE_STRIDE + c] = acc;
             if (c == 0) { res[g * SL::MERGE_STRIDE + D] = M; res[g * SL::MERGE_STRIDE + D + 1] = lsum; }
         } else {
@@ -300,7 +304,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
             if (c == 0) *reinterpret_cast<float2*>(p.part_ml + (item * G + g) * 2) = make_float2(M, lsum);
         }
     }
-    if (!p.direct) return;
+    if (!p.direct || p.n_splits == 1) return;
 
     // ---------------------------------------------------- the cluster merges: every CTA a part of the group's output
     cluster_sync();
@@ -396,10 +400,17 @@ struct DecodePlan {
 // Where a power of two of chunks (up to a portable cluster of 8) per (sequence, KV head) fits one wave, those CTAs are a
 // cluster and the step is one launch.  Two launches cost 2 to 10 us more: 32 query heads on 8 of 128, one sequence of 512 /
 // 4096 tokens 6.5 -> 4.2 / 11.2 -> 6.9 us, 3 ragged sequences up to 6000 12.3 -> 8.5, 16 of 2048 28.6 -> 24.2, 4 of 32768
-// 97 -> 81 (90.8 in two launches of the present kernels).  The exceptions:
-//   - fewer CTAs than SMs with long chunks: one sequence of 16384 takes 16.3 us in 64 chunks of 2048, 15.7 in two launches;
-//   - batches whose longest sequence is far above the mean (lengths are known on the device only): one CTA
-//     would stream its long chunk alone, so chunks are limited to 2048 tokens there.
+// 97 -> 81 (90.8 in two launches of the present kernels).  The exceptions, where two launches balance better:
+//   - even lengths, long chunks in CTAs that fill less than six tenths of the slots: one sequence of 16384 takes 16.3 us in 64
+//     chunks of 2048, 15.7 in two launches, 5 of 4500 19.1 / 17.2 (160 CTAs of 296), 15 of 5499 on 16 heads of 64 60.3 / 57.2 (240 of
+//     444); 6 of 4500 21.4 / 23.0 (192 of 296), 18 of 6000 on 8 heads of 64 39.4 / 42.2 (288 of 444);
+//   - a cluster size that would fill more than nine tenths of the slots with clusters of 4 or 8: 9 of 9000 62.7 / 58.3 (72
+//     clusters of 4), 8 of 9000 46.5 / 51.8;
+//   - uneven lengths (the longest more than 1.25 times the mean; lengths are known on the device only, their sum here), unless
+//     the chunks are short or no longer than 1.2 times an SM's share of all tokens: up to 3421 tokens on 19 / 34 sequences 28.6 /
+//     43.5 us against 18.0 / 45.6, up to 1500 on 22 16.6 / 12.9.
+// Where a chunk holds the longest sequence there is nothing to merge, whatever the number of waves (79 ragged sequences of up to
+// 377 tokens 16.5 -> 12.5 us, 100 of 200 19.5 -> 15.1).
 // Workspace: that of the two launches in every case, a function of batch, heads and max_seqlen alone.
 DecodePlan decode_plan(const seka_shape* s) {
     DecodePlan d;
@@ -425,13 +436,14 @@ DecodePlan decode_plan(const seka_shape* s) {
     d.total = d.o_off + d.o_bytes;
 
     d.direct = d.n_splits == 1;
-    int cl = 1;
-    while (cl < DEC_MAX_CLUSTER && pairs * 2 * cl <= slots && s->max_seqlen > 128 * cl) cl *= 2;
+    int cl = 1;                     // (clusters of 4 and 8 do not pack the last tenth of the SMs)
+    while (cl < DEC_MAX_CLUSTER && pairs * 2 * cl * 10 <= (cl > 1 ? 9LL : 10LL) * slots && s->max_seqlen > 128 * cl) cl *= 2;
     const int part = ((s->max_seqlen + cl - 1) / cl + DEC_STAGE_KEYS - 1) / DEC_STAGE_KEYS * DEC_STAGE_KEYS;
-    const bool even = (long long)s->max_seqlen * s->batch <= 3LL * shape_total_tokens(s);
-    if (pairs > 0 && pairs <= slots && part > 0 && (part <= 1024 || (pairs * cl >= DEC_SM_COUNT && (even || part <= 2048)))) {
-        d.chunk = part; d.n_splits = cl; d.direct = 1;
-    }
+    const long long T = shape_total_tokens(s);
+    const bool even = 4LL * s->max_seqlen * s->batch <= 5LL * T;
+    const bool full = even ? part <= 1024 || pairs * cl * 10 >= 6LL * slots
+                           : (cl > 1 && part <= 128 * cl + 256) || 5LL * part * slots <= 12LL * T * s->n_kv_heads;
+    if (pairs > 0 && pairs <= slots && part > 0 && full) { d.chunk = part; d.n_splits = cl; d.direct = 1; }
     return d;
 }
 

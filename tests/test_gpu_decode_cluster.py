@@ -21,12 +21,13 @@ def _launches(f):
 
 @pytest.mark.parametrize("d,Hq,Hkv,lens,launches", [
     (128, 1, 1, [128], 1), (128, 1, 1, [129], 1), (128, 4, 1, [1025, 0, 1, 128, 64], 1),        # clusters of 1, 2, 8 (ranks without tokens)
-    (128, 16, 1, [8192, 300], 1), (128, 9, 1, [8193, 7000], 2),                                 # the longest chunk of few CTAs
-    (64, 2, 2, [8192], 1), (64, 2, 2, [8193], 2),
-    (128, 8, 8, [700 - 17 * i for i in range(18)], 1), (128, 8, 8, [700 - 17 * i for i in range(19)], 1),       # 144 | 152 pairs: 2 | 1
-    (128, 8, 8, [1100 - 27 * i for i in range(37)], 1), (128, 8, 8, [1100 - 27 * i for i in range(38)], 2),         # 296 | 304 pairs: one wave
-    (64, 12, 12, [1100 - 27 * i for i in range(37)], 1), (64, 12, 12, [1100 - 27 * i for i in range(38)], 2),       # 444 | 456 pairs
-    (128, 8, 8, [2560] + [30] * 36, 2), (128, 8, 8, [2560] * 14 + [30] * 23, 1),                # 296 pairs of up to 2560: uneven | even
+    (128, 16, 1, [8192], 1), (128, 9, 1, [8193], 2), (64, 2, 2, [8192], 1), (64, 2, 2, [8193], 2),      # longest chunk of few CTAs
+    (128, 8, 8, [1500] * 5, 1), (128, 4, 4, [4500] * 11, 2), (128, 4, 4, [4500] * 12, 1),               # 176 | 192 CTAs in clusters of 4
+    (128, 8, 8, [2200] * 9, 2), (128, 8, 8, [2200] * 8, 1),                                             # clusters of 4 fit | do not
+    (128, 8, 8, [1100] * 37, 1), (128, 8, 8, [1100] * 38, 2),                                           # 296 | 304 pairs: one wave
+    (64, 12, 12, [1100] * 37, 1), (64, 12, 12, [1100] * 38, 2),                                         # 444 | 456 pairs
+    (128, 8, 8, [2560] + [30] * 36, 2), (128, 8, 8, [2560] * 20 + [30] * 17, 1),                        # uneven: far above an SM's share | not
+    (128, 8, 8, [1000] + [60] * 17, 1), (128, 8, 8, [1100] + [60] * 17, 2),                             # uneven: clusters of 2, chunks of 512 | more
 ])
 def test_decode_on_both_sides_of_its_dispatch(d, Hq, Hkv, lens, launches):
     w = inputs.make_custom(seed=41, dtype="bf16", lens=lens, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, rank=8)
