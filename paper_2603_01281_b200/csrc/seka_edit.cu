@@ -271,7 +271,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     return __all_sync(0xffffffffu, ok);
 }
 constexpr int ET_THREADS = 256, ET_SMALL = 512;
-constexpr int ET_UCOLS = 64;                // columns of U per block
+constexpr int ET_UCOLS = 64, ET_UBLOCKS = 4;        // columns of U per block; most blocks that stay in shared memory
 
 template <int D, bool SIDE, bool PACK = false>
 struct EtSmem {
@@ -349,7 +349,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     __shared__ int tok_s[2][SIDE ? 1 : 128], seq_s[2][SIDE ? 1 : 128];      // stand-alone: token (-1: none) and sequence of a row, per stage
     __shared__ float c_s[2][SIDE ? 1 : 128];            // stand-alone: gain (one expert: times its coefficient) of a row, per stage
     __shared__ UnitInfo look_s[NW];               // SIDE: the units looked at last
-    __shared__ unsigned short exp_s[2 * ET_UCOLS];      // expert of a column of the blocks in shared memory
+    __shared__ unsigned short exp_s[ET_UBLOCKS * ET_UCOLS];      // expert of a column of the blocks in shared memory
     __shared__ int pre_s[SIDE ? 1 : kMaxSegments + 1];  // stand-alone: highlighted tokens before each segment
     __shared__ int wsum_s[NW];
     volatile int* abort_flag = &abort_s;
@@ -385,11 +385,13 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     float cur_c = 0.f;
     int unit = blk, n_units = 0, n_hot = 0;
     int look_pos = NW;
-    // SIDE: a CTA keeps its (sequence, KV head) as long as there are enough CTAs (its block of U and its routed coefficients
-    // then serve all its units): `per` CTAs share the tiles of a pair, or a CTA takes several pairs one after another.
-    const int BH = p.B * Hkv, per = SIDE ? (p.n_tile_blocks >= BH ? p.n_tile_blocks / BH : 1) : 1;
+    // SIDE: the CTAs take the tiles of all pairs (sequence, KV head) in turn; their number is a multiple of the KV heads, so that
+    // a CTA keeps its head (and its blocks of U).  Routed: a CTA also keeps its pair, whose coefficients then serve all its
+    // units: `per` CTAs share the tiles of a pair, or a CTA takes several pairs one after another.
+    const int BH = p.B * Hkv, per = routed && p.n_tile_blocks >= BH ? p.n_tile_blocks / BH : 1;
     if constexpr (SIDE) {
         if (SMALL) n_units = 0;                         // (the only one is taken below)
+        else if (!routed) n_units = (BH * p.n_tiles - blk + p.n_tile_blocks - 1) / p.n_tile_blocks;
         else if (p.n_tile_blocks >= BH) n_units = blk < per * BH ? (p.n_tiles - blk / BH + per - 1) / per : 0;
         else n_units = (BH - blk + p.n_tile_blocks - 1) / p.n_tile_blocks * p.n_tiles;
         unit = 0;                                       // units are counted per CTA
@@ -413,6 +415,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         n_units = ((n_hot + 127) / 128) * Hkv;
     }
     auto unit_pair = [&](int u, int& t) -> int {        // (SIDE) pair b * Hkv + h and tile of unit u of this CTA
+        if (!routed) { const int v = blk + u * p.n_tile_blocks; t = v / BH; return v % BH; }
         if (p.n_tile_blocks >= BH) { t = blk / BH + u * per; return blk % BH; }
         t = u % p.n_tiles;
         return blk + u / p.n_tiles * p.n_tile_blocks;
@@ -587,8 +590,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         const bool one = M == 1 && p.alpha != nullptr && !routed;
         const float a1 = one ? p.alpha[bh] : 1.f;
         if (resident) {
-            stage_u(cur_h, 0, 0);
-            if (R > ET_UCOLS) stage_u(cur_h, ET_UCOLS, 1);
+            for (int j0 = 0; j0 < R; j0 += ET_UCOLS) stage_u(cur_h, j0, j0 / ET_UCOLS);
             u_head = cur_h;
         }
         const float amax = one ? fabsf(a1) : routed ? 1.f : alpha_max_of(p.alpha, (size_t)bh, M);       // (as in steer_byte)
@@ -624,8 +626,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         const int h = cur_h, b = cur_b, tok0 = cur_tok0, nvalid = cur_nvalid;
         const bool with_lo = SIDE && cur_lo != 0;
         if (u_head != h) {
-            stage_u(h, 0, 0);
-            if (resident && R > ET_UCOLS) stage_u(h, ET_UCOLS, 1);
+            for (int j0 = 0; j0 == 0 || (resident && j0 < R); j0 += ET_UCOLS) stage_u(h, j0, j0 / ET_UCOLS);
             u_head = resident ? h : -1;
         }
         const bool read_back = routed && BH > p.n_tile_blocks && p.route.alpha_out != nullptr;      // written by this CTA above
@@ -843,26 +844,31 @@ static seka_status launch_tiles_t(TileArgs& a, long long n_units, size_t smem, i
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return SEKA_ERR_CUDA;
     long long per_sm = (227 * 1024) / (smem + (SIDE ? 4 : 9) * 1024);
     per_sm = per_sm > CTAS ? CTAS : (per_sm < 1 ? 1 : per_sm);
-    // one wave; a multiple of the (sequence, KV head) pairs or at least of the KV heads, so that a CTA keeps its block of U
+    // one wave; a multiple of the KV heads or (routed) of the (sequence, KV head) pairs
     long long g = per_sm * n_sm;
     if (g > n_units) g = n_units;
-    if (SIDE && g >= (long long)a.B * a.Hkv) g -= g % ((long long)a.B * a.Hkv);
+    if (SIDE && a.route.sigma != nullptr && g >= (long long)a.B * a.Hkv) g -= g % ((long long)a.B * a.Hkv);
     else if (g > a.Hkv) g -= g % a.Hkv;
     a.n_tile_blocks = (int)g;
     return launch_kernel(true, kern, (unsigned)(g + extra_blocks), NTH, smem, st, a);
 }
 
-// Stacked ranks of 65 to 128 keep both blocks of U in shared memory at head_dim 64, where that leaves room for two CTAs (38
-// sequences of 487 tokens, 8 heads, 4 experts of rank 32, routed: see below); at head_dim 128 the blocks are replaced per step.
-static int u_blocks_of(const seka_shape* s) {
-    const int R = s->rank * s->n_experts;
-    return s->head_dim == 64 && R > ET_UCOLS && R <= 2 * ET_UCOLS ? 2 : 1;
+// Blocks of U that stay in shared memory.  Stacked ranks of 65 to 128 keep both at head_dim 64, where that leaves room for two
+// CTAs; at head_dim 128 they are replaced per step (one CTA per SM with both: 79 against 52 us on 12 x 1500 tokens, 8 heads, four
+// experts of rank 24).  Beyond 128 replacing them is what a step spends its time on.  A preparation of many steps (`many`) keeps up
+// to four at head_dim 128 (four experts of rank 64 on 51 x 423 tokens of 4 heads 143 -> 97 us, 81 with the routing apart) and,
+// where the CTAs do not route, three at head_dim 64 (rank 48, 51 x 423 tokens of 8 heads 68 -> 59; four would leave one CTA per
+// SM: rank 64, 82 -> 101).
+static int u_blocks_of(const seka_shape* s, bool many = false, bool routed = false) {
+    const int R = s->rank * s->n_experts, nb = (R + ET_UCOLS - 1) / ET_UCOLS;
+    if (many && nb > 2 && (s->head_dim == 128 ? nb <= ET_UBLOCKS : nb == 3 && !routed)) return nb;
+    return s->head_dim == 64 && nb == 2 ? 2 : 1;
 }
 
 template <int D, bool SIDE, bool PACK = false>
-static size_t tiles_smem(const seka_shape* s, bool routed, int k_route) {
+static size_t tiles_smem(const seka_shape* s, int u_blocks, bool routed, int k_route) {
     using SL = EtSmem<D, SIDE, PACK>;
-    return 1024 + SL::U + u_blocks_of(s) * SL::UBLK + (SIDE ? SL::TILE : 0) + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
+    return 1024 + SL::U + u_blocks * SL::UBLK + (SIDE ? SL::TILE : 0) + (routed ? align_up((size_t)s->n_experts * 4, 16) + route_smem_bytes(D, s->n_experts, k_route) : 0);
 }
 
 static TileArgs tile_args(const seka_shape* s, const WorkspaceLayout& w, const void* K, void* out, const uint8_t* mask, const float* U,
@@ -896,10 +902,10 @@ static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout&
     const long long units = (long long)((T + 127) / 128) * Hkv;
     // (the fused forward's preparation stays unpacked: its launches are a step or two per CTA, and gain nothing)
     if (s->rank * s->n_experts <= ET_UCOLS / 2)
-        return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16, true>(a, units, tiles_smem<128, false, true>(s, false, 0), 0, st)
-                        : launch_tiles_t<64, false, __nv_bfloat16, true>(a, units, tiles_smem<64, false, true>(s, false, 0), 0, st);
-    return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16>(a, units, tiles_smem<128, false>(s, false, 0), 0, st)
-                    : launch_tiles_t<64, false, __nv_bfloat16>(a, units, tiles_smem<64, false>(s, false, 0), 0, st);
+        return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16, true>(a, units, tiles_smem<128, false, true>(s, a.u_blocks, false, 0), 0, st)
+                        : launch_tiles_t<64, false, __nv_bfloat16, true>(a, units, tiles_smem<64, false, true>(s, a.u_blocks, false, 0), 0, st);
+    return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16>(a, units, tiles_smem<128, false>(s, a.u_blocks, false, 0), 0, st)
+                    : launch_tiles_t<64, false, __nv_bfloat16>(a, units, tiles_smem<64, false>(s, a.u_blocks, false, 0), 0, st);
 }
 
 // ---------------------------------------------------------------- many tiles, one projector: the preparation as a pipeline
@@ -1277,22 +1283,38 @@ seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, con
                                   : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st);
     TileArgs a = tile_args(s, w, K, ws + w.x_off, mask, U, alpha, gain, head_enable, ws);
     a.route = route; a.jobs = jobs;
-    const bool routed = route.sigma != nullptr;
+    const size_t n_alpha = (size_t)s->batch * s->n_kv_heads * s->n_experts;
+    const long long pairs = (long long)s->batch * s->n_kv_heads;
+    if (route.sigma != nullptr && s->rank * s->n_experts > 2 * ET_UCOLS && units > 2LL * n_sm && n_sm / pairs * pairs * 5 < 4 * n_sm &&
+        (route.alpha_out != nullptr || n_alpha * 4 <= w.list_bytes)) {
+        // Wide banks with many steps: Eq. 6 by the launch of adaseka_route (same bits), so that its 17000 to 23000 cycles are
+        // spent once per pair and no CTA is tied to a pair, where pairs do not go evenly into the SMs.  Four experts of rank 64,
+        // 12 x 1500 tokens of 8 / 4 heads of 128 (96 / 48 pairs): 83 / 61 us against 121 / 56 routed in the CTAs.
+        float* dst = route.alpha_out != nullptr ? route.alpha_out : reinterpret_cast<float*>(ws + w.list_off);
+        const seka_status stc = launch_route(s, route.Q, U, route.sigma, route.k_route, dst, st);
+        if (stc != SEKA_OK) return stc;
+        a.route = RouteArgs{};
+        a.alpha = dst;
+    }
+    const bool routed = a.route.sigma != nullptr;
     const int extra = jobs.n_items_blocks + jobs.n_conv_blocks;
     const bool f32 = s->dtype == SEKA_F32;
     if (units + extra <= n_sm) {                // one step per CTA, one CTA per SM: the small form (more CTAs than SMs would queue)
-        const size_t smem = s->head_dim == 128 ? tiles_smem<128, true>(s, routed, route.k_route) : tiles_smem<64, true>(s, routed, route.k_route);
+        const size_t smem = s->head_dim == 128 ? tiles_smem<128, true>(s, a.u_blocks, routed, route.k_route) : tiles_smem<64, true>(s, a.u_blocks, routed, route.k_route);
         if (s->head_dim == 128)
             return f32 ? launch_tiles_t<128, true, float, false, ET_SMALL>(a, units, smem, extra, st)
                        : launch_tiles_t<128, true, __nv_bfloat16, false, ET_SMALL>(a, units, smem, extra, st);
         return f32 ? launch_tiles_t<64, true, float, false, ET_SMALL>(a, units, smem, extra, st)
                    : launch_tiles_t<64, true, __nv_bfloat16, false, ET_SMALL>(a, units, smem, extra, st);
     }
+    a.u_blocks = u_blocks_of(s, units > 2LL * n_sm, routed);
+    if ((s->head_dim == 128 ? tiles_smem<128, true>(s, a.u_blocks, routed, route.k_route) : tiles_smem<64, true>(s, a.u_blocks, routed, route.k_route)) > 220 * 1024)
+        a.u_blocks = u_blocks_of(s);
     if (s->head_dim == 128) {
-        const size_t smem = tiles_smem<128, true>(s, routed, route.k_route);
+        const size_t smem = tiles_smem<128, true>(s, a.u_blocks, routed, route.k_route);
         return f32 ? launch_tiles_t<128, true, float>(a, units, smem, extra, st) : launch_tiles_t<128, true, __nv_bfloat16>(a, units, smem, extra, st);
     }
-    const size_t smem = tiles_smem<64, true>(s, routed, route.k_route);
+    const size_t smem = tiles_smem<64, true>(s, a.u_blocks, routed, route.k_route);
     return f32 ? launch_tiles_t<64, true, float>(a, units, smem, extra, st) : launch_tiles_t<64, true, __nv_bfloat16>(a, units, smem, extra, st);
 }
 

@@ -19,7 +19,12 @@ seka_status launch_route(const seka_shape* shape, const void* Q, const float* U,
     if (smem > 48 * 1024 &&      // very wide banks of rank-1 experts: up to 66 KB
         cudaFuncSetAttribute(route_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return SEKA_ERR_CUDA;
-    route_kernel<<<shape->batch * shape->n_kv_heads, 1024, smem, stream>>>(
+    // one pair's latency where every pair has an SM to itself, throughput otherwise (408 pairs of four experts
+    // of rank 64 at head_dim 128 in 13.7 us, at 64 in 8.4)
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
+    const int pairs = shape->batch * shape->n_kv_heads;
+    route_kernel<<<pairs, pairs <= n_sm ? 1024 : 256, smem, stream>>>(
         Q, shape->dtype == SEKA_F32 ? 1 : 0, U, sigma, shape->cu_seqlens, shape->max_seqlen, shape->n_q_heads,
         shape->n_kv_heads, shape->head_dim, shape->rank, shape->n_experts, k_route, alpha_out);
     ++g_launches;

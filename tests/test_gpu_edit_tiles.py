@@ -70,3 +70,29 @@ def test_small_preparation(d, seqs, kv, L, rank, experts, dtype, varlen):
     Oref, Lref, idx = H.oracle_rows(w, rows, alpha=alpha, head_enable=he)
     H.check_attention(O[idx], Oref, "d%d %d sequences" % (d, seqs))
     np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)       # the bound of the other forward tests
+
+
+@pytest.mark.parametrize("d,seqs,L,kv,rank,k_route", [
+    (128, 25, 400, 4, 43, 43), (128, 25, 400, 4, 64, 16),       # 100 pairs, 400 steps: blocks of U stay, Eq. 6 by a launch of its own
+    (128, 9, 1030, 4, 64, 64),                                  # 36 pairs: Eq. 6 in the CTAs
+    (64, 25, 400, 4, 48, 48), (64, 25, 400, 4, 64, 64), (64, 5, 2100, 4, 48, 7), (64, 25, 400, 4, 33, 4)])
+def test_wide_banks_with_many_steps(d, seqs, L, kv, rank, k_route):
+    """One call with routing against the coefficients of adaseka_route given by hand: the same bits, and the oracle's rows."""
+    w = inputs.make_custom(seed=98, dtype="bf16", lens=[L] * seqs, n_q_heads=kv, n_kv_heads=kv, head_dim=d, rank=rank, n_experts=4,
+                           mask_kind="runs", highlight=0.2, gain=[(0.5, 2.0, 0.0)[i % 3] for i in range(seqs)])
+    dev = H.device_tensors(w)
+    shp = H.shape_of(w, dev)
+    ws = binding.new_workspace(shp)
+    sigma = torch.from_numpy((0.9 ** np.arange(rank) * np.ones((4, kv, 1))).astype(np.float32)).cuda()
+    sigma *= torch.tensor([0.7, 1.0, 1.3, 0.9], device="cuda").view(4, 1, 1)
+    alpha = torch.empty((seqs, kv, 4), dtype=torch.float32, device="cuda")
+    binding.adaseka_route(shp, dev["Q"], dev["U"], sigma, k_route, alpha)
+    O = torch.full_like(dev["Q"], float("nan"))
+    for out in (torch.empty_like(alpha), None):
+        binding.seka_attention_fwd_routed(shp, dev["Q"], dev["K"], dev["V"], O, None, dev["mask"], dev["U"], sigma, k_route, out, dev["gain"],
+                                          None, ws)
+        assert binding.seka_poll_status(ws) == binding.SEKA_OK
+        assert out is None or torch.equal(out, alpha)
+        rows = H.sampled_rows(w, 4, seed=1)
+        Oref, _, idx = H.oracle_rows(w, rows, alpha=alpha.cpu().numpy())
+        H.check_attention(O.double().cpu().numpy()[idx], Oref, "d%d rank %d" % (d, rank))
