@@ -1177,7 +1177,9 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 }
 
 // First launch of that path: blocks [0, n_p) form a 32 x 32 tile of P[h] each (bf16, high parts of all heads, then low parts);
-// then blocks with a warp per (sequence, key tile) for the tile flags and the steering bytes; then the item table.
+// then blocks with a warp per (sequence, key tile) for the tile flags and the steering bytes; then the item table and the
+// conversion of fp32 inputs (11 ragged sequences of up to 11083 tokens of 8 heads of 64, nearly all
+// highlighted: 107 us for both launches, 232 for the chain with its conversion blocks).
 __global__ void __launch_bounds__(PREP_THREADS)
 prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ mask, __nv_bfloat16* __restrict__ P,
                       uint8_t* __restrict__ tile_hot, uint8_t* __restrict__ bh_info, int B, int L, int Hkv, int D, int r, int n_tiles,
@@ -1239,7 +1241,9 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
             for (int h = lane; h < Hkv; h += 32) bh_info[(size_t)b * Hkv + h] = (uint8_t)steer_byte(jobs.steer, b, h, Hkv);
         return;
     }
-    items_block(jobs.sched, jobs.cu, jobs.steer, jobs.items, jobs.item_count, blk - n_flag);
+    blk -= n_flag;
+    if (blk < jobs.n_items_blocks) items_block(jobs.sched, jobs.cu, jobs.steer, jobs.items, jobs.item_count, blk);
+    else convert_block(jobs.conv, blk - jobs.n_items_blocks, jobs.n_conv_blocks);
 }
 
 template <int D>
@@ -1253,9 +1257,10 @@ static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout&
     void* P = ws + w.w_off;
     uint8_t* tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off);
     CUtensorMap tk, tp;
-    if (!make_tile_map(&tk, K, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * Hkv * D, D)) return SEKA_ERR_CUDA;
+    const void* k16 = s->dtype == SEKA_F32 ? static_cast<const void*>(jobs.conv.out[1]) : K;       // (converted by the first launch)
+    if (!make_tile_map(&tk, k16, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * Hkv * D, D)) return SEKA_ERR_CUDA;
     const int n_p = Hkv * (D / 32) * (D / 32), n_flag = (s->batch * w.n_tiles + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
-    seka_status stc = launch_kernel(true, prep_projector_kernel, (unsigned)(n_p + n_flag + jobs.n_items_blocks), PREP_THREADS, 0, st, U, mask,
+    seka_status stc = launch_kernel(true, prep_projector_kernel, (unsigned)(n_p + n_flag + jobs.n_items_blocks + jobs.n_conv_blocks), PREP_THREADS, 0, st, U, mask,
                                     static_cast<__nv_bfloat16*>(P), tile_hot, reinterpret_cast<uint8_t*>(ws + w.info_off), s->batch,
                                     s->max_seqlen, Hkv, D, s->rank, w.n_tiles, n_p, n_flag, jobs);
     if (stc != SEKA_OK) return stc;
@@ -1278,7 +1283,7 @@ seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, con
     const long long units = (long long)s->batch * w.n_tiles * s->n_kv_heads;
     if (units > 0x7fffffffLL) return SEKA_ERR_UNSUPPORTED;
     const int chain_ctas = s->head_dim == 128 ? EtSmem<128, true>::CTAS : EtSmem<64, true>::CTAS;
-    if (s->n_experts == 1 && route.sigma == nullptr && s->dtype == SEKA_BF16 && s->n_kv_heads <= n_sm && units > 4LL * chain_ctas * n_sm)
+    if (s->n_experts == 1 && route.sigma == nullptr && s->n_kv_heads <= n_sm && units > 4LL * chain_ctas * n_sm)
         return s->head_dim == 128 ? launch_stage_pipe<128>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st)
                                   : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st);
     TileArgs a = tile_args(s, w, K, ws + w.x_off, mask, U, alpha, gain, head_enable, ws);

@@ -37,13 +37,15 @@ def test_edit_steps_and_blocks(d, rank, experts, kv, lens, mask, in_place):
     assert np.array_equal(got[same], w.K.astype(np.float64)[same])
 
 
-@pytest.mark.parametrize("d,seqs,kv", [(128, 74, 4), (128, 75, 4), (64, 111, 4), (64, 112, 4)])
-def test_preparation_on_both_sides_of_its_rule(d, seqs, kv):
+@pytest.mark.parametrize("d,seqs,kv,dtype", [(128, 74, 4, "bf16"), (128, 75, 4, "bf16"), (64, 111, 4, "bf16"), (64, 112, 4, "bf16"),
+                                             (128, 75, 4, "f32"), (64, 112, 4, "f32")])
+def test_preparation_on_both_sides_of_its_rule(d, seqs, kv, dtype):
     """Four key tiles a sequence, so that 74 | 75 (111 | 112) sequences lie on the two sides of the line between the chain and the
     pipelined preparation on a GPU of 148 SMs."""
     lens = [400 + (37 * i) % 113 for i in range(seqs - 1)] + [512]
-    w = inputs.make_custom(seed=95, dtype="bf16", lens=lens, n_q_heads=kv, n_kv_heads=kv, head_dim=d, rank=16, mask_kind="runs",
+    w = inputs.make_custom(seed=95, dtype=dtype, lens=lens, n_q_heads=kv, n_kv_heads=kv, head_dim=d, rank=16, mask_kind="runs",
                            highlight=0.1, gain=[(0.5, 2.0, 0.0)[i % 3] for i in range(seqs)])
+    w.Q, w.K, w.V = (inputs.round_to_bf16(x) for x in (w.Q, w.K, w.V))      # (fp32 inputs are rounded on the way in)
     he = np.array([1, 0] + [1] * (kv - 2), dtype=np.uint8)
     rows = H.sampled_rows(w, 8, seed=1)
     O, LSE = H.run_fused(w, head_enable=he)
