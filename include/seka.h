@@ -79,7 +79,7 @@ size_t seka_workspace_bytes(const seka_shape* shape);
  * for highlighted tokens t of enabled heads h; every other row of K_out equals K_in
  * bit for bit.  K_out may alias K_in (in place: only edited rows are written).
  * fp32 tensors are edited in fp32 arithmetic; bf16 tensors accumulate in fp32 and round
- * once.  Uses `workspace` for the list of highlighted tiles.
+ * once.  Uses `workspace` for the list of highlighted tokens.
  */
 seka_status seka_edit_keys(const seka_shape* shape, const void* K_in, void* K_out,
                            const uint8_t* mask, const float* U, const float* alpha,
@@ -119,8 +119,8 @@ seka_status seka_attention_fwd(const seka_shape* shape, const void* Q, const voi
                                void* workspace, size_t workspace_bytes, void* cuda_stream);
 
 /*
- * AdaSEKA in one call (Algorithm 2): seka_attention_fwd with the routing coefficients of Eq. 6 computed by further
- * blocks of the library's operand-preparation launch instead of by a separate adaseka_route call (one launch fewer).
+ * AdaSEKA in one call (Algorithm 2): seka_attention_fwd with the routing coefficients of Eq. 6 computed by the blocks
+ * of its preparation launch (wide expert banks over many sequences: by the launch of adaseka_route ahead of it).
  * sigma and k_route are those of adaseka_route; the result equals adaseka_route followed by seka_attention_fwd bit
  * for bit.  alpha_out, if not NULL, receives the coefficients (fp32 [B, Hkv, M]); without it they live in the
  * workspace.  mask, U and sigma are required.
@@ -195,7 +195,8 @@ seka_status seka_edit_keys_static(const seka_shape* shape, const void* K_in, voi
  * [T, Hkv, d] described above; lse, if not NULL, receives fp32 [B, Hq] (natural log).  A sequence without
  * cached tokens gets O = 0 and lse = -inf.  K and V are read once and never written.
  * Only SEKA_BF16, at most 16 query heads per KV head and at most 65535 sequences (SEKA_ERR_UNSUPPORTED
- * otherwise); rank and n_experts of the shape are not used.  `workspace` holds the per-chunk partial results:
+ * otherwise); rank and n_experts of the shape are not used.  `workspace` holds the per-chunk partial results
+ * where they are not merged on chip:
  * seka_decode_workspace_bytes(shape) bytes, 256-byte aligned, its first 256 bytes the status block that
  * seka_reset_status / seka_poll_status read.
  */
@@ -214,7 +215,7 @@ seka_status seka_decode_attention(const seka_shape* shape, const void* Q, const 
  *   U_pos[s], U_neg[s]          [d, d] row-major, COLUMNS = left singular vectors of Omega+ / Omega-, singular values
  *                               descending (the layout seka_edit_keys / seka_attention_fwd take as U with rank = d;
  *                               P+ of Eq. 2 uses columns [0, k_pos), P- columns [k_neg, d)); computed in fp64 from the
- *                               fp32 Omega by one-sided Jacobi; a singular vector is defined up to its sign; columns
+ *                               fp32 Omega by QR and one-sided Jacobi; a singular vector is defined up to its sign; columns
  *                               of exactly zero singular value are returned as zeros
  *   S_pos[s], S_neg[s]          [d] singular values
  *   k_pos[s], k_neg[s]          int32: the smallest k with sum_{i<=k} S_i >= gamma * sum_i S_i (Eq. 3), decided in fp64

@@ -258,8 +258,11 @@ static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void*
 //
 // The step is a chain (rows and U land, product, scale, product, add, write) that several CTAs per SM walk side by side; the
 // rows of a CTA's next step are fetched under the present one where shared memory has room for a second stage.
-// Registers and code are kept small (16 columns at a time, short unrolls): a launch is often one or two steps per CTA, bound
-// by fetching its instructions, and spilled registers tripled the time of a step at head_dim 64.
+// Registers and code are kept small (16 columns at a time, short unrolls): a preparation is often one or two steps per CTA, bound
+// by fetching its instructions, and spilled registers tripled the time of a step at head_dim 64.  The stand-alone edit, whose CTAs
+// take many steps, has its loads, drain and writes unrolled at head_dim 128 (64 x 3000 tokens of 8 heads, all highlighted 216 -> 195
+// us).  Dense spans are what whole tiles through a projector did better: all / six tenths / three tenths of those tokens 173 / 119 / 76
+// us against 195 / 121 / 66, a tenth 45 against 28, short runs 138 against 37.
 // Measured: 144 x 4096 tokens x 8 heads x 128 in place, a tenth highlighted, 94 -> 69 us per call (whole 128-row tiles
 // through a projector, of which 58 % of the rows were written); one prompt of 777 tokens on 32/8 heads 42 -> 31 us per call
 // (four launches and two memsets before, two launches now).
@@ -507,7 +510,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     auto load_rows = [&](int st) {
         const int c = tid % UPR;
         const uint32_t base = smem_u32(smem) + st * SL::TILE + (c >> 3) * EBLK;
-#pragma unroll 2
+#pragma unroll (SIDE ? 2 : D == 128 ? 8 : 2)
         for (int k = 0; k < 128 / RPP; ++k) {
             const int rr = tid / UPR + k * RPP;
             const int tok = SIDE ? cur_tok0 + rr : tok_s[st][SIDE ? 0 : rr];
@@ -727,7 +730,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         if (ok && (warp_hl || with_lo)) {
             // k' = k + dK[row] for highlighted rows, 1 / PARTS of a row per thread, in place in the staged rows; low parts beside them
             tc_fence_after();
-#pragma unroll 1
+#pragma unroll (SIDE ? 1 : D == 128 ? 4 : 2)
             for (int c = part * (D / 16 / PARTS); c < (part + 1) * (D / 16 / PARTS); ++c) {      // 16 columns
                 uint32_t v[16];
                 if (warp_hl) { tmem_ld16(tD + lane_off + c * 16, v); tmem_wait_ld_on16(v); }     // warp-wide: every lane takes part
@@ -756,7 +759,7 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
         ok = __syncthreads_and(ok);
         if (!ok) break;
         // write the rows out: D / 8 lanes per row, 16 bytes each
-#pragma unroll SMALL ? 4 : 2
+#pragma unroll (SMALL ? 4 : SIDE ? 2 : D == 128 ? 8 : 2)
         for (int k = 0; k < 128 / RPP; ++k) {
             const int rr = tid / UPR + k * RPP, c = tid % UPR;
             const int tok = SIDE ? tok0 + rr : tok_s[st][SIDE ? 0 : rr];
