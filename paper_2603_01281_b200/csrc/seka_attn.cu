@@ -71,8 +71,7 @@ struct Geo {
     // P is handed to the tensor core in two pieces, so that most of P V runs under the last exponentials; 16-key blocks in the
     // first piece (head_dim 64, whose P V is short: half)
     static constexpr int KP1 = D == 128 ? 6 : 4;
-    // K and V ring depth: what fits (64 ragged sequences on 16 heads of 64: 647 us with three stages, 638 with four)
-    static constexpr int NK = D == 128 ? 2 : 4;
+    static constexpr int NK = D == 128 ? 2 : 3;                    // K and V ring depth
     static constexpr uint32_t TILE = (D / 64) * BLK_BYTES;         // a [128 x D] tile
     static constexpr int NXMAX = 3;                                // most stages of the key-side operand
     static constexpr uint32_t NBARS = 14 + 2 * NK + NXMAX;
