@@ -25,6 +25,7 @@ namespace seka {
 //                     (sequence, KV head): steered / low parts used
 // then                item table of the fused kernel (32 bytes per unit, heaviest first)
 // then                (stand-alone edit) highlighted tokens, in segments: int32 per token; then a count per segment
+//                     (routed fused forward without an output for the coefficients: these, fp32, instead of the tokens)
 // then (fp32 inputs)  bf16 copies of Q, K, V
 // then                edited keys of the fused kernel, bf16 [T, Hkv, 2 d] (high | low parts; only rows of tiles that
 //                     hold a highlighted token are ever written or read)
@@ -165,7 +166,8 @@ static inline WorkspaceLayout workspace_layout(const seka_shape* s) {
     w.item_off = w.info_off + align_up((size_t)s->batch * s->n_kv_heads + 1, 256);
     w.item_bytes = align_up((size_t)sc.n_items_max * 32 + 32, 256);
     w.list_off = w.item_off + w.item_bytes;
-    w.list_bytes = align_up(T * 4 + 4, 256);
+    const size_t n_alpha = s->n_experts == 1 ? (size_t)s->batch * s->n_kv_heads : 0;       // (one expert: routed coefficients may live here)
+    w.list_bytes = align_up((T > n_alpha ? T : n_alpha) * 4 + 4, 256);
     w.count_off = w.list_off + w.list_bytes;
     w.cvt_off = w.count_off + kMaxSegments * 4;
     w.cvt_bytes = 0;

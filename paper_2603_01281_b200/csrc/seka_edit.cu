@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(EP_THREADS, EpSmem<D>::CTAS)
 stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmP, __nv_bfloat16* __restrict__ X,
                        const uint8_t* __restrict__ mask, const float* __restrict__ alpha, const float* __restrict__ gain,
                        const uint8_t* __restrict__ head_enable, const int* __restrict__ cu_seqlens,
-                       const uint8_t* __restrict__ tile_hot, int* status, int B, int L, int Hkv, int n_tiles) {
+                       const uint8_t* __restrict__ tile_hot, int* status, int B, int L, int Hkv, int n_tiles, int routed) {
     using SL = EpSmem<D>;
     constexpr int EP_NS = SL::NS;
     constexpr int NBLK = D / 64;
@@ -1043,7 +1043,7 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
                 hot_l = (tile_hot[bt] != 0 && g != 0.f) ? 1 : 0;
                 c_l = g * a;
                 tok0_l = seq0 + t * 128; nv_l = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
-                lo_l = (lo_needed(g, fabsf(a)) || t < kLoTiles) ? 1 : 0;
+                lo_l = (lo_needed(g, routed ? 1.f : fabsf(a)) || t < kLoTiles) ? 1 : 0;        // (as in steer_byte)
             }
             unsigned todo = __ballot_sync(0xffffffffu, hot_l != 0);
             uint32_t bits[4] = {0, 0, 0, 0};
@@ -1180,13 +1180,15 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 }
 
 // First launch of that path: blocks [0, n_p) form a 32 x 32 tile of P[h] each (bf16, high parts of all heads, then low parts);
-// then blocks with a warp per (sequence, key tile) for the tile flags and the steering bytes; then the item table and the
-// conversion of fp32 inputs (11 ragged sequences of up to 11083 tokens of 8 heads of 64, nearly all
+// then blocks with a warp per (sequence, key tile) for the tile flags and the steering bytes; then, in a routed call, a block
+// per (sequence, KV head) that leaves its coefficient (Eq. 6, the routine of adaseka_route: the same bits) for the launch
+// behind; then the item table and the conversion of fp32 inputs (11 ragged sequences of up to 11083 tokens of 8 heads of 64, nearly all
 // highlighted: 107 us for both launches, 232 for the chain with its conversion blocks).
 __global__ void __launch_bounds__(PREP_THREADS)
 prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ mask, __nv_bfloat16* __restrict__ P,
                       uint8_t* __restrict__ tile_hot, uint8_t* __restrict__ bh_info, int B, int L, int Hkv, int D, int r, int n_tiles,
-                      int n_p, int n_flag, const __grid_constant__ PrepJobs jobs) {
+                      int n_p, int n_flag, int n_route, const __grid_constant__ RouteArgs route, const __grid_constant__ PrepJobs jobs) {
+    extern __shared__ __align__(16) double route_sm[];
     const int tid = threadIdx.x;
     pdl_wait();
     pdl_release();
@@ -1245,6 +1247,13 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
         return;
     }
     blk -= n_flag;
+    if (blk < n_route) {
+        const double* a = route_group(route.Q, route.q_is_f32, U, route.sigma, jobs.cu, L, route.Hq, Hkv, D, r, 1, route.k_route, blk / Hkv,
+                                      blk % Hkv, route_sm);
+        if (tid == 0) route.alpha_out[blk] = (float)a[0];
+        return;
+    }
+    blk -= n_route;
     if (blk < jobs.n_items_blocks) items_block(jobs.sched, jobs.cu, jobs.steer, jobs.items, jobs.item_count, blk);
     else convert_block(jobs.conv, blk - jobs.n_items_blocks, jobs.n_conv_blocks);
 }
@@ -1252,7 +1261,7 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
 template <int D>
 static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
                                      const float* alpha, const float* gain, const uint8_t* he, char* ws, const PrepJobs& jobs,
-                                     cudaStream_t st) {
+                                     const RouteArgs& route_in, cudaStream_t st) {
     using PL = EpSmem<D>;
     const int T = shape_total_tokens(s), Hkv = s->n_kv_heads;
     int n_sm = 0;
@@ -1263,15 +1272,22 @@ static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout&
     const void* k16 = s->dtype == SEKA_F32 ? static_cast<const void*>(jobs.conv.out[1]) : K;       // (converted by the first launch)
     if (!make_tile_map(&tk, k16, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * Hkv * D, D)) return SEKA_ERR_CUDA;
     const int n_p = Hkv * (D / 32) * (D / 32), n_flag = (s->batch * w.n_tiles + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
-    seka_status stc = launch_kernel(true, prep_projector_kernel, (unsigned)(n_p + n_flag + jobs.n_items_blocks + jobs.n_conv_blocks), PREP_THREADS, 0, st, U, mask,
+    RouteArgs route = route_in;
+    const int n_route = route.sigma != nullptr ? s->batch * Hkv : 0;
+    if (n_route > 0) {          // without a place of the caller's the coefficients live in the list region, which has room for them
+        if (route.alpha_out == nullptr) route.alpha_out = reinterpret_cast<float*>(ws + w.list_off);
+        alpha = route.alpha_out;
+    }
+    seka_status stc = launch_kernel(true, prep_projector_kernel, (unsigned)(n_p + n_flag + n_route + jobs.n_items_blocks + jobs.n_conv_blocks), PREP_THREADS,
+                                    n_route > 0 ? route_smem_bytes(D, 1, route.k_route) : 0, st, U, mask,
                                     static_cast<__nv_bfloat16*>(P), tile_hot, reinterpret_cast<uint8_t*>(ws + w.info_off), s->batch,
-                                    s->max_seqlen, Hkv, D, s->rank, w.n_tiles, n_p, n_flag, jobs);
+                                    s->max_seqlen, Hkv, D, s->rank, w.n_tiles, n_p, n_flag, n_route, route, jobs);
     if (stc != SEKA_OK) return stc;
     auto kern = stage_keys_pipe_kernel<D>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::DYN_BYTES) != cudaSuccess) return SEKA_ERR_CUDA;
     const unsigned grid = (unsigned)(PL::CTAS * n_sm / Hkv * Hkv);
     return launch_kernel(true, kern, grid, EP_THREADS, PL::DYN_BYTES, st, tk, tp, reinterpret_cast<__nv_bfloat16*>(ws + w.x_off), mask, alpha,
-                         gain, he, s->cu_seqlens, tile_hot, reinterpret_cast<int*>(ws), s->batch, s->max_seqlen, Hkv, w.n_tiles);
+                         gain, he, s->cu_seqlens, tile_hot, reinterpret_cast<int*>(ws), s->batch, s->max_seqlen, Hkv, w.n_tiles, n_route > 0 ? 1 : 0);
 }
 
 seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
@@ -1286,9 +1302,9 @@ seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, con
     const long long units = (long long)s->batch * w.n_tiles * s->n_kv_heads;
     if (units > 0x7fffffffLL) return SEKA_ERR_UNSUPPORTED;
     const int chain_ctas = s->head_dim == 128 ? EtSmem<128, true>::CTAS : EtSmem<64, true>::CTAS;
-    if (s->n_experts == 1 && route.sigma == nullptr && s->n_kv_heads <= n_sm && units > 4LL * chain_ctas * n_sm)
-        return s->head_dim == 128 ? launch_stage_pipe<128>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st)
-                                  : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, st);
+    if (s->n_experts == 1 && s->n_kv_heads <= n_sm && units > 4LL * chain_ctas * n_sm)     // (routed or not: both forms give the same bits)
+        return s->head_dim == 128 ? launch_stage_pipe<128>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st)
+                                  : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st);
     TileArgs a = tile_args(s, w, K, ws + w.x_off, mask, U, alpha, gain, head_enable, ws);
     a.route = route; a.jobs = jobs;
     const size_t n_alpha = (size_t)s->batch * s->n_kv_heads * s->n_experts;

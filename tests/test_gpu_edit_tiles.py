@@ -98,3 +98,31 @@ def test_wide_banks_with_many_steps(d, seqs, L, kv, rank, k_route):
         rows = H.sampled_rows(w, 4, seed=1)
         Oref, _, idx = H.oracle_rows(w, rows, alpha=alpha.cpu().numpy())
         H.check_attention(O.double().cpu().numpy()[idx], Oref, "d%d rank %d" % (d, rank))
+
+
+@pytest.mark.parametrize("d,lens,dtype", [
+    (128, [512] * 74, "bf16"), (128, [512] * 75, "bf16"), (64, [512] * 112, "bf16"), (64, [512] * 112, "f32"),
+    (64, [1 + i % 3 for i in range(600)], "bf16")])            # fewer tokens than (sequence, KV head) pairs
+def test_one_routed_expert_on_both_sides_of_the_rule(d, lens, dtype):
+    """One expert, four KV heads, on both sides of the line between the chain and the pipelined preparation: one call with routing gives
+    the bits of adaseka_route followed by seka_attention_fwd."""
+    w = inputs.make_custom(seed=99, dtype=dtype, lens=lens, n_q_heads=4, n_kv_heads=4, head_dim=d, rank=16, mask_kind="runs", highlight=0.3,
+                           gain=[(0.5, 2.0, 0.0, -1.5)[i % 4] for i in range(len(lens))])
+    dev = H.device_tensors(w)
+    shp = H.shape_of(w, dev)
+    sigma = torch.from_numpy(0.9 ** np.arange(16, dtype=np.float32) * np.ones((1, 4, 1), dtype=np.float32)).cuda()
+    alpha = torch.empty((w.batch, 4, 1), dtype=torch.float32, device="cuda")
+    binding.adaseka_route(shp, dev["Q"], dev["U"], sigma, 0, alpha)
+    assert (alpha < 0).any() and (alpha > 0).any()
+    bits = torch.int16 if dtype == "bf16" else torch.int32
+    ref = torch.full_like(dev["Q"], float("nan"))
+    ws = binding.new_workspace(shp)
+    binding.seka_attention_fwd(shp, dev["Q"], dev["K"], dev["V"], ref, None, dev["mask"], dev["U"], alpha, dev["gain"], None, ws)
+    assert binding.seka_poll_status(ws) == binding.SEKA_OK
+    for out in (torch.full_like(alpha, float("nan")), None):
+        O = torch.full_like(ref, float("nan"))
+        ws = binding.new_workspace(shp)
+        binding.seka_attention_fwd_routed(shp, dev["Q"], dev["K"], dev["V"], O, None, dev["mask"], dev["U"], sigma, 0, out, dev["gain"], None, ws)
+        assert binding.seka_poll_status(ws) == binding.SEKA_OK
+        assert out is None or torch.equal(out, alpha)
+        assert torch.equal(O.view(bits), ref.view(bits))
