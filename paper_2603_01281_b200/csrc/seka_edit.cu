@@ -175,7 +175,7 @@ edit_rows_kernel(const T* K_in, T* K_out, const uint8_t* __restrict__ mask, cons
                         if (lane < rp) {
                             const int sb = seq_of[s];
                             const float a = gain[sb] * (alpha != nullptr ? alpha[((size_t)sb * Hkv + h) * M + m] : 1.f);
-                            Cs[s * ER_CP + j] = c[i] * a;
+                            Cs[s * ER_CP + j] = j < rn ? c[i] * a : 0.f;       // (an infinity times a zero column is not a zero)
                         }
                     }
                 }

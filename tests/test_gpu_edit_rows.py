@@ -39,3 +39,34 @@ def test_row_edit_tiles_and_chunks(dtype, d, rank, experts, lens, in_place):
         assert (np.abs(got - ref) / scale).max() <= tol
         same = (w.mask == 0)[:, None] | (he == 0)[None, :]
         assert np.array_equal(got[same], w.K.astype(np.float64)[same])
+
+
+@pytest.mark.parametrize("dtype,d,rank", [("f32", 64, 1), ("f32", 128, 3), ("f32", 64, 8), ("f32", 128, 13), ("f32", 64, 34), ("bf16", 64, 1), ("bf16", 128, 6)])
+def test_row_edit_infinities_and_nan(dtype, d, rank):
+    """A key with an infinity (or NaN) is edited as the sums over the stored columns say: the columns that fill up a chunk of the rank
+    add nothing, and no other row is touched."""
+    w = inputs.make_custom(seed=77, dtype=dtype, lens=[150], n_q_heads=2, n_kv_heads=2, head_dim=d, rank=rank, mask_kind="all", gain=0.5)
+    w.K[3, 0, 5] = np.inf; w.K[70, 1, 1] = -np.inf; w.K[149, 0, 9] = np.nan
+    with np.errstate(invalid="ignore"):
+        ref = oracle_edit(w)
+    for in_place in (False, True):
+        dev = H.device_tensors(w)
+        out = dev["K"] if in_place else torch.full_like(dev["K"], float("nan"))
+        binding.seka_edit_keys_static(H.shape_of(w, dev), dev["K"], out, dev["mask"], dev["U"], None, dev["gain"], None)
+        got = out.double().cpu().numpy()
+        assert np.array_equal(np.isnan(got), np.isnan(ref))
+        assert np.array_equal(np.isposinf(got), np.isposinf(ref)) and np.array_equal(np.isneginf(got), np.isneginf(ref))
+        fin = np.isfinite(ref)
+        assert np.isposinf(ref).any() or rank > 1
+        # the tolerances of the test above (entries of a unit-variance row stay below 8)
+        assert np.abs(got[fin] - ref[fin]).max() <= 8 * (2.0 ** -24 * (d + rank) * np.sqrt(d) if dtype == "f32" else 2.0 ** -8)
+
+
+def oracle_edit(w):
+    """k + g U (U^T k) in fp64, row by row (the oracle library is not asked for rows that are not finite)."""
+    K, U = w.K.astype(np.float64), w.U[0].astype(np.float64)
+    out = K.copy()
+    for h in range(K.shape[1]):
+        C = (K[:, h, :, None] * U[h][None]).sum(1)
+        out[:, h] = K[:, h] + float(w.gain[0]) * (C[:, None, :] * U[h][None]).sum(-1)
+    return out
