@@ -308,7 +308,8 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
 
     // ---------------------------------------------------- the cluster merges: every CTA a part of the group's output
     cluster_sync();
-    const int ns = (Lb + p.chunk - 1) / p.chunk;            // CTAs that held cached tokens (ranks 0 .. ns - 1)
+    // CTAs that held cached tokens (ranks 0 .. ns - 1; no further ones, also where max_seqlen understates the length)
+    const int ns = min((Lb + p.chunk - 1) / p.chunk, p.n_splits);
     const uint32_t res_addr = smem_u32(res);
     for (int idx = split * DEC_THREADS + threadIdx.x; idx < G * D; idx += p.n_splits * DEC_THREADS) {
         const int g = idx / D, c = idx - g * D;
@@ -353,7 +354,7 @@ decode_combine_kernel(const DecodeParams p) {
     const int b = row / p.Hq, hq = row - b * p.Hq;
     const int hkv = hq / p.G, g = hq - hkv * p.G;
     const int Lb = p.cu_seqlens != nullptr ? p.cu_seqlens[b + 1] - p.cu_seqlens[b] : p.L;
-    const int ns = (Lb + p.chunk - 1) / p.chunk;            // chunks that held cached tokens
+    const int ns = min((Lb + p.chunk - 1) / p.chunk, p.n_splits);       // chunks that held cached tokens (as above)
     const size_t item0 = ((size_t)b * p.Hkv + hkv) * p.n_splits;
     float M = -INFINITY, l = 0.f, acc[V] = {};
     for (int s0 = 0; s0 < ns; s0 += 32) {

@@ -40,3 +40,26 @@ def test_decode_on_both_sides_of_its_dispatch(d, Hq, Hkv, lens, launches):
     for b in np.flatnonzero(np.asarray(lens) == 0):
         assert np.all(O[b] == 0) and np.all(np.isneginf(LSE[b]))
     T._check(O, LSE, Oref, Lref)
+
+
+@pytest.mark.parametrize("d,kv,lens,max_len,covered", [
+    (128, 2, [3000] * 3, 129, 256), (64, 2, [3000, 20, 600], 500, 512),         # clusters of 2 and 4
+    (128, 8, [4000] + [30] * 36, 2560, 3072)])                                  # two launches, chunks of 1024
+def test_decode_of_lengths_beyond_max_seqlen(d, kv, lens, max_len, covered):
+    """cu_seqlens that runs ahead of the shape's max_seqlen: the step attends to the tokens that its chunks cover and reads no
+    chunk that does not exist."""
+    w = inputs.make_custom(seed=43, dtype="bf16", lens=lens, n_q_heads=kv, n_kv_heads=kv, head_dim=d, rank=8)
+    dev = H.device_tensors(w)
+    q = T._last_queries(w)
+    shp = H.shape_of(w, dev, force_varlen=True)
+    shp.max_seqlen = max_len
+    ws = torch.zeros(binding.seka_decode_workspace_bytes(shp), dtype=torch.uint8, device="cuda")
+    qd = torch.from_numpy(q).to(device="cuda", dtype=torch.bfloat16)
+    O = torch.full_like(qd, float("nan"))
+    binding.seka_decode_attention(shp, qd, dev["K"], dev["V"], O, None, ws)
+    assert binding.seka_poll_status(ws) == binding.SEKA_OK
+    seen = np.minimum(lens, covered)
+    rows = np.concatenate([s + np.arange(n) for s, n in zip(w.cu_seqlens[:-1].astype(np.int64), seen)])
+    Oref, _ = oracle.decode_attention(q, w.K[rows], w.V[rows], np.concatenate([[0], np.cumsum(seen)]).astype(np.int32))
+    err = np.abs(O.double().cpu().numpy() - Oref)
+    assert err.max() <= 1e-2 and err.mean() <= 1e-3, (err.max(), err.mean())       # the bounds of the other decode tests
