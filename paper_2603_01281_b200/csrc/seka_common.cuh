@@ -24,7 +24,7 @@ namespace seka {
 // then                one byte per (sequence, 128-key tile): the tile contains a highlighted token; then one byte per
 //                     (sequence, KV head): steered / low parts used
 // then                item table of the fused kernel (32 bytes per unit, heaviest first)
-// then                (stand-alone edit) highlighted tokens, in segments: int32 per token; then a count per segment
+// then                (stand-alone edit) highlighted tokens, in segments: int32 per token; their sequences; then a count per segment
 //                     (routed fused forward without an output for the coefficients: these, fp32, instead of the tokens)
 // then (fp32 inputs)  bf16 copies of Q, K, V
 // then                edited keys of the fused kernel, bf16 [T, Hkv, 2 d] (high | low parts; only rows of tiles that
@@ -139,12 +139,20 @@ static inline int edit_segment_tokens(long long T) {
     return (int)((T + (long long)kMaxSegments * 1024 - 1) / ((long long)kMaxSegments * 1024)) * 1024;
 }
 
+// Shapes that have projectors P[m][h] = U_m U_m^T in their workspace: one expert (pipelined preparation of the fused forward), and
+// several whose stand-alone edit takes them instead of the stacked columns (per 64 of these: nb) because that is less work.
+static inline bool edit_projectors(const seka_shape* s) {
+    const int nb = (s->rank * s->n_experts + 63) / 64;
+    return s->n_experts == 1 || (nb >= (s->head_dim == 128 ? 2 : 3) && 4 * nb >= 3 * s->n_experts);
+}
+
 struct WorkspaceLayout {
-    size_t w_off;                     // projectors P[h] as two bf16 parts (one expert)
+    size_t w_off;                     // projectors P[m][h] as two bf16 parts
     size_t hot_off;                   // uint8 [B, ceil(max_seqlen / 128)]
     size_t info_off;                  // uint8 [B, Hkv]: bit 0 steered, bit 1 with the low parts
     size_t item_off, item_bytes;      // ItemRecord [n_items_max]
     size_t list_off, list_bytes;      // int32 [total_tokens]
+    size_t seq_off;                   // int32 [total_tokens]
     size_t count_off;                 // int32 [kMaxSegments]
     size_t cvt_off, cvt_bytes;        // bf16 copies of Q, K, V (fp32 inputs only)
     size_t x_off, x_bytes;            // edited keys of the fused kernel
@@ -160,7 +168,7 @@ static inline WorkspaceLayout workspace_layout(const seka_shape* s) {
     const SteerPlan plan = make_steer_plan(s, true);
     w.n_tiles = (s->max_seqlen + 127) / 128;
     w.w_off = 1024;                   // (1024-byte aligned: read by TMA)
-    w.hot_off = w.w_off + (s->n_experts == 1 ? (size_t)2 * s->n_kv_heads * D * D * 2 : 0);
+    w.hot_off = w.w_off + (edit_projectors(s) ? (size_t)4 * s->n_experts * s->n_kv_heads * D * D : 0);
     w.info_off = w.hot_off + align_up((size_t)s->batch * w.n_tiles + 1, 256);
     const Sched sc = make_sched(s);
     w.item_off = w.info_off + align_up((size_t)s->batch * s->n_kv_heads + 1, 256);
@@ -168,7 +176,8 @@ static inline WorkspaceLayout workspace_layout(const seka_shape* s) {
     w.list_off = w.item_off + w.item_bytes;
     const size_t n_alpha = s->n_experts == 1 ? (size_t)s->batch * s->n_kv_heads : 0;       // (one expert: routed coefficients may live here)
     w.list_bytes = align_up((T > n_alpha ? T : n_alpha) * 4 + 4, 256);
-    w.count_off = w.list_off + w.list_bytes;
+    w.seq_off = w.list_off + w.list_bytes;
+    w.count_off = w.seq_off + align_up(T * 4 + 4, 256);
     w.cvt_off = w.count_off + kMaxSegments * 4;
     w.cvt_bytes = 0;
     if (s->dtype == SEKA_F32)
@@ -305,6 +314,13 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
+// Four rows of a 2-D tensor (box 64 x 1): coordinates are the first element (a multiple of 8) and the rows.
+__device__ __forceinline__ void tma_gather4(void* smem_dst, const CUtensorMap* m, uint64_t* bar, int x, int r0, int r1, int r2, int r3) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+        ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(x), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
         : "memory");
 }
 // generic-proxy writes to shared memory -> visible to the async proxy (UMMA / TMA)

@@ -259,13 +259,11 @@ static seka_status launch_edit_rows(const seka_shape* s, const void* K_in, void*
 // The step is a chain (rows and U land, product, scale, product, add, write) that several CTAs per SM walk side by side; the
 // rows of a CTA's next step are fetched under the present one where shared memory has room for a second stage.
 // Registers and code are kept small (16 columns at a time, short unrolls): a preparation is often one or two steps per CTA, bound
-// by fetching its instructions, and spilled registers tripled the time of a step at head_dim 64.  The stand-alone edit, whose CTAs
-// take many steps, has its loads, drain and writes unrolled at head_dim 128 (64 x 3000 tokens of 8 heads, all highlighted 216 -> 195
-// us).  Dense spans are what whole tiles through a projector did better: all / six tenths / three tenths of those tokens 173 / 119 / 76
-// us against 195 / 121 / 66, a tenth 45 against 28, short runs 138 against 37.
-// Measured: 144 x 4096 tokens x 8 heads x 128 in place, a tenth highlighted, 94 -> 69 us per call (whole 128-row tiles
-// through a projector, of which 58 % of the rows were written); one prompt of 777 tokens on 32/8 heads 42 -> 31 us per call
-// (four launches and two memsets before, two launches now).
+// by fetching its instructions, and many spilled registers tripled the time of a step at head_dim 64.  The stand-alone edit, whose
+// CTAs take many steps, has its loads, drain and writes unrolled at head_dim 128 (64 x 3000 tokens of 8 heads, all highlighted 216 ->
+// 200 us); where they are very many, or U is wide, the gathering kernel below takes over (see gather_edit).
+// Measured: one prompt of 777 tokens on 32/8 heads 42 -> 31 us per call of the fused forward (four launches and two memsets
+// before, two launches now).
 constexpr uint32_t EBLK = 128 * 128;        // one [128 x 64] bf16 block
 
 // all lanes of a warp wait on the same barrier and then agree on the outcome
@@ -274,6 +272,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     return __all_sync(0xffffffffu, ok);
 }
 constexpr int ET_THREADS = 256, ET_SMALL = 512;
+constexpr int kMaxGatherHeads = 256;
 constexpr int ET_UCOLS = 64, ET_UBLOCKS = 4;        // columns of U per block; most blocks that stay in shared memory
 
 template <int D, bool SIDE, bool PACK = false>
@@ -294,7 +293,7 @@ struct __align__(16) UnitInfo { uint32_t bits[4]; int work, b, tok0, nvalid; flo
 struct TileArgs {
     const void* K; __nv_bfloat16* out;
     const uint8_t* mask; const float* U; const float* alpha; const float* gain; const uint8_t* head_enable; const int* cu;
-    const int* list; const int* counts; int n_seg, seg_tokens;                   // stand-alone edit: the highlighted tokens
+    const int* list; const int* seqs; const int* counts; int n_seg, seg_tokens;  // stand-alone edit: the highlighted tokens, their sequences
     uint8_t* tile_hot; uint8_t* bh_info;                                         // SIDE: written for the fused kernel
     int* status;
     int B, L, Hkv, r, M, n_tiles;
@@ -784,17 +783,76 @@ edit_tiles_kernel(const __grid_constant__ TileArgs p) {
     if (warp == 0) tmem_dealloc(tC, SL::TMEM_COLS);
 }
 
+// A 32 x 32 tile of P = U U^T of one (expert, KV head), two bf16 parts: P = hi + lo to about 2^-17, so that the edit keeps
+// fp32-like accuracy on bf16 tensor cores.  Blocks of PREP_THREADS threads, (D / 32)^2 per matrix; the high parts of all matrices
+// come first, then the low parts.  Bound by one trip to memory per 64 columns of U.
+__device__ __forceinline__ void projector_block(const float* __restrict__ U, __nv_bfloat16* __restrict__ P, int blk, int n_mats, int D, int r) {
+    const int tid = threadIdx.x, tiles = D / 32;
+    const int mat = blk / (tiles * tiles), t = blk % (tiles * tiles);
+    const int i0 = (t / tiles) * 32, j0 = (t % tiles) * 32;
+    constexpr int KC = 64, LD = KC + 4;                     // columns of U at a time; float4 reads of 8 rows meet 32 banks
+    __shared__ __align__(16) float ui[32][LD], uj[32][LD];
+    const int tx = tid & 31, ty = tid >> 5;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    const float* Um = U + (size_t)mat * D * r;
+    for (int k0 = 0; k0 < r; k0 += KC) {
+        const int rc = r - k0 < KC ? r - k0 : KC;
+        float a[2][4], b[2][4];                             // all loads of the chunk in flight together
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = c * 32 + tx;
+                a[c][q] = k < rc ? Um[(size_t)(i0 + ty + 8 * q) * r + k0 + k] : 0.f;
+                b[c][q] = k < rc ? Um[(size_t)(j0 + ty + 8 * q) * r + k0 + k] : 0.f;
+            }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { ui[ty + 8 * q][c * 32 + tx] = a[c][q]; uj[ty + 8 * q][c * 32 + tx] = b[c][q]; }
+        __syncthreads();
+        const int kn = (rc + 3) & ~3;
+#pragma unroll 4
+        for (int k = 0; k < kn; k += 4) {
+            const float4 y = *reinterpret_cast<const float4*>(&uj[tx][k]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 x = *reinterpret_cast<const float4*>(&ui[ty + 8 * q][k]);
+                acc[q] = fmaf(x.x, y.x, acc[q]); acc[q] = fmaf(x.y, y.y, acc[q]);
+                acc[q] = fmaf(x.z, y.z, acc[q]); acc[q] = fmaf(x.w, y.w, acc[q]);
+            }
+        }
+    }
+    __nv_bfloat16* Phi = P + (size_t)mat * D * D;
+    __nv_bfloat16* Plo = P + ((size_t)n_mats + mat) * D * D;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(acc[q]);
+        Phi[(size_t)(i0 + ty + 8 * q) * D + j0 + tx] = hi;
+        Plo[(size_t)(i0 + ty + 8 * q) * D + j0 + tx] = __float2bfloat16_rn(acc[q] - __bfloat162float(hi));
+    }
+}
+
 // List of the highlighted tokens (of sequences with a gain), a block per segment of consecutive tokens; with a second output
-// tensor further blocks copy the keys meanwhile (the rows that change are overwritten by the launch behind).
-__global__ void __launch_bounds__(256)
+// tensor further blocks copy the keys meanwhile (the rows that change are overwritten by the launch behind); the last n_p blocks
+// form the projectors that the gathering kernel reads.
+template <bool PROJ>
+__global__ void __launch_bounds__(PREP_THREADS)
 edit_scan_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ gain, const int* __restrict__ cu, int T, int B, int L,
-                 int* __restrict__ list, int* __restrict__ counts, int seg_tokens, int n_seg, const uint4* __restrict__ src,
-                 uint4* __restrict__ dst, size_t n16) {
+                 int* __restrict__ list, int* __restrict__ seqs, int* __restrict__ counts, int seg_tokens, int n_seg, const uint4* __restrict__ src,
+                 uint4* __restrict__ dst, size_t n16, const float* __restrict__ U, __nv_bfloat16* __restrict__ P, int n_p, int n_mats, int D, int r) {
     pdl_wait();
     pdl_release();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if constexpr (PROJ) {
+        if ((int)blockIdx.x >= (int)gridDim.x - n_p) {
+            projector_block(U, P, (int)blockIdx.x - ((int)gridDim.x - n_p), n_mats, D, r);
+            return;
+        }
+    }
     if ((int)blockIdx.x >= n_seg) {
-        const size_t step = (size_t)(gridDim.x - n_seg) * 256;
+        const size_t step = (size_t)(gridDim.x - n_p - n_seg) * 256;
         for (size_t i0 = (size_t)(blockIdx.x - n_seg) * 256 + tid; i0 < n16; i0 += 4 * step) {
             uint4 v[4];
 #pragma unroll
@@ -813,12 +871,16 @@ edit_scan_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ gai
     for (int t0 = s0; t0 < s0 + seg_tokens && t0 < T; t0 += 1024) {        // 1024 tokens a round, four per thread
         const int t = t0 + tid * 4;
         unsigned bits = 0;
+        int seq[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) bits |= (t + q < T && mask[t + q] != 0) ? 1u << q : 0u;
         if (bits != 0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (((bits >> q) & 1u) && gain[find_sequence(cu, B, L, t + q)] == 0.f) bits &= ~(1u << q);
+                if ((bits >> q) & 1u) {
+                    seq[q] = find_sequence(cu, B, L, t + q);
+                    if (gain[seq[q]] == 0.f) bits &= ~(1u << q);
+                }
         }
         const int cnt = __popc(bits);
         int incl = cnt;
@@ -831,10 +893,411 @@ edit_scan_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ gai
         for (int w = 0; w < 8; ++w) { if (w < warp) base += wsum[w]; total += wsum[w]; }
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if ((bits >> q) & 1u) out[base++] = t + q;
+            if ((bits >> q) & 1u) { seqs[s0 + base] = seq[q]; out[base++] = t + q; }
         __syncthreads();
     }
     if (tid == 0) counts[blockIdx.x] = total;
+}
+
+// ---------------------------------------------------------------- many rows or wide banks: gathered rows through projectors
+//
+// Where the chain above has many steps, or its stacked rank is wide, the edit is a pipeline over the same list of highlighted
+// tokens, one CTA per SM with a KV head of its own, from projectors P_m = U_m U_m^T in two bf16 parts.  One expert's projector is
+// formed by the CTA itself, on the tensor cores, while its first rows are on their way (by blocks of the launch before it cost
+// small edits 4 to 6 us); those of several (MULTI) come from that launch:
+//   warps 17 ..  producers, one per shared-memory stage: each brings every NS-th 128-row step of the CTA into its stage by TMA (one
+//                box where the tokens are consecutive, four rows an instruction otherwise), the rows' tokens and coefficients
+//                beside it; the look-up of its next step runs under the product and the drain of this one;
+//   warp 16      MMA issuer: K P_m (two bf16 parts) into a ring of sets of tensor-memory columns; with more experts than
+//                projectors fit (MULTI), it also brings the next ones in;
+//   warps 0-15   drain: 32 columns of a row per thread (at head_dim 64 two groups of warps take every other step),
+//                k' = k + sum_m c_m (K P_m)[row] in place in the stage, then the warp writes the pieces of its own 32 rows, 16
+//                bytes per lane (no barrier among the warps).
+// What a step costs does not depend on the rank.  Bound at head_dim 128 by shared memory (operands, rows in and out: 60 % of its
+// bandwidth, which stretches every access to it), at 64 by the pace at which one thread issues products (about 130 cycles each).
+// 144 x 4096 tokens x 8 heads x 128 in place, a tenth / all highlighted: whole tiles through a projector 96 / 561-590 us, the chain
+// 68.5 / 600-619, this 61.5 / 529-546 (4.5 TB/s).  On the way: rows fetched by 16-byte asynchronous copies instead of TMA 100 us more (a
+// step's 64 instructions held a warp for 5000 cycles), a look-up by binary search per row 40 more, eight drain warps 50 more.
+template <int D, bool MULTI>
+struct EgSmem {
+    static constexpr uint32_t TILE = (D / 64) * EBLK;
+    static constexpr uint32_t PBLK = D * 128;
+    static constexpr uint32_t PMAT = (D / 64) * PBLK;
+    static constexpr int NS = D == 128 ? (MULTI ? 2 : 4) : (MULTI ? 6 : 8);        // stages of key rows, a producer warp each
+    static constexpr int NP = MULTI ? (D == 128 ? 2 : 4) : 1;                       // projectors in shared memory
+    static constexpr int NSET = 512 / D;
+    static constexpr int WPT = D / 8, GROUPS = 16 / WPT;                            // drain warps of a step, of 16 in all; groups of them
+    static constexpr int GSET = NSET / GROUPS;                                      // sets of columns of a group
+    static constexpr int THREADS = (17 + NS) * 32;
+    static constexpr uint32_t K = 0;
+    static constexpr uint32_t P = K + NS * TILE;                                    // high part, then low part of each
+    static constexpr uint32_t META = P + NP * 2 * PMAT;                             // per stage: token, coefficient, sequence of a row
+    static constexpr uint32_t META_BYTES = 128 * 12;
+    static constexpr uint32_t BARS = META + NS * META_BYTES;        // full[NS], free[NS], done[NSET], cols[NSET], p_full[NP], drain, u_full, p_mma
+    static constexpr uint32_t NBARS = 2 * NS + 2 * NSET + NP + 3;
+    static constexpr uint32_t MISC = BARS + NBARS * 8;
+    static constexpr uint32_t DYN_BYTES = MISC + 16 + 1024;
+    static_assert(NS % GROUPS == 0, "a stage belongs to one group of drain warps");
+};
+
+template <int D, bool MULTI>
+__global__ void __launch_bounds__(EgSmem<D, MULTI>::THREADS, 1)
+edit_gather_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmP,
+                   const __grid_constant__ TileArgs p) {
+    using SL = EgSmem<D, MULTI>;
+    constexpr int NS = SL::NS, NP = SL::NP, NSET = SL::NSET, GROUPS = SL::GROUPS, GSET = SL::GSET, NBLK = D / 64;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + SL::BARS);      // [NS]  rows, tokens and coefficients of a step are in place
+    uint64_t* freeb = full + NS;               // [NS]    WPT drain-warp arrivals: the stage may be refilled
+    uint64_t* done = freeb + NS;               // [NSET]  a product is in its columns
+    uint64_t* cols = done + NSET;              // [NSET]  WPT drain-warp arrivals: the columns have been read
+    uint64_t* p_full = cols + NSET;            // [NP]    projector in place (MULTI: TMA bytes; else 16 drain-warp arrivals)
+    uint64_t* drain = p_full + NP;             // [1]     (teardown after an abort) every product issued has finished
+    uint64_t* u_full = drain + 1;              // [1]     (one expert) 16 drain-warp arrivals: both parts of U are staged
+    uint64_t* p_mma = u_full + 1;              // [1]     (one expert) U U^T is in the first set of columns
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + SL::MISC);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::MISC + 4);
+    __shared__ int pre_s[kMaxSegments];        // highlighted tokens before each segment
+    __shared__ int wsum_s[8];
+    __shared__ unsigned short on_s[kMaxGatherHeads];   // enabled heads
+    __shared__ int n_on_s;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int Hkv = p.Hkv, M = MULTI ? p.M : 1;
+    if (tid == 0) {
+        for (int i = 0; i < NS; ++i) { mbar_init(full + i, 2); mbar_init(freeb + i, SL::WPT); }
+        for (int i = 0; i < NSET; ++i) { mbar_init(done + i, 1); mbar_init(cols + i, SL::WPT); }
+        for (int i = 0; i < NP; ++i) mbar_init(p_full + i, MULTI ? 1 : 16);
+        mbar_init(drain, 1); mbar_init(u_full, 16); mbar_init(p_mma, 1);
+        *abort_flag = 0;
+        mbar_fence_init();
+        tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmT);
+        if (MULTI) tma_prefetch_desc(&tmP);
+    }
+    __syncwarp();
+    if (warp == 0) { tmem_alloc(tmem_holder, 512); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+    pdl_wait();
+    pdl_release();
+    // The first reads make one trip to memory together: the status, the counts of the list, the enabled heads and, where all are
+    // enabled (the CTA's head is known), this thread's first piece of U.
+    const int dead_word = *reinterpret_cast<volatile int*>(p.status);
+    const int nu = (p.r + 15) / 16 * 2;        // 8-column units of a row of U (zero up to the next multiple of 16 columns)
+    const bool u_vec = (p.r & 7) == 0 && (reinterpret_cast<uintptr_t>(p.U) & 15) == 0;
+    auto load_u = [&](int head, int u, float (&f)[8]) {
+        const int i = u / nu, c8 = (u - i * nu) * 8;
+        const float* src = p.U + ((size_t)head * D + i) * p.r + c8;
+        if (u_vec) {
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 a = c8 < p.r ? __ldg(reinterpret_cast<const float4*>(src)) : z, b = c8 < p.r ? __ldg(reinterpret_cast<const float4*>(src) + 1) : z;
+            f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) f[e] = c8 + e < p.r ? __ldg(src + e) : 0.f;
+        }
+    };
+    float u_first[8];
+    const bool u_early = !MULTI && p.head_enable == nullptr && tid < 512 && tid < D * nu;
+    if (u_early) load_u((int)blockIdx.x % Hkv, tid, u_first);
+
+    // highlighted tokens before each segment, and in all; enabled heads
+    constexpr int PT = kMaxSegments / 256;
+    int c[PT], sum = 0, incl = 0, n_hot = 0;
+    if (tid < 256) {
+#pragma unroll
+        for (int q = 0; q < PT; ++q) { c[q] = tid * PT + q < p.n_seg ? p.counts[tid * PT + q] : 0; sum += c[q]; }
+        incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        if (lane == 31) wsum_s[warp] = incl;
+    } else if (warp == 16) {
+        int n = 0;
+        for (int h0 = 0; h0 < Hkv; h0 += 32) {
+            const bool on = h0 + lane < Hkv && (p.head_enable == nullptr || p.head_enable[h0 + lane] != 0);
+            const unsigned bal = __ballot_sync(0xffffffffu, on);
+            if (on) on_s[n + __popc(bal & ((1u << lane) - 1))] = (unsigned short)(h0 + lane);
+            n += __popc(bal);
+        }
+        if (lane == 0) n_on_s = n;
+    }
+    const bool dead = __syncthreads_or(dead_word != 0);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) n_hot += wsum_s[w];
+    if (tid < 256) {
+        int base = incl - sum;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) if (w < warp) base += wsum_s[w];
+#pragma unroll
+        for (int q = 0; q < PT; ++q) { pre_s[tid * PT + q] = base; base += c[q]; }
+    }
+    __syncthreads();
+    // Product m of step i stands in the columns set_of(i, m): every group of drain warps has sets of its own, so that it sees each
+    // phase of their barriers (a parity wait cannot tell a phase from the one two later).
+    auto nth_of = [&](int i, int m) -> int { return i / GROUPS * M + m; };
+    auto set_of = [&](int i, int m) -> int { return i % GROUPS * GSET + nth_of(i, m) % GSET; };
+    auto phase_of = [&](int i, int m) -> uint32_t { return (uint32_t)(nth_of(i, m) / GSET) & 1u; };
+    // this CTA: every `step`-th chunk of 128 listed tokens of one enabled head
+    const int n_on = n_on_s, n_chunks = (n_hot + 127) / 128;
+    int h = 0, c0 = 0, step = 1, n_my = 0;
+    if (n_on > 0 && !dead) {
+        const int hi = (int)blockIdx.x % n_on;
+        h = on_s[hi]; c0 = (int)blockIdx.x / n_on; step = ((int)gridDim.x - hi + n_on - 1) / n_on;
+        n_my = c0 < n_chunks ? (n_chunks - c0 + step - 1) / step : 0;
+    }
+
+    if (warp > 16) {
+        // ------------------------------------------------------------ producers
+        // rows 4 lane .. 4 lane + 3 of a step: token (-1: none), sequence, coefficient
+        int tok[4], seq[4];
+        float cf[4];
+        auto look = [&](int i) {
+            const int q0 = (c0 + i * step) * 128, q = q0 + 4 * lane;           // (q0 < n_hot)
+            // largest segment with pre_s[seg] <= q0 (an empty one is never the largest): among every 32nd, then among the 32
+            const int blk = 32 * (__popc(__ballot_sync(0xffffffffu, 32 * lane < p.n_seg && pre_s[32 * lane] <= q0)) - 1);
+            const int lo = blk + __popc(__ballot_sync(0xffffffffu, blk + lane < p.n_seg && pre_s[blk + lane] <= q0)) - 1;
+            const int base = pre_s[lo];
+            int pos[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) pos[e] = lo * p.seg_tokens + q + e - base;
+            // the segments that begin inside the step
+            for (int s0 = lo + 1; s0 < p.n_seg; s0 += 32) {
+                const int w = s0 + lane < p.n_seg ? pre_s[s0 + lane] : 0x7fffffff;
+                const int n = __popc(__ballot_sync(0xffffffffu, w < q0 + 128));
+                for (int k = 0; k < n; ++k) {
+                    const int first = __shfl_sync(0xffffffffu, w, k);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) pos[e] = q + e >= first ? (s0 + k) * p.seg_tokens + q + e - first : pos[e];
+                }
+                if (n < 32) break;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                tok[e] = -1; seq[e] = 0;
+                if (q + e < n_hot) { tok[e] = p.list[pos[e]]; seq[e] = p.seqs[pos[e]]; }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cf[e] = p.gain[seq[e]];
+            if (!MULTI && p.alpha != nullptr) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) cf[e] *= p.alpha[(size_t)seq[e] * Hkv + h];
+            }
+        };
+        int i = warp - 17;
+        const int s = i;                       // this producer's stage
+        if (i < n_my) look(i);
+        for (; i < n_my; i += NS) {
+            if (i >= NS && !warp_wait(freeb + s, ((i / NS) - 1) & 1, abort_flag, p.status, 80)) break;
+            if (lane == 0) mbar_expect_tx(full + s, SL::TILE);
+            __syncwarp();
+            uint8_t* dst = smem + SL::K + s * SL::TILE;
+            const int t0 = __shfl_sync(0xffffffffu, tok[0], 0);
+            if (__shfl_sync(0xffffffffu, tok[3], 31) == t0 + 127) {         // the tokens are consecutive: one box
+                if (lane == 0) {
+#pragma unroll
+                    for (int cb = 0; cb < NBLK; ++cb) tma_load_3d(dst + cb * EBLK, &tmT, full + s, cb * 64, h, t0);
+                }
+            } else {                                                        // four rows a lane (beyond the list: any row, never written)
+#pragma unroll
+                for (int cb = 0; cb < NBLK; ++cb)
+                    tma_gather4(dst + lane * 512 + cb * EBLK, &tmK, full + s, h * D + cb * 64, max(tok[0], 0), max(tok[1], 0), max(tok[2], 0), max(tok[3], 0));
+            }
+            // second arrival: tokens and coefficients (the rows are not held up by the loads of these)
+            int* mt = reinterpret_cast<int*>(smem + SL::META + s * SL::META_BYTES);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                mt[4 * lane + e] = tok[e];
+                mt[128 + 4 * lane + e] = __float_as_int(cf[e]);
+                if (MULTI) mt[256 + 4 * lane + e] = seq[e];
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full + s);
+            if (i + NS < n_my) look(i + NS);
+        }
+        // the last rows asked for have landed before the shared memory is released (also after an abort)
+        if (i >= NS) mbar_wait_limit(full + s, ((i / NS) - 1) & 1, nullptr, nullptr, 0, kWaitLimitNs);
+    } else if (warp == 16) {
+        // ------------------------------------------------------------ MMA issuer
+        constexpr uint32_t IDESC = umma_idesc_bf16(D, false);
+        constexpr uint32_t DESC_HI = umma_desc_hi_sw128(1024);
+        const uint32_t dK = umma_desc_lo(smem_u32(smem + SL::K), 16), dP = umma_desc_lo(smem_u32(smem + SL::P), 16);
+        // projector loads: number u is that of product u (i * M + m) where they do not all stay, else of expert u
+        const bool stay = !MULTI || M <= NP;
+        const int n_load = !MULTI || n_my == 0 ? 0 : stay ? M : n_my * M;
+        int n_pushed = 0;
+        auto load_p = [&]() {
+            const int slot = n_pushed % NP, m = n_pushed % M;
+            mbar_expect_tx(p_full + slot, 2 * SL::PMAT);
+#pragma unroll
+            for (int part = 0; part < 2; ++part)
+#pragma unroll
+                for (int cb = 0; cb < NBLK; ++cb)
+                    tma_load_3d(smem + SL::P + (slot * 2 + part) * SL::PMAT + cb * SL::PBLK, &tmP, p_full + slot, cb * 64, 0,
+                                ((part * M + m) * Hkv + h) * D);
+            ++n_pushed;
+        };
+        if (lane == 0) {            // (one lane runs the whole loop: nothing to agree on between its waits)
+            while (n_pushed < n_load && n_pushed < NP) load_p();
+            bool ok = true;
+            if (!MULTI && n_my > 0) {           // P = U_hi U_hi^T + U_hi U_lo^T + U_lo U_hi^T (to about 2^-17)
+                ok = mbar_wait(u_full, 0, abort_flag, p.status, 87);
+                if (ok) {
+                    for (int t = 0; t < 3; ++t)
+                        for (int ks = 0; ks < (p.r + 15) / 16; ++ks) {
+                            const uint32_t off = ((uint32_t)(ks >> 2) * SL::PBLK + (uint32_t)(ks & 3) * 32) >> 4;
+                            umma_ss(tmem_base, dP + (t == 2 ? SL::PMAT >> 4 : 0u) + off, DESC_HI, dP + (t == 1 ? SL::PMAT >> 4 : 0u) + off, DESC_HI, IDESC,
+                                    (t > 0 || ks > 0) ? 1u : 0u);
+                        }
+                    umma_commit(p_mma);
+                }
+            }
+            for (int i = 0, u = 0; i < n_my && ok; ++i) {
+                const int s = i % NS;
+                ok = mbar_wait(full + s, (i / NS) & 1, abort_flag, p.status, 81);
+                if (!ok) break;
+                for (int m = 0; m < M; ++m, ++u) {
+                    const int set = set_of(i, m), slot = stay ? m : u % NP;
+                    if (!stay || i == 0) ok = mbar_wait(p_full + slot, stay ? 0 : (u / NP) & 1, abort_flag, p.status, 82);
+                    if (ok && nth_of(i, m) >= GSET) ok = mbar_wait(cols + set, phase_of(i, m) ^ 1u, abort_flag, p.status, 83);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t kd = dK + s * (SL::TILE >> 4), pd = dP + slot * (2 * SL::PMAT >> 4);
+#pragma unroll
+                    for (int part = 0; part < 2; ++part)
+#pragma unroll
+                        for (int ks = 0; ks < D / 16; ++ks) {
+                            const uint32_t offk = ((uint32_t)(ks >> 2) * EBLK + (uint32_t)(ks & 3) * 32) >> 4;
+                            const uint32_t offp = ((uint32_t)part * SL::PMAT + (uint32_t)(ks >> 2) * SL::PBLK + (uint32_t)(ks & 3) * 32) >> 4;
+                            umma_ss(tmem_base + set * D, kd + offk, DESC_HI, pd + offp, DESC_HI, IDESC, (ks > 0 || part) ? 1u : 0u);
+                        }
+                    umma_commit(done + set);
+                    if (!stay && u > 0 && n_pushed < n_load) {      // the product before is through: its projector makes room
+                        const int ip = (u - 1) / M, mp = (u - 1) % M;
+                        ok = mbar_wait(done + set_of(ip, mp), phase_of(ip, mp), abort_flag, p.status, 84);
+                        if (!ok) break;
+                        load_p();
+                    }
+                }
+            }
+            if (*abort_flag) {
+                // projectors on their way land, and products issued finish, before shared and tensor memory are released
+                for (int u = n_pushed > NP ? n_pushed - NP : 0; u < n_pushed; ++u)
+                    mbar_wait_limit(p_full + u % NP, (u / NP) & 1, nullptr, nullptr, 0, kWaitLimitNs);
+                umma_commit(drain);
+                mbar_wait_limit(drain, 0, nullptr, nullptr, 0, kWaitLimitNs);
+            }
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------------ drain and write-out
+        const int row = tid & 127, col0 = ((warp % SL::WPT) >> 2) * 32;          // row of the step, first of this thread's 32 columns
+        const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + col0;
+        const uint32_t off0 = (uint32_t)(col0 >> 6) * EBLK + sw128_offset(row, col0 & 63);
+        bool ready = true;
+        if constexpr (!MULTI) {
+            if (n_my > 0) {
+                // both parts of U, [D x 64] blocks where the projector will stand
+                uint8_t* sP = smem + SL::P;
+#pragma unroll 1
+                for (int u = tid; u < D * nu; u += 512) {
+                    const int i = u / nu, c8 = (u - i * nu) * 8;
+                    if (!u_early || u != tid) load_u(h, u, u_first);
+                    uint32_t hi[4], lo[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) split_pair(u_first[2 * e], u_first[2 * e + 1], hi[e], lo[e]);
+                    const uint32_t off = (uint32_t)(c8 >> 6) * SL::PBLK + sw128_offset(i, c8 & 63);
+                    *reinterpret_cast<uint4*>(sP + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                    *reinterpret_cast<uint4*>(sP + SL::PMAT + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                }
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(u_full);
+                // the projector in two parts over them
+                ready = warp_wait(p_mma, 0, abort_flag, p.status, 88);
+                const int pc = (warp >> 2) * 32;
+                if (ready && pc < D && (warp & 3) * 32 < D) {
+                    tc_fence_after();
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + pc, v);
+                    tmem_wait_ld_on(v);
+                    tc_fence_before();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        uint32_t hi[4], lo[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) split_pair(__uint_as_float(v[q * 8 + 2 * e]), __uint_as_float(v[q * 8 + 2 * e + 1]), hi[e], lo[e]);
+                        const uint32_t off = (uint32_t)(pc >> 6) * SL::PBLK + sw128_offset(row, (pc & 63) + q * 8);
+                        *reinterpret_cast<uint4*>(sP + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                        *reinterpret_cast<uint4*>(sP + SL::PMAT + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                    }
+                    fence_proxy_async();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(p_full);
+            }
+        }
+        for (int i = warp / SL::WPT; ready && i < n_my; i += GROUPS) {
+            const int s = i % NS;
+            if (!warp_wait(full + s, (i / NS) & 1, abort_flag, p.status, 85)) break;
+            const int* mt = reinterpret_cast<const int*>(smem + SL::META + s * SL::META_BYTES);
+            const int tok = mt[row];
+            const float cf = __int_as_float(mt[128 + row]);
+            uint8_t* sK = smem + SL::K + s * SL::TILE;
+            bool ok = true;
+            uint4 kv[4];                                // this thread's 32 columns of the row (before anything waits for the product)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) kv[q] = *reinterpret_cast<const uint4*>(sK + (off0 ^ (q << 4)));
+            float acc[32];
+            const float* al = MULTI && p.alpha != nullptr ? p.alpha + ((size_t)mt[256 + row] * Hkv + h) * M : nullptr;
+#pragma unroll 1
+            for (int m = 0; m < M; ++m) {
+                const int set = set_of(i, m);
+                const float cm = cf * (MULTI && al != nullptr ? al[m] : 1.f);
+                ok = warp_wait(done + set, phase_of(i, m), abort_flag, p.status, 86);
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t v[32];
+                tmem_ld32(t_lane + set * D, v);
+                tmem_wait_ld_on(v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(cols + set);
+#pragma unroll
+                for (int e = 0; e < 32; ++e) acc[e] = MULTI ? fmaf(cm, __uint_as_float(v[e]), m == 0 ? 0.f : acc[e]) : __uint_as_float(v[e]);
+            }
+            if (!ok) break;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {               // 8 elements = one 16-byte unit of the swizzled row
+                uint32_t* w = reinterpret_cast<uint32_t*>(&kv[q]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 k2 = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[e]));
+                    const float v0 = acc[q * 8 + 2 * e], v1 = acc[q * 8 + 2 * e + 1];
+                    w[e] = MULTI ? pack_bf16(k2.x + v0, k2.y + v1) : pack_bf16(fmaf(cf, v0, k2.x), fmaf(cf, v1, k2.y));
+                }
+                *reinterpret_cast<uint4*>(sK + (off0 ^ (q << 4))) = kv[q];
+            }
+            fence_proxy_async();            // (the stage is written by TMA next; here no global store is on its way yet)
+            __syncwarp();
+            // four lanes write the 64 bytes of a row, eight rows an instruction
+            uint4 v[4];
+            const uint32_t rd = (uint32_t)(col0 >> 6) * EBLK + sw128_offset((warp & 3) * 32 + (lane >> 2), (col0 & 63) + (lane & 3) * 8);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4*>(sK + rd + k * 1024);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(freeb + s);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int t = __shfl_sync(0xffffffffu, tok, k * 8 + (lane >> 2));
+                if (t >= 0) *reinterpret_cast<uint4*>(p.out + ((size_t)(uint32_t)t * Hkv + h) * D + col0 + (lane & 3) * 8) = v[k];
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem_base, 512);
 }
 
 template <int D, bool SIDE, typename KT, bool PACK = false, int NTH = ET_THREADS>
@@ -879,13 +1342,43 @@ static TileArgs tile_args(const seka_shape* s, const WorkspaceLayout& w, const v
     TileArgs a = {};
     a.K = K; a.out = static_cast<__nv_bfloat16*>(out);
     a.mask = mask; a.U = U; a.alpha = alpha; a.gain = gain; a.head_enable = he; a.cu = s->cu_seqlens;
-    a.list = reinterpret_cast<int*>(ws + w.list_off); a.counts = reinterpret_cast<int*>(ws + w.count_off);
+    a.list = reinterpret_cast<int*>(ws + w.list_off); a.seqs = reinterpret_cast<int*>(ws + w.seq_off); a.counts = reinterpret_cast<int*>(ws + w.count_off);
     a.seg_tokens = edit_segment_tokens(shape_total_tokens(s));
     a.n_seg = (shape_total_tokens(s) + a.seg_tokens - 1) / a.seg_tokens;
     a.tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off); a.bh_info = reinterpret_cast<uint8_t*>(ws + w.info_off);
     a.status = reinterpret_cast<int*>(ws); a.u_blocks = u_blocks_of(s);
     a.B = s->batch; a.L = s->max_seqlen; a.Hkv = s->n_kv_heads; a.r = s->rank; a.M = s->n_experts; a.n_tiles = w.n_tiles;
     return a;
+}
+
+template <int D, bool MULTI>
+static seka_status launch_gather_t(const TileArgs& a, const void* P, int T, long long units, int n_sm, cudaStream_t st) {
+    using SL = EgSmem<D, MULTI>;
+    CUtensorMap tk, tt, tp;        // gathered rows, 128 consecutive rows, projectors
+    if (!make_row_map(&tk, a.K, a.Hkv * D, T) || !make_tile_map(&tt, a.K, D, a.Hkv, T)) return SEKA_ERR_CUDA;
+    tp = tt;                       // (not used with one expert)
+    if (MULTI && !make_tile_map(&tp, P, D, 1, (long long)2 * a.M * a.Hkv * D, D)) return SEKA_ERR_CUDA;
+    auto kern = edit_gather_kernel<D, MULTI>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SL::DYN_BYTES) != cudaSuccess) return SEKA_ERR_CUDA;
+    return launch_kernel(true, kern, (unsigned)(units < n_sm ? units : n_sm), SL::THREADS, SL::DYN_BYTES, st, tk, tt, tp, a);
+}
+
+// The gathering kernel instead of the chain.  `units`: (128 tokens, KV head) pairs if every token were highlighted (how many are
+// is known on the device only).  Chain against gathering, us per call in place, 8 heads of 128 unless said otherwise:
+//   one expert, rank of at most 32 (packed chain): 144 x 4096 tokens, 2 % / 10 % / all highlighted 20.7 / 68.5 / 619 against 20.7 / 62 /
+//     546; 64 x 3000 (12000 units) 11.3 / 30 / 204 against 14 / 26 / 183, where the sparse edit would pay 3 us for its larger CTAs;
+//   rank of 33 to 64: 64 x 3000, rank 64, 10 % / all 35 / 245 against 30 / 187; 16 x 4096 (4096 units) 10 % even; 64 x 4096 x 16 of 64,
+//     10 % / all 45 / 371 against 34 / 199;
+//   rank beyond 64 (the chain replaces U in every step): 1 x 4096, rank 128, 10 % 13.7 against 11, 64 x 3000 all 472 against 163;
+//   several experts: a step costs the chain about 130 + 195 and the gathering kernel 150 (all of 64 x 3000) per block of stacked
+//     columns / per expert: four of rank 32 / 64 / 128 523 / 909 / 1682 against 624 / 625 / 592, two of rank 64 516 against 292 (14.5
+//     against 16 on 1 x 4096), eight of rank 64 1691 against 1128; at head_dim 64, where the chain keeps two blocks, four of rank 48 /
+//     64 on 32 x 4096 x 16 545 / 680 against 324, two of rank 64 10 % on 8 x 4096 x 16 15.7 against 17.7.
+static bool gather_edit(const seka_shape* s, long long units, int n_sm) {
+    if (s->n_kv_heads > n_sm || s->n_kv_heads > kMaxGatherHeads) return false;
+    const long long size = units * s->head_dim;
+    if (s->n_experts > 1) return edit_projectors(s) && (s->rank * s->n_experts > 2 * ET_UCOLS || size >= 2048 * 128);
+    return s->rank > 64 || size > (s->rank > 32 ? 4095 : 32768) * 128LL;
 }
 
 static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout& w, const void* K_in, void* K_out, const uint8_t* mask,
@@ -898,11 +1391,18 @@ static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout&
     const size_t n16 = copy ? (size_t)T * Hkv * D / 8 : 0;
     size_t n_copy = (n16 + 4 * 256 - 1) / (4 * 256);
     if (n_copy > (size_t)n_sm * 8) n_copy = (size_t)n_sm * 8;
-    seka_status stc = launch_kernel(true, edit_scan_kernel, (unsigned)(a.n_seg + n_copy), 256, 0, st, mask, gain, s->cu_seqlens, T, s->batch,
-                                    s->max_seqlen, const_cast<int*>(a.list), const_cast<int*>(a.counts), a.seg_tokens, a.n_seg,
-                                    static_cast<const uint4*>(K_in), static_cast<uint4*>(K_out), n16);
-    if (stc != SEKA_OK) return stc;
     const long long units = (long long)((T + 127) / 128) * Hkv;
+    const bool gather = gather_edit(s, units, n_sm) && (s->n_experts == 1 || (reinterpret_cast<uintptr_t>(ws) & 15) == 0);
+    const int n_mats = s->n_experts * Hkv, n_p = gather && s->n_experts > 1 ? n_mats * (D / 32) * (D / 32) : 0;
+    __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + w.w_off);
+    seka_status stc = launch_kernel(true, n_p > 0 ? edit_scan_kernel<true> : edit_scan_kernel<false>, (unsigned)(a.n_seg + n_copy + n_p), PREP_THREADS, 0, st, mask, gain, s->cu_seqlens, T, s->batch,
+                                    s->max_seqlen, const_cast<int*>(a.list), const_cast<int*>(a.seqs), const_cast<int*>(a.counts), a.seg_tokens, a.n_seg,
+                                    static_cast<const uint4*>(K_in), static_cast<uint4*>(K_out), n16, U, P, n_p, n_mats, D, s->rank);
+    if (stc != SEKA_OK) return stc;
+    if (gather) {
+        if (D == 128) return s->n_experts == 1 ? launch_gather_t<128, false>(a, P, T, units, n_sm, st) : launch_gather_t<128, true>(a, P, T, units, n_sm, st);
+        return s->n_experts == 1 ? launch_gather_t<64, false>(a, P, T, units, n_sm, st) : launch_gather_t<64, true>(a, P, T, units, n_sm, st);
+    }
     // (the fused forward's preparation stays unpacked: its launches are a step or two per CTA, and gain nothing)
     if (s->rank * s->n_experts <= ET_UCOLS / 2)
         return D == 128 ? launch_tiles_t<128, false, __nv_bfloat16, true>(a, units, tiles_smem<128, false, true>(s, a.u_blocks, false, 0), 0, st)
@@ -1194,37 +1694,7 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
     pdl_release();
     int blk = blockIdx.x;
     if (blk < n_p) {
-        const int tiles = D / 32;
-        const int h = blk / (tiles * tiles), t = blk % (tiles * tiles);
-        const int i0 = (t / tiles) * 32, j0 = (t % tiles) * 32;
-        __shared__ float ui[32][33], uj[32][33];
-        const int tx = tid & 31, ty = tid >> 5;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        const float* Uh = U + (size_t)h * D * r;
-        for (int k0 = 0; k0 < r; k0 += 32) {
-            __syncthreads();
-            for (int q = ty; q < 32; q += 8) {
-                const bool in = k0 + tx < r;
-                ui[q][tx] = in ? Uh[(size_t)(i0 + q) * r + k0 + tx] : 0.f;
-                uj[q][tx] = in ? Uh[(size_t)(j0 + q) * r + k0 + tx] : 0.f;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = ty + 8 * q;
-#pragma unroll 8
-                for (int k = 0; k < 32; ++k) acc[q] = fmaf(ui[i][k], uj[tx][k], acc[q]);
-            }
-        }
-        // two bf16 parts, P = hi + lo to about 2^-17: the edit keeps fp32-like accuracy on bf16 tensor cores
-        __nv_bfloat16* Phi = P + (size_t)h * D * D;
-        __nv_bfloat16* Plo = P + ((size_t)Hkv + h) * D * D;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const __nv_bfloat16 hi = __float2bfloat16_rn(acc[q]);
-            Phi[(size_t)(i0 + ty + 8 * q) * D + j0 + tx] = hi;
-            Plo[(size_t)(i0 + ty + 8 * q) * D + j0 + tx] = __float2bfloat16_rn(acc[q] - __bfloat162float(hi));
-        }
+        projector_block(U, P, blk, Hkv, D, r);
         return;
     }
     blk -= n_p;

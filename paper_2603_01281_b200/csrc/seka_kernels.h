@@ -42,6 +42,9 @@ seka_status launch_route(const seka_shape* s, const void* Q, const float* U, con
 // bf16 tensor [T, H, d] viewed as (d, H, T) for TMA: tiles of 64 x 1 x box_rows with the 128-byte swizzle.
 bool make_tile_map(CUtensorMap* m, const void* base, int d, int H, long long T, int box_rows = 128);
 
+// bf16 tensor [T, cols] for gathers of four rows x 64 columns at a time, 128-byte swizzle.
+bool make_row_map(CUtensorMap* m, const void* base, int cols, long long T);
+
 seka_status validate_shape(const seka_shape* s);
 
 // Number of SMs of the current device (looked up once per device, thread-safe).
