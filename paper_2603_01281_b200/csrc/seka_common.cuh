@@ -143,7 +143,11 @@ static inline int edit_segment_tokens(long long T) {
 // several whose stand-alone edit takes them instead of the stacked columns (per 64 of these: nb) because that is less work.
 static inline bool edit_projectors(const seka_shape* s) {
     const int nb = (s->rank * s->n_experts + 63) / 64;
-    return s->n_experts == 1 || (nb >= (s->head_dim == 128 ? 2 : 3) && 4 * nb >= 3 * s->n_experts);
+    return s->n_experts == 1 || (nb >= 2 && 4 * nb >= 3 * s->n_experts);
+}
+// ... and those whose pipelined preparation takes several experts: what fits beside the key tiles
+static inline bool pipe_experts(const seka_shape* s) {
+    return s->head_dim == 64 && s->n_experts > 1 && s->n_experts <= 8 && edit_projectors(s);
 }
 
 struct WorkspaceLayout {
@@ -174,7 +178,8 @@ static inline WorkspaceLayout workspace_layout(const seka_shape* s) {
     w.item_off = w.info_off + align_up((size_t)s->batch * s->n_kv_heads + 1, 256);
     w.item_bytes = align_up((size_t)sc.n_items_max * 32 + 32, 256);
     w.list_off = w.item_off + w.item_bytes;
-    const size_t n_alpha = s->n_experts == 1 ? (size_t)s->batch * s->n_kv_heads : 0;       // (one expert: routed coefficients may live here)
+    // (routed coefficients may live here)
+    const size_t n_alpha = s->n_experts == 1 || pipe_experts(s) ? (size_t)s->batch * s->n_kv_heads * s->n_experts : 0;
     w.list_bytes = align_up((T > n_alpha ? T : n_alpha) * 4 + 4, 256);
     w.seq_off = w.list_off + w.list_bytes;
     w.count_off = w.seq_off + align_up(T * 4 + 4, 256);

@@ -1377,7 +1377,7 @@ static seka_status launch_gather_t(const TileArgs& a, const void* P, int T, long
 static bool gather_edit(const seka_shape* s, long long units, int n_sm) {
     if (s->n_kv_heads > n_sm || s->n_kv_heads > kMaxGatherHeads) return false;
     const long long size = units * s->head_dim;
-    if (s->n_experts > 1) return edit_projectors(s) && (s->rank * s->n_experts > 2 * ET_UCOLS || size >= 2048 * 128);
+    if (s->n_experts > 1) return edit_projectors(s) && (s->rank * s->n_experts > 2 * ET_UCOLS || (s->head_dim == 128 && size >= 2048 * 128));
     return s->rank > 64 || size > (s->rank > 32 ? 4095 : 32768) * 128LL;
 }
 
@@ -1411,7 +1411,7 @@ static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout&
                     : launch_tiles_t<64, false, __nv_bfloat16>(a, units, tiles_smem<64, false>(s, a.u_blocks, false, 0), 0, st);
 }
 
-// ---------------------------------------------------------------- many tiles, one projector: the preparation as a pipeline
+// ---------------------------------------------------------------- many tiles, few projectors: the preparation as a pipeline
 //
 // Where the tiles of a plain-SEKA forward are many waves of CTAs, the chain above is bound by its instruction latencies
 // (about 5000 cycles per tile and SM at head_dim 64).  There one persistent CTA per SM with three roles does the same work from
@@ -1428,19 +1428,22 @@ static seka_status launch_edit_tiles(const seka_shape* s, const WorkspaceLayout&
 constexpr int EP_THREADS = 320;
 
 // per stage: highlighted rows, first token, rows inside the sequence, end marker, low parts wanted, g * alpha
-struct __align__(16) EpMeta { uint32_t bits[4]; int tok0, nvalid, valid, with_lo; float c; int pad[3]; };
+// (several experts: the gain alone, and the sequence)
+struct __align__(16) EpMeta { uint32_t bits[4]; int tok0, nvalid, valid, with_lo; float c; int b, pad[2]; };
 
-template <int D>
+// NP: most projectors (experts).  Several of them (head_dim 64) leave room for one CTA per SM.
+template <int D, int NP>
 struct EpSmem {
     static constexpr uint32_t TILE = (D / 64) * EBLK;
     static constexpr uint32_t PBLK = D * 128;
     static constexpr uint32_t PMAT = (D / 64) * PBLK;
-    static constexpr int NS = D == 128 ? 4 : 3;             // stages of key tiles
-    static constexpr int CTAS = D == 128 ? 1 : 2;           // per SM (the projector of 128 leaves room for one)
+    static constexpr int NS = D == 128 ? 4 : NP == 4 ? 6 : 3;       // stages of key tiles
+    static constexpr int CTAS = D == 128 || NP > 1 ? 1 : 2; // per SM (the projector of 128 leaves room for one)
+    static constexpr int CS = NP * D > 256 ? 1 : 2;         // sets of tensor-memory columns (NP products each)
     static constexpr uint32_t K = 0;                        // NS stages
-    static constexpr uint32_t P = K + NS * TILE;            // high part, then low part
+    static constexpr uint32_t P = K + NS * TILE;            // high part, then low part of each
     static constexpr bool LOW = D == 64;                    // the low parts go out through shared memory (two tiles), as whole rows
-    static constexpr uint32_t L = P + 2 * PMAT;
+    static constexpr uint32_t L = P + NP * 2 * PMAT;
     static constexpr uint32_t META = L + (LOW ? 2 * TILE : 0);        // NS x 48 bytes
     static constexpr uint32_t BARS = META + NS * 48;        // full[NS], free[NS], mma_done[2], cols_free[2], p_full, meet[2]
     static constexpr uint32_t NBARS = 2 * NS + 7;
@@ -1448,22 +1451,23 @@ struct EpSmem {
     static constexpr uint32_t DYN_BYTES = MISC + 16 + 1024;
 };
 
-template <int D>
-__global__ void __launch_bounds__(EP_THREADS, EpSmem<D>::CTAS)
+template <int D, int NP>
+__global__ void __launch_bounds__(EP_THREADS, EpSmem<D, NP>::CTAS)
 stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmP, __nv_bfloat16* __restrict__ X,
                        const uint8_t* __restrict__ mask, const float* __restrict__ alpha, const float* __restrict__ gain,
                        const uint8_t* __restrict__ head_enable, const int* __restrict__ cu_seqlens,
-                       const uint8_t* __restrict__ tile_hot, int* status, int B, int L, int Hkv, int n_tiles, int routed) {
-    using SL = EpSmem<D>;
-    constexpr int EP_NS = SL::NS;
+                       const uint8_t* __restrict__ tile_hot, int* status, int B, int L, int Hkv, int n_tiles, int routed, int n_experts) {
+    using SL = EpSmem<D, NP>;
+    constexpr int EP_NS = SL::NS, CS = SL::CS;
     constexpr int NBLK = D / 64;
-    constexpr uint32_t TMEM_COLS = 2 * D < 32 ? 32 : 2 * D;
+    constexpr uint32_t TMEM_COLS = CS * NP * D;
+    const int M = NP == 1 ? 1 : n_experts;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SL::BARS);
     uint64_t* full = bars;                     // [NS]  tile landed (TMA bytes) and flags / coordinates written (producer)
     uint64_t* freeb = full + EP_NS;            // [NS]  8 drain-warp arrivals: the stage may be refilled
-    uint64_t* mma_done = freeb + EP_NS;        // [2]   K P of a tile is in column set c
+    uint64_t* mma_done = freeb + EP_NS;        // [2]   K P of a tile (of every expert) is in column set c
     uint64_t* cols_free = mma_done + 2;        // [2]   8 drain-warp arrivals: column set c has been read
     uint64_t* p_full = cols_free + 2;          // [1]   projector landed
     uint64_t* meetb = p_full + 1;              // [2]   8 drain-warp arrivals: all rows of the tile are updated
@@ -1500,15 +1504,16 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         bool ok = true;
         const bool on = head_enable == nullptr || head_enable[h] != 0;
         if (lane == 0 && on) {
-            mbar_expect_tx(p_full, 2 * SL::PMAT);
+            mbar_expect_tx(p_full, M * 2 * SL::PMAT);
+            for (int m = 0; m < M; ++m)
 #pragma unroll
-            for (int part = 0; part < 2; ++part)
+                for (int part = 0; part < 2; ++part)
 #pragma unroll
-                for (int cb = 0; cb < NBLK; ++cb)
-                    tma_load_3d(smem + SL::P + part * SL::PMAT + cb * SL::PBLK, &tmP, p_full, cb * 64, 0, (part * Hkv + h) * D);
+                    for (int cb = 0; cb < NBLK; ++cb)
+                        tma_load_3d(smem + SL::P + (m * 2 + part) * SL::PMAT + cb * SL::PBLK, &tmP, p_full, cb * 64, 0, ((part * M + m) * Hkv + h) * D);
         }
         __syncwarp();
-        auto push = [&](bool last, int tok0, int nvalid, int with_lo, float c, const uint32_t (&bits)[4]) {
+        auto push = [&](bool last, int tok0, int nvalid, int with_lo, float c, int b, const uint32_t (&bits)[4]) {
             const uint32_t s = n_push % EP_NS;
             if (n_push >= EP_NS) {
                 ok = warp_wait(freeb + s, ((n_push / EP_NS) - 1) & 1, abort_flag, status, 63);
@@ -1516,7 +1521,7 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
             }
             if (lane == 0) {
                 EpMeta* m = reinterpret_cast<EpMeta*>(smem + SL::META + s * 48);
-                m->tok0 = tok0; m->valid = last ? 0 : 1; m->c = c; m->nvalid = nvalid; m->with_lo = with_lo;
+                m->tok0 = tok0; m->valid = last ? 0 : 1; m->c = c; m->nvalid = nvalid; m->with_lo = with_lo; m->b = b;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) m->bits[q] = bits[q];
                 if (!last) {
@@ -1533,15 +1538,16 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         };
         for (long long base = (int)blockIdx.x / Hkv; base < n_bt && ok && on; base += 32LL * bt_step) {
             const long long my = base + (long long)lane * bt_step;
-            int tok0_l = 0, nv_l = 0, lo_l = 0, hot_l = 0;
+            int tok0_l = 0, nv_l = 0, lo_l = 0, hot_l = 0, b_l = 0;
             float c_l = 0.f;
             if (my < n_bt) {
                 const int bt = (int)my, b = bt / n_tiles, t = bt - b * n_tiles;
                 const int seq0 = cu_seqlens ? cu_seqlens[b] : b * L;
                 const int Lb = (cu_seqlens ? cu_seqlens[b + 1] : (b + 1) * L) - seq0;
-                const float g = gain[b], a = alpha != nullptr ? alpha[(size_t)b * Hkv + h] : 1.f;
+                const float g = gain[b], a = NP > 1 ? alpha_max_of(alpha, (size_t)b * Hkv + h, M) : alpha != nullptr ? alpha[(size_t)b * Hkv + h] : 1.f;
                 hot_l = (tile_hot[bt] != 0 && g != 0.f) ? 1 : 0;
-                c_l = g * a;
+                b_l = b;
+                c_l = NP > 1 ? g : g * a;
                 tok0_l = seq0 + t * 128; nv_l = Lb - t * 128 < 128 ? Lb - t * 128 : 128;
                 lo_l = (lo_needed(g, routed ? 1.f : fabsf(a)) || t < kLoTiles) ? 1 : 0;        // (as in steer_byte)
             }
@@ -1562,10 +1568,10 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 #pragma unroll
                 for (int q = 0; q < 4; ++q) { bits[q] = __ballot_sync(0xffffffffu, fl[q] != 0); fl[q] = fl_next[q]; }
                 push(false, __shfl_sync(0xffffffffu, tok0_l, k), __shfl_sync(0xffffffffu, nv_l, k), __shfl_sync(0xffffffffu, lo_l, k),
-                     __shfl_sync(0xffffffffu, c_l, k), bits);
+                     __shfl_sync(0xffffffffu, c_l, k), __shfl_sync(0xffffffffu, b_l, k), bits);
             }
         }
-        if (ok) { const uint32_t none[4] = {0, 0, 0, 0}; push(true, 0, 0, 0, 0.f, none); }      // the end marker
+        if (ok) { const uint32_t none[4] = {0, 0, 0, 0}; push(true, 0, 0, 0, 0.f, 0, none); }      // the end marker
         if (on) warp_wait(p_full, 0, abort_flag, status, 62);      // (a CTA without work leaves only when the projector has landed)
     } else if (warp == 9) {
         // ------------------------------------------------------------ MMA issuer
@@ -1574,7 +1580,7 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         const uint32_t dK = umma_desc_lo(smem_u32(smem + SL::K), 16), dP = umma_desc_lo(smem_u32(smem + SL::P), 16);
         bool ok = true;
         for (uint32_t n = 0; ok; ++n) {
-            const uint32_t s = n % EP_NS, cset = n & 1;
+            const uint32_t s = n % EP_NS, cset = n % CS;
             ok = warp_wait(full + s, (n / EP_NS) & 1, abort_flag, status, 64);
             if (!ok) break;
             const EpMeta m = *reinterpret_cast<const EpMeta*>(smem + SL::META + s * 48);
@@ -1583,21 +1589,23 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
                 ok = warp_wait(p_full, 0, abort_flag, status, 65);
                 if (!ok) break;
             }
-            if (n >= 2) {
-                ok = warp_wait(cols_free + cset, ((n >> 1) - 1) & 1, abort_flag, status, 66);
+            if (n >= CS) {
+                ok = warp_wait(cols_free + cset, ((n / CS) - 1) & 1, abort_flag, status, 66);
                 if (!ok) break;
             }
             tc_fence_after();
             if (lane == 0) {
                 const uint32_t kd = dK + s * (SL::TILE >> 4);
+#pragma unroll 1
+                for (int m = 0; m < M; ++m)
 #pragma unroll
-                for (int part = 0; part < 2; ++part)
+                    for (int part = 0; part < 2; ++part)
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) {
-                        const uint32_t offk = ((uint32_t)(ks >> 2) * EBLK + (uint32_t)(ks & 3) * 32) >> 4;
-                        const uint32_t offp = ((uint32_t)part * SL::PMAT + (uint32_t)(ks >> 2) * SL::PBLK + (uint32_t)(ks & 3) * 32) >> 4;
-                        umma_ss(tmem_base + cset * D, kd + offk, DESC_HI, dP + offp, DESC_HI, IDESC, (ks > 0 || part) ? 1u : 0u);
-                    }
+                        for (int ks = 0; ks < D / 16; ++ks) {
+                            const uint32_t offk = ((uint32_t)(ks >> 2) * EBLK + (uint32_t)(ks & 3) * 32) >> 4;
+                            const uint32_t offp = ((uint32_t)part * SL::PMAT + (uint32_t)(ks >> 2) * SL::PBLK + (uint32_t)(ks & 3) * 32) >> 4;
+                            umma_ss(tmem_base + (cset * NP + m) * D, kd + offk, DESC_HI, dP + m * (2 * SL::PMAT >> 4) + offp, DESC_HI, IDESC, (ks > 0 || part) ? 1u : 0u);
+                        }
                 umma_commit(mma_done + cset);
             }
             __syncwarp();
@@ -1608,7 +1616,7 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         bool ok = true;
         for (uint32_t n = 0; ok; ++n) {
-            const uint32_t s = n % EP_NS, cset = n & 1;
+            const uint32_t s = n % EP_NS, cset = n % CS, lset = n & 1;
             ok = warp_wait(full + s, (n / EP_NS) & 1, abort_flag, status, 67);
             if (!ok) break;
             const EpMeta m = *reinterpret_cast<const EpMeta*>(smem + SL::META + s * 48);
@@ -1616,7 +1624,7 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
             uint8_t* sK = smem + SL::K + s * SL::TILE;
             const uint32_t hl_bits = reinterpret_cast<const EpMeta*>(smem + SL::META + s * 48)->bits[warp & 3];
             const bool hl = ((hl_bits >> lane) & 1u) != 0, warp_hl = hl_bits != 0, with_lo = m.with_lo != 0;
-            ok = warp_wait(mma_done + cset, (n >> 1) & 1, abort_flag, status, 68);
+            ok = warp_wait(mma_done + cset, (n / CS) & 1, abort_flag, status, 68);
             if (!ok) break;
             tc_fence_after();
             const bool side_lo = with_lo && row < m.nvalid;
@@ -1625,7 +1633,20 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 #pragma unroll 1
                 for (int c = half * (D / 64); c < (half + 1) * (D / 64); ++c) {
                     uint32_t v[32];
-                    if (warp_hl) { tmem_ld32(t_lane + cset * D + c * 32, v); tmem_wait_ld_on(v); }     // warp-wide: every lane takes part
+                    float acc[NP > 1 ? 32 : 1];
+                    if constexpr (NP == 1) {
+                        if (warp_hl) { tmem_ld32(t_lane + cset * D + c * 32, v); tmem_wait_ld_on(v); }     // warp-wide: every lane takes part
+                    } else if (warp_hl) {               // sum_m c_m K P_m
+                        const float* al = alpha != nullptr ? alpha + ((size_t)m.b * Hkv + h) * M : nullptr;
+#pragma unroll 1
+                        for (int e = 0; e < M; ++e) {
+                            const float cm = m.c * (al != nullptr ? al[e] : 1.f);
+                            tmem_ld32(t_lane + (cset * NP + e) * D + c * 32, v);
+                            tmem_wait_ld_on(v);
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) acc[k] = fmaf(cm, __uint_as_float(v[k]), e == 0 ? 0.f : acc[k]);
+                        }
+                    }
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {          // 8 elements = one 16-byte unit of the swizzled row
                         const int col = c * 32 + q * 8;
@@ -1637,12 +1658,13 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 const float2 k2 = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[e]));
-                                split_pair(fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e]), k2.x), fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e + 1]), k2.y), w[e], lo[e]);
+                                if constexpr (NP == 1) split_pair(fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e]), k2.x), fmaf(m.c, __uint_as_float(v[q * 8 + 2 * e + 1]), k2.y), w[e], lo[e]);
+                                else split_pair(k2.x + acc[q * 8 + 2 * e], k2.y + acc[q * 8 + 2 * e + 1], w[e], lo[e]);
                             }
                             *ptr = kv;
                         }
                         if (SL::LOW) {          // (the tile before last is out: its writers have met since)
-                            if (with_lo) *reinterpret_cast<uint4*>(smem + SL::L + cset * SL::TILE + (col >> 6) * EBLK + sw128_offset(row, col & 63)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                            if (with_lo) *reinterpret_cast<uint4*>(smem + SL::L + lset * SL::TILE + (col >> 6) * EBLK + sw128_offset(row, col & 63)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                         } else if (side_lo) {
                             *reinterpret_cast<uint4*>(xlo + col) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                         }
@@ -1653,8 +1675,8 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
             // the columns are read: the next product may use them; all rows updated: the tile may be written out
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) { mbar_arrive(cols_free + cset); mbar_arrive(meetb + cset); }
-            ok = warp_wait(meetb + cset, (n >> 1) & 1, abort_flag, status, 69);
+            if (lane == 0) { mbar_arrive(cols_free + cset); mbar_arrive(meetb + lset); }
+            ok = warp_wait(meetb + lset, (n >> 1) & 1, abort_flag, status, 69);
             if (!ok) break;
             constexpr int LPR = D / 8, RPI = 32 / LPR;
 #pragma unroll 1
@@ -1664,7 +1686,7 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
                     const uint4 v = *reinterpret_cast<const uint4*>(sK + (col >> 6) * EBLK + sw128_offset(r, col & 63));
                     __nv_bfloat16* dst = X + ((size_t)(m.tok0 + r) * Hkv + h) * (2 * D) + col;
                     *reinterpret_cast<uint4*>(dst) = v;
-                    if (SL::LOW && with_lo) *reinterpret_cast<uint4*>(dst + D) = *reinterpret_cast<const uint4*>(smem + SL::L + cset * SL::TILE + (col >> 6) * EBLK + sw128_offset(r, col & 63));
+                    if (SL::LOW && with_lo) *reinterpret_cast<uint4*>(dst + D) = *reinterpret_cast<const uint4*>(smem + SL::L + lset * SL::TILE + (col >> 6) * EBLK + sw128_offset(r, col & 63));
                 }
             }
             __syncwarp();
@@ -1681,12 +1703,12 @@ stage_keys_pipe_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
 
 // First launch of that path: blocks [0, n_p) form a 32 x 32 tile of P[h] each (bf16, high parts of all heads, then low parts);
 // then blocks with a warp per (sequence, key tile) for the tile flags and the steering bytes; then, in a routed call, a block
-// per (sequence, KV head) that leaves its coefficient (Eq. 6, the routine of adaseka_route: the same bits) for the launch
+// per (sequence, KV head) that leaves its coefficients (Eq. 6, the routine of adaseka_route: the same bits) for the launch
 // behind; then the item table and the conversion of fp32 inputs (11 ragged sequences of up to 11083 tokens of 8 heads of 64, nearly all
 // highlighted: 107 us for both launches, 232 for the chain with its conversion blocks).
 __global__ void __launch_bounds__(PREP_THREADS)
 prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ mask, __nv_bfloat16* __restrict__ P,
-                      uint8_t* __restrict__ tile_hot, uint8_t* __restrict__ bh_info, int B, int L, int Hkv, int D, int r, int n_tiles,
+                      uint8_t* __restrict__ tile_hot, uint8_t* __restrict__ bh_info, int B, int L, int Hkv, int D, int r, int M, int n_tiles,
                       int n_p, int n_flag, int n_route, const __grid_constant__ RouteArgs route, const __grid_constant__ PrepJobs jobs) {
     extern __shared__ __align__(16) double route_sm[];
     const int tid = threadIdx.x;
@@ -1694,7 +1716,7 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
     pdl_release();
     int blk = blockIdx.x;
     if (blk < n_p) {
-        projector_block(U, P, blk, Hkv, D, r);
+        projector_block(U, P, blk, M * Hkv, D, r);
         return;
     }
     blk -= n_p;
@@ -1718,9 +1740,9 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
     }
     blk -= n_flag;
     if (blk < n_route) {
-        const double* a = route_group(route.Q, route.q_is_f32, U, route.sigma, jobs.cu, L, route.Hq, Hkv, D, r, 1, route.k_route, blk / Hkv,
+        const double* a = route_group(route.Q, route.q_is_f32, U, route.sigma, jobs.cu, L, route.Hq, Hkv, D, r, M, route.k_route, blk / Hkv,
                                       blk % Hkv, route_sm);
-        if (tid == 0) route.alpha_out[blk] = (float)a[0];
+        for (int m = tid; m < M; m += PREP_THREADS) route.alpha_out[(size_t)blk * M + m] = (float)a[m];
         return;
     }
     blk -= n_route;
@@ -1728,11 +1750,11 @@ prep_projector_kernel(const float* __restrict__ U, const uint8_t* __restrict__ m
     else convert_block(jobs.conv, blk - jobs.n_items_blocks, jobs.n_conv_blocks);
 }
 
-template <int D>
+template <int D, int NP>
 static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
                                      const float* alpha, const float* gain, const uint8_t* he, char* ws, const PrepJobs& jobs,
                                      const RouteArgs& route_in, cudaStream_t st) {
-    using PL = EpSmem<D>;
+    using PL = EpSmem<D, NP>;
     const int T = shape_total_tokens(s), Hkv = s->n_kv_heads;
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
@@ -1740,41 +1762,51 @@ static seka_status launch_stage_pipe(const seka_shape* s, const WorkspaceLayout&
     uint8_t* tile_hot = reinterpret_cast<uint8_t*>(ws + w.hot_off);
     CUtensorMap tk, tp;
     const void* k16 = s->dtype == SEKA_F32 ? static_cast<const void*>(jobs.conv.out[1]) : K;       // (converted by the first launch)
-    if (!make_tile_map(&tk, k16, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * Hkv * D, D)) return SEKA_ERR_CUDA;
-    const int n_p = Hkv * (D / 32) * (D / 32), n_flag = (s->batch * w.n_tiles + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
+    if (!make_tile_map(&tk, k16, D, Hkv, T) || !make_tile_map(&tp, P, D, 1, (long long)2 * s->n_experts * Hkv * D, D)) return SEKA_ERR_CUDA;
+    const int n_p = s->n_experts * Hkv * (D / 32) * (D / 32), n_flag = (s->batch * w.n_tiles + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
     RouteArgs route = route_in;
     const int n_route = route.sigma != nullptr ? s->batch * Hkv : 0;
     if (n_route > 0) {          // without a place of the caller's the coefficients live in the list region, which has room for them
         if (route.alpha_out == nullptr) route.alpha_out = reinterpret_cast<float*>(ws + w.list_off);
         alpha = route.alpha_out;
     }
+    const size_t route_smem = n_route > 0 ? route_smem_bytes(D, s->n_experts, route.k_route) : 0;       // (at most 34 KB, on top of 19 of its own)
+    if (route_smem > 24 * 1024 &&
+        cudaFuncSetAttribute(prep_projector_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)route_smem) != cudaSuccess) return SEKA_ERR_CUDA;
     seka_status stc = launch_kernel(true, prep_projector_kernel, (unsigned)(n_p + n_flag + n_route + jobs.n_items_blocks + jobs.n_conv_blocks), PREP_THREADS,
-                                    n_route > 0 ? route_smem_bytes(D, 1, route.k_route) : 0, st, U, mask,
+                                    route_smem, st, U, mask,
                                     static_cast<__nv_bfloat16*>(P), tile_hot, reinterpret_cast<uint8_t*>(ws + w.info_off), s->batch,
-                                    s->max_seqlen, Hkv, D, s->rank, w.n_tiles, n_p, n_flag, n_route, route, jobs);
+                                    s->max_seqlen, Hkv, D, s->rank, s->n_experts, w.n_tiles, n_p, n_flag, n_route, route, jobs);
     if (stc != SEKA_OK) return stc;
-    auto kern = stage_keys_pipe_kernel<D>;
+    auto kern = stage_keys_pipe_kernel<D, NP>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::DYN_BYTES) != cudaSuccess) return SEKA_ERR_CUDA;
     const unsigned grid = (unsigned)(PL::CTAS * n_sm / Hkv * Hkv);
     return launch_kernel(true, kern, grid, EP_THREADS, PL::DYN_BYTES, st, tk, tp, reinterpret_cast<__nv_bfloat16*>(ws + w.x_off), mask, alpha,
-                         gain, he, s->cu_seqlens, tile_hot, reinterpret_cast<int*>(ws), s->batch, s->max_seqlen, Hkv, w.n_tiles, n_route > 0 ? 1 : 0);
+                         gain, he, s->cu_seqlens, tile_hot, reinterpret_cast<int*>(ws), s->batch, s->max_seqlen, Hkv, w.n_tiles, n_route > 0 ? 1 : 0, s->n_experts);
 }
 
 seka_status launch_stage_keys(const seka_shape* s, const WorkspaceLayout& w, const void* K, const uint8_t* mask, const float* U,
                               const float* alpha, const float* gain, const uint8_t* head_enable, char* ws, const PrepJobs& jobs,
                               const RouteArgs& route, cudaStream_t st) {
-    // The pipelined pair of launches from four waves of the chain on.  Measured preparations, pipeline against chain: packed
+    // One expert: the pipelined pair of launches from four waves of the chain on.  Measured preparations, pipeline against chain: packed
     // batch of 64 sequences, 16 heads of 64, short runs (16384 units) 84 against 132 us; 64 x 1024 tokens, 4 heads of 64 /
     // 128, all highlighted (2048 units) 26 against 36 / 50 against 56; 46 x 500, 8 heads of 64, 44 % (1472 units) 29 against
     // 30, 12 x 500 (384 units) 15 against 13; 4 x 4096 tokens, 8 heads of 128, a tenth (1024 units) 18 against 16; 4362 tokens, 8 heads (280) 19 against 13.
+    // Several experts at head_dim 64 (up to the eight whose projectors fit, where they are less work than the stacked columns): from four
+    // tiles per SM on.  Calls of the fused forward, pipeline against chain: four of rank 64 on 64 packed sequences of up to 2048 tokens of
+    // 16 heads 760 against 1015 us, 16 x 1024 x 16 130 against 167, 8 x 2048 x 8 (1024 units) 102 against 119, 51 x 423 x 4 57 against 76;
+    // two of rank 48 on 64 x 512 x 16 218 against 259.
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     const long long units = (long long)s->batch * w.n_tiles * s->n_kv_heads;
     if (units > 0x7fffffffLL) return SEKA_ERR_UNSUPPORTED;
     const int chain_ctas = s->head_dim == 128 ? EtSmem<128, true>::CTAS : EtSmem<64, true>::CTAS;
     if (s->n_experts == 1 && s->n_kv_heads <= n_sm && units > 4LL * chain_ctas * n_sm)     // (routed or not: both forms give the same bits)
-        return s->head_dim == 128 ? launch_stage_pipe<128>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st)
-                                  : launch_stage_pipe<64>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st);
+        return s->head_dim == 128 ? launch_stage_pipe<128, 1>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st)
+                                  : launch_stage_pipe<64, 1>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st);
+    if (pipe_experts(s) && s->n_kv_heads <= n_sm && units > 4LL * n_sm)
+        return s->n_experts <= 4 ? launch_stage_pipe<64, 4>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st)
+                                 : launch_stage_pipe<64, 8>(s, w, K, mask, U, alpha, gain, head_enable, ws, jobs, route, st);
     TileArgs a = tile_args(s, w, K, ws + w.x_off, mask, U, alpha, gain, head_enable, ws);
     a.route = route; a.jobs = jobs;
     const size_t n_alpha = (size_t)s->batch * s->n_kv_heads * s->n_experts;

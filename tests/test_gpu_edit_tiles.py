@@ -126,3 +126,37 @@ def test_one_routed_expert_on_both_sides_of_the_rule(d, lens, dtype):
         assert binding.seka_poll_status(ws) == binding.SEKA_OK
         assert out is None or torch.equal(out, alpha)
         assert torch.equal(O.view(bits), ref.view(bits))
+
+
+@pytest.mark.parametrize("seqs,experts,rank,k_route,dtype,varlen", [
+    (37, 4, 64, 64, "bf16", False), (38, 4, 64, 16, "bf16", False),            # 592 | 608 tiles: chain | pipeline
+    (60, 2, 64, 64, "bf16", True), (45, 3, 57, 57, "bf16", False), (40, 5, 64, 3, "bf16", True), (70, 8, 64, 64, "bf16", False),
+    (38, 8, 48, 48, "f32", True)])
+def test_preparation_with_several_projectors(seqs, experts, rank, k_route, dtype, varlen):
+    """Banks at head_dim 64 on both sides of the line between the chain and the pipelined preparation: the oracle's rows, and one call
+    with routing gives the bits of the coefficients of adaseka_route given by hand."""
+    lens = [512 if i == 0 or not varlen else 385 + (53 * i) % 127 for i in range(seqs)]
+    w = inputs.make_custom(seed=96, dtype=dtype, lens=lens, n_q_heads=4, n_kv_heads=4, head_dim=64, rank=rank, n_experts=experts,
+                           mask_kind="runs", highlight=0.15, gain=[(0.5, 2.0, 0.0, -1.0)[i % 4] for i in range(seqs)])
+    w.Q, w.K, w.V = (inputs.round_to_bf16(x) for x in (w.Q, w.K, w.V))      # (fp32 inputs are rounded on the way in)
+    dev = H.device_tensors(w)
+    shp = H.shape_of(w, dev, force_varlen=varlen)
+    he = torch.tensor([1, 1, 0, 1], dtype=torch.uint8, device="cuda")
+    sigma = torch.rand((experts, 4, rank), generator=torch.Generator().manual_seed(1)).cuda() + 0.5
+    alpha = torch.empty((seqs, 4, experts), dtype=torch.float32, device="cuda")
+    binding.adaseka_route(shp, dev["Q"], dev["U"], sigma, k_route, alpha)
+    ref = torch.full_like(dev["Q"], float("nan"))
+    ws = binding.new_workspace(shp)
+    binding.seka_attention_fwd(shp, dev["Q"], dev["K"], dev["V"], ref, None, dev["mask"], dev["U"], alpha, dev["gain"], he, ws)
+    assert binding.seka_poll_status(ws) == binding.SEKA_OK
+    rows = H.sampled_rows(w, 4, seed=1)
+    Oref, _, idx = H.oracle_rows(w, rows, alpha=alpha.cpu().numpy(), head_enable=he.cpu().numpy())
+    H.check_attention(ref.double().cpu().numpy()[idx], Oref, "%d experts of rank %d" % (experts, rank))
+    bits = torch.int16 if dtype == "bf16" else torch.int32
+    for out in (torch.full_like(alpha, float("nan")), None):
+        O = torch.full_like(ref, float("nan"))
+        ws = binding.new_workspace(shp)
+        binding.seka_attention_fwd_routed(shp, dev["Q"], dev["K"], dev["V"], O, None, dev["mask"], dev["U"], sigma, k_route, out, dev["gain"], he, ws)
+        assert binding.seka_poll_status(ws) == binding.SEKA_OK
+        assert out is None or torch.equal(out, alpha)
+        assert torch.equal(O.view(bits), ref.view(bits))
