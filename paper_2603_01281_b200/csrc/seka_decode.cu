@@ -248,6 +248,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constan
                 mma_16816(o[2 * jp], pa, b0, b1);
                 mma_16816(o[2 * jp + 1], pa, b2, b3);
             }
+            fence_proxy_async();            // the reads of this stage come before the copies that refill it
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[s]);
         }
