@@ -26,8 +26,8 @@
 // item's first key tile travels with this item's last value tile, its Q tiles follow the last score products, and the
 // first scores of a tile's next item are issued right behind its last P V, under the store of its output (before, every
 // item began with an empty tensor pipe and its operands on the way, about 8000 cycles).  Measured on 32 / 8 heads of 128:
-// 4 x 4096 tokens 0.495 -> 0.466 ms, one prompt of 4362 tokens 148 -> 139 us, 28 / 4 heads 1 x 32768 5.93 -> 5.69 ms
-// (unsteered, GPU rested between blocks).
+// 4 x 4096 tokens 0.495 -> 0.466 ms, one prompt of 4362 tokens 148 -> 139 us (unsteered, GPU rested between blocks); 1 x 32768
+// level.  About 2 us per item remain beside its steps.
 // Every wait is bounded: a wait that runs out raises the CTA's abort flag, every role leaves its loop, and the status word
 // reports it.
 #include <math.h>
@@ -184,8 +184,8 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     uint64_t* kv_free = kv_full + NK;        // [NK]  one event per step: the tensor core is done with K(g+1) and V(g)
     uint64_t* x_full = kv_free + NK;         // [3]   low parts of an edited tile landed
     uint64_t* s_full = x_full + G::NXMAX;    // [2]   scores of tile x are in tensor memory
-    uint64_t* p_full = s_full + 2;           // [2]   4 softmax-warp arrivals (O_x rescaled, keys 0-95 of P_x written) + 1 from the relay
-    uint64_t* p_last = p_full + 2;           // [2]   4 softmax-warp arrivals: keys 96-127 of P_x written
+    uint64_t* p_full = s_full + 2;           // [2]   4 softmax-warp arrivals (O_x rescaled, the first 16 KP1 keys of P_x written) + 1 from the relay
+    uint64_t* p_last = p_full + 2;           // [2]   4 softmax-warp arrivals: the other keys of P_x written
     uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished
     uint64_t* o_drained = o_full + 2;        // [2]   4 softmax-warp arrivals: O_x of the item has been read
     uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles of the item landed

@@ -22,7 +22,7 @@ constexpr int DEC_STAGE_KEYS = 64;
 constexpr int DEC_CONSUMERS = 4;                       // warps; each owns 16 tokens of a stage
 constexpr int DEC_THREADS = (DEC_CONSUMERS + 1) * 32;  // + one producer warp
 constexpr int DEC_MAX_GROUP = 16;                      // query heads per KV head (rows of one MMA)
-constexpr int DEC_SM_COUNT = 148;                      // used for sizing the split only
+constexpr int DEC_SM_COUNT = 148;                      // sizing of the split, and the line between its two forms
 constexpr int DEC_MAX_CLUSTER = 8;                     // chunks of a (sequence, KV head) that merge in a cluster
 
 template <int D>

@@ -2,9 +2,7 @@
 
 A serving process that gave all of its memory to a KV-cache pool at start-up, or a plug-in running
 inside someone else's stream callback, has no buffer to offer as workspace and may not call
-cudaMalloc.  The variant keeps its scratch (the list of highlighted tokens) in a fixed array
-inside the library.  It must give what seka_edit_keys gives, on a first call and on a second call
-that finds the previous call's contents in the array.  Collected last on purpose (file name), so a
+cudaMalloc.  The variant needs no scratch and keeps no state.  It must give what seka_edit_keys gives.  Collected last on purpose (file name), so a
 run that stops at the first failure has already run every other test.
 """
 import ctypes
@@ -34,8 +32,7 @@ def _both(w):
 
 def test_static_scratch_edit_matches_workspace_edit_twice():
     assert torch.cuda.is_available()
-    # first call: many highlighted tokens; second call: fewer and elsewhere, so a stale list or a
-    # counter that was not cleared would edit the wrong rows
+    # many highlighted tokens, then fewer and elsewhere
     w1 = inputs.make_custom(seed=31, dtype="bf16", lens=[700, 300], n_q_heads=4, n_kv_heads=2, head_dim=128, rank=32,
                             gain=1.0, mask_kind="runs", highlight=0.6)
     w2 = inputs.make_custom(seed=32, dtype="bf16", lens=[500, 450], n_q_heads=4, n_kv_heads=2, head_dim=128, rank=32,
