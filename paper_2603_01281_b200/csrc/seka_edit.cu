@@ -1286,6 +1286,7 @@ edit_gather_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
             const uint32_t rd = (uint32_t)(col0 >> 6) * EBLK + sw128_offset((warp & 3) * 32 + (lane >> 2), (col0 & 63) + (lane & 3) * 8);
 #pragma unroll
             for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4*>(sK + rd + k * 1024);
+            fence_proxy_async();            // (these reads come before the copies that refill the stage)
             __syncwarp();
             if (lane == 0) mbar_arrive(freeb + s);
 #pragma unroll

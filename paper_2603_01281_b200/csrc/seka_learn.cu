@@ -233,6 +233,7 @@ learn_cov_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant_
                     }
                     ++count;
                 }
+                fence_proxy_async();            // (the reads of this stage come before the copies that refill it)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + s);
                 ++n_pop;
