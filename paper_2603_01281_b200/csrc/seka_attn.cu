@@ -290,7 +290,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         return true;
     };
 
-    if (tid == 0) *abort_flag = 0;
+    if (tid == 0) { *abort_flag = 0; *reinterpret_cast<volatile float*>(smem + sl.misc + 8) = p.scale_log2; }
     // steering info into shared memory
     if (info_local)
         for (int i = tid; i < p.sched.B * p.sched.Hkv; i += NTHREADS) info_bh[i] = p.bh_info[i];
@@ -724,6 +724,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         tmem_st32(tO + c * 32, o);
                     }
                 }
+                float2 sc_piece = sc2;
                 const float2 nm2 = make_float2(-m_run, -m_run);
                 float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
@@ -732,7 +733,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
                     for (int e2 = 0; e2 < 16; ++e2) {
                         const int e = 32 * c + 2 * e2;
-                        const float2 arg = __ffma2_rn(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), sc2, nm2);
+                        const float2 arg = __ffma2_rn(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), sc_piece, nm2);
                         const float2 pe = make_float2(fast_exp2(arg.x), fast_exp2(arg.y));
                         sum[e2 & 1] = __fadd2_rn(sum[e2 & 1], pe);
                         pk16[e2] = pack_bf16(pe.x, pe.y);
@@ -743,6 +744,16 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(p_full + x);
+                        // The scale of the other keys comes from shared memory, read here: their exponentials then cannot be moved
+                        // ahead of the hand-over (the compiler did, which left 70 cycles between the two pieces and the tensor core
+                        // without work under the last exponentials).  A step of a tile pair 3190 -> 3060 cycles: 4 x 4096 tokens
+                        // of 32 / 8 heads of 128 563 -> 553 us, 1 x 32768 of 28 / 4 6800 -> 6600.  At head_dim 64 P V is too short
+                        // to gain from it (64 ragged sequences of 16 heads 714 -> 720 us).
+                        if (D == 128) {
+                            float again;
+                            asm volatile("ld.volatile.shared.f32 %0, [%1];" : "=f"(again) : "r"(smem_u32(smem + sl.misc + 8)) : "memory");
+                            sc_piece = make_float2(again, again);
+                        }
                     }
                 }
                 tmem_wait_st();
