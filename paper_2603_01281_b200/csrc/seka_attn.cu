@@ -16,11 +16,11 @@
 //   warp 1        MMA issuer: S_x = Q_x K^T (+ the low-part steps) and O_x += P_x V on tcgen05 with all accumulators
 //                 in tensor memory (S_A, S_B, O_A, O_B = 512 columns); P_x is read from tensor memory;
 //   warp 2        operand relay: tells the issuer when the operands have landed, so that it waits on one barrier per
-//                 hand-off;
+//                 hand-off (head_dim 64: warps 1 and 2 issue for tile A and tile B and see to their operands themselves);
 //   warps 4-7 / 8-11  softmax of tile A / B, one query row per thread: causal mask on the diagonal tile, online
 //                 softmax in base 2 with a lazily updated running maximum, P written back as bf16 over the consumed
-//                 score columns, O rescaled in tensor memory only when the maximum moved by more than 2^8; final
-//                 normalisation and store.
+//                 score columns (head_dim 64: to columns of its own), O rescaled in tensor memory only when the maximum
+//                 moved by more than 2^8; final normalisation and store.
 // (Warp 3 only gives its registers to the softmax warps.)
 // While one tile's softmax runs, the tensor core works on the other tile.  Items follow each other without a seam: the next
 // item's first key tile travels with this item's last value tile, its Q tiles follow the last score products, and the
@@ -68,13 +68,21 @@ constexpr uint32_t SMEM_LIMIT = 227 * 1024;
 // Shared memory of one CTA.  Tiles first (each a multiple of 1024 bytes), then barriers and per-warp item slots.
 template <int D>
 struct Geo {
-    // P is handed to the tensor core in two pieces, so that most of P V runs under the last exponentials; 16-key blocks in the
-    // first piece (head_dim 64, whose P V is short: half)
-    static constexpr int KP1 = D == 128 ? 6 : 4;
+    // head_dim 128: P is handed to the tensor core in two pieces, so that most of P V runs under the last exponentials; 16-key
+    // blocks in the first piece
+    static constexpr int KP1 = 6;
+    // Head_dim 64 leaves room in tensor memory for the weights P beside the scores.  The next scores of a tile are then formed as
+    // soon as the present ones are in registers, under their softmax, instead of behind P V: the softmax warps wait for nothing
+    // but one another's use of the special-function units.  Each tile has an issuer of its own (one for both would hold one
+    // tile's scores back until the other's weights are there), and the output of an item is stored behind the first weights of
+    // the next.  64 ragged sequences of 16 heads 710 -> 672 us (preparation included), one prompt of 8192 tokens of 32 / 8 heads
+    // 407 -> 384, a toy layer in fp32 16.3 -> 14.6.  Without the late store: 667, 431, 14.4; with the two tiles' exponentials
+    // kept apart by a lock per scheduler: 681, 442.
+    static constexpr bool APART = D == 64;
     static constexpr int NK = D == 128 ? 2 : 3;                    // K and V ring depth
     static constexpr uint32_t TILE = (D / 64) * BLK_BYTES;         // a [128 x D] tile
     static constexpr int NXMAX = 3;                                // most stages of the key-side operand
-    static constexpr uint32_t NBARS = 14 + 2 * NK + NXMAX;
+    static constexpr uint32_t NBARS = 15 + 2 * NK + NXMAX;
     // shared-memory copy of the per-(sequence, KV head) steering bytes and of the tile flags, a bit each (what fits beside the
     // tiles; larger batches look them up in global memory)
     static constexpr int INFO_HEADS = D == 128 ? 768 : 2048, INFO_WORDS = D == 128 ? 128 : 512;
@@ -175,6 +183,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     constexpr int NBLK = D / 64;
     constexpr uint32_t TMEM_COLS = 512;
     constexpr uint32_t COL_S = 0, COL_O = 256;     // S_x at COL_S + 128 x, O_x at COL_O + D x
+    constexpr uint32_t COL_P = G::APART ? 384 : COL_S, P_PITCH = G::APART ? 64 : 128;      // P_x at COL_P + P_PITCH x
     extern __shared__ __align__(1024) uint8_t smem[];
     const SmemPlan sl = smem_plan<D>(p.plan);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sl.bars);
@@ -186,7 +195,8 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     uint64_t* s_full = x_full + G::NXMAX;    // [2]   scores of tile x are in tensor memory
     uint64_t* p_full = s_full + 2;           // [2]   4 softmax-warp arrivals (O_x rescaled, the first 16 KP1 keys of P_x written) + 1 from the relay
     uint64_t* p_last = p_full + 2;           // [2]   4 softmax-warp arrivals: the other keys of P_x written
-    uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished
+    uint64_t* s_free = p_last;               // [2]   (APART) 4 softmax-warp arrivals: the scores of tile x are in registers
+    uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished; (APART) a P V of tile x finished
     uint64_t* o_drained = o_full + 2;        // [2]   4 softmax-warp arrivals: O_x of the item has been read
     uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles of the item landed
     uint64_t* drain = start_full + 1;        // [1]   every product issued has finished
@@ -197,13 +207,13 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     // what does not depend on the launch before: barriers, tensor memory
     if (tid == 0) {
         mbar_init(q_full + 0, 1); mbar_init(q_full + 1, 1); mbar_init(k0_full, 1);
-        for (int i = 0; i < NK; ++i) { mbar_init(kv_full + i, 1); mbar_init(kv_free + i, 1); }
+        for (int i = 0; i < NK; ++i) { mbar_init(kv_full + i, 1); mbar_init(kv_free + i, G::APART ? 2 : 1); }
         for (int i = 0; i < G::NXMAX; ++i) mbar_init(x_full + i, 1);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(s_full + i, 1); mbar_init(p_full + i, 5); mbar_init(p_last + i, 4); mbar_init(o_full + i, 1);
+            mbar_init(s_full + i, 1); mbar_init(p_full + i, G::APART ? 4 : 5); mbar_init(p_last + i, 4); mbar_init(o_full + i, 1);
             mbar_init(o_drained + i, 4);
         }
-        mbar_init(start_full, 1); mbar_init(drain, 1);
+        mbar_init(start_full, 1); mbar_init(drain, G::APART ? 2 : 1);
         mbar_fence_init();
         tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
         if (p.plan.mode) tma_prefetch_desc(&tmX);
@@ -320,18 +330,17 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     //   cx[x]  steps of tile x so far (phases of s_full, p_full, p_last)
     Item it;
 
-    // final normalisation and store of this warp's 32 rows of tile x of item `w` (`inv`: 1 / row sum of the lane's row)
-    auto store_tile = [&](int x, const Item& w, float inv) {
+    // final normalisation and store of this warp's 32 rows of tile x: `rows` of them exist, the first goes to `dst` (`inv`: 1 / row
+    // sum of the lane's row)
+    auto store_tile = [&](int x, OutT* dst, int rows, float inv) {
         tc_fence_after();
-        const int q0 = (x ? w.qtB : w.qtA) * BM + (warp & 3) * 32;       // first query of the warp
         const uint32_t tO = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + COL_O + D * x;
-        OutT* dst = static_cast<OutT*>(p.O) + ((size_t)(w.seq0 + q0) * p.sched.Hq + (x ? w.hqB : w.hqA)) * D;
 #pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
             uint32_t o[32];
             tmem_ld32(tO + c * 32, o);
             tmem_wait_ld_on(o);
-            store_chunk32<OutT>(dst + c * 32, (size_t)p.sched.Hq * D, w.Lb - q0, o, inv, lane);
+            store_chunk32<OutT>(dst + c * 32, (size_t)p.sched.Hq * D, rows, o, inv, lane);
         }
         tc_fence_before();
         // O_x may be written again (the next item's first P V)
@@ -474,7 +483,128 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
                 for (int i = 0; i < G::NXMAX; ++i) settle(x_full + i, armed_x[i]);
             }
-        } else if (warp == 1) {
+        } else if (G::APART && warp < 3) {
+            // ------------------------------------------------------------ MMA issuer of tile x
+            constexpr uint32_t IDESC_S = umma_idesc_bf16(BN, false);
+            constexpr uint32_t IDESC_PV = umma_idesc_bf16(D, true);
+            constexpr uint32_t DESC_HI = umma_desc_hi_sw128(1024);
+            const int x = warp - 1;
+            const uint32_t dQ = umma_desc_lo(smem_u32(smem + x * G::TILE), 16), dK = umma_desc_lo(smem_u32(smem + sl.k), 16);
+            const uint32_t dX = umma_desc_lo(smem_u32(smem + sl.x), 16);
+            const uint32_t dV = umma_desc_lo(smem_u32(smem + sl.v), BLK_BYTES);
+            const uint32_t tS = tmem_base + COL_S + 128 * x, tO = tmem_base + COL_O + D * x, tP = tmem_base + COL_P + P_PITCH * x;
+            const uint32_t n_x = p.plan.nx > 0 ? (uint32_t)p.plan.nx : 1u;
+            uint32_t g = 0, n_q = 0, n_hot = 0, cx = 0, n_o = 0, n_s = 0;
+            bool ok = !dead;
+            uint32_t x_stage = 0;         // stage that holds the low parts of the key tile being multiplied
+            // the low parts of the next edited key tile have landed (each of them is seen, in order, whether the tile uses it or not)
+            auto see_x = [&]() {
+                x_stage = n_hot % n_x;
+                ok = warp_wait(x_full + x_stage, (n_hot / n_x) & 1, 32);
+                ++n_hot;
+            };
+            auto see_q = [&](const Item& w) {
+                if (x == 0 || w.nB > 0) { ok = warp_wait(q_full + x, n_q & 1, 20 + x); ++n_q; }
+            };
+            // scores against the key tile in stage `st`; `hot`: the tile is an edited one whose low parts are multiplied too
+            auto issue_S = [&](uint32_t st, bool hot) {
+                if (n_s > 0) {          // the scores before are in registers (each phase is seen, in order)
+                    ok = warp_wait(s_free + x, (n_s - 1) & 1, 28 + x);
+                    if (!ok) return;
+                }
+                ++n_s;
+                const uint32_t kd = dK + st * (G::TILE >> 4);
+                tc_fence_after();
+                if (leader) {
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        // 16 elements along the contraction = 32 bytes inside a 64-element block
+                        const uint32_t off = ((uint32_t)(ks >> 2) * BLK_BYTES + (uint32_t)(ks & 3) * 32) >> 4;
+                        umma_ss(tS, dQ + off, DESC_HI, kd + off, DESC_HI, IDESC_S, ks > 0 ? 1u : 0u);
+                    }
+                    if (hot) {        // ... + Q (k'_lo)^T
+                        const uint32_t xd = dX + x_stage * (sl.xb >> 4);
+#pragma unroll
+                        for (int ks = 0; ks < D / 16; ++ks) {
+                            const uint32_t off = ((uint32_t)(ks >> 2) * BLK_BYTES + (uint32_t)(ks & 3) * 32) >> 4;
+                            umma_ss(tS, dQ + off, DESC_HI, xd + off, DESC_HI, IDESC_S, 1u);
+                        }
+                    }
+                    umma_commit(s_full + x);
+                }
+                __syncwarp();
+            };
+            // P of step j has been handed over: P V with the value tile in stage `st` (blocks of 16 keys: 2048 bytes of V, 8
+            // columns of P).  Before an item's first P V writes O_x, the O_x of the last item that had a tile x has been read (its
+            // phases count those items only, and each is seen, in order, by the next item that has the tile: a parity wait cannot
+            // tell a phase from the one two later).
+            auto step_PV = [&](uint32_t st, int j) {
+                ok = warp_wait(p_full + x, (cx + j) & 1, 24 + 2 * x);
+                if (ok && j == 0 && n_o > 0) ok = warp_wait(o_drained + x, (n_o - 1) & 1, 46 + x);
+                if (!ok) return;
+                const uint32_t vd = dV + st * (G::TILE >> 4);
+                tc_fence_after();
+                if (leader) {
+#pragma unroll
+                    for (int ks = 0; ks < BN / 16; ++ks)
+                        umma_ts(tO, tP + (uint32_t)ks * 8, vd + (uint32_t)ks * (2048 >> 4), DESC_HI, IDESC_PV, (j > 0 || ks > 0) ? 1u : 0u);
+                    umma_commit(o_full + x);
+                }
+                __syncwarp();
+            };
+            auto commit_event = [&](uint32_t st) {
+                if (leader) umma_commit(kv_free + st);
+                __syncwarp();
+            };
+            uint32_t st = 0;              // stage of the present value tile (of key tile g; the next key tile is in the stage after it)
+            bool have = ok && next_item(it, true);
+            if (have) {
+                see_q(it);
+                if (ok) ok = warp_wait(k0_full, 0, 23);
+                const bool hot = it.need_lo && tile_is_hot(it.b, 0);
+                if (ok && hot) see_x();
+                if (ok) {
+                    if (x == 0 || it.nB > 0) issue_S(0, hot);
+                    commit_event(0);
+                }
+            }
+            while (ok && have) {
+                Item nx;
+                const bool more = next_item(nx, true);
+                const int n = x ? it.nB : it.nA, n_kv = it.n_kv, n_nx = x ? nx.nB : nx.nA;
+                bool hot_nxt = it.need_lo && n_kv > 1 && tile_is_hot(it.b, 1);
+#pragma unroll 1
+                for (int j = 0; j < n_kv; ++j, ++g) {
+                    const int j1 = j + 1;
+                    const uint32_t st1 = st + 1 == (uint32_t)NK ? 0u : st + 1;
+                    const bool turn = j1 == n_kv && more;      // on to the next item's scores
+                    bool hot = hot_nxt && j1 < n_kv;
+                    hot_nxt = it.need_lo && j + 2 < n_kv && tile_is_hot(it.b, j + 2);
+                    ok = warp_wait(kv_full + g % NK, (g / NK) & 1, 25);       // V of this step and K of the next
+                    if (!ok) break;
+                    // inside an item the next scores go first: they only wait for the present ones to be in registers
+                    if (!turn) {
+                        if (hot) { see_x(); if (!ok) break; }
+                        if (j1 < n) issue_S(st1, hot);
+                        if (ok && j < n) step_PV(st, j);
+                    } else {
+                        if (j < n) step_PV(st, j);
+                        if (ok) see_q(nx);
+                        if (!ok) break;
+                        hot = nx.need_lo && tile_is_hot(nx.b, 0);
+                        if (hot) { see_x(); if (!ok) break; }
+                        if (n_nx > 0) issue_S(st1, hot);
+                    }
+                    if (!ok) break;
+                    commit_event(st1);     // K(g+1) and V(g) may be overwritten, as far as this tile goes
+                    st = st1;
+                }
+                if (!ok) break;
+                cx += n;
+                if (n > 0) ++n_o;
+                it = nx; have = more;
+            }
+        } else if (!G::APART && warp == 1) {
             // ------------------------------------------------------------ MMA issuer
             constexpr uint32_t IDESC_S = umma_idesc_bf16(BN, false);
             constexpr uint32_t IDESC_PV = umma_idesc_bf16(D, true);
@@ -630,7 +760,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 if (nB > 0) ++n_o[1];
                 it = nx; have = more;
             }
-        } else if (warp == 2) {
+        } else if (!G::APART && warp == 2) {
             // ------------------------------------------------------------ operand relay: "the operands have landed", once per
             // item for Q (and the CTA's first K), and per step "V(g) and K(g+1) landed" as a fifth arrival on the
             // P hand-off barrier, so that the MMA issuer waits on one barrier per hand-off
@@ -677,9 +807,12 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const int x = (warp - 4) >> 2;
         const int row = (warp & 3) * 32 + lane;
         const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t tS = t_lane + COL_S + 128 * x, tO = t_lane + COL_O + D * x;
+        const uint32_t tS = t_lane + COL_S + 128 * x, tO = t_lane + COL_O + D * x, tP = t_lane + COL_P + P_PITCH * x;
         const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
         uint32_t cX = 0, n_o = 0;       // steps and items of this tile so far
+        OutT* pend_dst = nullptr;       // (APART) the last item's output: where it goes (null: nothing to store), its rows, 1 / row sum
+        int pend_rows = 0;
+        float pend_inv = 0.f;
         bool ok = !dead;
         while (ok && next_item(it)) {
             const int nX = x ? it.nB : it.nA;
@@ -695,6 +828,11 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, reinterpret_cast<uint32_t(&)[32]>(v[32 * c]));
                 tmem_wait_ld();
+                if (G::APART) {         // the next scores may be formed
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(s_free + x);
+                }
                 if (j == nX - 1) {       // diagonal tile: keys after the query are masked
 #pragma unroll
                     for (int e = 0; e < 128; ++e)
@@ -713,6 +851,11 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 const bool raise = (m_new - m_run) > LAZY_RESCALE_LOG2;      // true on the first tile (m_run = -inf)
                 const float factor = raise ? fast_exp2(m_run - m_new) : 1.f;
                 if (raise) m_run = m_new;
+                if (G::APART && (j > 0 || pend_dst != nullptr)) {       // the P V before is through: P may be written, O read or written
+                    ok = warp_wait(o_full + x, (cX + j - 1) & 1, 48 + x);
+                    if (!ok) break;
+                    tc_fence_after();
+                }
                 if (j > 0 && __any_sync(0xffffffffu, raise)) {
                     uint32_t o[32];
 #pragma unroll 1
@@ -738,8 +881,8 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         sum[e2 & 1] = __fadd2_rn(sum[e2 & 1], pe);
                         pk16[e2] = pack_bf16(pe.x, pe.y);
                     }
-                    tmem_st16(tS + c * 16, pk16);     // P (bf16 pairs) over score columns that are already in registers
-                    if (2 * c + 2 == G::KP1) {      // the first piece is in place: the tensor core may start on it
+                    tmem_st16(tP + c * 16, pk16);     // P (bf16 pairs); head_dim 128: over score columns that are already in registers
+                    if (!G::APART && 2 * c + 2 == G::KP1) {      // the first piece is in place: the tensor core may start on it
                         tmem_wait_st();
                         tc_fence_before();
                         __syncwarp();
@@ -747,34 +890,45 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         // The scale of the other keys comes from shared memory, read here: their exponentials then cannot be moved
                         // ahead of the hand-over (the compiler did, which left 70 cycles between the two pieces and the tensor core
                         // without work under the last exponentials).  A step of a tile pair 3190 -> 3060 cycles: 4 x 4096 tokens
-                        // of 32 / 8 heads of 128 563 -> 553 us, 1 x 32768 of 28 / 4 6800 -> 6600.  At head_dim 64 P V is too short
-                        // to gain from it (64 ragged sequences of 16 heads 714 -> 720 us).
-                        if (D == 128) {
-                            float again;
-                            asm volatile("ld.volatile.shared.f32 %0, [%1];" : "=f"(again) : "r"(smem_u32(smem + sl.misc + 8)) : "memory");
-                            sc_piece = make_float2(again, again);
-                        }
+                        // of 32 / 8 heads of 128 563 -> 553 us, 1 x 32768 of 28 / 4 6800 -> 6600.
+                        float again;
+                        asm volatile("ld.volatile.shared.f32 %0, [%1];" : "=f"(again) : "r"(smem_u32(smem + sl.misc + 8)) : "memory");
+                        sc_piece = make_float2(again, again);
                     }
                 }
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(p_last + x);
+                if (lane == 0) mbar_arrive((G::APART ? p_full : p_last) + x);
                 const float2 s2 = __fadd2_rn(sum[0], sum[1]);
                 l_run = l_run * factor + (s2.x + s2.y);
+                if (G::APART && j == 0 && pend_dst != nullptr) {
+                    store_tile(x, pend_dst, pend_rows, pend_inv);
+                    pend_dst = nullptr;
+                }
             }
             if (!ok) break;
             cX += nX;
             if (nX > 0) {
                 const float inv = 1.f / l_run;
-                const int qpos = qtX * BM + row;
+                const int qpos = qtX * BM + row, q0 = qtX * BM + (warp & 3) * 32;
+                OutT* dst = static_cast<OutT*>(p.O) + ((size_t)(it.seq0 + q0) * p.sched.Hq + hqX) * D;
                 if (p.lse != nullptr && qpos < it.Lb)
                     p.lse[(size_t)(it.seq0 + qpos) * p.sched.Hq + hqX] = (m_run + log2f(l_run)) * 0.6931471805599453f;
-                ok = warp_wait(o_full + x, n_o & 1, 44 + x);
-                if (!ok) break;
-                store_tile(x, it, inv);
-                ++n_o;
+                if (G::APART) {
+                    // the last P V runs on; its output is stored behind the first weights of the next item
+                    pend_dst = dst; pend_rows = it.Lb - q0; pend_inv = inv;
+                } else {
+                    ok = warp_wait(o_full + x, n_o & 1, 44 + x);
+                    if (!ok) break;
+                    store_tile(x, dst, it.Lb - q0, inv);
+                    ++n_o;
+                }
             }
+        }
+        if (G::APART && ok && pend_dst != nullptr) {
+            ok = warp_wait(o_full + x, (cX - 1) & 1, 44 + x);
+            if (ok) store_tile(x, pend_dst, pend_rows, pend_inv);
         }
     }
 
@@ -782,7 +936,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     pdl_release();
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 1 || (G::APART && warp == 2)) {
         // every product issued has finished before tensor and shared memory are released
         if (elect_one()) umma_commit(drain);
         __syncwarp();
