@@ -69,7 +69,7 @@ constexpr uint32_t SMEM_LIMIT = 227 * 1024;
 template <int D>
 struct Geo {
     // head_dim 128: P is handed to the tensor core in two pieces, so that most of P V runs under the last exponentials; 16-key
-    // blocks in the first piece
+    // blocks in the first piece (5: level; 7: 2 % slower)
     static constexpr int KP1 = 6;
     // Head_dim 64 leaves room in tensor memory for the weights P beside the scores.  The next scores of a tile are then formed as
     // soon as the present ones are in registers, under their softmax, instead of behind P V: the softmax warps wait for nothing
@@ -327,7 +327,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     //   n_o[x] items that had a tile x so far (phases of o_full, o_drained)
     //   n_qb   items with a tile B so far (phase of q_full[1])
     //   n_hot  edited key tiles whose low parts were loaded / used so far, over all items (stage and phase of x_full)
-    //   cx[x]  steps of tile x so far (phases of s_full, p_full, p_last)
+    //   cx[x]  steps of tile x so far (phases of s_full, p_full, p_last; of s_free and, with a phase per step, o_full in head_dim 64)
     Item it;
 
     // final normalisation and store of this warp's 32 rows of tile x: `rows` of them exist, the first goes to `dst` (`inv`: 1 / row
@@ -571,7 +571,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             while (ok && have) {
                 Item nx;
                 const bool more = next_item(nx, true);
-                const int n = x ? it.nB : it.nA, n_kv = it.n_kv, n_nx = x ? nx.nB : nx.nA;
+                const int n = x ? it.nB : it.nA, n_kv = it.n_kv, n_nx = !more ? 0 : x ? nx.nB : nx.nA;
                 bool hot_nxt = it.need_lo && n_kv > 1 && tile_is_hot(it.b, 1);
 #pragma unroll 1
                 for (int j = 0; j < n_kv; ++j, ++g) {
