@@ -58,7 +58,7 @@ constexpr uint32_t BLK_BYTES = 128 * 128;   // one [128 x 64] bf16 block
 constexpr float LAZY_RESCALE_LOG2 = 8.0f;   // the running maximum is only raised when it moved by more than this
 // registers per thread after the roles split, out of the launch's 168 per thread (3 x 168 = 104 + 2 x 200)
 constexpr int REGS_CTRL = 104, REGS_SOFTMAX = 200;
-// Plain polls of a wait before it parks (see mbar_wait_limit).  One: a warp that polls takes issue slots from the softmax
+// Plain polls of a wait before it parks (see mbar_wait_within).  One: a warp that polls takes issue slots from the softmax
 // warps of its scheduler (eight polls cost 1 % on 4 x 4096 tokens of 32 heads of 128, polling without end 4 %).
 constexpr int PLAIN_POLLS = 1;
 
@@ -228,7 +228,14 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     bool dead = false;
     if (TABLE) dead = __syncthreads_or(status0 != 0);
     const int hook_skip = p.status[4];
-    const uint64_t limit_ns = p.status[5] > 0 ? (uint64_t)p.status[5] * 1000ull : kWaitLimitNs;
+    const uint64_t limit_set = p.status[5] > 0 ? (uint64_t)p.status[5] * 1000ull : kWaitLimitNs;
+    // The limit of a wait: only one that has parked in vain asks for it.  Packed launches keep it in shared memory: the item
+    // records leave them no registers for it, and the compiler spilled around it.  Three sequences of 1000 to 8000 tokens at
+    // head_dim 128: 28 / 4 heads 667 -> 656 us, 16 / 16 heads 407 -> 404; 64 of 256 to 2048 tokens of 32 / 8 heads 1135 -> 1068
+    // (1.9 GHz).  Fixed-length launches have the registers, and the store would wait for the word's first read (0.3 us of a
+    // short steered call).
+    volatile uint64_t* limit_smem = reinterpret_cast<volatile uint64_t*>(smem + sl.misc + 16);
+    auto limit_ns = [&]() -> uint64_t { return TABLE ? *limit_smem : limit_set; };
     // steering info is kept in shared memory when it fits (a look-up then costs no trip to the caches): a byte per (sequence,
     // KV head) and a bit per (sequence, key tile)
     const bool info_local = p.steer && p.sched.B * p.sched.Hkv <= G::INFO_HEADS;
@@ -242,7 +249,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
     // all lanes of a warp wait on the same barrier and then agree on the outcome
     auto warp_wait = [&](uint64_t* bar, uint32_t parity, int where) -> bool {
-        const bool ok = mbar_wait_limit(bar, parity, abort_flag, p.status, where, limit_ns, PLAIN_POLLS);
+        const bool ok = mbar_wait_within(bar, parity, abort_flag, p.status, where, limit_ns, PLAIN_POLLS);
         return __all_sync(0xffffffffu, ok);
     };
 
@@ -300,7 +307,10 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         return true;
     };
 
-    if (tid == 0) { *abort_flag = 0; *reinterpret_cast<volatile float*>(smem + sl.misc + 8) = p.scale_log2; }
+    if (tid == 0) {
+        *abort_flag = 0; *reinterpret_cast<volatile float*>(smem + sl.misc + 8) = p.scale_log2;
+        if (TABLE) *limit_smem = limit_set;
+    }
     // steering info into shared memory
     if (info_local)
         for (int i = tid; i < p.sched.B * p.sched.Hkv; i += NTHREADS) info_bh[i] = p.bh_info[i];
@@ -475,7 +485,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             if (*abort_flag) {
                 // loads that were armed may still be in flight: let them land before the shared memory is released
                 auto settle = [&](uint64_t* bar, uint32_t armed) {
-                    if (armed) mbar_wait_limit(bar, armed - 1, nullptr, nullptr, 0, limit_ns);
+                    if (armed) mbar_wait_within(bar, armed - 1, nullptr, nullptr, 0, limit_ns);
                 };
                 settle(q_full + 0, armed_q[0]); settle(q_full + 1, armed_q[1]); settle(k0_full, armed_k0);
 #pragma unroll
@@ -940,7 +950,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         // every product issued has finished before tensor and shared memory are released
         if (elect_one()) umma_commit(drain);
         __syncwarp();
-        mbar_wait_limit(drain, 0, nullptr, p.status, 90, limit_ns);
+        mbar_wait_within(drain, 0, nullptr, p.status, 90, limit_ns);
     }
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem_base, TMEM_COLS);

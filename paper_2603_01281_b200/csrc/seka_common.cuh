@@ -282,8 +282,10 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint64_t* bar, uint32_t par
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s; a whole launch takes milliseconds
 constexpr int kPlainPolls = 8;
 
-__device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                int* status, int where, uint64_t limit_ns, int plain_polls = kPlainPolls) {
+// `limit_ns()` is called only where a parked poll came back empty-handed
+template <typename Limit>
+__device__ __forceinline__ bool mbar_wait_within(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                 int* status, int where, const Limit& limit_ns, int plain_polls = kPlainPolls) {
 #pragma unroll 1
     for (int i = 0; i < plain_polls; ++i)
         if (mbar_try_wait(bar, parity)) return true;
@@ -296,12 +298,17 @@ __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, 
         const uint64_t now = global_timer_ns();
         if (t0 == 0) {
             t0 = now;
-        } else if (now - t0 > limit_ns) {
+        } else if (now - t0 > limit_ns()) {
             if (abort_flag != nullptr) *abort_flag = 1;
             report_timeout(status, where);
             return false;
         }
     }
+}
+
+__device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                int* status, int where, uint64_t limit_ns, int plain_polls = kPlainPolls) {
+    return mbar_wait_within(bar, parity, abort_flag, status, where, [=]() { return limit_ns; }, plain_polls);
 }
 
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,

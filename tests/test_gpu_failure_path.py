@@ -21,12 +21,22 @@ HOOK_SKIP_PAIR_WORD, WAIT_LIMIT_US_WORD = 4, 5      # int32 words of the 256-byt
 
 @pytest.mark.parametrize("d", [128, 64])
 def test_wait_runs_out_and_the_workspace_recovers(d):
+    _wait_runs_out(d, packed=False)
+
+
+# a packed launch looks its limit up in shared memory
+@pytest.mark.parametrize("d", [128, 64])
+def test_wait_of_a_packed_launch_runs_out(d):
+    _wait_runs_out(d, packed=True)
+
+
+def _wait_runs_out(d, packed):
     binding.load()
     # two row tiles of one head pair: CTA 0 takes the item with two key tiles, CTA 1 the one with a single tile
     w = inputs.make_custom(seed=31, dtype="bf16", lens=[256], n_q_heads=2, n_kv_heads=1, head_dim=d, rank=16,
                            gain=1.0, highlight=0.2)
     dev = H.device_tensors(w)
-    shp = H.shape_of(w, dev)
+    shp = H.shape_of(w, dev, packed)
     ws = binding.new_workspace(shp)
     words = ws[:256].view(torch.int32)
     O = torch.full_like(dev["Q"], float("nan"))
