@@ -173,12 +173,15 @@ struct Item {
     bool need_lo;               // ... and the low parts of the edited keys are multiplied too
 };
 
-template <int D, typename OutT, bool TABLE>
+// LEAD (head_dim 64, one item per CTA, both tiles equally long): tile B starts its first exponentials when tile A is three
+// quarters through its own, see launch_attn_t.
+template <int D, typename OutT, bool TABLE, bool LEAD = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmX,
                      const __grid_constant__ AttnParams p) {
     using G = Geo<D>;
+    static_assert(!LEAD || (G::APART && !TABLE), "the lead barrier has one phase, and head_dim 128 uses it otherwise");
     constexpr int NK = G::NK;
     constexpr int NBLK = D / 64;
     constexpr uint32_t TMEM_COLS = 512;
@@ -199,6 +202,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished; (APART) a P V of tile x finished
     uint64_t* o_drained = o_full + 2;        // [2]   4 softmax-warp arrivals: O_x of the item has been read
     uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles of the item landed
+    uint64_t* lead = start_full;             // [1]   (LEAD) 4 softmax-warp arrivals: tile A is three quarters through its first exponentials
     uint64_t* drain = start_full + 1;        // [1]   every product issued has finished
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sl.misc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + sl.misc + 4);
@@ -213,7 +217,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             mbar_init(s_full + i, 1); mbar_init(p_full + i, G::APART ? 4 : 5); mbar_init(p_last + i, 4); mbar_init(o_full + i, 1);
             mbar_init(o_drained + i, 4);
         }
-        mbar_init(start_full, 1); mbar_init(drain, G::APART ? 2 : 1);
+        mbar_init(start_full, LEAD ? 4 : 1); mbar_init(drain, G::APART ? 2 : 1);
         mbar_fence_init();
         tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
         if (p.plan.mode) tma_prefetch_desc(&tmX);
@@ -877,6 +881,10 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         tmem_st32(tO + c * 32, o);
                     }
                 }
+                if (LEAD && x == 1 && j == 0) {
+                    ok = warp_wait(lead, 0, 36);
+                    if (!ok) break;
+                }
                 float2 sc_piece = sc2;
                 const float2 nm2 = make_float2(-m_run, -m_run);
                 float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -891,6 +899,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         sum[e2 & 1] = __fadd2_rn(sum[e2 & 1], pe);
                         pk16[e2] = pack_bf16(pe.x, pe.y);
                     }
+                    if (LEAD && c == 2 && x == 0 && j == 0 && lane == 0) mbar_arrive(lead);
                     tmem_st16(tP + c * 16, pk16);     // P (bf16 pairs); head_dim 128: over score columns that are already in registers
                     if (!G::APART && 2 * c + 2 == G::KP1) {      // the first piece is in place: the tensor core may start on it
                         tmem_wait_st();
@@ -1022,12 +1031,25 @@ static seka_status launch_attn_t(const TileMaps& tm, const AttnParams& p, cudaSt
     const SmemPlan sl = smem_plan<D>(p.plan);
     const uint32_t dyn = sl.total;
     if (dyn > SMEM_LIMIT) return SEKA_ERR_UNSUPPORTED;
+    int n_sm = 0;
+    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     auto kern = seka_attn_fwd_kernel<D, OutT, TABLE>;
+    if constexpr (Geo<D>::APART && !TABLE) {
+        // One item per CTA, two query heads at the same rows: without the aliasing of P and S nothing keeps such tiles apart, so
+        // they load, search their maximum and use the special-function unit in step, each half idle.  The lead undoes that.
+        // Unsteered, us (P over S / in step / with the lead, 1.9 GHz): 16 / 8 heads, 257 tokens 9.6 / 9.9 / 9.1, 512 tokens
+        // 11.3 / 11.7 / 10.6, 1024 tokens 18.2 / 18.7 / 16.8; 32 / 8 heads, 512 tokens 11.7 / 12.0 / 10.9; 4 / 2 heads, 2048 tokens
+        // 30.0 / 30.5 / 28.2.  A lead of half of the exponentials 1 to 4 % slower, of a quarter 10 %.  Steered launches, which start
+        // under their preparation, up to 1024 tokens only (16 / 8 heads 777 tokens 23.3 / 23.3 / 22.2; 1500 tokens 33.8 / 32.3 /
+        // 33.0, 8 / 4 heads 3000 tokens 52.9 / 49.1 / 53.0).  Not with several items per CTA: the tiles are better off in step
+        // there (8192 tokens of 32 / 8 heads 383 -> 440).
+        const int most = p.steer ? 8 : 16;
+        if (p.sched.pair_heads && p.sched.n_items_max <= (long long)n_sm && p.sched.n_qt > 1 && p.sched.n_qt <= most)
+            kern = seka_attn_fwd_kernel<D, OutT, false, true>;
+    }
     // the attribute belongs to the function on the current device: set on every call (a cheap driver call), so that a
     // process that drives several devices, or calls from several threads, needs no bookkeeping here
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return SEKA_ERR_CUDA;
-    int n_sm = 0;
-    if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     // persistent CTAs, one per SM (the kernel needs the whole SM: all of tensor memory and most of shared memory)
     const unsigned grid = (unsigned)(p.sched.n_items_max < (long long)n_sm ? p.sched.n_items_max : (long long)n_sm);
     if (grid == 0) return SEKA_OK;

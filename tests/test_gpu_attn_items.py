@@ -47,3 +47,26 @@ def test_growing_scores(d, Hq, Hkv):
     err = np.abs(O[idx] - Oref)
     assert (err <= 2.0 ** -7 * Oabs + 1e-3).all(), (err / (2.0 ** -7 * Oabs + 1e-3)).max()
     np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)
+
+
+# One item per CTA whose tiles are two heads at the same rows, head_dim 64: tile B follows tile A.  The lengths at either end of
+# the rule (two key tiles; 8 steered, 16 unsteered; one tile more; one more item than SMs), with a last tile of one row and of 128.
+# Which kernel runs changes no bit: the same sequence as a packed batch takes another.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("steer", [True, False])
+@pytest.mark.parametrize("L,Hq,Hkv", [(128, 4, 2), (129, 4, 2), (256, 8, 2), (257, 2, 1), (1024, 4, 2), (1025, 4, 2), (2048, 4, 1),
+                                      (2049, 2, 1), (200, 148, 74), (200, 152, 76)])
+def test_one_item_per_cta(L, Hq, Hkv, steer, dtype):
+    w = inputs.make_custom(seed=47, dtype=dtype, lens=[L], n_q_heads=Hq, n_kv_heads=Hkv, head_dim=64, rank=16, gain=1.5,
+                           mask_kind="runs", highlight=0.15)
+    # fp32 inputs reach the tensor core as bf16; a row that attends to one key shows that rounding of V in full, 2^-9 |v| or 8e-3 at
+    # |v| = 4, which leaves nothing of the 1e-2 for the kernel: the values are bf16 ones, so that the conversion is exact
+    w.Q, w.K, w.V = inputs.round_to_bf16(w.Q), inputs.round_to_bf16(w.K), inputs.round_to_bf16(w.V)
+    O, LSE = H.run_fused(w, steer=steer)
+    Op, Lp = H.run_fused(w, steer=steer, force_varlen=True)
+    assert np.array_equal(O, Op) and np.array_equal(LSE, Lp)
+    if not steer:
+        w.mask[:] = 0
+    Oref, Lref, idx = H.oracle_rows(w, H.sampled_rows(w, 24))
+    H.check_attention(O[idx], Oref, "%d tokens %d/%d" % (L, Hq, Hkv))
+    np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)
