@@ -181,7 +181,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmX,
                      const __grid_constant__ AttnParams p) {
     using G = Geo<D>;
-    static_assert(!LEAD || (G::APART && !TABLE), "the lead barrier has one phase, and head_dim 128 uses it otherwise");
+    static_assert(!LEAD || G::APART, "head_dim 128 uses the lead barrier otherwise");
     constexpr int NK = G::NK;
     constexpr int NBLK = D / 64;
     constexpr uint32_t TMEM_COLS = 512;
@@ -202,7 +202,7 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished; (APART) a P V of tile x finished
     uint64_t* o_drained = o_full + 2;        // [2]   4 softmax-warp arrivals: O_x of the item has been read
     uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles of the item landed
-    uint64_t* lead = start_full;             // [1]   (LEAD) 4 softmax-warp arrivals: tile A is three quarters through its first exponentials
+    uint64_t* lead = start_full;             // [1]   (LEAD) 4 softmax-warp arrivals, once: tile A is three quarters through its first exponentials
     uint64_t* drain = start_full + 1;        // [1]   every product issued has finished
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sl.misc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + sl.misc + 4);
@@ -1034,18 +1034,19 @@ static seka_status launch_attn_t(const TileMaps& tm, const AttnParams& p, cudaSt
     int n_sm = 0;
     if (!device_info(&n_sm)) return SEKA_ERR_CUDA;
     auto kern = seka_attn_fwd_kernel<D, OutT, TABLE>;
-    if constexpr (Geo<D>::APART && !TABLE) {
+    if constexpr (Geo<D>::APART) {
         // One item per CTA, two query heads at the same rows: without the aliasing of P and S nothing keeps such tiles apart, so
         // they load, search their maximum and use the special-function unit in step, each half idle.  The lead undoes that.
         // Unsteered, us (P over S / in step / with the lead, 1.9 GHz): 16 / 8 heads, 257 tokens 9.6 / 9.9 / 9.1, 512 tokens
         // 11.3 / 11.7 / 10.6, 1024 tokens 18.2 / 18.7 / 16.8; 32 / 8 heads, 512 tokens 11.7 / 12.0 / 10.9; 4 / 2 heads, 2048 tokens
-        // 30.0 / 30.5 / 28.2.  A lead of half of the exponentials 1 to 4 % slower, of a quarter 10 %.  Steered launches, which start
+        // 30.0 / 30.5 / 28.2; three packed sequences of 100 to 900 tokens of 8 / 2 heads 17.5 / 18.5 / 16.7 (a packed launch has at
+        // most n_items_max items).  A lead of half of the exponentials 1 to 4 % slower, of a quarter 10 %.  Steered launches, which start
         // under their preparation, up to 1024 tokens only (16 / 8 heads 777 tokens 23.3 / 23.3 / 22.2; 1500 tokens 33.8 / 32.3 /
         // 33.0, 8 / 4 heads 3000 tokens 52.9 / 49.1 / 53.0).  Not with several items per CTA: the tiles are better off in step
         // there (8192 tokens of 32 / 8 heads 383 -> 440).
         const int most = p.steer ? 8 : 16;
         if (p.sched.pair_heads && p.sched.n_items_max <= (long long)n_sm && p.sched.n_qt > 1 && p.sched.n_qt <= most)
-            kern = seka_attn_fwd_kernel<D, OutT, false, true>;
+            kern = seka_attn_fwd_kernel<D, OutT, TABLE, true>;
     }
     // the attribute belongs to the function on the current device: set on every call (a cheap driver call), so that a
     // process that drives several devices, or calls from several threads, needs no bookkeeping here

@@ -1,7 +1,10 @@
 """Items that follow each other in one CTA of the attention kernel: late stores, items without a second tile, and a running
 maximum that is raised on the way, against the fp64 oracle."""
+import dataclasses
+
 import numpy as np
 import pytest
+import torch
 
 from paper_2603_01281_b200 import inputs
 
@@ -50,8 +53,9 @@ def test_growing_scores(d, Hq, Hkv):
 
 
 # One item per CTA whose tiles are two heads at the same rows, head_dim 64: tile B follows tile A.  The lengths at either end of
-# the rule (two key tiles; 8 steered, 16 unsteered; one tile more; one more item than SMs), with a last tile of one row and of 128.
-# Which kernel runs changes no bit: the same sequence as a packed batch takes another.
+# the rule (two key tiles; 8 steered, 16 unsteered; one tile more; one more item than SMs), with a last tile of one row and of 128,
+# as a fixed-length and as a packed launch.  Which kernel runs changes no bit: as one of many sequences of a packed batch the same
+# one goes through CTAs of several items.
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("steer", [True, False])
 @pytest.mark.parametrize("L,Hq,Hkv", [(128, 4, 2), (129, 4, 2), (256, 8, 2), (257, 2, 1), (1024, 4, 2), (1025, 4, 2), (2048, 4, 1),
@@ -65,7 +69,14 @@ def test_one_item_per_cta(L, Hq, Hkv, steer, dtype):
     O, LSE = H.run_fused(w, steer=steer)
     Op, Lp = H.run_fused(w, steer=steer, force_varlen=True)
     assert np.array_equal(O, Op) and np.array_equal(LSE, Lp)
-    if not steer:
+    if not steer:       # (the preparation of a large batch may round the edited keys elsewhere)
+        n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+        n = n_sm // (Hq // 2 * ((L + 127) // 128)) + 2
+        many = dataclasses.replace(w, Q=np.tile(w.Q, (n, 1, 1)), K=np.tile(w.K, (n, 1, 1)), V=np.tile(w.V, (n, 1, 1)), mask=np.tile(w.mask, n),
+                                   gain=np.tile(w.gain, n), cu_seqlens=(np.arange(n + 1) * L).astype(np.int32))
+        Om, Lm = H.run_fused(many, steer=False, force_varlen=True)
+        for b in range(n):
+            assert np.array_equal(O, Om[b * L:(b + 1) * L]) and np.array_equal(LSE, Lm[b * L:(b + 1) * L])
         w.mask[:] = 0
     Oref, Lref, idx = H.oracle_rows(w, H.sampled_rows(w, 24))
     H.check_attention(O[idx], Oref, "%d tokens %d/%d" % (L, Hq, Hkv))
