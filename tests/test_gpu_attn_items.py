@@ -29,8 +29,8 @@ def test_items_follow_each_other(d, Hq, Hkv, lens):
     assert np.isfinite(O).all() and np.isfinite(LSE).all()
 
 
-# Keys that grow along the sequence: the maximum of a row passes the threshold of 2^8 in tile after tile, so O is rescaled while
-# products are in flight.  Few keys then share a row, so the roundings to bf16 (8 significant bits: at most 2^-8 of a value) no
+# Keys that grow along the sequence: the maximum of a row passes the threshold of 2^8 in tile after tile, so O is rescaled between
+# the products (head_dim 128: the next scores are committed behind the P V before; head_dim 64: the softmax waits for it).  Few keys then share a row, so the roundings to bf16 (8 significant bits: at most 2^-8 of a value) no
 # longer average out: the weights' moves the result by up to 2^-8 sum p |v|, the output's by up to 2^-8 |o|, together 2^-7
 # sum p |v|; 1e-3 for the scores' fp32 sums and exp2.  (The same computation on the CPU with bf16 weights and output, everything
 # else in fp64, reaches 0.80 of this bound.)
@@ -47,6 +47,32 @@ def test_growing_scores(d, Hq, Hkv):
     Oref, Lref, idx = H.oracle_rows(w, H.all_rows(w))
     w.V = np.abs(w.V)
     Oabs = H.oracle_rows(w, H.all_rows(w))[0]
+    err = np.abs(O[idx] - Oref)
+    assert (err <= 2.0 ** -7 * Oabs + 1e-3).all(), (err / (2.0 ** -7 * Oabs + 1e-3)).max()
+    np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)
+
+
+# The same with several items per CTA: O is rescaled after the output of the item before was still to be stored, and the phases of
+# a tile's barriers go on from item to item.  Bounds as above.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("Hq,Hkv", [(16, 4), (9, 3)])
+@pytest.mark.parametrize("lens", [[1100, 513, 128] * 6, [900] * 10])
+def test_growing_scores_over_items(d, Hq, Hkv, lens, dtype):
+    w = inputs.make_custom(seed=44, dtype=dtype, lens=lens, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, rank=8, gain=1.0, mask_kind="none")
+    tiles = [(n + 127) // 128 for n in lens]
+    items = sum(Hq // 2 * t if (Hq // Hkv) % 2 == 0 else Hq * ((t + 1) // 2) for t in tiles)
+    assert items >= 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    for b in range(w.batch):
+        s, e = int(w.cu_seqlens[b]), int(w.cu_seqlens[b + 1])
+        w.K[s:e] *= (1.0 + 12.0 * np.arange(e - s)[:, None, None] / 1100.0).astype(np.float32)
+    w.Q, w.K, w.V = inputs.round_to_bf16(w.Q), inputs.round_to_bf16(w.K), inputs.round_to_bf16(w.V)
+    O, LSE = H.run_fused(w)
+    assert np.isfinite(O).all() and np.isfinite(LSE).all()
+    rows = H.sampled_rows(w, 16)
+    Oref, Lref, idx = H.oracle_rows(w, rows)
+    w.V = np.abs(w.V)
+    Oabs = H.oracle_rows(w, rows)[0]
     err = np.abs(O[idx] - Oref)
     assert (err <= 2.0 ** -7 * Oabs + 1e-3).all(), (err / (2.0 ** -7 * Oabs + 1e-3)).max()
     np.testing.assert_allclose(LSE[idx], Lref, atol=2e-2)
