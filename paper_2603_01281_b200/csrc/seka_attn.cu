@@ -14,7 +14,8 @@
 //                 shared-memory rings, throttled by "free" mbarriers the tensor core signals, and the low parts of
 //                 edited tiles through a ring of their own;
 //   warp 1        MMA issuer: S_x = Q_x K^T (+ the low-part steps) and O_x += P_x V on tcgen05 with all accumulators
-//                 in tensor memory (S_A, S_B, O_A, O_B = 512 columns); P_x is read from tensor memory;
+//                 in tensor memory (head_dim 128: S_A, S_B, O_A, O_B = 512 columns, P_x over S_x; head_dim 64: 384, P_A and P_B
+//                 the other 128); P_x is read from tensor memory;
 //   warp 2        operand relay: tells the issuer when the operands have landed, so that it waits on one barrier per
 //                 hand-off (head_dim 64: warps 1 and 2 issue for tile A and tile B and see to their operands themselves);
 //   warps 4-7 / 8-11  softmax of tile A / B, one query row per thread: causal mask on the diagonal tile, online
@@ -24,10 +25,10 @@
 // (Warp 3 only gives its registers to the softmax warps.)
 // While one tile's softmax runs, the tensor core works on the other tile.  Items follow each other without a seam: the next
 // item's first key tile travels with this item's last value tile, its Q tiles follow the last score products, and the
-// first scores of a tile's next item are issued right behind its last P V, under the store of its output (before, every
-// item began with an empty tensor pipe and its operands on the way, about 8000 cycles).  Measured on 32 / 8 heads of 128:
-// 4 x 4096 tokens 0.495 -> 0.466 ms, one prompt of 4362 tokens 148 -> 139 us (unsteered, GPU rested between blocks); 1 x 32768
-// level.  About 2 us per item remain beside its steps.
+// first scores of a tile's next item are issued right behind its last P V, under the store of its output (head_dim 64: that
+// store waits for the next item's first weights).  Before, every item began with an empty tensor pipe and its operands on the
+// way, about 8000 cycles.  Measured on 32 / 8 heads of 128: 4 x 4096 tokens 0.495 -> 0.466 ms, one prompt of 4362 tokens
+// 148 -> 139 us (unsteered, GPU rested between blocks); 1 x 32768 level.  About 4200 cycles per item remain beside its steps.
 // Every wait is bounded: a wait that runs out raises the CTA's abort flag, every role leaves its loop, and the status word
 // reports it.
 #include <math.h>
@@ -69,15 +70,21 @@ constexpr uint32_t SMEM_LIMIT = 227 * 1024;
 template <int D>
 struct Geo {
     // head_dim 128: P is handed to the tensor core in two pieces, so that most of P V runs under the last exponentials; 16-key
-    // blocks in the first piece (5: level; 7: 2 % slower)
+    // blocks in the first piece.  The exponentials come 32 keys at a time, so an even number; 5 and 7, with that loop cut at 16
+    // keys, were level and 2 % slower.  (head_dim 64 hands P over whole: in two pieces 64 ragged sequences 590 -> 601 us, one
+    // prompt of 8192 tokens 380 -> 434.)
     static constexpr int KP1 = 6;
+    static_assert(KP1 % 2 == 0 && KP1 > 0 && KP1 < 8, "the first hand-over lies behind 32 or 64 or 96 of 128 keys");
     // Head_dim 64 leaves room in tensor memory for the weights P beside the scores.  The next scores of a tile are then formed as
     // soon as the present ones are in registers, under their softmax, instead of behind P V: the softmax warps wait for nothing
     // but one another's use of the special-function units.  Each tile has an issuer of its own (one for both would hold one
     // tile's scores back until the other's weights are there), and the output of an item is stored behind the first weights of
-    // the next.  64 ragged sequences of 16 heads 710 -> 672 us (preparation included), one prompt of 8192 tokens of 32 / 8 heads
-    // 407 -> 384, a toy layer in fp32 16.3 -> 14.6.  Without the late store: 667, 431, 14.4; with the two tiles' exponentials
-    // kept apart by a lock per scheduler: 681, 442.
+    // the next.  64 ragged sequences of 16 heads 646 -> 590 us (preparation included), one prompt of 8192 tokens of 32 / 8 heads
+    // 412 -> 382, a toy layer in fp32 16.0 -> 14.6 (both sides in turn, 1.9 GHz).  Of that the late store costs the ragged batch
+    // 0.7 % and the toy 1 %, and gives the long prompt 11 %: it pays where a CTA walks several items of many steps.  The two tiles'
+    // exponentials kept apart by a lock per scheduler: 1 and 15 % slower.
+    // With several items per CTA and an even head group the tiles run in step or half a period apart, whichever small delays of the
+    // control warps lead to; in step is faster there (8192 tokens 380 us against 400 to 440).  Check both after any change here.
     static constexpr bool APART = D == 64;
     static constexpr int NK = D == 128 ? 2 : 3;                    // K and V ring depth
     static constexpr uint32_t TILE = (D / 64) * BLK_BYTES;         // a [128 x D] tile
@@ -193,17 +200,17 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     uint64_t* q_full = bars;                 // [2]   Q tile landed
     uint64_t* k0_full = q_full + 2;          // [1]   first key tile of the CTA's first item landed
     uint64_t* kv_full = k0_full + 1;         // [NK]  V(g) and K(g+1) landed (they are loaded as a pair)
-    uint64_t* kv_free = kv_full + NK;        // [NK]  one event per step: the tensor core is done with K(g+1) and V(g)
+    uint64_t* kv_free = kv_full + NK;        // [NK]  one event per step: the tensor core is done with K(g+1) and V(g); (APART) an arrival from each issuer
     uint64_t* x_full = kv_free + NK;         // [3]   low parts of an edited tile landed
     uint64_t* s_full = x_full + G::NXMAX;    // [2]   scores of tile x are in tensor memory
-    uint64_t* p_full = s_full + 2;           // [2]   4 softmax-warp arrivals (O_x rescaled, the first 16 KP1 keys of P_x written) + 1 from the relay
+    uint64_t* p_full = s_full + 2;           // [2]   4 softmax-warp arrivals (O_x rescaled, the first 16 KP1 keys of P_x written) + 1 from the relay; (APART) 4: all of P_x written
     uint64_t* p_last = p_full + 2;           // [2]   4 softmax-warp arrivals: the other keys of P_x written
     uint64_t* s_free = p_last;               // [2]   (APART) 4 softmax-warp arrivals: the scores of tile x are in registers
     uint64_t* o_full = p_last + 2;           // [2]   last P V of tile x finished; (APART) a P V of tile x finished
     uint64_t* o_drained = o_full + 2;        // [2]   4 softmax-warp arrivals: O_x of the item has been read
     uint64_t* start_full = o_drained + 2;    // [1]   relay: Q tiles of the item landed
     uint64_t* lead = start_full;             // [1]   (LEAD) 4 softmax-warp arrivals, once: tile A is three quarters through its first exponentials
-    uint64_t* drain = start_full + 1;        // [1]   every product issued has finished
+    uint64_t* drain = start_full + 1;        // [1]   every product issued has finished; (APART) an arrival from each issuer
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sl.misc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + sl.misc + 4);
 
@@ -236,8 +243,9 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     // The limit of a wait: only one that has parked in vain asks for it.  Packed launches keep it in shared memory: the item
     // records leave them no registers for it, and the compiler spilled around it.  Three sequences of 1000 to 8000 tokens at
     // head_dim 128: 28 / 4 heads 667 -> 656 us, 16 / 16 heads 407 -> 404; 64 of 256 to 2048 tokens of 32 / 8 heads 1135 -> 1068
-    // (1.9 GHz).  Fixed-length launches have the registers, and the store would wait for the word's first read (0.3 us of a
-    // short steered call).
+    // (1.9 GHz).  Fixed-length launches keep it: at head_dim 128 they have the registers; at head_dim 64 they spill it (8 bytes
+    // stored, 232 loaded), but only the comparison on that slow path reads it, while the store would wait for the word's first read (0.3 us
+    // of a short steered call) and moved the tiles of long prompts out of step (8192 tokens of 32 / 8 heads 380 -> 435 us).
     volatile uint64_t* limit_smem = reinterpret_cast<volatile uint64_t*>(smem + sl.misc + 16);
     auto limit_ns = [&]() -> uint64_t { return TABLE ? *limit_smem : limit_set; };
     // steering info is kept in shared memory when it fits (a look-up then costs no trip to the caches): a byte per (sequence,
@@ -338,9 +346,10 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     //   kv_free event g: the score products of key tile g and the P V of tile g - 1 are through (event 0: after the CTA's
     //          first score products; event g + 1: after step g)
     //   n_it   items so far (phases of start_full, q_full[0])
-    //   n_o[x] items that had a tile x so far (phases of o_full, o_drained)
+    //   n_o[x] items that had a tile x so far (phases of o_drained; of o_full too in head_dim 128)
     //   n_qb   items with a tile B so far (phase of q_full[1])
-    //   n_hot  edited key tiles whose low parts were loaded / used so far, over all items (stage and phase of x_full)
+    //   n_hot  edited key tiles whose low parts were loaded / seen so far, over all items (stage and phase of x_full; both issuers of
+    //          head_dim 64 see each, used or not)
     //   cx[x]  steps of tile x so far (phases of s_full, p_full, p_last; of s_free and, with a phase per step, o_full in head_dim 64)
     Item it;
 
@@ -908,8 +917,9 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                         if (lane == 0) mbar_arrive(p_full + x);
                         // The scale of the other keys comes from shared memory, read here: their exponentials then cannot be moved
                         // ahead of the hand-over (the compiler did, which left 70 cycles between the two pieces and the tensor core
-                        // without work under the last exponentials).  A step of a tile pair 3190 -> 3060 cycles: 4 x 4096 tokens
-                        // of 32 / 8 heads of 128 563 -> 553 us, 1 x 32768 of 28 / 4 6800 -> 6600.
+                        // without work under the last exponentials).  A traced step of a tile pair 3190 -> 3060 cycles (2970 on
+                        // average over CTAs and steps, plus 4200 an item): 4 x 4096 tokens of 32 / 8 heads of 128 563 -> 553 us,
+                        // 1 x 32768 of 28 / 4 6800 -> 6600 (back to back, about 1.5 GHz).
                         float again;
                         asm volatile("ld.volatile.shared.f32 %0, [%1];" : "=f"(again) : "r"(smem_u32(smem + sl.misc + 8)) : "memory");
                         sc_piece = make_float2(again, again);
