@@ -239,15 +239,20 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     bool dead = false;
     if (TABLE) dead = __syncthreads_or(status0 != 0);
     const int hook_skip = p.status[4];
+    // The limit of a wait: only one that has parked in vain asks for it.  Packed launches carry it as the 32-bit word it comes as: the
+    // item records leave them one register less, and around 64 bits the compiler spilled at head_dim 128.  Three sequences of 1000 to
+    // 8000 tokens at head_dim 128, unsteered: 28 / 4 heads 670 -> 654 us, 16 / 16 heads 413 -> 406; 64 of 256 to 2048 tokens of 32 / 8
+    // heads 1140 -> 1068, of 50 to 500 tokens of 28 / 4 heads 142.7 -> 140.4; 200 of up to 128 tokens 159 -> 161; at head_dim 64 up to
+    // 7 % faster (1.9 GHz).  Fixed-length launches keep 64 bits.  At head_dim 128 they have the registers (the word: level); at
+    // head_dim 64 they spill them (8 bytes stored, 232 loaded), but only the comparison on that slow path reads them, and with the
+    // word the tiles of long prompts went out of step (8192 tokens of 32 / 8 heads 383 -> 389 to 409 us).  In shared memory instead:
+    // 200 packed sequences of up to 128 tokens 2 % slower.
     const uint64_t limit_set = p.status[5] > 0 ? (uint64_t)p.status[5] * 1000ull : kWaitLimitNs;
-    // The limit of a wait: only one that has parked in vain asks for it.  Packed launches keep it in shared memory: the item
-    // records leave them no registers for it, and the compiler spilled around it.  Three sequences of 1000 to 8000 tokens at
-    // head_dim 128: 28 / 4 heads 667 -> 656 us, 16 / 16 heads 407 -> 404; 64 of 256 to 2048 tokens of 32 / 8 heads 1135 -> 1068
-    // (1.9 GHz).  Fixed-length launches keep it: at head_dim 128 they have the registers; at head_dim 64 they spill it (8 bytes
-    // stored, 232 loaded), but only the comparison on that slow path reads it, while the store would wait for the word's first read (0.3 us
-    // of a short steered call) and moved the tiles of long prompts out of step (8192 tokens of 32 / 8 heads 380 -> 435 us).
-    volatile uint64_t* limit_smem = reinterpret_cast<volatile uint64_t*>(smem + sl.misc + 16);
-    auto limit_ns = [&]() -> uint64_t { return TABLE ? *limit_smem : limit_set; };
+    const int limit_us = TABLE ? p.status[5] : 0;
+    auto limit_ns = [&]() -> uint64_t {
+        if (!TABLE) return limit_set;
+        return limit_us > 0 ? (uint64_t)limit_us * 1000ull : kWaitLimitNs;
+    };
     // steering info is kept in shared memory when it fits (a look-up then costs no trip to the caches): a byte per (sequence,
     // KV head) and a bit per (sequence, key tile)
     const bool info_local = p.steer && p.sched.B * p.sched.Hkv <= G::INFO_HEADS;
@@ -321,7 +326,6 @@ seka_attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
     if (tid == 0) {
         *abort_flag = 0; *reinterpret_cast<volatile float*>(smem + sl.misc + 8) = p.scale_log2;
-        if (TABLE) *limit_smem = limit_set;
     }
     // steering info into shared memory
     if (info_local)

@@ -24,7 +24,7 @@ def test_wait_runs_out_and_the_workspace_recovers(d):
     _wait_runs_out(d, packed=False)
 
 
-# a packed launch looks its limit up in shared memory
+# a packed launch carries its limit as the 32-bit word of the status block
 @pytest.mark.parametrize("d", [128, 64])
 def test_wait_of_a_packed_launch_runs_out(d):
     _wait_runs_out(d, packed=True)
